@@ -363,6 +363,7 @@ scatter_status launch_adjoint_sep(scatter_plan_t p, float* grad, cudaStream_t st
   a.n_mt = p->adj_sep_mt;
   a.partial = p->d.adj_sep_partial;
   a.status = p->d.status;
+  a.flush = kSepFlush;
   dim3 grid((unsigned)(n_mp * p->adj_sep_ntiles), (unsigned)p->adj_sep_chunks);
   timing_begin(p, st);
   const cudaError_t le = sep_launch_core(a, grid, st, p->side_stream, p->side_fork, p->side_join);

@@ -92,7 +92,8 @@ __global__ void k_prep(const double* __restrict__ xyz, const float* __restrict__
                        const int32_t* __restrict__ slot_src, const int32_t* __restrict__ slot_inst,
                        const int64_t* __restrict__ inst_slot_begin, const double* __restrict__ inst_H,
                        const unsigned long long* __restrict__ bbox, double* inst_shift, float4* atom4,
-                       float4* atom_lo, float* atom_w, int64_t n_slots, unsigned* status) {
+                       float4* atom_lo, float* atom_w, int64_t n_slots, unsigned* status, float4* rec_a,
+                       double mid0, double mid1, double mid2) {
   const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (slot >= n_slots) return;
   const int inst = slot_inst[slot];
@@ -111,6 +112,7 @@ __global__ void k_prep(const double* __restrict__ xyz, const float* __restrict__
     atom4[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
     atom_lo[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
     atom_w[slot] = 0.f;
+    if (rec_a) rec_a[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
     return;
   }
   const double* H = inst_H + 3 * inst;
@@ -131,6 +133,7 @@ __global__ void k_prep(const double* __restrict__ xyz, const float* __restrict__
     atom4[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
     atom_lo[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
     atom_w[slot] = 0.f;
+    if (rec_a) rec_a[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
     return;
   }
   c -= rint(c);
@@ -138,6 +141,13 @@ __global__ void k_prep(const double* __restrict__ xyz, const float* __restrict__
   atom4[slot] = make_float4(x0, x1, x2, (float)c);
   atom_lo[slot] = make_float4((float)(r[0] - (double)x0), (float)(r[1] - (double)x1), (float)(r[2] - (double)x2), 0.f);
   atom_w[slot] = w;
+  if (rec_a) {
+    // the folded forward's A record: x' as a double-float and W = w e^{2 pi i (c + (mid - H).x')}
+    const double ph = fma(mid2, r[2], fma(mid1, r[1], fma(mid0, r[0], c)));
+    float sn, cs;
+    sincospif(2.0f * (float)(ph - rint(ph)), &sn, &cs);
+    rec_a[slot] = make_float4(x0, (float)(r[0] - (double)x0), w * cs, w * sn);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -395,7 +405,8 @@ scatter_status launch_prep(scatter_plan_t p, const double* xyz, const float* occ
     const int64_t nb = (p->n_slots + 255) / 256;
     k_prep<<<(unsigned)nb, 256, 0, st>>>(xyz, occ, p->d.slot_src, p->d.slot_inst, p->d.inst_slot_begin,
                                          p->d.inst_H, p->d.inst_bbox, p->d.inst_shift, p->d.atom4,
-                                         p->d.atom_lo, p->d.atom_w, p->n_slots, p->d.status);
+                                         p->d.atom_lo, p->d.atom_w, p->n_slots, p->d.status, p->d.sep_rec,
+                                         p->sep_mid[0], p->sep_mid[1], p->sep_mid[2]);
     p->last_launches += 1;
   }
   return cuda_status(cudaGetLastError(), "prep launch");

@@ -318,6 +318,9 @@ extern "C" void scatter_plan_destroy(scatter_plan_t p) {
   release(d.ftab64);
   release(d.sep_axis_s);
   release(d.sep_axis_lo);
+  release(d.sep_axis_d);
+  release(d.sep_axis_dlo);
+  release(d.sep_rec);
   release(d.sep_virt);
   release(d.batch_inst);
   release(d.batch_items);

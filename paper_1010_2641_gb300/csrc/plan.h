@@ -136,6 +136,9 @@ struct DeviceBuffers {
   double* ftab64 = nullptr;         // the same in FP64 (re, im) for the FP64 kernel
   float* sep_axis_s = nullptr;      // separable grid axes, s = axis - H (virtual for GID)
   float* sep_axis_lo = nullptr;     // their FP32 rounding errors
+  float* sep_axis_d = nullptr;      // folded forward: offsets from the axes' middles [n0 | n1 | n2]
+  float* sep_axis_dlo = nullptr;    // their FP32 rounding errors
+  float4* sep_rec = nullptr;        // folded forward: (x', its rounding error, Re W, Im W) per slot (written by prep)
   float2* sep_virt = nullptr;       // GID: map over the virtual (h, k, 4 beams x alpha_f) grid
   // batches
   BatchInst* batch_inst = nullptr;
@@ -208,6 +211,10 @@ struct scatter_plan_s {
   int64_t sep_n[3] = {0, 0, 0};                  // separable grid shape (GID: n_h, n_k, 4 n_af)
   int64_t sep_ns = 0;
   int32_t sep_n_chunks = 0;
+  bool sep_fold = false, sep_fold_h = false;     // folded over the (k, l) axes' middles, over h's too (sep_common.cuh)
+  int64_t sep_lanes = 0, sep_pairs = 0;          // h values with rows of their own, mirror pairs of (k, l) points
+  int sep_flush = 0;                             // steps between TMEM flushes
+  double sep_mid[3] = {0, 0, 0};                 // the axes' middles - H
   bool sep_form_a = false;                       // A formed inside the CTA-pair kernel, no A table
   float sep_smax[2] = {0.f, 0.f};               // max |s| of the separable grid's b and c axes
   int32_t ap_n_blocks = 0;

@@ -11,6 +11,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <cstdint>
+#include <vector>
 #include "device_common.cuh"
 #include "plan.h"
 
@@ -21,6 +22,9 @@ constexpr int kSepThreads = 32 * (kSepFormWarps + 2);  // + the MMA warp + the c
 constexpr int kSepM = 128;                 // MMA M (rows of A per CTA)
 constexpr int kSepN = 256;                 // MMA N (columns per CTA)
 constexpr int kSepStep = 16;               // K records per pipeline step (K' = 32)
+constexpr int kSepFoldStep = 32;           // the folded forward: one K value per atom, 32 atoms per step
+constexpr int kSepFoldPairs = 128;         // mirror pairs of points per N tile (cos and sin columns each)
+constexpr int kSepFoldRows = 64;           // h values per M tile (two rows each)
 constexpr int kSepFlush = 256;             // steps between TMEM flushes
 constexpr uint32_t kSepABytes = 16384;     // A block of one M tile: hi + lo, 128 x 32 f16 each
 constexpr int kSepPair = 2;                // M tiles per CTA (one formed B tile feeds both)
@@ -132,6 +136,121 @@ __device__ __forceinline__ void sep_a_row(float sa, float sal, bool ok, int ri, 
   split2(v[6], v[7], hi.w, lo.w);
 }
 
+// ---------------------------------------------------------------------------
+// Folded forward: the (k, l) axes symmetric about their middles.
+//
+// A point p = (s_b, s_c) and its mirror p' about the middle (mid_b, mid_c) have
+// the phases +-phi_p around that of the middle, so with X_aj = w_j
+// e^{2 pi i (s_a x'_j + c_j + (mid - H).r'_j)}
+//   A(a, p), A(a, p') = C +- i S,
+//   C = sum_j X_aj cos(2 pi phi_pj),  S = sum_j X_aj sin(2 pi phi_pj):
+// four real sums for two complex values, half the multiply-adds of the direct
+// form (two K values per atom: Re, Im), half the sin/cos of the B formation
+// and half the A table.  The contraction is the same D = A B^T with one K
+// value per atom: rows Re X, Im X, columns cos, sin.
+// Where the h axis is symmetric too (`fold_h`), with W_j = w_j e^{2 pi i (c_j +
+// (mid - H).r'_j)} the rows are W_j cos, W_j sin of the offset d_a from its
+// middle, four rows for the two values a, a' = n0 - 1 - a and one sin/cos for
+// both: C(a), C(a') = Zc +- i Zs, and S likewise.
+//   rows of M tile T, in four blocks of 32 (l = 0 .. 31):
+//     h direct: Re X, Im X of a = 64 T + l, then of a = 64 T + 32 + l
+//     fold_h:   Re W cos, Im W cos, Re W sin, Im W sin of a = 32 T + l
+//     so that one thread forms the four rows of a lane and every store of a
+//     warp covers 512 contiguous bytes, and one thread of the reduction reads
+//     them with no exchange;
+//   columns: groups of 64 pairs, [cos of 64 | sin of 64], so that the two
+//     columns of a pair are stores of one thread and 128 columns (one CTA of
+//     the pair kernel) hold whole pairs.
+// The accumulator loses up to an ulp of its value per MMA (it truncates), so a
+// strong point leaves its error on its mirror: an axis is folded only where
+// its middle is near H (sep_axis_middle), where the mirror of a strong point
+// is a strong point.
+// ---------------------------------------------------------------------------
+__host__ __device__ __forceinline__ int64_t sep_fold_cols(int64_t n_pairs) { return (n_pairs + 63) / 64 * 128; }
+
+// The four rows of one lane over a K block of 8 atoms with records (x', x'
+// rounding error, Re W, Im W): hi[r], lo[r] are the 16-byte core-matrix rows of
+// row block r.  FOLD_H: the offset d[0] + dl[0] from the middle; else the
+// offsets of two h values.  The phase's products are exact before the MUFU
+// sin/cos, as in sep_a_row.  The table kernel and the CTA pair's A warps both
+// form A through it.
+template <bool FOLD_H>
+__device__ __forceinline__ void sep_a_fold(const float (&d)[2], const float (&dl)[2], const bool (&ok)[2],
+                                           const float4* rec, uint4 (&hi)[4], uint4 (&lo)[4]) {
+  uint32_t h[4][4], l[4][4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    float v[4][2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const float4 a = rec[2 * q + u];
+      float sn, cs;
+      dev::sincos_cycles_mufu(dev::frac_of_product2(d[0], dl[0], a.x) + d[0] * a.y, &sn, &cs);
+      if (!ok[0]) sn = cs = 0.f;
+      if (FOLD_H) {
+        v[0][u] = a.z * cs;
+        v[1][u] = a.w * cs;
+        v[2][u] = a.z * sn;
+        v[3][u] = a.w * sn;
+      } else {
+        v[0][u] = fmaf(a.z, cs, -a.w * sn);
+        v[1][u] = fmaf(a.z, sn, a.w * cs);
+        dev::sincos_cycles_mufu(dev::frac_of_product2(d[1], dl[1], a.x) + d[1] * a.y, &sn, &cs);
+        if (!ok[1]) sn = cs = 0.f;
+        v[2][u] = fmaf(a.z, cs, -a.w * sn);
+        v[3][u] = fmaf(a.z, sn, a.w * cs);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) split2(v[r][0], v[r][1], h[r][q], l[r][q]);
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    hi[r] = make_uint4(h[r][0], h[r][1], h[r][2], h[r][3]);
+    lo[r] = make_uint4(l[r][0], l[r][1], l[r][2], l[r][3]);
+  }
+}
+
+// h values of lane l of M tile T (the second one of a folded axis is the mirror)
+__host__ __device__ __forceinline__ int64_t sep_fold_a(int64_t T, int l, int which, int fold_h, int64_t n0) {
+  return fold_h ? (which ? n0 - 1 - (32 * T + l) : 32 * T + l) : 64 * T + 32 * which + l;
+}
+
+// The cos and sin columns of one pair (offsets sb + sbl, sc + scl from the
+// middle) over a K block of 8 atoms (y', z' read), as 16-byte rows.  MODE 0:
+// raw phase, 1: reduced mod 1, 2: exact products, reduced.
+template <int MODE>
+__device__ __forceinline__ void sep_b_fold(float sb, float sc, float sbl, float scl, const float4* at, uint4 (&hi)[2],
+                                           uint4 (&lo)[2]) {
+  uint32_t h[2][4], l[2][4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    float sn[2], cs[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const float4 v = at[2 * q + u];
+      const float ph = MODE == 2 ? dev::frac_rn(dev::frac_product2_plus(sb, sbl, v.y,
+                                                                        dev::frac_product2_plus(sc, scl, v.z, 0.f)))
+                       : MODE == 1 ? dev::frac_rn(fmaf(sb, v.y, sc * v.z))
+                                   : fmaf(sb, v.y, sc * v.z);
+      dev::sincos_cycles_mufu(ph, &sn[u], &cs[u]);
+    }
+    split2(cs[0], cs[1], h[0][q], l[0][q]);
+    split2(sn[0], sn[1], h[1][q], l[1][q]);
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    hi[r] = make_uint4(h[r][0], h[r][1], h[r][2], h[r][3]);
+    lo[r] = make_uint4(l[r][0], l[r][1], l[r][2], l[r][3]);
+  }
+}
+
+// Middle of an axis that may be folded: symmetric about it, |v_i + v_{n-1-i} -
+// 2 mid| below 2e-13 of its largest value (a phase error under 1e-8 cycles for
+// crystals of 1e5 cells at |S| = 1; evenly spaced axes miss by a few ulp), and
+// the middle within a quarter of the axis' half width of H.
+bool sep_axis_middle(const std::vector<double>& v, double H, double* mid);
+
 struct SepArgs {
   const uint4* A;         // A blocks [species][M-tile pair][step][2 tiles][hi|lo] of 16 KB per tile
   int64_t a_sp_stride;    // uint4 per species table of A (0: one table, the forward)
@@ -159,6 +278,13 @@ struct SepArgs {
                           // records (rec_lo, rec_w beside them) instead of streamed from `A`
   const float4* rec_lo;   //   the records' position rounding errors (x' error read)
   const float* rec_w;     //   the atoms' occupancies
+  int fold;               // folded forward: axis_s, axis_lo hold the offsets d from the axes' middles,
+                          // 32 records per step
+  int64_t n_pairs;        //   mirror pairs of (k, l) points
+  int fold_h;             //   the h axis folded too
+  int64_t n_lanes;        //   h values (fold_h: of the axis' first half) that have rows
+  int flush;              // steps between TMEM flushes
+  const float4* rec_a;    //   form_a: A records (x', its rounding error, Re W, Im W)
 };
 
 // Partials in the accumulator's own blocking.  D row m (TMEM lane of its M
@@ -177,11 +303,12 @@ inline int64_t sep_part_floats(int64_t n_mt, int64_t n_cols) {
   return ((n_mt + 1) / 2) * 2 * 128 * ((n_cols + 31) / 32) * 32;
 }
 
-// Accumulation groups: the steps between two TMEM flushes (every kSepFlush
+// Accumulation groups: the steps between two TMEM flushes (every `flush`
 // steps and at the end of the chunk).  Every role walks them identically.
 struct SepGroups {
   int64_t ks_end, grp_start;
-  __device__ bool ends_at(int64_t ks) const { return ks + 1 == ks_end || ks + 1 - grp_start >= kSepFlush; }
+  int flush;
+  __device__ bool ends_at(int64_t ks) const { return ks + 1 == ks_end || ks + 1 - grp_start >= flush; }
   __device__ void advance(int64_t ks) { grp_start = ks + 1; }
 };
 

@@ -138,8 +138,18 @@ __device__ __forceinline__ void commit_pair(uint64_t* bar) {
 // occupancies) instead of the copy warp streaming them from the table (a
 // grid of one N tile, where the table would be written and read once); they
 // wait and signal like the B warps, and take no part in the read-outs.
-template <bool FORM_A>
+// FOLD: the folded forward (sep_common.cuh).  A step is 32 atoms with one K
+// value each instead of 16 with two, and the CTA's 128 columns are the cos and
+// sin columns of 64 mirror pairs of points: per step the same copies, MMAs and
+// sin/cos, for twice the atoms and the same points.  B thread (q, kb) forms
+// both columns of pair q over the K block kb of 8 atoms; an A thread the four
+// rows of one lane over one K block.  Measured on the strained sphere (134,009
+// atoms x 256 x 256 x 64): 6.23 ms direct, 3.08-3.13 ms folded; on 1e6 atoms x
+// 200 x 1 x 200 with the A tiles formed here: 1.06 ms direct, 0.45 ms folded
+// (tensor pipe 73 % active, the formation's latency the rest).
+template <bool FORM_A, bool FOLD>
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(FORM_A ? 112 : 168) k_sep_pair(const SepArgs a) {
+  constexpr int kRec = FOLD ? kSepFoldStep : kSepStep;  // records (atoms or points) per step
   extern __shared__ __align__(1024) unsigned char pair_smem_raw[];
   __shared__ __align__(8) uint64_t bar_ready[kPairAStages];
   __shared__ __align__(8) uint64_t bar_done[kPairAStages];
@@ -147,10 +157,11 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(FORM_A ? 112 : 168) k_sep_
   __shared__ __align__(8) uint64_t bar_tempty[kPairTStages];
   __shared__ __align__(8) uint64_t bar_tread;
   __shared__ __align__(8) uint64_t bar_pfree;
-  __shared__ __align__(16) float4 ring_atom[kPairTStages][kSepStep];
-  // FORM_A: the records' x' errors and occupancies (one unused stage otherwise)
-  __shared__ __align__(16) float4 ring_lo[FORM_A ? kPairTStages : 1][kSepStep];
-  __shared__ __align__(16) float ring_w[FORM_A ? kPairTStages : 1][kSepStep];
+  __shared__ __align__(16) float4 ring_atom[kPairTStages][kRec];
+  // FORM_A: the records' x' errors and occupancies, folded: the A records
+  // (one unused stage otherwise)
+  __shared__ __align__(16) float4 ring_lo[FORM_A ? kPairTStages : 1][kRec];
+  __shared__ __align__(16) float ring_w[FORM_A && !FOLD ? kPairTStages : 1][kSepStep];
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_abort;
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -169,9 +180,9 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(FORM_A ? 112 : 168) k_sep_
   const int64_t mp0 = a.mp_first + 2 * mq;   // the quad's first M-tile pair
   const int chunk = blockIdx.y;
   const int64_t nbc = a.n1 * a.n2;
-  int64_t col_base = nt * kSepN, col_end = nbc;
+  int64_t col_base = nt * kSepN, col_end = FOLD ? sep_fold_cols(a.n_pairs) : nbc;
   int a_species = 0;
-  if (a.ntiles) {
+  if (!FOLD && a.ntiles) {
     const Segment t = a.ntiles[nt];
     col_base = t.begin;
     col_end = t.end;
@@ -205,8 +216,8 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(FORM_A ? 112 : 168) k_sep_
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
 
-  const int64_t ks_begin = a.chunks[chunk].begin / kSepStep, ks_end = a.chunks[chunk].end / kSepStep;
-  SepGroups grp{ks_end, ks_begin};
+  const int64_t ks_begin = a.chunks[chunk].begin / kRec, ks_end = a.chunks[chunk].end / kRec;
+  SepGroups grp{ks_end, ks_begin, FOLD ? a.flush : kSepFlush};
   bool ok = true;
   int64_t a_issued = 0, t_issued = 0, g_committed = 0;
 
@@ -232,15 +243,17 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(FORM_A ? 112 : 168) k_sep_
         if constexpr (FORM_A) {
           // the records, their x' errors and occupancies: the formation warps
           // build the step's A tiles from them
-          dev::mbar_arrive_expect_tx(&bar_atom[tst], kSepStep * (2 * sizeof(float4) + sizeof(float)));
-          dev::bulk_g2s(&ring_atom[tst][0], a.rec + ks * kSepStep, kSepStep * sizeof(float4), &bar_atom[tst]);
-          dev::bulk_g2s(&ring_lo[tst][0], a.rec_lo + ks * kSepStep, kSepStep * sizeof(float4), &bar_atom[tst]);
-          dev::bulk_g2s(&ring_w[tst][0], a.rec_w + ks * kSepStep, kSepStep * sizeof(float), &bar_atom[tst]);
+          dev::mbar_arrive_expect_tx(&bar_atom[tst], kRec * (2 * sizeof(float4) + (FOLD ? 0 : sizeof(float))));
+          dev::bulk_g2s(&ring_atom[tst][0], a.rec + ks * kRec, kRec * sizeof(float4), &bar_atom[tst]);
+          dev::bulk_g2s(&ring_lo[tst][0], (FOLD ? a.rec_a : a.rec_lo) + ks * kRec, kRec * sizeof(float4),
+                        &bar_atom[tst]);
+          if constexpr (!FOLD)
+            dev::bulk_g2s(&ring_w[tst][0], a.rec_w + ks * kSepStep, kSepStep * sizeof(float), &bar_atom[tst]);
           t_issued = g + 1;
           continue;
         }
-        dev::mbar_arrive_expect_tx(&bar_atom[tst], kSepStep * sizeof(float4));
-        dev::bulk_g2s(&ring_atom[tst][0], a.rec + ks * kSepStep, kSepStep * sizeof(float4), &bar_atom[tst]);
+        dev::mbar_arrive_expect_tx(&bar_atom[tst], kRec * sizeof(float4));
+        dev::bulk_g2s(&ring_atom[tst][0], a.rec + ks * kRec, kRec * sizeof(float4), &bar_atom[tst]);
         t_issued = g + 1;
         if (g >= kPairAStages &&
             !dev::mbar_wait_bounded(&bar_done[ast], (uint32_t)(((g - kPairAStages) / kPairAStages) & 1))) {
@@ -335,11 +348,23 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(FORM_A ? 112 : 168) k_sep_
     // m = 2 a + {Re, Im}, and the two lanes of a row pair share
     // X = w e^{2 pi i s_a x'} of their 4 atoms
     const int atid = tid - 32 * (kSepFormWarps + 2);
-    constexpr int kAUnits = 4;
+    // folded: one unit, (tile pair atid / 128, K block, lane of the tile)
+    constexpr int kAUnits = FOLD ? 2 : 4;  // folded: the h values of the thread's rows
     float a_s[kAUnits], a_sl[kAUnits];
     bool a_ok[kAUnits];
+    if constexpr (FOLD) {
+      const int tp = atid >> 7;
+      const int64_t tile = 2 * (mp0 + tp) + (int)rank;
 #pragma unroll
-    for (int i = 0; i < kAUnits; ++i) {
+      for (int i = 0; i < 2; ++i) {
+        const int64_t ah = sep_fold_a(tile, lane, i, a.fold_h, a.n0);
+        a_ok[i] = tp < ntp && (a.fold_h ? 32 * tile + lane < a.n_lanes : ah < a.n_lanes);
+        a_s[i] = a_ok[i] ? a.axis_s[ah] : 0.f;
+        a_sl[i] = a_ok[i] ? a.axis_lo[ah] : 0.f;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kAUnits && !FOLD; ++i) {
       const int unit = i * 256 + atid, tp = unit >> 9, u = unit & 511;
       const int64_t m = (int64_t)(2 * (mp0 + tp) + (int)rank) * kSepM + ((u >> 3) & 15) * 8 + (u & 7);
       const int64_t ah = m >> 1;
@@ -364,9 +389,25 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(FORM_A ? 112 : 168) k_sep_
       // phase s_a x' with its products' rounding errors restored, MUFU
       // sin/cos, the occupancy, rows Re (Xr, -Xi) and Im (Xi, Xr), f16 hi, lo
       const float4* atl = ring_lo[tst];
-      const float* atw = ring_w[tst];
+      const float* atw = ring_w[FOLD ? 0 : tst];
+      if constexpr (FOLD) {
+        const int tp = atid >> 7, kb = (atid >> 5) & 3;
+        if (tp < ntp) {  // the same for the whole warp
+          uint4 hi[4], lo[4];
+          if (a.fold_h)
+            sep_a_fold<true>(a_s, a_sl, a_ok, atl + kb * 8, hi, lo);
+          else
+            sep_a_fold<false>(a_s, a_sl, a_ok, atl + kb * 8, hi, lo);
+          uint4* blk = reinterpret_cast<uint4*>(ringA + (bst * 2 + tp) * kPairTileBytes) + kb * 128 + lane;
 #pragma unroll
-      for (int i = 0; i < kAUnits; ++i) {
+          for (int r = 0; r < 4; ++r) {
+            blk[32 * r] = hi[r];
+            blk[512 + 32 * r] = lo[r];
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < kAUnits && !FOLD; ++i) {
         const int unit = i * 256 + atid, tp = unit >> 9, u = unit & 511;
         if (tp >= ntp) continue;  // the same for the whole warp
         const int kb = u >> 7, ri = u & 1;
@@ -396,13 +437,15 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(FORM_A ? 112 : 168) k_sep_
     // column col of this CTA's half: forward the point (b, c) with offsets
     // (s_b, s_c) from H, adjoint the atom's (y', z'); two threads per column,
     // thread half h forms the step's atoms 8 h .. 8 h + 7 (K blocks 2 h, 2 h + 1)
-    const int c_loc = tid & (kPairHalfN - 1), half = tid / kPairHalfN;
-    const int64_t col = col_base + (int64_t)rank * kPairHalfN + c_loc;
-    const bool row_ok = col < col_end;
+    const int c_loc = FOLD ? tid & 63 : tid & (kPairHalfN - 1), half = FOLD ? tid >> 6 : tid / kPairHalfN;
+    // folded: c_loc is the CTA's mirror pair, col its first point, half the K block
+    const int64_t col = FOLD ? nt * kSepFoldPairs + (int64_t)rank * 64 + c_loc
+                             : col_base + (int64_t)rank * kPairHalfN + c_loc;
+    const bool row_ok = col < (FOLD ? a.n_pairs : col_end);
     float sb, sc, sbl = 0.f, scl = 0.f;  // sbl, scl: low parts of a double-float s (forward)
     float att = 0.f;                     // buried object: 2 pi Im(sigma) of the column's beam
     bool att_over = false;               // an attenuation exponent passed kSepAttMax
-    if (a.ntiles) {
+    if (!FOLD && a.ntiles) {
       const float4 at = row_ok ? a.atom4[col] : make_float4(0.f, 0.f, 0.f, 0.f);
       sb = at.y;
       sc = at.z;
@@ -410,7 +453,7 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(FORM_A ? 112 : 168) k_sep_
       const int64_t rb = row_ok ? col / a.n2 : 0, rc = row_ok ? col % a.n2 : 0;
       sb = a.axis_s[a.n0 + rb];
       sc = a.axis_s[a.n0 + a.n1 + rc];
-      if (a.axis_att) att = a.axis_att[rc];
+      if (!FOLD && a.axis_att) att = a.axis_att[rc];
       if (a.axis_lo) {
         sbl = a.axis_lo[a.n0 + rb];
         scl = a.axis_lo[a.n0 + a.n1 + rc];
@@ -448,6 +491,25 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(FORM_A ? 112 : 168) k_sep_
       }
       unsigned char* sB = ringB + bst * kPairBBytes;
       const float4* at = ring_atom[tst] + half * 8;
+      if constexpr (FOLD) {
+        uint4 hi[2], lo[2];
+        hi[0] = hi[1] = lo[0] = lo[1] = make_uint4(0u, 0u, 0u, 0u);
+        if (row_ok) {
+          if (exact)
+            sep_b_fold<2>(sb, sc, sbl, scl, at, hi, lo);
+          else if (reduce)
+            sep_b_fold<1>(sb, sc, sbl, scl, at, hi, lo);
+          else
+            sep_b_fold<0>(sb, sc, sbl, scl, at, hi, lo);
+        }
+        // columns c_loc (cos) and 64 + c_loc (sin) of the CTA's 128
+        unsigned char* q = sB + half * 2048 + b_row_off;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          *reinterpret_cast<uint4*>(q + u * 1024) = hi[u];
+          *reinterpret_cast<uint4*>(q + 8192 + u * 1024) = lo[u];
+        }
+      } else {
       // mode 0: raw phase, 1: reduced mod 1, 2: exact products, reduced
       // kAtt: a buried object's rows carry exp(-att z')
       auto form = [&](auto mode_tag, auto att_tag) {
@@ -497,6 +559,7 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(FORM_A ? 112 : 168) k_sep_
         form_all(std::true_type{});
       else
         form_all(std::false_type{});
+      }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) {
@@ -589,22 +652,27 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(FORM_A ? 112 : 168) k_sep_
 }
 
 cudaError_t sep_pair_prepare_kernel() {
-  static_assert(kPairSmem + 8192 <= 227 * 1024, "dynamic + static shared memory of k_sep_pair");
-  const cudaError_t e =
-      cudaFuncSetAttribute(k_sep_pair<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem);
-  return e != cudaSuccess
-             ? e
-             : cudaFuncSetAttribute(k_sep_pair<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem);
+  static_assert(kPairSmem + 12288 <= 227 * 1024, "dynamic + static shared memory of k_sep_pair");
+  for (const void* fn : {(const void*)&k_sep_pair<false, false>, (const void*)&k_sep_pair<true, false>,
+                         (const void*)&k_sep_pair<false, true>, (const void*)&k_sep_pair<true, true>}) {
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // Grid: x = 2 CTAs x M quads x N tiles (cluster pairs along x), y = chunks.
 cudaError_t sep_pair_launch_core(const SepArgs& a, int64_t n_nt, int n_chunks, cudaStream_t st) {
   const int64_t n_mq = ((a.mp_count > 0 ? a.mp_count : (a.n_mt + 1) / 2) + 1) / 2;
   dim3 grid((unsigned)(2 * n_mq * n_nt), (unsigned)n_chunks);
-  if (a.form_a)
-    k_sep_pair<true><<<grid, kPairThreadsA, kPairSmem, st>>>(a);
+  if (a.fold && a.form_a)
+    k_sep_pair<true, true><<<grid, kPairThreadsA, kPairSmem, st>>>(a);
+  else if (a.fold)
+    k_sep_pair<false, true><<<grid, kSepThreads, kPairSmem, st>>>(a);
+  else if (a.form_a)
+    k_sep_pair<true, false><<<grid, kPairThreadsA, kPairSmem, st>>>(a);
   else
-    k_sep_pair<false><<<grid, kSepThreads, kPairSmem, st>>>(a);
+    k_sep_pair<false, false><<<grid, kSepThreads, kPairSmem, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -100,6 +100,38 @@ __global__ void k_sep_tab_a(const SepTabArgs t) {
   blk[512 + off] = lo;
 }
 
+// The folded A operand (sep_common.cuh): one thread per (M tile, step, K block
+// of 8 atoms, lane), the lane's four rows; a warp is the 32 lanes of one K
+// block, so the records are broadcast loads and each of the eight stores
+// covers 512 contiguous bytes.  Bound by the table's write: 275 MB in 42 us on the
+// strained sphere (the direct form's k_sep_tab_a: 549 MB in 116 us).
+template <bool FOLD_H>
+__global__ void __launch_bounds__(256) k_sep_tab_fold(const float4* __restrict__ rec_a, const float* __restrict__ axis_d,
+                                                      const float* __restrict__ axis_dlo, int64_t n0, int64_t n_lanes,
+                                                      int64_t n_steps, int64_t n_mt, uint4* __restrict__ A) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n_mt * n_steps * 128) return;  // whole warps
+  const int lane = (int)(i & 31), kb = (int)((i >> 5) & 3);
+  const int64_t ks = (i >> 7) % n_steps, mt = (i >> 7) / n_steps;
+  float d[2], dl[2];
+  bool ok[2];
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    const int64_t ah = sep_fold_a(mt, lane, w, FOLD_H, n0);
+    ok[w] = FOLD_H ? 32 * mt + lane < n_lanes : ah < n_lanes;
+    d[w] = ok[w] ? axis_d[ah] : 0.f;
+    dl[w] = ok[w] ? axis_dlo[ah] : 0.f;
+  }
+  uint4 hi[4], lo[4];
+  sep_a_fold<FOLD_H>(d, dl, ok, rec_a + ks * kSepFoldStep + kb * 8, hi, lo);
+  uint4* blk = A + (((mt >> 1) * n_steps + ks) * kSepPair + (mt & 1)) * (kSepABytes / 16) + kb * 128 + lane;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    blk[32 * r] = hi[r];
+    blk[512 + 32 * r] = lo[r];
+  }
+}
+
 // -------------------------------------------------------------------------
 // main kernel
 // -------------------------------------------------------------------------
@@ -116,7 +148,12 @@ __global__ void k_sep_tab_a(const SepTabArgs t) {
 //   bar_tempty[t] atom records read by the formation   (8 warps)
 //   bar_bfull[b]  B block of a step formed             (8 warps)
 //   bar_tfree     accumulators read out after a group end (8 warps)
+// FOLD: the folded forward (sep_common.cuh): 32 atoms per step, the 256 columns
+// are the cos and sin columns of 128 mirror pairs of points; thread (p, half)
+// forms both columns of pair p over two of the four K blocks.
+template <bool FOLD>
 __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
+  constexpr int kRec = FOLD ? kSepFoldStep : kSepStep;  // records per step
   // a B stage is freed by the done barrier of the step that read it: the A
   // ring (and with it the done ring) must be at least as deep as the B ring
   static_assert(kSepBStages <= kSepAStages, "B-stage reuse is tracked on the done ring");
@@ -127,7 +164,7 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
   __shared__ __align__(8) uint64_t bar_tempty[kSepTStages];
   __shared__ __align__(8) uint64_t bar_bfull[kSepBStages];
   __shared__ __align__(8) uint64_t bar_tfree;
-  __shared__ __align__(16) float4 ring_atom[kSepTStages][kSepStep];
+  __shared__ __align__(16) float4 ring_atom[kSepTStages][kRec];
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_abort;
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -142,9 +179,9 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
   const int chunk = blockIdx.y;
   const int64_t nbc = a.n1 * a.n2;
   // this CTA's columns [col_base, col_end) and the species of its A table
-  int64_t col_base = nt * kSepN, col_end = nbc;
+  int64_t col_base = nt * kSepN, col_end = FOLD ? sep_fold_cols(a.n_pairs) : nbc;
   int a_species = 0;
-  if (a.ntiles) {
+  if (!FOLD && a.ntiles) {
     const Segment t = a.ntiles[nt];
     col_base = t.begin;
     col_end = t.end;
@@ -178,8 +215,8 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
   const uint32_t tmem = tmem_slot;
 
   // the chunk's steps (record bounds on step edges)
-  const int64_t ks_begin = a.chunks[chunk].begin / kSepStep, ks_end = a.chunks[chunk].end / kSepStep;
-  SepGroups grp{ks_end, ks_begin};
+  const int64_t ks_begin = a.chunks[chunk].begin / kRec, ks_end = a.chunks[chunk].end / kRec;
+  SepGroups grp{ks_end, ks_begin, FOLD ? a.flush : kSepFlush};
   bool ok = true;
   // copies issued and MMA steps committed (steps), for the drain on abort
   int64_t a_issued = 0, t_issued = 0, g_committed = 0;
@@ -202,8 +239,8 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
           ok = false;
           break;
         }
-        dev::mbar_arrive_expect_tx(&bar_atom[tst], kSepStep * sizeof(float4));
-        dev::bulk_g2s(&ring_atom[tst][0], a.rec + ks * kSepStep, kSepStep * sizeof(float4), &bar_atom[tst]);
+        dev::mbar_arrive_expect_tx(&bar_atom[tst], kRec * sizeof(float4));
+        dev::bulk_g2s(&ring_atom[tst][0], a.rec + ks * kRec, kRec * sizeof(float4), &bar_atom[tst]);
         t_issued = g + 1;
         if (g >= kSepAStages &&
             !dev::mbar_wait_bounded(&bar_done[ast], (uint32_t)(((g - kSepAStages) / kSepAStages) & 1))) {
@@ -269,12 +306,14 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
     // ---- formation warps ---------------------------------------------------
     // this thread's B row (column col of D): forward the point (b, c) with
     // offsets (s_b, s_c) from H, adjoint the atom's (y', z')
-    const int64_t col = col_base + tid;
-    const bool row_ok = col < col_end;
+    // (folded: the first point of the thread's mirror pair)
+    const int p_loc = tid & (kSepFoldPairs - 1);
+    const int64_t col = FOLD ? nt * kSepFoldPairs + p_loc : col_base + tid;
+    const bool row_ok = col < (FOLD ? a.n_pairs : col_end);
     float sb, sc, sbl = 0.f, scl = 0.f;  // sbl, scl: low parts of a double-float s (forward)
     float att = 0.f;                     // buried object: 2 pi Im(sigma) of the column's beam
     bool att_over = false;               // an attenuation exponent passed kSepAttMax
-    if (a.ntiles) {
+    if (!FOLD && a.ntiles) {
       const float4 at = row_ok ? a.atom4[col] : make_float4(0.f, 0.f, 0.f, 0.f);
       sb = at.y;
       sc = at.z;
@@ -282,13 +321,14 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
       const int64_t rb = row_ok ? col / a.n2 : 0, rc = row_ok ? col % a.n2 : 0;
       sb = a.axis_s[a.n0 + rb];
       sc = a.axis_s[a.n0 + a.n1 + rc];
-      if (a.axis_att) att = a.axis_att[rc];
+      if (!FOLD && a.axis_att) att = a.axis_att[rc];
       if (a.axis_lo) {
         sbl = a.axis_lo[a.n0 + rb];
         scl = a.axis_lo[a.n0 + a.n1 + rc];
       }
     }
-    const uint32_t b_row_off = (uint32_t)((tid >> 3) * 128 + (tid & 7) * 16);
+    const int b_row = FOLD ? (p_loc >> 6) * 128 + (p_loc & 63) : tid;  // folded: the cos column, the sin column 64 on
+    const uint32_t b_row_off = (uint32_t)((b_row >> 3) * 128 + (b_row & 7) * 16);
     // |s_b y' + s_c z' + c| of every B element of this call stays below
     // kSepPhaseLim cycles when the centred extent is small: the exact mod-1
     // reduction is then skipped (MUFU sin/cos of an argument of L cycles errs
@@ -325,6 +365,28 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
       // B[col, k] = e^{2 pi i (s_b y' + s_c z' + c)}, zero past the last column
       unsigned char* sB = ringB + bst * kSepBBytes;
       const float4* at = ring_atom[tst];
+      if constexpr (FOLD) {
+#pragma unroll
+        for (int kq = 0; kq < 2; ++kq) {
+          const int kb = 2 * (tid / kSepFoldPairs) + kq;
+          uint4 hi[2], lo[2];
+          hi[0] = hi[1] = lo[0] = lo[1] = make_uint4(0u, 0u, 0u, 0u);
+          if (row_ok) {
+            if (exact)
+              sep_b_fold<2>(sb, sc, sbl, scl, at + kb * 8, hi, lo);
+            else if (reduce)
+              sep_b_fold<1>(sb, sc, sbl, scl, at + kb * 8, hi, lo);
+            else
+              sep_b_fold<0>(sb, sc, sbl, scl, at + kb * 8, hi, lo);
+          }
+          unsigned char* q = sB + kb * 4096 + b_row_off;
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            *reinterpret_cast<uint4*>(q + u * 1024) = hi[u];
+            *reinterpret_cast<uint4*>(q + 16384 + u * 1024) = lo[u];
+          }
+        }
+      } else {
       // mode 0: raw phase, 1: reduced mod 1, 2: exact products, reduced
       // kAtt: a buried object's rows carry exp(-att z')
       auto form = [&](auto mode_tag, auto att_tag) {
@@ -373,6 +435,7 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
         form_all(std::true_type{});
       else
         form_all(std::false_type{});
+      }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) {
@@ -563,13 +626,230 @@ __global__ void __launch_bounds__(256) k_sep_reduce(const float* __restrict__ pa
   }
 }
 
+struct SepFoldReduceArgs {
+  const float* partial;
+  int64_t chunk_floats, n_cb;
+  const Segment* chunks;
+  int n_chunks;
+  const float* coef;
+  const float2* ftab;
+  float inv4a2;
+  const float* axis_s;   // [n0 | n1 | n2] s = axis - H, and rounding errors
+  const float* axis_lo;
+  int64_t n0, n1, n2, n_pairs, n_lanes;
+  int fold_h;
+  float H[3];
+  const double* shift;
+  int64_t l8_base;       // first block of 8 lanes of this launch
+  float2* out_amp;
+  float* out_int;
+};
+
+// The reduction of the folded forward: per species run of the chunks the
+// eight real sums of every (lane, pair), then their four points (two h values,
+// a point and its mirror) with f_s at each point's own |S|, and at the end the
+// centring phase and |A|^2.  A thread holds one lane's rows and four pairs:
+// rows l % 8 and quad l / 8 of pairs, so a read covers 128 contiguous bytes
+// per quad, and the four row blocks and the two columns of a pair (blocks of
+// the partials that the same thread reads) combine with no exchange.  GROUPS threads share a quadruple's chunks on small maps and meet
+// in shared memory in a fixed order (a 16-value row range of the strained
+// sphere's map: 21.5 us with one thread per quadruple, 12.7 us with four).
+template <int GROUPS>
+__global__ void __launch_bounds__(256) k_sep_reduce_fold(const SepFoldReduceArgs a) {
+  constexpr int kCols = 256 / GROUPS;  // threads over (alpha, quad)
+  __shared__ float sh_t[3];
+  __shared__ int sh_shifted;
+  __shared__ float sh_v[GROUPS > 1 ? GROUPS - 1 : 1][GROUPS > 1 ? 32 : 1][GROUPS > 1 ? kCols : 1];
+  if (threadIdx.x == 0) {
+    sh_t[0] = (float)a.shift[0];
+    sh_t[1] = (float)a.shift[1];
+    sh_t[2] = (float)a.shift[2];
+    sh_shifted = a.shift[0] != 0.0 || a.shift[1] != 0.0 || a.shift[2] != 0.0;
+  }
+  const int t = threadIdx.x % kCols, grp = threadIdx.x / kCols;
+  const int64_t lg = (a.l8_base + blockIdx.y) * 8 + (t & 7);  // lane of the map: 32 per M tile
+  const int64_t p0 = ((int64_t)blockIdx.x * (kCols / 8) + (t >> 3)) * 4;
+  const int64_t ncols = a.n1 * a.n2, n_s = a.n0 * ncols;
+  int64_t ia[2];
+  bool a_ok[2];
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    ia[w] = sep_fold_a(lg >> 5, (int)(lg & 31), w, a.fold_h, a.n0);
+    a_ok[w] = a.fold_h ? lg < a.n_lanes && (w == 0 || ia[1] != ia[0]) : ia[w] < a.n_lanes;
+    if (!a_ok[w]) ia[w] = 0;
+  }
+  const bool l_ok = a_ok[0] || a_ok[1];
+  // |S|^2 parts in FP32 (S = H + s): of the two h values, of the points p and p'
+  float h2[2], q2[4][2];
+  auto s_of = [&](int64_t i, int d) { return a.H[d] + (a.axis_s[i] + a.axis_lo[i]); };
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const float x = s_of(ia[u], 0);
+    h2[u] = x * x;
+  }
+  bool p_ok[4];
+  int64_t pt[4][2];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    p_ok[j] = l_ok && p0 + j < a.n_pairs;
+    pt[j][0] = p_ok[j] ? p0 + j : 0;
+    pt[j][1] = ncols - 1 - pt[j][0];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const float y = s_of(a.n0 + pt[j][u] / a.n2, 1), z = s_of(a.n0 + a.n1 + pt[j][u] % a.n2, 2);
+      q2[j][u] = y * y + z * z;
+    }
+  }
+  // block (row block r, cos | sin) of this thread's lane and pairs: the M tile
+  // lg / 32 has four consecutive 32-row blocks, the pair group p0 / 64 its cos
+  // and sin columns in two pairs of 32-column blocks
+  const int64_t c = (p0 >> 6) * 128 + (p0 & 63);
+  const bool in = l_ok && p0 < (a.n_pairs + 63) / 64 * 64;
+  const float* base = a.partial + sep_part_off((lg >> 5) * 128 + (lg & 31), c, a.n_cb);
+  const int64_t r_off = a.n_cb * 1024, s_off = 2 * 1024;
+  float2 v[4][4];  // [pair][first h value: p, p' | second: p, p']
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[j][k] = make_float2(0.f, 0.f);
+  float4 z[4][2];
+  auto zero = [&]() {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) z[r][0] = z[r][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  zero();
+  const int per = (a.n_chunks + GROUPS - 1) / GROUPS;
+  const int c_lo = grp * per, c_hi = min(a.n_chunks, c_lo + per);
+  for (int ch = c_lo; ch < c_hi; ++ch) {
+    const int sp = a.chunks[ch].species;
+    if (in) {
+      const float* q = base + (int64_t)ch * a.chunk_floats;
+      float4 x[4][2];
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int y = 0; y < 2; ++y) x[r][y] = __ldcs(reinterpret_cast<const float4*>(q + r * r_off + y * s_off));
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+          z[r][y].x += x[r][y].x;
+          z[r][y].y += x[r][y].y;
+          z[r][y].z += x[r][y].z;
+          z[r][y].w += x[r][y].w;
+        }
+    }
+    if (ch + 1 < c_hi && a.chunks[ch + 1].species == sp) continue;  // uniform over the group
+    const float* cf = a.coef + kNCoef * sp;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      auto e = [&](const float4& f) { return j == 0 ? f.x : j == 1 ? f.y : j == 2 ? f.z : f.w; };
+      // C and S of the two h values
+      float cr[2], ci[2], sr[2], si[2];
+      const float c0 = e(z[0][0]), c1 = e(z[1][0]), c2 = e(z[2][0]), c3 = e(z[3][0]);
+      const float s0 = e(z[0][1]), s1 = e(z[1][1]), s2 = e(z[2][1]), s3 = e(z[3][1]);
+      cr[0] = a.fold_h ? c0 - c3 : c0;
+      ci[0] = a.fold_h ? c1 + c2 : c1;
+      cr[1] = a.fold_h ? c0 + c3 : c2;
+      ci[1] = a.fold_h ? c1 - c2 : c3;
+      sr[0] = a.fold_h ? s0 - s3 : s0;
+      si[0] = a.fold_h ? s1 + s2 : s1;
+      sr[1] = a.fold_h ? s0 + s3 : s2;
+      si[1] = a.fold_h ? s1 - s2 : s3;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        // p runs over the first half of the points, whose offsets are the formed ones: C + i S, its mirror C - i S
+        const int w = k >> 1;
+        const float re = k & 1 ? cr[w] + si[w] : cr[w] - si[w];
+        const float im = k & 1 ? ci[w] - sr[w] : ci[w] + sr[w];
+        const float2 F = a.ftab ? (p_ok[j] ? a.ftab[(int64_t)sp * n_s + ia[k >> 1] * ncols + pt[j][k & 1]]
+                                           : make_float2(0.f, 0.f))
+                                : dev::form_factor(cf, (h2[k >> 1] + q2[j][k & 1]) * a.inv4a2);
+        v[j][k].x += F.x * re - F.y * im;
+        v[j][k].y += F.x * im + F.y * re;
+      }
+    }
+    zero();
+  }
+  __syncthreads();  // sh_t; and before the groups' exchange
+  if constexpr (GROUPS > 1) {
+    if (grp > 0) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          sh_v[grp - 1][8 * j + 2 * k][t] = v[j][k].x;
+          sh_v[grp - 1][8 * j + 2 * k + 1][t] = v[j][k].y;
+        }
+    }
+    __syncthreads();
+    if (grp > 0) return;
+    for (int g = 0; g < GROUPS - 1; ++g)
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          v[j][k].x += sh_v[g][8 * j + 2 * k][t];
+          v[j][k].y += sh_v[g][8 * j + 2 * k + 1][t];
+        }
+  }
+  if (!l_ok) return;
+  if (sh_shifted) {
+    // e^{2 pi i s.t}: the products' fractional parts per axis value
+    float fh[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) fh[u] = dev::frac_of_product2(a.axis_s[ia[u]], a.axis_lo[ia[u]], sh_t[0]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int64_t iy = a.n0 + pt[j][u] / a.n2, iz = a.n0 + a.n1 + pt[j][u] % a.n2;
+        const float fy = dev::frac_of_product2(a.axis_s[iy], a.axis_lo[iy], sh_t[1]);
+        const float fz = dev::frac_of_product2(a.axis_s[iz], a.axis_lo[iz], sh_t[2]);
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+          float sn, cs;
+          sincospif(2.0f * dev::frac_rn(fh[w] + fy + fz), &sn, &cs);
+          v[j][2 * w + u] = dev::cmul(make_float2(cs, sn), v[j][2 * w + u]);
+        }
+      }
+  }
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    if (!a_ok[w]) continue;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        if (!p_ok[j] || (u == 1 && pt[j][1] == pt[j][0])) continue;  // the middle point of an odd plane
+        const int64_t m = ia[w] * ncols + pt[j][u];
+        const float2 x = v[j][2 * w + u];
+        if (a.out_amp) a.out_amp[m] = x;
+        if (a.out_int) a.out_int[m] = x.x * x.x + x.y * x.y;
+      }
+  }
+}
+
 // -------------------------------------------------------------------------
 // host side
 // -------------------------------------------------------------------------
 
+bool sep_axis_middle(const std::vector<double>& v, double H, double* mid) {
+  if (v.empty()) return false;
+  double top = 1.0;
+  for (double x : v) top = std::max(top, std::fabs(x));
+  const size_t n = v.size();
+  *mid = 0.5 * (v.front() + v.back());
+  for (size_t i = 0; i < n; ++i)
+    if (std::fabs(v[i] + v[n - 1 - i] - 2.0 * *mid) > 2e-13 * top) return false;
+  return std::fabs(*mid - H) <= 0.125 * std::fabs(v.back() - v.front()) + 2e-13 * top || n == 1;
+}
+
 cudaError_t sep_prepare_kernel() {
-  static_assert(kSepSmem + 4096 <= 227 * 1024, "dynamic + static shared memory of k_sep");
-  const cudaError_t e = cudaFuncSetAttribute(k_sep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSepSmem);
+  static_assert(kSepSmem + 8192 <= 227 * 1024, "dynamic + static shared memory of k_sep");
+  cudaError_t e = cudaFuncSetAttribute(k_sep<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSepSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_sep<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSepSmem);
   return e != cudaSuccess ? e : sep_pair_prepare_kernel();
 }
 
@@ -579,13 +859,20 @@ cudaError_t sep_prepare_kernel() {
 // accumulator tile would form all of its B columns for half the MMA work),
 // on the side stream where one is given, so that its CTAs take the SMs the
 // pair kernel's last clusters leave idle.
+static void launch_one_cta(const SepArgs& a, dim3 grid, cudaStream_t st) {
+  if (a.fold)
+    k_sep<true><<<grid, kSepThreads, kSepSmem, st>>>(a);
+  else
+    k_sep<false><<<grid, kSepThreads, kSepSmem, st>>>(a);
+}
+
 cudaError_t sep_launch_core(const SepArgs& a, dim3 grid, cudaStream_t st, cudaStream_t side, cudaEvent_t fork,
                             cudaEvent_t join) {
   const int64_t n_mp = (a.n_mt + 1) / 2;
   const int64_t n_nt = (int64_t)grid.x / n_mp;
   const int64_t n_even = n_mp & ~int64_t(1);
   if (!sep_pair_enabled() || n_even == 0) {
-    k_sep<<<grid, kSepThreads, kSepSmem, st>>>(a);
+    launch_one_cta(a, grid, st);
     return cudaGetLastError();
   }
   SepArgs pa = a;
@@ -602,7 +889,7 @@ cudaError_t sep_launch_core(const SepArgs& a, dim3 grid, cudaStream_t st, cudaSt
   e = sep_pair_launch_core(pa, n_nt, (int)grid.y, st);
   if (split) {
     if (e == cudaSuccess) {
-      k_sep<<<dim3((unsigned)n_nt, grid.y), kSepThreads, kSepSmem, beside ? side : st>>>(sa);
+      launch_one_cta(sa, dim3((unsigned)n_nt, grid.y), beside ? side : st);
       e = cudaGetLastError();
     }
     if (beside) {  // join even after a failed launch: a capture needs the side stream back
@@ -632,15 +919,23 @@ int sep_core_launches(int64_t n_mt) {
 
 namespace {
 
-int sep_best_split(const scatter_plan_s* p, int64_t tiles) {
+// Smallest crystal (atom slots) whose map is folded: AUTO's own line below
+// which a grid is not sent to the tensor cores, a few hundred steps of atoms
+// bound by fixed costs that the fold does not change.
+constexpr int64_t kSepFoldMinSlots = 4096;
+
+// Atom chunks (split over K) of `steps` steps in all that minimise the waves
+// of CTAs x steps per CTA, each chunk at least min_steps long; *cost_out in
+// steps.
+int sep_best_split(const scatter_plan_s* p, int64_t tiles, int64_t n_steps, double min_steps, double* cost_out) {
   const double cap = (double)p->n_sm;  // one CTA per SM (TMEM + shared memory)
-  const double steps = (double)std::max<int64_t>(p->n_slots / kSepStep, 1);
+  const double steps = (double)std::max<int64_t>(n_steps, 1);
   double best = 1e300;
   int best_k = 1;
   // up to two chunks per SM: a grid of one N tile and one M quad (a few
   // columns, a long atom list) needs ~n_sm / 2 chunks to give every SM a CTA
   for (int k = 1; k <= 2 * p->n_sm; ++k) {
-    if (k > 1 && steps / k < 64) break;
+    if (k > 1 && steps / k < min_steps) break;
     // one step ~1 us of MMA; an extra chunk costs one partial of the
     // map (8 B per point written once, read once by the reduction)
     const double part_steps = 16.0 * (double)p->sep_ns / 6.0e12 / 1.0e-6;
@@ -650,6 +945,7 @@ int sep_best_split(const scatter_plan_s* p, int64_t tiles) {
       best_k = k;
     }
   }
+  *cost_out = best;
   return best_k;
 }
 
@@ -701,16 +997,68 @@ scatter_status prepare_separable(scatter_plan_s* p, int split_override) {
     }
   }
   p->sep_ns = p->sep_n[0] * p->sep_n[1] * p->sep_n[2];
+  // The direct form's tiles and chunks
+  const int64_t steps_d = p->n_slots / kSepStep, nbc = p->sep_n[1] * p->sep_n[2];
+  const int64_t mt_d = (2 * p->sep_n[0] + kSepM - 1) / kSepM;
+  double cost_d = 0.0, cost_f = 0.0;
+  int split = split_override > 0 ? split_override
+                                 : sep_best_split(p, (mt_d + 1) / 2 * ((nbc + kSepN - 1) / kSepN), steps_d, 64.0, &cost_d);
+  p->sep_flush = kSepFlush;
+  // Fold where the (k, l) axes are symmetric (evenly spaced axes) and the
+  // crystal has at least kSepFoldMinSlots slots.  Not on grazing incidence:
+  // near the critical angle the four beams nearly cancel, and the errors of a
+  // point and its mirror (opposite beams), one sum's in the fold, no longer
+  // cancel with them (2-3 times the direct form's scatter on some maps).  The
+  // accumulators' truncation grows with the steps of a group, so the fold
+  // keeps 7/8 of the direct form's group length (its chunks are at least 0.8
+  // of that form's groups long), which keeps the error of the map where the
+  // direct form has it; it is taken where that leaves it the cheaper form by
+  // the cost model.
+  double mid[3] = {0, 0, 0};
+  p->sep_fold = !gid && p->n_slots >= kSepFoldMinSlots && p->n_slots % kSepFoldStep == 0 &&
+                sep_axis_middle(ax64[1], p->inst[0].H[1], &mid[1]) && sep_axis_middle(ax64[2], p->inst[0].H[2], &mid[2]);
+  if (p->sep_fold) {
+    p->sep_fold_h = sep_axis_middle(ax64[0], p->inst[0].H[0], &mid[0]);
+    p->sep_lanes = p->sep_fold_h ? (p->sep_n[0] + 1) / 2 : p->sep_n[0];
+    p->sep_pairs = (nbc + 1) / 2;
+    const int64_t mt_f = p->sep_fold_h ? (p->sep_lanes + 31) / 32 : (p->sep_lanes + kSepFoldRows - 1) / kSepFoldRows;
+    const int64_t nt_f = (sep_fold_cols(p->sep_pairs) + kSepN - 1) / kSepN;
+    const double group = std::min<double>(kSepFlush, (double)((steps_d + split - 1) / split));
+    if (split_override <= 0) {
+      const int split_f =
+          sep_best_split(p, (mt_f + 1) / 2 * nt_f, p->n_slots / kSepFoldStep, 0.8 * group, &cost_f);
+      p->sep_fold = cost_f < 0.95 * cost_d && (double)(p->n_slots / kSepFoldStep) >= 0.8 * group;
+      if (p->sep_fold) split = split_f;
+    }
+    if (p->sep_fold) p->sep_flush = std::max(1, (int)(0.875 * group));
+  }
+  std::vector<float> dvals, dvals_lo;
+  if (p->sep_fold) {
+    for (int d = 0; d < 3; ++d) {
+      const bool fold_d = d > 0 || p->sep_fold_h;
+      if (!fold_d) mid[d] = p->inst[0].H[d];  // an h axis that is not folded: offsets from H
+      p->sep_mid[d] = mid[d] - p->inst[0].H[d];
+      const size_t n = ax64[d].size();
+      for (size_t i = 0; i < n; ++i) {
+        const double dv = fold_d ? 0.5 * (ax64[d][i] - ax64[d][n - 1 - i]) : ax64[d][i] - mid[d];
+        dvals.push_back((float)dv);
+        dvals_lo.push_back((float)(dv - (double)(float)dv));
+      }
+    }
+  }
+  const std::vector<float>& form = p->sep_fold ? dvals : alls;  // offsets that the kernels form phases from
   p->sep_smax[0] = p->sep_smax[1] = 0.f;
   for (int64_t i = 0; i < p->sep_n[1]; ++i)
-    p->sep_smax[0] = std::max(p->sep_smax[0], std::fabs(alls[p->sep_n[0] + i]));
+    p->sep_smax[0] = std::max(p->sep_smax[0], std::fabs(form[p->sep_n[0] + i]));
   for (int64_t i = 0; i < p->sep_n[2]; ++i)
-    p->sep_smax[1] = std::max(p->sep_smax[1], std::fabs(alls[p->sep_n[0] + p->sep_n[1] + i]));
-  const int64_t n_steps = p->n_slots / kSepStep;
-  const int64_t n_mt = (2 * p->sep_n[0] + kSepM - 1) / kSepM;
-  const int64_t n_nt = (p->sep_n[1] * p->sep_n[2] + kSepN - 1) / kSepN;
+    p->sep_smax[1] = std::max(p->sep_smax[1], std::fabs(form[p->sep_n[0] + p->sep_n[1] + i]));
+  const int step = p->sep_fold ? kSepFoldStep : kSepStep;
+  const int64_t n_steps = p->n_slots / step;
+  const int64_t n_mt = !p->sep_fold ? mt_d : p->sep_fold_h ? (p->sep_lanes + 31) / 32
+                                                           : (p->sep_lanes + kSepFoldRows - 1) / kSepFoldRows;
+  const int64_t n_cols = p->sep_fold ? sep_fold_cols(p->sep_pairs) : nbc;
+  const int64_t n_nt = (n_cols + kSepN - 1) / kSepN;
   const int64_t n_mp = (n_mt + 1) / 2;
-  const int split = split_override > 0 ? split_override : sep_best_split(p, n_mp * n_nt);
   Tiling t;
   t.threads = 256;
   t.R = 8;
@@ -740,19 +1088,19 @@ scatter_status prepare_separable(scatter_plan_s* p, int split_override) {
   std::vector<Segment> chunks;
   int64_t total_steps = 0;
   for (const Segment& sg : p->all_segs)
-    if (sg.instance == 0 && sg.end > sg.begin) total_steps += (sg.end - sg.begin) / kSepStep;
+    if (sg.instance == 0 && sg.end > sg.begin) total_steps += (sg.end - sg.begin) / step;
   for (const Segment& sg : p->all_segs) {
     if (sg.instance != 0 || sg.end <= sg.begin) continue;
-    const int64_t steps = (sg.end - sg.begin) / kSepStep;
+    const int64_t steps = (sg.end - sg.begin) / step;
     const int64_t k = std::max<int64_t>(1, std::llround((double)split * (double)steps / (double)total_steps));
     const int64_t per = (steps + k - 1) / k;
     for (int64_t b = 0; b < steps; b += per)
-      chunks.push_back(Segment{sg.begin + b * kSepStep, sg.begin + std::min(steps, b + per) * kSepStep, sg.species, 0});
+      chunks.push_back(Segment{sg.begin + b * step, sg.begin + std::min(steps, b + per) * step, sg.species, 0});
   }
   if (chunks.empty()) chunks.push_back(Segment{0, 0, 0, 0});  // no atoms: one empty chunk, zero partials
   p->sep_n_chunks = (int32_t)chunks.size();
   const size_t part_bytes =
-      (size_t)p->sep_n_chunks * (size_t)sep_part_floats(n_mt, p->sep_n[1] * p->sep_n[2]) * sizeof(float);
+      (size_t)p->sep_n_chunks * (size_t)sep_part_floats(n_mt, n_cols) * sizeof(float);
   const size_t chunk_bytes = chunks.size() * sizeof(Segment);
   if (a_bytes) {
     if ((e = cudaMalloc(&p->d.sep_A, a_bytes)) != cudaSuccess) return cuda_status(e, "cudaMalloc separable A");
@@ -768,6 +1116,16 @@ scatter_status prepare_separable(scatter_plan_s* p, int split_override) {
   if ((e = cudaMalloc(&p->d.sep_axis_lo, alls_lo.size() * sizeof(float))) != cudaSuccess) return cuda_status(e, "axes");
   cudaMemcpy(p->d.sep_axis_s, alls.data(), alls.size() * sizeof(float), cudaMemcpyHostToDevice);
   cudaMemcpy(p->d.sep_axis_lo, alls_lo.data(), alls_lo.size() * sizeof(float), cudaMemcpyHostToDevice);
+  size_t fold_bytes = 0;
+  if (p->sep_fold) {
+    const size_t rb = (size_t)p->n_slots * sizeof(float4), db = dvals.size() * sizeof(float);
+    if ((e = cudaMalloc(&p->d.sep_rec, rb)) != cudaSuccess) return cuda_status(e, "cudaMalloc folded records");
+    if ((e = cudaMalloc(&p->d.sep_axis_d, db)) != cudaSuccess) return cuda_status(e, "folded axes");
+    if ((e = cudaMalloc(&p->d.sep_axis_dlo, db)) != cudaSuccess) return cuda_status(e, "folded axes");
+    cudaMemcpy(p->d.sep_axis_d, dvals.data(), db, cudaMemcpyHostToDevice);
+    cudaMemcpy(p->d.sep_axis_dlo, dvals_lo.data(), db, cudaMemcpyHostToDevice);
+    fold_bytes = rb + 2 * db;
+  }
   size_t virt_bytes = 0;
   if (gid) {
     virt_bytes = (size_t)p->sep_ns * sizeof(float2);
@@ -781,7 +1139,7 @@ scatter_status prepare_separable(scatter_plan_s* p, int split_override) {
     cudaMemcpy(p->d.sep_szf, szf.data(), tb, cudaMemcpyHostToDevice);
     virt_bytes += 2 * tb;
   }
-  p->base_bytes += (int64_t)(a_bytes + part_bytes + chunk_bytes + virt_bytes);
+  p->base_bytes += (int64_t)(a_bytes + part_bytes + chunk_bytes + virt_bytes + fold_bytes);
   if ((e = sep_prepare_kernel()) != cudaSuccess) return cuda_status(e, "separable shared memory attribute");
   return sep_prepare_side(p, n_mt);
 }
@@ -801,7 +1159,13 @@ scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_ou
   t.n_mt = p->sep_mt;
   t.A = static_cast<uint4*>(p->d.sep_A);
   const int n_chunks = p->sep_n_chunks;
-  if (p->n_slots > 0 && !p->sep_form_a) {
+  if (p->sep_fold && !p->sep_form_a) {
+    const int64_t na = p->sep_mt * p->sep_steps * 128;
+    const auto kernel = p->sep_fold_h ? k_sep_tab_fold<true> : k_sep_tab_fold<false>;
+    kernel<<<(unsigned)((na + 255) / 256), 256, 0, st>>>(p->d.sep_rec, p->d.sep_axis_d, p->d.sep_axis_dlo, p->sep_n[0],
+                                                         p->sep_lanes, p->sep_steps, p->sep_mt, t.A);
+    p->last_launches += 1;
+  } else if (p->n_slots > 0 && !p->sep_form_a) {
     const int64_t na = p->sep_mt * p->sep_steps * 4 * kSepM;  // real tiles; a padding tile is never read
     k_sep_tab_a<<<(unsigned)((na + 255) / 256), 256, 0, st>>>(t);
     p->last_launches += 1;
@@ -816,13 +1180,20 @@ scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_ou
   a.shift = p->d.inst_shift;
   a.smax_b = p->sep_smax[0];
   a.smax_c = p->sep_smax[1];
-  a.axis_s = p->d.sep_axis_s;
-  a.axis_lo = p->d.sep_axis_lo;
+  const int64_t n_cols = p->sep_fold ? sep_fold_cols(p->sep_pairs) : p->sep_n[1] * p->sep_n[2];
+  a.axis_s = p->sep_fold ? p->d.sep_axis_d : p->d.sep_axis_s;
+  a.axis_lo = p->sep_fold ? p->d.sep_axis_dlo : p->d.sep_axis_lo;
   a.n0 = p->sep_n[0];
   a.n1 = p->sep_n[1];
   a.n2 = p->sep_n[2];
-  a.n_cb = (p->sep_n[1] * p->sep_n[2] + 31) / 32;
-  a.chunk_floats = sep_part_floats(p->sep_mt, p->sep_n[1] * p->sep_n[2]);
+  a.n_cb = (n_cols + 31) / 32;
+  a.chunk_floats = sep_part_floats(p->sep_mt, n_cols);
+  a.fold = p->sep_fold ? 1 : 0;
+  a.n_pairs = p->sep_pairs;
+  a.n_lanes = p->sep_lanes;
+  a.fold_h = p->sep_fold_h ? 1 : 0;
+  a.flush = p->sep_flush;
+  a.rec_a = p->d.sep_rec;
   a.n_steps = p->sep_steps;
   a.n_mt = p->sep_mt;
   a.partial = p->d.sep_partial;
@@ -838,31 +1209,85 @@ scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_ou
   if (le != cudaSuccess) return cuda_status(le, "separable kernel launch");
   p->last_launches += sep_core_launches(p->sep_mt);
   const bool gid = p->s_kind == SCATTER_S_GID_GRID;
-  const int64_t n_cb = (p->sep_n[1] * p->sep_n[2] + 31) / 32;
-  const int64_t n_bm = (2 * p->sep_n[0] + 31) / 32;  // 32-row blocks holding map rows
+  const int64_t n_cb = a.n_cb, ncols = p->sep_n[1] * p->sep_n[2];
+  // row blocks of the reduction: 16 h values (32 partial rows); folded 8 lanes, 32 per
+  // M tile: the h values of a tile's second half (or their mirrors) with those of its first
+  const int64_t n_bm = !p->sep_fold ? (2 * p->sep_n[0] + 31) / 32
+                       : p->sep_fold_h ? (p->sep_lanes + 7) / 8 : 4 * p->sep_mt;
   // a host call copies each row range to the host while the next is reduced
   const bool pieces = p->host_out && !gid;
   const int n_pieces = pieces ? (int)std::min<int64_t>(kHostPieces, n_bm) : 1;
-  const int64_t ncols = p->sep_n[1] * p->sep_n[2];
+  float2* amp_dst = gid ? p->d.sep_virt : amp_out;
+  float* int_dst = gid ? nullptr : int_out;
   for (int k = 0; k < n_pieces; ++k) {
     const int64_t b0 = n_bm * k / n_pieces, b1 = n_bm * (k + 1) / n_pieces;
-    const dim3 rgrid((unsigned)n_cb, (unsigned)(b1 - b0));
-    k_sep_reduce<<<rgrid, 256, 0, st>>>(
-        p->d.sep_partial, sep_part_floats(p->sep_mt, ncols), n_cb, p->d.sep_chunks, n_chunks, p->d.coef, p->d.ftab,
-        (float)(1.0 / (4.0 * p->lattice_a * p->lattice_a)), p->d.sep_axis_s, p->d.sep_axis_lo, p->sep_n[0],
-        p->sep_n[1], p->sep_n[2],
-        make_float3((float)p->inst[0].H[0], (float)p->inst[0].H[1], (float)p->inst[0].H[2]), p->d.inst_shift,
-        p->d.sep_att, p->d.sep_szf, b0, gid ? p->d.sep_virt : amp_out, gid ? nullptr : int_out);
+    if (p->sep_fold) {
+      SepFoldReduceArgs r{};
+      r.partial = p->d.sep_partial;
+      r.chunk_floats = a.chunk_floats;
+      r.n_cb = n_cb;
+      r.chunks = p->d.sep_chunks;
+      r.n_chunks = n_chunks;
+      r.coef = p->d.coef;
+      r.ftab = p->d.ftab;
+      r.inv4a2 = (float)(1.0 / (4.0 * p->lattice_a * p->lattice_a));
+      r.axis_s = p->d.sep_axis_s;
+      r.axis_lo = p->d.sep_axis_lo;
+      r.n0 = p->sep_n[0];
+      r.n1 = p->sep_n[1];
+      r.n2 = p->sep_n[2];
+      r.n_pairs = p->sep_pairs;
+      r.n_lanes = p->sep_lanes;
+      r.fold_h = p->sep_fold_h ? 1 : 0;
+      for (int d = 0; d < 3; ++d) r.H[d] = (float)p->inst[0].H[d];
+      r.shift = p->d.inst_shift;
+      r.l8_base = b0;
+      r.out_amp = amp_dst;
+      r.out_int = int_dst;
+      // small launches (a row range of a host call, a small map of a large crystal):
+      // several threads share each quadruple's chunks until the launch has two
+      // CTAs per SM
+      const int64_t quads = (p->sep_pairs + 3) / 4, want = 2 * (int64_t)p->n_sm;
+      int groups = 1;
+      while (groups < 8 && 2 * groups <= n_chunks && (quads + 31) / 32 * (b1 - b0) * groups < want) groups *= 2;
+      const auto kernel = groups == 1   ? k_sep_reduce_fold<1>
+                          : groups == 2 ? k_sep_reduce_fold<2>
+                          : groups == 4 ? k_sep_reduce_fold<4>
+                                        : k_sep_reduce_fold<8>;
+      const int64_t per_cta = 32 / groups;  // quads per CTA
+      kernel<<<dim3((unsigned)((quads + per_cta - 1) / per_cta), (unsigned)(b1 - b0)), 256, 0, st>>>(r);
+    } else {
+      const dim3 rgrid((unsigned)n_cb, (unsigned)(b1 - b0));
+      k_sep_reduce<<<rgrid, 256, 0, st>>>(
+          p->d.sep_partial, a.chunk_floats, n_cb, p->d.sep_chunks, n_chunks, p->d.coef, p->d.ftab,
+          (float)(1.0 / (4.0 * p->lattice_a * p->lattice_a)), p->d.sep_axis_s, p->d.sep_axis_lo, p->sep_n[0],
+          p->sep_n[1], p->sep_n[2],
+          make_float3((float)p->inst[0].H[0], (float)p->inst[0].H[1], (float)p->inst[0].H[2]), p->d.inst_shift,
+          p->d.sep_att, p->d.sep_szf, b0, amp_dst, int_dst);
+    }
     p->last_launches += 1;
     if (pieces) {
-      // h rows 16 b0 .. 16 b1 of the map: a contiguous range of points
-      const int64_t m0 = std::min<int64_t>(16 * b0, p->sep_n[0]) * ncols;
-      const int64_t m1 = std::min<int64_t>(16 * b1, p->sep_n[0]) * ncols;
+      const int64_t n0 = p->sep_n[0];
       cudaError_t e = cudaEventRecord(p->copy_ev[k], st);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(p->copy_stream, p->copy_ev[k], 0);
-      if (e == cudaSuccess && m1 > m0)
-        e = cudaMemcpyAsync(static_cast<float2*>(p->host_out) + m0, amp_out + m0, (size_t)(m1 - m0) * sizeof(float2),
-                            cudaMemcpyDeviceToHost, p->copy_stream);
+      auto copy_rows = [&](int64_t r0, int64_t r1) {
+        r1 = std::min(r1, n0);
+        if (e == cudaSuccess && r1 > r0)
+          e = cudaMemcpyAsync(static_cast<float2*>(p->host_out) + r0 * ncols, amp_out + r0 * ncols,
+                              (size_t)((r1 - r0) * ncols) * sizeof(float2), cudaMemcpyDeviceToHost, p->copy_stream);
+      };
+      if (!p->sep_fold) {
+        copy_rows(16 * b0, 16 * b1);
+      } else if (p->sep_fold_h) {
+        // h rows 8 b0 .. 8 b1 of the axis' first half and their mirror rows
+        const int64_t i0 = std::min(8 * b0, p->sep_lanes), i1 = std::min(8 * b1, p->sep_lanes);
+        copy_rows(i0, i1);
+        copy_rows(std::max(i1, n0 - i1), n0 - i0);
+      } else {
+        // per block of 8 lanes, the rows of the tile's first and second 32 h values
+        for (int64_t b = b0; b < b1; ++b)
+          for (int w = 0; w < 2; ++w) copy_rows(64 * (b / 4) + 32 * w + 8 * (b % 4), 64 * (b / 4) + 32 * w + 8 * (b % 4) + 8);
+      }
       if (e != cudaSuccess) return cuda_status(e, "map range to the host");
     }
   }
