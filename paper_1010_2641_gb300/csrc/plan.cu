@@ -312,7 +312,8 @@ extern "C" void scatter_plan_destroy(scatter_plan_t p) {
   release(d.ztab);
   release(d.sep_A);
   release(d.sep_partial);
-  release(d.sep_chunks);
+  release(p->sep_direct.chunks);
+  release(p->sep_folded.chunks);
   release(d.ap_blocks);
   release(d.ftab);
   release(d.ftab64);

@@ -86,6 +86,21 @@ struct Tiling {
 // more ranges, the less of the map's copy is left after the last reduction
 constexpr int kHostPieces = 16;
 
+// One form of the separable contraction: its tiles, atom chunks and launch
+// choices.  The A table and the partials are the plan's, sized for the larger.
+struct SepForm {
+  bool fold = false, fold_h = false;  // folded over the (k, l) axes' middles, over h's too (sep_common.cuh)
+  int64_t mt = 0, nt = 0, steps = 0;  // M tiles, N tiles, K steps
+  int64_t cols = 0;                   // columns of the partials
+  int64_t lanes = 0, pairs = 0;       // fold: h values with rows of their own, mirror pairs of (k, l) points
+  int split = 1;
+  int32_t n_chunks = 0;
+  Segment* chunks = nullptr;          // device: atom chunks, one species each, step-aligned slots
+  int flush = 0;                      // steps between TMEM flushes
+  bool form_a = false;                // A formed inside the CTA-pair kernel, no A table
+  float smax[2] = {0.f, 0.f};         // max offset of the b and c axes
+};
+
 struct DeviceBuffers {
   int32_t* slot_src = nullptr;      // [n_slots]
   int32_t* slot_inst = nullptr;     // [n_slots]
@@ -130,7 +145,6 @@ struct DeviceBuffers {
   // separable path
   void* sep_A = nullptr;            // A operand blocks (f16 hi/lo)
   float* sep_partial = nullptr;     // [chunk][2][sep_ns] planar
-  Segment* sep_chunks = nullptr;    // separable atom chunks: one species each, step-aligned slots
   Segment* ap_blocks = nullptr;     // atom-parallel blocks: one species each, <= 256 K slots
   float2* ftab = nullptr;           // Eq. 4 factor table [n_species][M], or null (form factors)
   double* ftab64 = nullptr;         // the same in FP64 (re, im) for the FP64 kernel
@@ -207,16 +221,10 @@ struct scatter_plan_s {
   cudaStream_t graph_stream = nullptr;
   cudaEvent_t graph_in = nullptr, graph_out = nullptr;
   int32_t graph_launches = 0;
-  int64_t sep_mt = 0, sep_nt = 0, sep_steps = 0;
   int64_t sep_n[3] = {0, 0, 0};                  // separable grid shape (GID: n_h, n_k, 4 n_af)
   int64_t sep_ns = 0;
-  int32_t sep_n_chunks = 0;
-  bool sep_fold = false, sep_fold_h = false;     // folded over the (k, l) axes' middles, over h's too (sep_common.cuh)
-  int64_t sep_lanes = 0, sep_pairs = 0;          // h values with rows of their own, mirror pairs of (k, l) points
-  int sep_flush = 0;                             // steps between TMEM flushes
-  double sep_mid[3] = {0, 0, 0};                 // the axes' middles - H
-  bool sep_form_a = false;                       // A formed inside the CTA-pair kernel, no A table
-  float sep_smax[2] = {0.f, 0.f};               // max |s| of the separable grid's b and c axes
+  scatter::SepForm sep_direct, sep_folded;       // sep_folded.fold: the folded form exists (amplitude calls)
+  double sep_mid[3] = {0, 0, 0};                 // the folded axes' middles - H
   int32_t ap_n_blocks = 0;
   int32_t ap_tile = 0;               // reflections per atom-parallel CTA (<= kApPts)
   std::vector<double> gid_sz_host;               // [2][n_af] Sz1, Sz2 (r.l.u.)
@@ -231,6 +239,9 @@ struct scatter_plan_s {
   float adj_ds = 0.f;               // its l step
   int64_t adj_lines_per_chunk = 0;
   bool adj_sep = false;             // SEPARABLE grid plan: the adjoint runs on k_sep
+  bool adj_sep_fold = false;        // its points folded over the middle of the (k, l) plane
+  int64_t adj_sep_k = 0;            // points (mirror pairs) of a plane
+  double adj_sep_mid[2] = {0, 0};   // the middles of the k and l axes - H
   int64_t adj_sep_ksteps = 0, adj_sep_mt = 0;
   int32_t adj_sep_ntiles = 0, adj_sep_chunks = 0;
   float adj_sep_smax[2] = {0.f, 0.f};

@@ -652,8 +652,8 @@ struct SepFoldReduceArgs {
 // rows l % 8 and quad l / 8 of pairs, so a read covers 128 contiguous bytes
 // per quad, and the four row blocks and the two columns of a pair (blocks of
 // the partials that the same thread reads) combine with no exchange.  GROUPS threads share a quadruple's chunks on small maps and meet
-// in shared memory in a fixed order (a 16-value row range of the strained
-// sphere's map: 21.5 us with one thread per quadruple, 12.7 us with four).
+// in shared memory in a fixed order (64 CTAs of seven chunks: 21.5 us with one
+// thread per quadruple, 12.7 us with four).
 template <int GROUPS>
 __global__ void __launch_bounds__(256) k_sep_reduce_fold(const SepFoldReduceArgs a) {
   constexpr int kCols = 256 / GROUPS;  // threads over (alpha, quad)
@@ -924,6 +924,36 @@ namespace {
 // bound by fixed costs that the fold does not change.
 constexpr int64_t kSepFoldMinSlots = 4096;
 
+// Atom chunks: every species segment split into step-aligned pieces, about
+// `split` pieces in all, so that each chunk carries a single form factor.
+std::vector<Segment> sep_chunks(const scatter_plan_s* p, int split, int step) {
+  std::vector<Segment> chunks;
+  int64_t total_steps = 0;
+  for (const Segment& sg : p->all_segs)
+    if (sg.instance == 0 && sg.end > sg.begin) total_steps += (sg.end - sg.begin) / step;
+  for (const Segment& sg : p->all_segs) {
+    if (sg.instance != 0 || sg.end <= sg.begin) continue;
+    const int64_t steps = (sg.end - sg.begin) / step;
+    const int64_t k = std::max<int64_t>(1, std::llround((double)split * (double)steps / (double)total_steps));
+    const int64_t per = (steps + k - 1) / k;
+    for (int64_t b = 0; b < steps; b += per)
+      chunks.push_back(Segment{sg.begin + b * step, sg.begin + std::min(steps, b + per) * step, sg.species, 0});
+  }
+  return chunks;
+}
+
+// Mean steps of the accumulation group that a step lies in, for chunks flushed
+// every `flush` steps: the truncation error of a map grows with it.
+double sep_mean_group(const std::vector<Segment>& chunks, int step, int64_t flush) {
+  double sq = 0.0, all = 0.0;
+  for (const Segment& c : chunks) {
+    const int64_t n = (c.end - c.begin) / step, full = n / flush, rest = n % flush;
+    sq += (double)full * (double)flush * (double)flush + (double)rest * (double)rest;
+    all += (double)n;
+  }
+  return all > 0.0 ? sq / all : 0.0;
+}
+
 // Atom chunks (split over K) of `steps` steps in all that minimise the waves
 // of CTAs x steps per CTA, each chunk at least min_steps long; *cost_out in
 // steps.
@@ -997,45 +1027,60 @@ scatter_status prepare_separable(scatter_plan_s* p, int split_override) {
     }
   }
   p->sep_ns = p->sep_n[0] * p->sep_n[1] * p->sep_n[2];
-  // The direct form's tiles and chunks
-  const int64_t steps_d = p->n_slots / kSepStep, nbc = p->sep_n[1] * p->sep_n[2];
-  const int64_t mt_d = (2 * p->sep_n[0] + kSepM - 1) / kSepM;
+  const int64_t nbc = p->sep_n[1] * p->sep_n[2];
+  // The direct form
+  SepForm& fd = p->sep_direct;
+  fd.mt = (2 * p->sep_n[0] + kSepM - 1) / kSepM;
+  fd.cols = nbc;
+  fd.nt = (fd.cols + kSepN - 1) / kSepN;
+  fd.steps = p->n_slots / kSepStep;
+  fd.flush = kSepFlush;
   double cost_d = 0.0, cost_f = 0.0;
-  int split = split_override > 0 ? split_override
-                                 : sep_best_split(p, (mt_d + 1) / 2 * ((nbc + kSepN - 1) / kSepN), steps_d, 64.0, &cost_d);
-  p->sep_flush = kSepFlush;
-  // Fold where the (k, l) axes are symmetric (evenly spaced axes) and the
-  // crystal has at least kSepFoldMinSlots slots.  Not on grazing incidence:
-  // near the critical angle the four beams nearly cancel, and the errors of a
-  // point and its mirror (opposite beams), one sum's in the fold, no longer
-  // cancel with them (2-3 times the direct form's scatter on some maps).  The
-  // accumulators' truncation grows with the steps of a group, so the fold
-  // keeps 7/8 of the direct form's group length (its chunks are at least 0.8
-  // of that form's groups long), which keeps the error of the map where the
-  // direct form has it; it is taken where that leaves it the cheaper form by
-  // the cost model.
+  fd.split = split_override > 0 ? split_override
+                                : sep_best_split(p, (fd.mt + 1) / 2 * fd.nt, fd.steps, 64.0, &cost_d);
+  // The folded form, where the (k, l) axes are symmetric (evenly spaced axes)
+  // and the crystal has at least kSepFoldMinSlots slots, for amplitude calls.
+  // Not on grazing incidence: near the critical angle the four beams nearly
+  // cancel, and the errors of a point and its mirror (opposite beams), one
+  // sum's in the fold, no longer cancel with them (2-3 times the direct form's
+  // scatter on some maps).  The accumulators' truncation grows with the steps
+  // of a group, so the fold takes chunks and a flush interval that come to
+  // 0.95 of the direct form's mean group, which keeps the error of the map
+  // where the direct form has it (the two forms' amplitudes agree to ~1.3e-5);
+  // it is taken where that leaves it the cheaper form by the cost model.
+  // Intensities keep the direct form: |A|^2 doubles the forms' difference.
+  SepForm& ff = p->sep_folded;
   double mid[3] = {0, 0, 0};
-  p->sep_fold = !gid && p->n_slots >= kSepFoldMinSlots && p->n_slots % kSepFoldStep == 0 &&
-                sep_axis_middle(ax64[1], p->inst[0].H[1], &mid[1]) && sep_axis_middle(ax64[2], p->inst[0].H[2], &mid[2]);
-  if (p->sep_fold) {
-    p->sep_fold_h = sep_axis_middle(ax64[0], p->inst[0].H[0], &mid[0]);
-    p->sep_lanes = p->sep_fold_h ? (p->sep_n[0] + 1) / 2 : p->sep_n[0];
-    p->sep_pairs = (nbc + 1) / 2;
-    const int64_t mt_f = p->sep_fold_h ? (p->sep_lanes + 31) / 32 : (p->sep_lanes + kSepFoldRows - 1) / kSepFoldRows;
-    const int64_t nt_f = (sep_fold_cols(p->sep_pairs) + kSepN - 1) / kSepN;
-    const double group = std::min<double>(kSepFlush, (double)((steps_d + split - 1) / split));
+  ff.fold = !gid && p->n_slots >= kSepFoldMinSlots && p->n_slots % kSepFoldStep == 0 &&
+            sep_axis_middle(ax64[1], p->inst[0].H[1], &mid[1]) && sep_axis_middle(ax64[2], p->inst[0].H[2], &mid[2]);
+  if (ff.fold) {
+    ff.fold_h = sep_axis_middle(ax64[0], p->inst[0].H[0], &mid[0]);
+    ff.lanes = ff.fold_h ? (p->sep_n[0] + 1) / 2 : p->sep_n[0];
+    ff.pairs = (nbc + 1) / 2;
+    ff.mt = ff.fold_h ? (ff.lanes + 31) / 32 : (ff.lanes + kSepFoldRows - 1) / kSepFoldRows;
+    ff.cols = sep_fold_cols(ff.pairs);
+    ff.nt = (ff.cols + kSepN - 1) / kSepN;
+    ff.steps = p->n_slots / kSepFoldStep;
+    const double group = 0.95 * sep_mean_group(sep_chunks(p, fd.split, kSepStep), kSepStep, kSepFlush);
+    ff.split = fd.split;
     if (split_override <= 0) {
-      const int split_f =
-          sep_best_split(p, (mt_f + 1) / 2 * nt_f, p->n_slots / kSepFoldStep, 0.8 * group, &cost_f);
-      p->sep_fold = cost_f < 0.95 * cost_d && (double)(p->n_slots / kSepFoldStep) >= 0.8 * group;
-      if (p->sep_fold) split = split_f;
+      ff.split = sep_best_split(p, (ff.mt + 1) / 2 * ff.nt, ff.steps, group, &cost_f);
+      ff.fold = cost_f < 0.95 * cost_d && (double)ff.steps >= 0.9 * group;
     }
-    if (p->sep_fold) p->sep_flush = std::max(1, (int)(0.875 * group));
+    const std::vector<Segment> cf = sep_chunks(p, ff.split, kSepFoldStep);
+    double off = 1e300;
+    for (int f = 1; f <= kSepFlush + kSepFlush / 2; ++f) {
+      const double d = std::fabs(sep_mean_group(cf, kSepFoldStep, f) - group);
+      if (d < off) {
+        off = d;
+        ff.flush = f;
+      }
+    }
   }
   std::vector<float> dvals, dvals_lo;
-  if (p->sep_fold) {
+  if (ff.fold) {
     for (int d = 0; d < 3; ++d) {
-      const bool fold_d = d > 0 || p->sep_fold_h;
+      const bool fold_d = d > 0 || ff.fold_h;
       if (!fold_d) mid[d] = p->inst[0].H[d];  // an h axis that is not folded: offsets from H
       p->sep_mid[d] = mid[d] - p->inst[0].H[d];
       const size_t n = ax64[d].size();
@@ -1046,23 +1091,10 @@ scatter_status prepare_separable(scatter_plan_s* p, int split_override) {
       }
     }
   }
-  const std::vector<float>& form = p->sep_fold ? dvals : alls;  // offsets that the kernels form phases from
-  p->sep_smax[0] = p->sep_smax[1] = 0.f;
-  for (int64_t i = 0; i < p->sep_n[1]; ++i)
-    p->sep_smax[0] = std::max(p->sep_smax[0], std::fabs(form[p->sep_n[0] + i]));
-  for (int64_t i = 0; i < p->sep_n[2]; ++i)
-    p->sep_smax[1] = std::max(p->sep_smax[1], std::fabs(form[p->sep_n[0] + p->sep_n[1] + i]));
-  const int step = p->sep_fold ? kSepFoldStep : kSepStep;
-  const int64_t n_steps = p->n_slots / step;
-  const int64_t n_mt = !p->sep_fold ? mt_d : p->sep_fold_h ? (p->sep_lanes + 31) / 32
-                                                           : (p->sep_lanes + kSepFoldRows - 1) / kSepFoldRows;
-  const int64_t n_cols = p->sep_fold ? sep_fold_cols(p->sep_pairs) : nbc;
-  const int64_t n_nt = (n_cols + kSepN - 1) / kSepN;
-  const int64_t n_mp = (n_mt + 1) / 2;
   Tiling t;
   t.threads = 256;
   t.R = 8;
-  t.split_k = split;
+  t.split_k = fd.split;
   // chunk tables (segments) as for the generic path; the partial buffer is blocked
   scatter_status st = apply_tiling(p, t);
   if (st != SCATTER_OK) return st;
@@ -1070,54 +1102,48 @@ scatter_status prepare_separable(scatter_plan_s* p, int split_override) {
     cudaFree(p->d.partial);
     p->d.partial = nullptr;
   }
-  p->sep_mt = n_mt;
-  p->sep_nt = n_nt;
-  p->sep_steps = n_steps;
   cudaError_t e;
-  // With one N tile every A tile is read by one cluster only: the CTA pair
-  // then forms its A tiles itself from the atom records (the same arithmetic
-  // as k_sep_tab_a), and the table, written and read once, is not kept.
-  // With several N tiles that formation would repeat per tile, so the table
-  // stays; an odd pair count runs its last pair on the one-CTA kernel, which
-  // reads the table.
-  p->sep_form_a = sep_pair_enabled() && n_mp % 2 == 0 && n_nt == 1;
-  const size_t a_bytes =
-      p->sep_form_a ? 0 : (size_t)(2 * n_mp) * (size_t)std::max<int64_t>(n_steps, 1) * kSepABytes;
-  // atom chunks: every species segment split into step-aligned pieces, about
-  // `split` pieces in all, so that each chunk carries a single form factor
-  std::vector<Segment> chunks;
-  int64_t total_steps = 0;
-  for (const Segment& sg : p->all_segs)
-    if (sg.instance == 0 && sg.end > sg.begin) total_steps += (sg.end - sg.begin) / step;
-  for (const Segment& sg : p->all_segs) {
-    if (sg.instance != 0 || sg.end <= sg.begin) continue;
-    const int64_t steps = (sg.end - sg.begin) / step;
-    const int64_t k = std::max<int64_t>(1, std::llround((double)split * (double)steps / (double)total_steps));
-    const int64_t per = (steps + k - 1) / k;
-    for (int64_t b = 0; b < steps; b += per)
-      chunks.push_back(Segment{sg.begin + b * step, sg.begin + std::min(steps, b + per) * step, sg.species, 0});
+  size_t a_bytes = 0, part_bytes = 0, chunk_bytes = 0;
+  for (SepForm* f : {&fd, &ff}) {
+    if (f == &ff && !ff.fold) break;
+    const std::vector<float>& off = f->fold ? dvals : alls;  // offsets that the kernels form phases from
+    for (int64_t i = 0; i < p->sep_n[1]; ++i) f->smax[0] = std::max(f->smax[0], std::fabs(off[p->sep_n[0] + i]));
+    for (int64_t i = 0; i < p->sep_n[2]; ++i)
+      f->smax[1] = std::max(f->smax[1], std::fabs(off[p->sep_n[0] + p->sep_n[1] + i]));
+    // With one N tile every A tile is read by one cluster only: the CTA pair
+    // then forms its A tiles itself from the atom records (the same arithmetic
+    // as k_sep_tab_a), and the table, written and read once, is not kept.
+    // With several N tiles that formation would repeat per tile, so the table
+    // stays; an odd pair count runs its last pair on the one-CTA kernel, which
+    // reads the table.
+    const int64_t n_mp = (f->mt + 1) / 2;
+    f->form_a = sep_pair_enabled() && n_mp % 2 == 0 && f->nt == 1;
+    if (!f->form_a)
+      a_bytes = std::max(a_bytes, (size_t)(2 * n_mp) * (size_t)std::max<int64_t>(f->steps, 1) * kSepABytes);
+    std::vector<Segment> chunks = sep_chunks(p, f->split, f->fold ? kSepFoldStep : kSepStep);
+    if (chunks.empty()) chunks.push_back(Segment{0, 0, 0, 0});  // no atoms: one empty chunk, zero partials
+    f->n_chunks = (int32_t)chunks.size();
+    part_bytes = std::max(part_bytes, (size_t)f->n_chunks * (size_t)sep_part_floats(f->mt, f->cols) * sizeof(float));
+    const size_t cb = chunks.size() * sizeof(Segment);
+    if ((e = cudaMalloc(&f->chunks, cb)) != cudaSuccess) return cuda_status(e, "cudaMalloc chunks");
+    cudaMemcpy(f->chunks, chunks.data(), cb, cudaMemcpyHostToDevice);
+    chunk_bytes += cb;
   }
-  if (chunks.empty()) chunks.push_back(Segment{0, 0, 0, 0});  // no atoms: one empty chunk, zero partials
-  p->sep_n_chunks = (int32_t)chunks.size();
-  const size_t part_bytes =
-      (size_t)p->sep_n_chunks * (size_t)sep_part_floats(n_mt, n_cols) * sizeof(float);
-  const size_t chunk_bytes = chunks.size() * sizeof(Segment);
   if (a_bytes) {
     if ((e = cudaMalloc(&p->d.sep_A, a_bytes)) != cudaSuccess) return cuda_status(e, "cudaMalloc separable A");
-    // tiles past the last row are never written by the table kernel: zero
-    // them once (the CTA-pair kernel streams the second tile of a pair always)
+    // tiles past the last row are never written by the table kernel (the
+    // CTA-pair kernel streams the second tile of a pair always; its rows are
+    // never read): zero them once
     if ((e = cudaMemset(p->d.sep_A, 0, a_bytes)) != cudaSuccess) return cuda_status(e, "memset separable A");
   }
   if ((e = cudaMalloc(&p->d.sep_partial, part_bytes)) != cudaSuccess)
     return cuda_status(e, "cudaMalloc separable partials");
-  if ((e = cudaMalloc(&p->d.sep_chunks, chunk_bytes)) != cudaSuccess) return cuda_status(e, "cudaMalloc chunks");
-  cudaMemcpy(p->d.sep_chunks, chunks.data(), chunk_bytes, cudaMemcpyHostToDevice);
   if ((e = cudaMalloc(&p->d.sep_axis_s, alls.size() * sizeof(float))) != cudaSuccess) return cuda_status(e, "axes");
   if ((e = cudaMalloc(&p->d.sep_axis_lo, alls_lo.size() * sizeof(float))) != cudaSuccess) return cuda_status(e, "axes");
   cudaMemcpy(p->d.sep_axis_s, alls.data(), alls.size() * sizeof(float), cudaMemcpyHostToDevice);
   cudaMemcpy(p->d.sep_axis_lo, alls_lo.data(), alls_lo.size() * sizeof(float), cudaMemcpyHostToDevice);
   size_t fold_bytes = 0;
-  if (p->sep_fold) {
+  if (ff.fold) {
     const size_t rb = (size_t)p->n_slots * sizeof(float4), db = dvals.size() * sizeof(float);
     if ((e = cudaMalloc(&p->d.sep_rec, rb)) != cudaSuccess) return cuda_status(e, "cudaMalloc folded records");
     if ((e = cudaMalloc(&p->d.sep_axis_d, db)) != cudaSuccess) return cuda_status(e, "folded axes");
@@ -1141,10 +1167,12 @@ scatter_status prepare_separable(scatter_plan_s* p, int split_override) {
   }
   p->base_bytes += (int64_t)(a_bytes + part_bytes + chunk_bytes + virt_bytes + fold_bytes);
   if ((e = sep_prepare_kernel()) != cudaSuccess) return cuda_status(e, "separable shared memory attribute");
-  return sep_prepare_side(p, n_mt);
+  st = sep_prepare_side(p, fd.mt);
+  return st == SCATTER_OK && ff.fold ? sep_prepare_side(p, ff.mt) : st;
 }
 
 scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st) {
+  const SepForm& fm = p->sep_folded.fold && amp_out ? p->sep_folded : p->sep_direct;
   SepTabArgs t{};
   t.atom4 = p->d.atom4;
   t.atom_lo = p->d.atom_lo;
@@ -1155,18 +1183,18 @@ scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_ou
   t.n1 = p->sep_n[1];
   t.n2 = p->sep_n[2];
   t.n_slots = p->n_slots;
-  t.n_steps = p->sep_steps;
-  t.n_mt = p->sep_mt;
+  t.n_steps = fm.steps;
+  t.n_mt = fm.mt;
   t.A = static_cast<uint4*>(p->d.sep_A);
-  const int n_chunks = p->sep_n_chunks;
-  if (p->sep_fold && !p->sep_form_a) {
-    const int64_t na = p->sep_mt * p->sep_steps * 128;
-    const auto kernel = p->sep_fold_h ? k_sep_tab_fold<true> : k_sep_tab_fold<false>;
+  const int n_chunks = fm.n_chunks;
+  if (fm.fold && !fm.form_a) {
+    const int64_t na = fm.mt * fm.steps * 128;
+    const auto kernel = fm.fold_h ? k_sep_tab_fold<true> : k_sep_tab_fold<false>;
     kernel<<<(unsigned)((na + 255) / 256), 256, 0, st>>>(p->d.sep_rec, p->d.sep_axis_d, p->d.sep_axis_dlo, p->sep_n[0],
-                                                         p->sep_lanes, p->sep_steps, p->sep_mt, t.A);
+                                                         fm.lanes, fm.steps, fm.mt, t.A);
     p->last_launches += 1;
-  } else if (p->n_slots > 0 && !p->sep_form_a) {
-    const int64_t na = p->sep_mt * p->sep_steps * 4 * kSepM;  // real tiles; a padding tile is never read
+  } else if (p->n_slots > 0 && !fm.form_a) {
+    const int64_t na = fm.mt * fm.steps * 4 * kSepM;  // real tiles; a padding tile is never read
     k_sep_tab_a<<<(unsigned)((na + 255) / 256), 256, 0, st>>>(t);
     p->last_launches += 1;
   }
@@ -1174,59 +1202,61 @@ scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_ou
   a.A = static_cast<const uint4*>(p->d.sep_A);
   a.a_sp_stride = 0;
   a.rec = p->d.atom4;
-  a.chunks = p->d.sep_chunks;
+  a.chunks = fm.chunks;
   a.ntiles = nullptr;
   a.bbox = p->d.inst_bbox;
   a.shift = p->d.inst_shift;
-  a.smax_b = p->sep_smax[0];
-  a.smax_c = p->sep_smax[1];
-  const int64_t n_cols = p->sep_fold ? sep_fold_cols(p->sep_pairs) : p->sep_n[1] * p->sep_n[2];
-  a.axis_s = p->sep_fold ? p->d.sep_axis_d : p->d.sep_axis_s;
-  a.axis_lo = p->sep_fold ? p->d.sep_axis_dlo : p->d.sep_axis_lo;
+  a.smax_b = fm.smax[0];
+  a.smax_c = fm.smax[1];
+  a.axis_s = fm.fold ? p->d.sep_axis_d : p->d.sep_axis_s;
+  a.axis_lo = fm.fold ? p->d.sep_axis_dlo : p->d.sep_axis_lo;
   a.n0 = p->sep_n[0];
   a.n1 = p->sep_n[1];
   a.n2 = p->sep_n[2];
-  a.n_cb = (n_cols + 31) / 32;
-  a.chunk_floats = sep_part_floats(p->sep_mt, n_cols);
-  a.fold = p->sep_fold ? 1 : 0;
-  a.n_pairs = p->sep_pairs;
-  a.n_lanes = p->sep_lanes;
-  a.fold_h = p->sep_fold_h ? 1 : 0;
-  a.flush = p->sep_flush;
+  a.n_cb = (fm.cols + 31) / 32;
+  a.chunk_floats = sep_part_floats(fm.mt, fm.cols);
+  a.fold = fm.fold ? 1 : 0;
+  a.n_pairs = fm.pairs;
+  a.n_lanes = fm.lanes;
+  a.fold_h = fm.fold_h ? 1 : 0;
+  a.flush = fm.flush;
   a.rec_a = p->d.sep_rec;
-  a.n_steps = p->sep_steps;
-  a.n_mt = p->sep_mt;
+  a.n_steps = fm.steps;
+  a.n_mt = fm.mt;
   a.partial = p->d.sep_partial;
   a.status = p->d.status;
   a.axis_att = p->d.sep_att;
-  a.form_a = p->sep_form_a ? 1 : 0;
+  a.form_a = fm.form_a ? 1 : 0;
   a.rec_lo = p->d.atom_lo;
   a.rec_w = p->d.atom_w;
-  dim3 grid((unsigned)(((p->sep_mt + 1) / 2) * p->sep_nt), (unsigned)n_chunks);
+  dim3 grid((unsigned)(((fm.mt + 1) / 2) * fm.nt), (unsigned)n_chunks);
   timing_begin(p, st);
   const cudaError_t le = sep_launch_core(a, grid, st, p->side_stream, p->side_fork, p->side_join);
   timing_end(p, st);
   if (le != cudaSuccess) return cuda_status(le, "separable kernel launch");
-  p->last_launches += sep_core_launches(p->sep_mt);
+  p->last_launches += sep_core_launches(fm.mt);
   const bool gid = p->s_kind == SCATTER_S_GID_GRID;
   const int64_t n_cb = a.n_cb, ncols = p->sep_n[1] * p->sep_n[2];
   // row blocks of the reduction: 16 h values (32 partial rows); folded 8 lanes, 32 per
   // M tile: the h values of a tile's second half (or their mirrors) with those of its first
-  const int64_t n_bm = !p->sep_fold ? (2 * p->sep_n[0] + 31) / 32
-                       : p->sep_fold_h ? (p->sep_lanes + 7) / 8 : 4 * p->sep_mt;
+  const int64_t n_bm = !fm.fold ? (2 * p->sep_n[0] + 31) / 32
+                       : fm.fold_h ? (fm.lanes + 7) / 8 : 4 * fm.mt;
   // a host call copies each row range to the host while the next is reduced
   const bool pieces = p->host_out && !gid;
-  const int n_pieces = pieces ? (int)std::min<int64_t>(kHostPieces, n_bm) : 1;
+  // (folded: four; 2 to 16 ranges measured the same 3.59 ms on the strained
+  // sphere, and fewer leave each reduction more CTAs)
+  const int max_pieces = (int)std::min<int64_t>(fm.fold ? 4 : kHostPieces, n_bm);
+  const int n_pieces = pieces ? max_pieces : 1;
   float2* amp_dst = gid ? p->d.sep_virt : amp_out;
   float* int_dst = gid ? nullptr : int_out;
   for (int k = 0; k < n_pieces; ++k) {
     const int64_t b0 = n_bm * k / n_pieces, b1 = n_bm * (k + 1) / n_pieces;
-    if (p->sep_fold) {
+    if (fm.fold) {
       SepFoldReduceArgs r{};
       r.partial = p->d.sep_partial;
       r.chunk_floats = a.chunk_floats;
       r.n_cb = n_cb;
-      r.chunks = p->d.sep_chunks;
+      r.chunks = fm.chunks;
       r.n_chunks = n_chunks;
       r.coef = p->d.coef;
       r.ftab = p->d.ftab;
@@ -1236,20 +1266,20 @@ scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_ou
       r.n0 = p->sep_n[0];
       r.n1 = p->sep_n[1];
       r.n2 = p->sep_n[2];
-      r.n_pairs = p->sep_pairs;
-      r.n_lanes = p->sep_lanes;
-      r.fold_h = p->sep_fold_h ? 1 : 0;
+      r.n_pairs = fm.pairs;
+      r.n_lanes = fm.lanes;
+      r.fold_h = fm.fold_h ? 1 : 0;
       for (int d = 0; d < 3; ++d) r.H[d] = (float)p->inst[0].H[d];
       r.shift = p->d.inst_shift;
       r.l8_base = b0;
       r.out_amp = amp_dst;
       r.out_int = int_dst;
-      // small launches (a row range of a host call, a small map of a large crystal):
-      // several threads share each quadruple's chunks until the launch has two
-      // CTAs per SM
-      const int64_t quads = (p->sep_pairs + 3) / 4, want = 2 * (int64_t)p->n_sm;
+      // small maps: several threads share each quadruple's chunks until a row
+      // range's launch has a CTA per SM (the same choice with and without
+      // ranges: a host call's map equals the device call's bit for bit)
+      const int64_t quads = (fm.pairs + 3) / 4, range = (n_bm + max_pieces - 1) / max_pieces;
       int groups = 1;
-      while (groups < 8 && 2 * groups <= n_chunks && (quads + 31) / 32 * (b1 - b0) * groups < want) groups *= 2;
+      while (groups < 8 && 2 * groups <= n_chunks && (quads + 31) / 32 * range * groups < p->n_sm) groups *= 2;
       const auto kernel = groups == 1   ? k_sep_reduce_fold<1>
                           : groups == 2 ? k_sep_reduce_fold<2>
                           : groups == 4 ? k_sep_reduce_fold<4>
@@ -1259,7 +1289,7 @@ scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_ou
     } else {
       const dim3 rgrid((unsigned)n_cb, (unsigned)(b1 - b0));
       k_sep_reduce<<<rgrid, 256, 0, st>>>(
-          p->d.sep_partial, a.chunk_floats, n_cb, p->d.sep_chunks, n_chunks, p->d.coef, p->d.ftab,
+          p->d.sep_partial, a.chunk_floats, n_cb, fm.chunks, n_chunks, p->d.coef, p->d.ftab,
           (float)(1.0 / (4.0 * p->lattice_a * p->lattice_a)), p->d.sep_axis_s, p->d.sep_axis_lo, p->sep_n[0],
           p->sep_n[1], p->sep_n[2],
           make_float3((float)p->inst[0].H[0], (float)p->inst[0].H[1], (float)p->inst[0].H[2]), p->d.inst_shift,
@@ -1276,11 +1306,11 @@ scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_ou
           e = cudaMemcpyAsync(static_cast<float2*>(p->host_out) + r0 * ncols, amp_out + r0 * ncols,
                               (size_t)((r1 - r0) * ncols) * sizeof(float2), cudaMemcpyDeviceToHost, p->copy_stream);
       };
-      if (!p->sep_fold) {
+      if (!fm.fold) {
         copy_rows(16 * b0, 16 * b1);
-      } else if (p->sep_fold_h) {
+      } else if (fm.fold_h) {
         // h rows 8 b0 .. 8 b1 of the axis' first half and their mirror rows
-        const int64_t i0 = std::min(8 * b0, p->sep_lanes), i1 = std::min(8 * b1, p->sep_lanes);
+        const int64_t i0 = std::min(8 * b0, fm.lanes), i1 = std::min(8 * b1, fm.lanes);
         copy_rows(i0, i1);
         copy_rows(std::max(i1, n0 - i1), n0 - i0);
       } else {
