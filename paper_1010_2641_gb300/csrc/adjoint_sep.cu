@@ -18,6 +18,15 @@
 // 2^14 (f16 keeps 22 bits of it in hi + lo down to 2^-17 of the row's
 // maximum); the epilogue undoes the scale exactly.
 //
+// Where the (k, l) axes are symmetric about their middles (offsets +-d of a
+// point p and its mirror p', phases +-phi_p around the middle's) the products
+// of the two share their cos and sin:
+//   U_w e^{-2 pi i (mid - H).r'} = sum over half the points of P cos phi + i M sin phi,
+//   P, M = omega(p) gF(p) +- omega(p') gF(p'),  omega_1 = d_b, omega_2 = d_c
+// (odd, so their sums take the other sign): the same rows over half the K, half
+// the MMAs, formation and A table.  The epilogue turns the result by the
+// middle's phase and adds the middle to H.
+//
 // k_adj_sep_scale  per (species, a): the exponents of the three rows' scales
 // k_adj_sep_tab    A blocks of every species in the tcgen05 no-swizzle layout
 // k_sep            U for every (M-tile pair, 256-atom tile, point chunk)
@@ -32,57 +41,84 @@ namespace scatter {
 
 constexpr int kAdjSepRowMax = 14;  // binary exponent of a row's largest |element| after scaling
 
-// One CTA per (species, a): the largest |Re|, |Im| of gF, s_b gF and s_c gF
-// over the plane's n1 n2 points, as the exponent e of 2^e >= max (frexp),
-// stored as the shift k = e - kAdjSepRowMax of the row's scale 2^k.
-__global__ void __launch_bounds__(256) k_adj_sep_scale(const float2* __restrict__ gf, const float* __restrict__ axis_s,
-                                                       int64_t n0, int64_t n1, int64_t n2, int64_t n_s,
-                                                       int* __restrict__ sexp) {
+// P and M of a point (fold: of the pair p, p'; else P = M = omega gF), for the
+// weight row w; gp, gm: gF at p and p', om: omega_w(p).
+struct AdjPair {
+  float2 P, M;
+};
+__device__ __forceinline__ AdjPair adj_pair(float2 gp, float2 gm, float om, int w, bool fold, bool self) {
+  AdjPair r;
+  if (!fold) {
+    r.P = r.M = make_float2(gp.x * om, gp.y * om);
+  } else if (self) {  // the middle point: phase 0, offsets 0
+    r.P = w == 0 ? gp : make_float2(0.f, 0.f);
+    r.M = make_float2(0.f, 0.f);
+  } else {
+    const float2 sum = make_float2(gp.x + gm.x, gp.y + gm.y), dif = make_float2(gp.x - gm.x, gp.y - gm.y);
+    r.P = w == 0 ? sum : make_float2(om * dif.x, om * dif.y);
+    r.M = w == 0 ? dif : make_float2(om * sum.x, om * sum.y);
+  }
+  return r;
+}
+
+// x 2^k in two exact steps (k beyond a float's exponents; a subnormal result
+// may round twice): ldexpf without its branches
+__device__ __forceinline__ float scale2(float x, int k) {
+  const int k1 = k / 2;
+  return x * __int_as_float((k1 + 127) << 23) * __int_as_float((k - k1 + 127) << 23);
+}
+
+// One CTA per (species, a): the largest |Re|, |Im| of the three weights' P and
+// M over the plane's points, as the exponent e of 2^e >= max (frexp), stored
+// as the shift k = e - kAdjSepRowMax of the row's scale 2^k.  Latency-bound
+// (128 planes of 131 KB on the 128^3 cube): 1024 threads keep the loads in
+// flight, 37.7 us with 256, 7.3 us with 1024.
+__global__ void __launch_bounds__(1024) k_adj_sep_scale(const float2* __restrict__ gf, const float4* __restrict__ rec,
+                                                        int64_t n0, int64_t nbc, int64_t n_k, int fold, int64_t n_s,
+                                                        int* __restrict__ sexp) {
   const int64_t sp = blockIdx.x / n0, a = blockIdx.x % n0;
-  const int64_t nbc = n1 * n2;
   const float2* row = gf + sp * n_s + a * nbc;
-  float m0 = 0.f, m1 = 0.f, m2 = 0.f;
-  for (int64_t p = threadIdx.x; p < nbc; p += blockDim.x) {
-    const float2 v = row[p];
-    const float g = fmaxf(fabsf(v.x), fabsf(v.y));
-    m0 = fmaxf(m0, g);
-    m1 = fmaxf(m1, g * fabsf(axis_s[n0 + p / n2]));
-    m2 = fmaxf(m2, g * fabsf(axis_s[n0 + n1 + p % n2]));
+  float m[3] = {0.f, 0.f, 0.f};
+#pragma unroll 4
+  for (int64_t p = threadIdx.x; p < n_k; p += blockDim.x) {
+    const float2 gp = row[p], gm = fold ? row[nbc - 1 - p] : gp;
+    const float4 r = rec[p];
+#pragma unroll
+    for (int w = 0; w < 3; ++w) {
+      const AdjPair q = adj_pair(gp, gm, w == 0 ? 1.f : w == 1 ? r.y : r.z, w, fold, 2 * p + 1 == nbc);
+      m[w] = fmaxf(m[w], fmaxf(fmaxf(fabsf(q.P.x), fabsf(q.P.y)), fmaxf(fabsf(q.M.x), fabsf(q.M.y))));
+    }
   }
-  __shared__ float sh[3][8];
-  for (int o = 16; o > 0; o >>= 1) {
-    m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, o));
-    m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
-    m2 = fmaxf(m2, __shfl_xor_sync(0xffffffffu, m2, o));
-  }
+  __shared__ float sh[3][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) {
-    sh[0][warp] = m0;
-    sh[1][warp] = m1;
-    sh[2][warp] = m2;
+#pragma unroll
+  for (int w = 0; w < 3; ++w) {
+    for (int o = 16; o > 0; o >>= 1) m[w] = fmaxf(m[w], __shfl_xor_sync(0xffffffffu, m[w], o));
+    if (lane == 0) sh[w][warp] = m[w];
   }
   __syncthreads();
   if (threadIdx.x < 3) {
-    float m = 0.f;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) m = fmaxf(m, sh[threadIdx.x][q]);
+    float v = 0.f;
+    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) v = fmaxf(v, sh[threadIdx.x][q]);
     int e = 0;
-    if (m > 0.f && m <= 3.0e38f) frexpf(m, &e);  // zero or non-finite rows: scale 2^-14
+    if (v > 0.f && v <= 3.0e38f) frexpf(v, &e);  // zero or non-finite rows: scale 2^-14
     sexp[(sp * 3 + threadIdx.x) * n0 + a] = e - kAdjSepRowMax;
   }
 }
 
 struct AdjSepTabArgs {
   const float2* gf;     // [n_species][M] gF_s, M = n0 n1 n2 row-major
-  const float* axis_s;  // [n0 | n1 | n2] s = axis - H
+  const float4* rec;    // point records (0, omega_1, omega_2, 0)
   const int* sexp;      // [n_species][3][n0] row scale exponents
-  int64_t n0, n1, n2, n_s;
+  int64_t n0, nbc, n_k, n_s;  // n_k: points (fold: mirror pairs) of a plane
+  int fold;
   int64_t n_ksteps, n_mt, n_mp;
   int64_t total;        // threads: n_species x n_mt x n_ksteps x 512
   uint4* A;             // [species][n_mp][n_ksteps][2 tiles][hi|lo][4 kb][16 mg][8 rows] of 16 B
 };
 
 // One thread per 16-byte row of a core matrix (4 points x Re/Im of one A row).
-// Row 2 pa: (Gr, -Gi); row 2 pa + 1: (Gi, Gr) with G = gF omega_w 2^-k.
+// Row 2 pa: (Pr, -Mi); row 2 pa + 1: (Pi, Mr) with P, M scaled by 2^-k.
 __global__ void k_adj_sep_tab(const AdjSepTabArgs t) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= t.total) return;
@@ -92,25 +128,25 @@ __global__ void k_adj_sep_tab(const AdjSepTabArgs t) {
   const int64_t m = mt * kSepM + mg * 8 + r;
   const int64_t pa = m >> 1;
   const int ri = (int)(m & 1);
-  const int64_t nbc = t.n1 * t.n2;
   const bool in_row = pa < 3 * t.n0;
   const int w = in_row ? (int)(pa / t.n0) : 0;
   const int64_t a = in_row ? pa % t.n0 : 0;
   const int k = in_row ? t.sexp[(sp * 3 + w) * t.n0 + a] : 0;
-  const float2* row = t.gf + sp * t.n_s + a * nbc;
+  const float2* row = t.gf + sp * t.n_s + a * t.nbc;
   float v[8];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int64_t p = ks * kSepStep + kb * 4 + q;
-    float gr = 0.f, gi = 0.f;
-    if (in_row && p < nbc) {
-      const float2 g = row[p];
-      const float om = w == 0 ? 1.f : (w == 1 ? t.axis_s[t.n0 + p / t.n2] : t.axis_s[t.n0 + t.n1 + p % t.n2]);
-      gr = ldexpf(g.x * om, -k);
-      gi = ldexpf(g.y * om, -k);
+    float c0 = 0.f, c1 = 0.f;
+    if (in_row && p < t.n_k) {
+      const float2 gp = row[p], gm = t.fold ? row[t.nbc - 1 - p] : gp;
+      const float4 rc = t.rec[p];
+      const AdjPair g = adj_pair(gp, gm, w == 0 ? 1.f : w == 1 ? rc.y : rc.z, w, t.fold, 2 * p + 1 == t.nbc);
+      c0 = scale2(ri ? g.P.y : g.P.x, -k);
+      c1 = scale2(ri ? g.M.x : -g.M.y, -k);
     }
-    v[2 * q] = ri ? gi : gr;
-    v[2 * q + 1] = ri ? gr : -gi;
+    v[2 * q] = c0;
+    v[2 * q + 1] = c1;
   }
   uint4 hi, lo;
   split2(v[0], v[1], hi.x, lo.x);
@@ -130,88 +166,117 @@ struct AdjSepFinalArgs {
   const Segment* ntiles;
   const int* sexp;
   const float4* atom4;
+  const float4* atom_lo;
   const float* atom_w;
   const int32_t* slot_src;
   const float* axis_s;
   int64_t n0, n_slots;
-  double H[3];
+  float H[3], H_lo[3];     // as double-floats; fold: k and l at the middles of their axes
+  float mid[2], mid_lo[2]; // fold: those middles - H as double-floats, else 0
   float* grad;             // [n_atoms][3] caller order
 };
 
-// One thread per atom slot of an N tile: the sum over a (and over the point
-// chunks) with FP32 products and double-float (TwoSum) FP32 sums (FP64 runs
-// at ~1/75 of the FP32 rate here; the 3 n0 terms are already contracted
-// values whose own error is ~1e-6), the row factor e^{2 i pi s_a x'} from
-// MUFU sin/cos of the exactly reduced phase (|error| < 4e-7), then the
-// rotation by e^{2 i pi c} and the H terms in FP64.  Four values of a per
-// iteration keep 24 loads in flight per thread.
-__global__ void __launch_bounds__(kSepN) k_adj_sep_final(const AdjSepFinalArgs f) {
+// One warp per four atom slots: lane 2 i + ri holds row (Re or Im) of a = a0 + i
+// of a block of 16 values, so a read of one weight's rows is 512 contiguous
+// bytes (the partials keep four columns of a 32-row block together).  One
+// exchange gives the even lane (Re, Im) of the first two slots and the odd
+// lane of the last two.  The sum over a (and over the point chunks) runs with
+// FP32 products and double-float (TwoSum) FP32 sums (FP64 runs at ~1/75 of
+// the FP32 rate here; the 3 n0 terms are already contracted values whose own
+// error is ~1e-6).  Only Im(e^{2 pi i theta} X) is wanted, so the atom's phase
+// c + (mid - H).r' joins the row factor's (exactly reduced, MUFU sin/cos,
+// |error| < 4e-7) and four imaginary sums are enough; the 16 lanes' sums meet
+// in a fixed order.  116 us on the 102,400-atom cube x 128^3 (315 MB of
+// partials, 47 us at the copy rate; 217 us with one thread per slot, whose
+// reads were 16-byte pieces).
+constexpr int kAdjFinalWarps = 8;
+__global__ void __launch_bounds__(32 * kAdjFinalWarps) k_adj_sep_final(const AdjSepFinalArgs f) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = lane >> 1, ri = lane & 1;
   const Segment t = f.ntiles[blockIdx.x];
-  const int64_t slot = t.begin + threadIdx.x;
-  if (slot >= t.end) return;
-  const int32_t src = f.slot_src[slot];
-  if (src < 0) return;
-  const float4 at = f.atom4[slot];
+  const int64_t slot0 = t.begin + 4 * ((int64_t)blockIdx.y * kAdjFinalWarps + warp);
+  if (slot0 >= t.end) return;  // segments are multiples of 32 slots
+  const int64_t slot = slot0 + 2 * ri;  // this lane's two slots
   const int64_t rows = 3 * f.n0;
   const int* se = f.sexp + (int64_t)t.species * rows;
-  dev::DFloatSum V[2], Wd[3][2];
-  // the partials' offset of D entry (m, slot) is the column's part plus the
-  // row's (sep_part_off): the column part once per thread, and rows 2 r and
-  // 2 r + 1 (Re, Im) are neighbours in the same 32-row block, 4 floats apart
-  const int64_t col_off = sep_part_off(0, slot, f.n_cb);
+  float x[2], th[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const float4 at = f.atom4[slot + u], lo = f.atom_lo[slot + u];
+    x[u] = at.x;
+    const float py = dev::frac_of_product2(f.mid[0], f.mid_lo[0], at.y) + f.mid[0] * lo.y;
+    const float pz = dev::frac_of_product2(f.mid[1], f.mid_lo[1], at.z) + f.mid[1] * lo.z;
+    th[u] = dev::frac_rn(at.w + (py + pz));
+  }
+  // sums of Im P_0, s_a Im P_0, Im P_1, Im P_2
+  dev::DFloatSum sum[2][4];
+  const float* base = f.partial + sep_part_off(0, slot0, f.n_cb);
   const int64_t row_block = f.n_cb << 10;  // floats per 32-row block
-  constexpr int kU = 4;
-  for (int64_t a0 = 0; a0 < f.n0; a0 += kU) {
-    float U[kU][3][2];
+  for (int64_t a0 = 0; a0 < f.n0; a0 += 16) {
+    const int64_t a = a0 + i;
+    const bool ok = a < f.n0;
+    float4 U[3];
+    int k[3];
 #pragma unroll
-    for (int u = 0; u < kU; ++u)
-#pragma unroll
-      for (int w = 0; w < 3; ++w) {
-        U[u][w][0] = U[u][w][1] = 0.f;
-        const int64_t a = a0 + u;
-        if (a < f.n0) {
-          const int64_t m = 2 * (w * f.n0 + a);
-          const float* pc = f.partial + col_off + (m >> 5) * row_block + ((m & 31) << 2);
-          for (int c = 0; c < f.n_chunks; ++c, pc += f.chunk_floats) {
-            U[u][w][0] += pc[0];
-            U[u][w][1] += pc[4];
-          }
+    for (int w = 0; w < 3; ++w) {
+      U[w] = make_float4(0.f, 0.f, 0.f, 0.f);
+      k[w] = 0;
+      if (ok) {
+        const int64_t m = 2 * (w * f.n0 + a) + ri;
+        const float* pc = base + (m >> 5) * row_block + ((m & 31) << 2);
+        U[w] = __ldcs(reinterpret_cast<const float4*>(pc));
+        for (int c = 1; c < f.n_chunks; ++c) {
+          const float4 v = __ldcs(reinterpret_cast<const float4*>(pc + c * f.chunk_floats));
+          U[w].x += v.x;
+          U[w].y += v.y;
+          U[w].z += v.z;
+          U[w].w += v.w;
         }
+        k[w] = se[w * f.n0 + a];
       }
+    }
+    const float sa = ok ? f.axis_s[a] : 0.f;
+    float sn[2], cs[2];
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int64_t a = a0 + u;
-      if (a >= f.n0) break;
-      const float sa = f.axis_s[a];
-      float sn, cs;
-      dev::sincos_cycles_mufu(dev::frac_of_product(sa, at.x), &sn, &cs);
-      float P[3][2];
+    for (int u = 0; u < 2; ++u) dev::sincos_cycles_mufu(dev::frac_rn(dev::frac_of_product(sa, x[u]) + th[u]), &sn[u], &cs[u]);
 #pragma unroll
-      for (int w = 0; w < 3; ++w) {
-        const int k = se[w * f.n0 + a];
-        const float re = ldexpf(U[u][w][0], k), im = ldexpf(U[u][w][1], k);
-        P[w][0] = fmaf(cs, re, -sn * im);
-        P[w][1] = fmaf(cs, im, sn * re);
+    for (int w = 0; w < 3; ++w) {
+      const float rx = __shfl_xor_sync(0xffffffffu, ri ? U[w].x : U[w].z, 1);
+      const float ry = __shfl_xor_sync(0xffffffffu, ri ? U[w].y : U[w].w, 1);
+      const float re[2] = {ri ? rx : U[w].x, ri ? ry : U[w].y}, im[2] = {ri ? U[w].z : rx, ri ? U[w].w : ry};
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const float v = scale2(fmaf(cs[u], im[u], sn[u] * re[u]), k[w]);
+        sum[u][w == 0 ? 0 : w + 1].add(v);
+        if (w == 0) sum[u][1].add(sa * v);
       }
-      V[0].add(P[0][0]);
-      V[1].add(P[0][1]);
-      Wd[0][0].add(sa * P[0][0]);
-      Wd[0][1].add(sa * P[0][1]);
-      Wd[1][0].add(P[1][0]);
-      Wd[1][1].add(P[1][1]);
-      Wd[2][0].add(P[2][0]);
-      Wd[2][1].add(P[2][1]);
     }
   }
-  double sn, cs;
-  sincospi(2.0 * (double)at.w, &sn, &cs);
-  const double scale = -2.0 * 3.14159265358979323846 * (double)f.atom_w[slot];
-  auto dval = [](const dev::DFloatSum& q) { return (double)q.hi + (double)q.lo; };
-  const double vr = dval(V[0]), vi = dval(V[1]);
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const double xr = f.H[d] * vr + dval(Wd[d][0]), xi = f.H[d] * vi + dval(Wd[d][1]);
-    f.grad[3 * (int64_t)src + d] = (float)(scale * (cs * xi + sn * xr));  // Im(e^{2 i pi c} X)
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int o = 2; o < 32; o <<= 1) {
+        const float h = __shfl_xor_sync(0xffffffffu, sum[u][q].hi, o), l = __shfl_xor_sync(0xffffffffu, sum[u][q].lo, o);
+        sum[u][q].add(h);
+        sum[u][q].lo = __fadd_rn(sum[u][q].lo, l);
+      }
+  if (i > 0) return;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int32_t src = f.slot_src[slot + u];
+    if (src < 0) continue;
+    // -2 pi w (H_d V + W_d) in double-floats (an FP64 operation of two lanes
+    // costs the whole warp's 19 cycles here), H_d exact in two floats
+    const float scale = -6.28318530717958647692f * f.atom_w[slot + u];
+    const dev::DFloatSum v = sum[u][0];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      dev::DFloatSum g = sum[u][d + 1];
+      g.add_product(f.H[d], v.hi);
+      g.lo = __fadd_rn(g.lo, fmaf(f.H[d], v.lo, f.H_lo[d] * v.hi));
+      f.grad[3 * (int64_t)src + d] = scale * g.value();
+    }
   }
 }
 
@@ -225,13 +290,16 @@ constexpr size_t kAdjSepMaxBytes = (size_t)32 << 30;  // A tables + partials; la
 
 // Point chunks (split over K) that minimise waves x steps per CTA plus the
 // cost of one more set of partials (written once, read once).
-int adj_sep_split(const scatter_plan_s* p, int64_t tiles, int64_t n_ksteps, size_t part_bytes) {
+// A folded plane has half the steps: its chunks may be half as long, which
+// keeps the points per chunk and with them the accumulators' truncation no
+// larger than the direct form's.
+int adj_sep_split(const scatter_plan_s* p, int64_t tiles, int64_t n_ksteps, size_t part_bytes, bool fold) {
   const double cap = (double)p->n_sm;
   const double part_steps = 2.0 * (double)part_bytes / 6.0e12 / 1.0e-6;  // ~1 us per step
   double best = 1e300;
   int best_k = 1;
   for (int k = 1; k <= 64; ++k) {
-    if (k > 1 && (double)n_ksteps / k < 64) break;
+    if (k > 1 && (double)n_ksteps / k < (fold ? 32 : 64)) break;
     const double cost = std::ceil((double)tiles * k / cap) * ((double)n_ksteps / k + 40.0) + (k - 1) * part_steps;
     if (cost < best * 0.995) {
       best = cost;
@@ -255,7 +323,12 @@ scatter_status prepare_adjoint_sep(scatter_plan_s* p) {
   if (!adjoint_sep_applicable(p)) return SCATTER_OK;
   const int64_t n0 = p->n_axis[0], n1 = p->n_axis[1], n2 = p->n_axis[2];
   const int64_t nbc = n1 * n2;
-  const int64_t n_ksteps = (nbc + kSepStep - 1) / kSepStep;
+  // fold the (k, l) plane over its middle where both axes are symmetric
+  double mid[2] = {0, 0};
+  const bool fold = sep_axis_middle(p->axis_host[1], p->inst[0].H[1], &mid[0]) &&
+                    sep_axis_middle(p->axis_host[2], p->inst[0].H[2], &mid[1]);
+  const int64_t n_k = fold ? (nbc + 1) / 2 : nbc;
+  const int64_t n_ksteps = (n_k + kSepStep - 1) / kSepStep;
   const int64_t n_mt = (2 * 3 * n0 + kSepM - 1) / kSepM;
   const int64_t n_mp = (n_mt + 1) / 2;
   // N tiles: 256 slots of one species
@@ -268,7 +341,7 @@ scatter_status prepare_adjoint_sep(scatter_plan_s* p) {
   if (ntiles.empty()) return SCATTER_OK;  // no atoms: the FP32 path writes the empty gradient
   const size_t a_bytes = (size_t)p->n_species * (size_t)n_mp * (size_t)n_ksteps * kSepPair * kSepABytes;
   const size_t part1 = (size_t)sep_part_floats(n_mt, p->n_slots) * sizeof(float);
-  const int split = adj_sep_split(p, n_mp * (int64_t)ntiles.size(), n_ksteps, part1);
+  const int split = adj_sep_split(p, n_mp * (int64_t)ntiles.size(), n_ksteps, part1, fold);
   std::vector<Segment> chunks;
   const int64_t per = (n_ksteps + split - 1) / split;
   for (int64_t b = 0; b < n_ksteps; b += per)
@@ -276,12 +349,14 @@ scatter_status prepare_adjoint_sep(scatter_plan_s* p) {
   const size_t part_bytes = chunks.size() * part1;
   if (a_bytes + part_bytes > kAdjSepMaxBytes) return SCATTER_OK;
   if (ntiles.size() * (size_t)n_mp > 0x7fffffffULL || chunks.size() > 65535) return SCATTER_OK;
-  // point records (0, s_b, s_c, 0), zero past the last point
+  // point records (0, s_b, s_c, 0), folded (0, d_b, d_c, 0), zero past the last point
   std::vector<float4> rec((size_t)n_ksteps * kSepStep, make_float4(0.f, 0.f, 0.f, 0.f));
   float smax_b = 0.f, smax_c = 0.f;
-  for (int64_t q = 0; q < nbc; ++q) {
-    const float sb = (float)(p->axis_host[1][q / n2] - p->inst[0].H[1]);
-    const float sc = (float)(p->axis_host[2][q % n2] - p->inst[0].H[2]);
+  const std::vector<double>&k64 = p->axis_host[1], &l64 = p->axis_host[2];
+  for (int64_t q = 0; q < n_k; ++q) {
+    const int64_t b = q / n2, c = q % n2;
+    const float sb = (float)(fold ? 0.5 * (k64[b] - k64[n1 - 1 - b]) : k64[b] - p->inst[0].H[1]);
+    const float sc = (float)(fold ? 0.5 * (l64[c] - l64[n2 - 1 - c]) : l64[c] - p->inst[0].H[2]);
     rec[q] = make_float4(0.f, sb, sc, 0.f);
     smax_b = std::max(smax_b, std::fabs(sb));
     smax_c = std::max(smax_c, std::fabs(sc));
@@ -311,6 +386,9 @@ scatter_status prepare_adjoint_sep(scatter_plan_s* p) {
   if (const scatter_status ss = sep_prepare_side(p, n_mt); ss != SCATTER_OK) return ss;
   p->base_bytes += (int64_t)(gf_bytes + sexp_bytes + a_bytes + part_bytes + rec.size() * sizeof(float4) +
                              (ntiles.size() + chunks.size()) * sizeof(Segment));
+  p->adj_sep_fold = fold;
+  p->adj_sep_k = n_k;
+  for (int d = 0; d < 2; ++d) p->adj_sep_mid[d] = fold ? mid[d] - p->inst[0].H[d + 1] : 0.0;
   p->adj_sep_ksteps = n_ksteps;
   p->adj_sep_mt = n_mt;
   p->adj_sep_ntiles = (int32_t)ntiles.size();
@@ -326,15 +404,16 @@ scatter_status prepare_adjoint_sep(scatter_plan_s* p) {
 scatter_status launch_adjoint_sep(scatter_plan_t p, float* grad, cudaStream_t st) {
   const int64_t n0 = p->n_axis[0], n1 = p->n_axis[1], n2 = p->n_axis[2];
   const int64_t n_mp = (p->adj_sep_mt + 1) / 2;
-  k_adj_sep_scale<<<(unsigned)(p->n_species * n0), 256, 0, st>>>(p->d.adj_gf, p->d.axis_s, n0, n1, n2, p->n_s,
-                                                                  p->d.adj_sexp);
+  k_adj_sep_scale<<<(unsigned)(p->n_species * n0), 1024, 0, st>>>(p->d.adj_gf, p->d.adj_rec, n0, n1 * n2, p->adj_sep_k,
+                                                                   p->adj_sep_fold, p->n_s, p->d.adj_sexp);
   AdjSepTabArgs t{};
   t.gf = p->d.adj_gf;
-  t.axis_s = p->d.axis_s;
+  t.rec = p->d.adj_rec;
   t.sexp = p->d.adj_sexp;
   t.n0 = n0;
-  t.n1 = n1;
-  t.n2 = n2;
+  t.nbc = n1 * n2;
+  t.n_k = p->adj_sep_k;
+  t.fold = p->adj_sep_fold;
   t.n_s = p->n_s;
   t.n_ksteps = p->adj_sep_ksteps;
   t.n_mt = p->adj_sep_mt;
@@ -363,7 +442,6 @@ scatter_status launch_adjoint_sep(scatter_plan_t p, float* grad, cudaStream_t st
   a.n_mt = p->adj_sep_mt;
   a.partial = p->d.adj_sep_partial;
   a.status = p->d.status;
-  a.flush = kSepFlush;
   dim3 grid((unsigned)(n_mp * p->adj_sep_ntiles), (unsigned)p->adj_sep_chunks);
   timing_begin(p, st);
   const cudaError_t le = sep_launch_core(a, grid, st, p->side_stream, p->side_fork, p->side_join);
@@ -377,14 +455,23 @@ scatter_status launch_adjoint_sep(scatter_plan_t p, float* grad, cudaStream_t st
   f.ntiles = p->d.adj_ntiles;
   f.sexp = p->d.adj_sexp;
   f.atom4 = p->d.atom4;
+  f.atom_lo = p->d.atom_lo;
   f.atom_w = p->d.atom_w;
   f.slot_src = p->d.slot_src;
   f.axis_s = p->d.axis_s;
   f.n0 = n0;
   f.n_slots = p->n_slots;
-  for (int d = 0; d < 3; ++d) f.H[d] = p->inst[0].H[d];
+  for (int d = 0; d < 3; ++d) {
+    const double h = p->inst[0].H[d] + (d > 0 ? p->adj_sep_mid[d - 1] : 0.0);
+    f.H[d] = (float)h;
+    f.H_lo[d] = (float)(h - (double)f.H[d]);
+  }
+  for (int d = 0; d < 2; ++d) {
+    f.mid[d] = (float)p->adj_sep_mid[d];
+    f.mid_lo[d] = (float)(p->adj_sep_mid[d] - (double)f.mid[d]);
+  }
   f.grad = grad;
-  k_adj_sep_final<<<(unsigned)p->adj_sep_ntiles, kSepN, 0, st>>>(f);
+  k_adj_sep_final<<<dim3((unsigned)p->adj_sep_ntiles, kSepN / (4 * kAdjFinalWarps)), 32 * kAdjFinalWarps, 0, st>>>(f);
   p->last_launches += 3 + sep_core_launches(p->adj_sep_mt);
   return cuda_status(cudaGetLastError(), "adjoint launch");
 }
