@@ -434,6 +434,7 @@ scatter_status launch_generic_reduce(scatter_plan_t p, int n_chunks, float2* amp
 }
 
 scatter_status launch_generic(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st) {
+  if (p->gs.active) return launch_gridsum(p, amp_out, int_out, st);
   if (p->tiling.atom_k > 0) return launch_atompar(p, amp_out, int_out, st);
   const Tiling& t = p->tiling;
   void* fn = pick_generic(mode_of(p), t.R, t.threads);

@@ -26,6 +26,16 @@ scatter_status launch_generic(scatter_plan_t p, float2* amp_out, float* int_out,
 scatter_status launch_generic_reduce(scatter_plan_t p, int n_chunks, float2* amp_out, float* int_out,
                                      cudaStream_t st);
 
+// Factorised FP32 sum on single GRID plans (gridsum.cu).
+bool gridsum_preferred(const scatter_plan_s* p);
+scatter_status prepare_gridsum(scatter_plan_s* p, int split_override);
+scatter_status launch_gridsum(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st);
+
+// Middle of an axis that is symmetric about it: |v_i + v_{n-1-i} - 2 mid| below
+// 2e-13 of its largest value (a phase error under 1e-8 cycles for crystals of
+// 1e5 cells at |S| = 1; evenly spaced axes miss by a few ulp).
+bool axis_symmetric(const std::vector<double>& v, double* mid);
+
 // Atom-parallel form of the generic sum for short S lists (atompar.cu).
 bool atompar_applicable(const scatter_plan_s* p);
 bool atompar_preferred(const scatter_plan_s* p, const Tiling& s_parallel);

@@ -312,6 +312,9 @@ extern "C" void scatter_plan_destroy(scatter_plan_t p) {
   release(d.ztab);
   release(d.sep_A);
   release(d.sep_partial);
+  release(p->gs.chunks);
+  release(p->gs.d);
+  release(p->gs.dlo);
   release(p->sep_direct.chunks);
   release(p->sep_folded.chunks);
   release(d.ap_blocks);
@@ -568,16 +571,23 @@ extern "C" scatter_status scatter_plan(const scatter_problem* pr, const scatter_
     t.split_k = op && op->split_k ? op->split_k : dwba_best_split(p.get());
     if ((st = apply_tiling(p.get(), t))) return st;
   } else if (path == SCATTER_PATH_GENERIC) {
-    Tiling t = heuristic_tiling(p.get());
+    // single grids: the factorised sum, unless the caller asks for a tile of the
+    // sincos forms or the grid is too small for it
+    const bool tile_asked = op && (op->threads || op->points_per_thread || op->atoms_per_thread > 0);
+    const bool factorised = !tile_asked && gridsum_preferred(p.get());
+    Tiling t = factorised ? Tiling{} : heuristic_tiling(p.get());
     if (op && op->threads) t.threads = op->threads;
     if (op && op->points_per_thread) t.R = op->points_per_thread;
-    if (op && op->split_k) t.split_k = op->split_k;
+    if (op && op->split_k && !factorised) t.split_k = op->split_k;
     if (op && (op->threads || op->points_per_thread || op->split_k || op->atoms_per_thread < 0)) t.atom_k = 0;
     if (op && op->atoms_per_thread > 0) t.atom_k = op->atoms_per_thread;
     if (!generic_tiling_supported(t))
       return fail(SCATTER_ERR_INVALID_ARG, "unsupported tile override (threads=%d R=%d)", t.threads, t.R);
     if ((st = apply_tiling(p.get(), t))) return st;
-    if (pr->batch > 1) {
+    if (factorised) {
+      if ((st = prepare_gridsum(p.get(), op ? op->split_k : 0))) return st;
+      if (op && op->autotune && !op->split_k && (st = autotune_gridsum(p.get(), op->tune_cache))) return st;
+    } else if (pr->batch > 1) {
       if ((st = prepare_batch(p.get()))) return st;
       if (op && op->autotune && !(op->threads || op->points_per_thread) &&
           (st = autotune_batch(p.get(), op->tune_cache)))

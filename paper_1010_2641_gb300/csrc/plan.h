@@ -86,6 +86,20 @@ struct Tiling {
 // more ranges, the less of the map's copy is left after the last reduction
 constexpr int kHostPieces = 16;
 
+// The factorised FP32 grid sum (gridsum.cu).
+struct GridSum {
+  bool active = false;
+  int q = 2, R = 1, threads = 256;  // column axis, columns and rows per thread block
+  bool mirror = false;              // the columns of a symmetric axis: half of them, each with its mirror
+  int64_t n_cols = 0, row_tiles = 0, col_tiles = 0;
+  int split = 1, n_chunks = 0;      // chunks asked for, chunks (one species each)
+  int64_t bytes = 0;                // its device memory (in tiling_bytes)
+  double mid = 0.0;                 // mirror: the axis' middle - H
+  Segment* chunks = nullptr;        // device
+  float* d = nullptr;               // device: column offsets and their rounding errors
+  float* dlo = nullptr;
+};
+
 // One form of the separable contraction: its tiles, atom chunks and launch
 // choices.  The A table and the partials are the plan's, sized for the larger.
 struct SepForm {
@@ -204,6 +218,7 @@ struct scatter_plan_s {
   double wavelength = 0, alpha_i = 0, delta = 0, beta = 0;
   int gid_mode = 0;                              // 0: on the substrate (four beams), 1: buried (one beam)
   scatter::DeviceBuffers d;
+  scatter::GridSum gs;
   int64_t base_bytes = 0;                        // tables and backward workspace
   int64_t tiling_bytes = 0;                      // chunk tables and split-K partials
   double s_max[3] = {0, 0, 0};                   // max |S - H| per axis (error model)

@@ -245,10 +245,8 @@ __device__ __forceinline__ void sep_b_fold(float sb, float sc, float sbl, float 
   }
 }
 
-// Middle of an axis that may be folded: symmetric about it, |v_i + v_{n-1-i} -
-// 2 mid| below 2e-13 of its largest value (a phase error under 1e-8 cycles for
-// crystals of 1e5 cells at |S| = 1; evenly spaced axes miss by a few ulp), and
-// the middle within a quarter of the axis' half width of H.
+// Middle of an axis that may be folded: symmetric (axis_symmetric), and the
+// middle within a quarter of the axis' half width of H.
 bool sep_axis_middle(const std::vector<double>& v, double H, double* mid);
 
 struct SepArgs {

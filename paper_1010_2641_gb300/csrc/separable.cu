@@ -835,14 +835,8 @@ __global__ void __launch_bounds__(256) k_sep_reduce_fold(const SepFoldReduceArgs
 // -------------------------------------------------------------------------
 
 bool sep_axis_middle(const std::vector<double>& v, double H, double* mid) {
-  if (v.empty()) return false;
-  double top = 1.0;
-  for (double x : v) top = std::max(top, std::fabs(x));
-  const size_t n = v.size();
-  *mid = 0.5 * (v.front() + v.back());
-  for (size_t i = 0; i < n; ++i)
-    if (std::fabs(v[i] + v[n - 1 - i] - 2.0 * *mid) > 2e-13 * top) return false;
-  return std::fabs(*mid - H) <= 0.125 * std::fabs(v.back() - v.front()) + 2e-13 * top || n == 1;
+  if (!axis_symmetric(v, mid)) return false;
+  return v.size() == 1 || std::fabs(*mid - H) <= 0.125 * std::fabs(v.back() - v.front()) + 1e-12;
 }
 
 cudaError_t sep_prepare_kernel() {

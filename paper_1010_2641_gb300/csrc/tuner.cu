@@ -193,6 +193,41 @@ scatter_status autotune_generic(scatter_plan_s* p, const char* cache_path) {
   return apply_tiling(p, best);
 }
 
+scatter_status autotune_gridsum(scatter_plan_s* p, const char* cache_path) {
+  if (p->n_s == 0 || p->n_slots == 0) return SCATTER_OK;
+  std::string key = cache_key(p);
+  key.replace(0, 7, "gridsum");
+  Tiling t;
+  if (cache_lookup(cache_path, key, &t)) return prepare_gridsum(p, t.split_k);
+  cudaEvent_t e0, e1;
+  cudaEventCreate(&e0);
+  cudaEventCreate(&e1);
+  const int start = p->gs.split;
+  double best_ms = 1e30;
+  for (int k : {start, std::max(1, start / 2), 2 * start}) {
+    if (prepare_gridsum(p, k) != SCATTER_OK) continue;
+    launch_gridsum(p, p->d.amp, nullptr, nullptr);  // warm-up
+    for (int i = 0; i < 2; ++i) {
+      cudaEventRecord(e0, nullptr);
+      launch_gridsum(p, p->d.amp, nullptr, nullptr);
+      cudaEventRecord(e1, nullptr);
+      if (cudaEventSynchronize(e1) != cudaSuccess) break;
+      float ms = 1e30f;
+      cudaEventElapsedTime(&ms, e0, e1);
+      if (ms < best_ms) {
+        best_ms = ms;
+        t.split_k = k;
+      }
+    }
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  const cudaError_t e = cudaDeviceSynchronize();
+  if (e != cudaSuccess) return cuda_status(e, "autotune");
+  cache_store(cache_path, key, t, best_ms);
+  return prepare_gridsum(p, t.split_k);
+}
+
 scatter_status autotune_batch(scatter_plan_s* p, const char* cache_path) {
   if (p->n_s == 0 || p->n_slots == 0) return SCATTER_OK;
   std::string key = cache_key(p);
