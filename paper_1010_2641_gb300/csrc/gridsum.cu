@@ -11,16 +11,21 @@
 // T - R): where the column axis is symmetric about its middle the same four
 // sums give a column and its mirror (the middle's phase joins c_j), two
 // multiply-adds per point.  All in FP32 like the sincos form (forward.cu), the
-// table's entries to ~1 ulp, the sums blocked by 64 atoms.
+// table's entries to ~1 ulp, the sums blocked by 128 atoms.
 //
 // CTA: up to 256 rows (one per thread) x R columns (in registers) x one chunk
-// of atoms of one species.  A tile of 64 atoms is staged in shared memory:
-// the rows' records (u, v, phase) and the R table entries per atom, formed by
-// the CTA itself from the atoms (64 R sincospif per 64 x 256 x R products), read
-// as broadcasts; two stages, one barrier per tile.  Bound by the FMA pipe
-// (4 R + 9 lane-operations per row and atom) and, below R = 6, by issue.
-// Strained sphere (134,009 atoms) x 61 x 47 x 33: 1.73 ms per call against 6.69 ms in
-// the sincos form; 1000 atoms x 32^3: 36 against 67 us.
+// of atoms of one species.  A tile of 128 atoms is staged in shared memory:
+// the rows' records (u, v, phase) and the R table entries per atom, read as
+// broadcasts; two stages, one barrier per tile.  On small sums the CTA forms
+// them itself from the atoms (128 R sincospif per tile and CTA: a sixth of the
+// instructions with 64 rows per CTA); on larger ones (TAB) a kernel writes them
+// once per call and the TMA engine copies them in.  Bound by issue (R = 6:
+// 33 instructions per row and atom for 12 points, 3.3 per clock).  The loop
+// is unrolled over 16 atoms: with 8 warps per SM the sincos latency is hidden
+// inside a warp (1.33 ms with 4 atoms, 1.19 ms with 16).
+// Strained sphere (134,009 atoms) x 61 x 47 x 33: 1.19 ms per call against 6.69 ms in
+// the sincos form (1.73 ms with 64 rows per CTA forming their own tables);
+// 1000 atoms x 32^3: 33 against 67 us.
 #include <cuda_runtime.h>
 #include <algorithm>
 #include <cmath>
@@ -33,8 +38,8 @@ namespace scatter {
 
 namespace {
 
-constexpr int kGsTile = 64;    // atoms per stage
-constexpr int kGsMaxR = 10;    // columns per thread
+constexpr int kGsTile = 128;   // atoms per stage
+constexpr int kGsMaxR = 8;     // columns per thread
 constexpr int kGsChunk = 32;   // chunk granularity (slots)
 
 struct GridSumArgs {
@@ -58,17 +63,51 @@ struct GridSumArgs {
   const double* shift;
   float smax[3];               // max |s| per axis, 0 for the columns' (their products are exact)
   float2* partial;             // [chunk][M], without f_s
+  // TAB: the tiles' contents, written by k_gridsum_tab
+  float4* rec;                 // [slot] (u, v, phase, 0)
+  float2* rec_lo;              // [slot] rounding errors of u, v
+  float2* ztab;                // [column tile][slot][RS]
+  int64_t n_slots;
+  unsigned* status;
 };
 
 __device__ __forceinline__ float comp(const float4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : v.z; }
 
-template <int R>
+// The record and the table entry of a slot (shared by the table kernel and the
+// CTAs that form their own tiles: the two routes agree bit for bit).
+__device__ __forceinline__ void gs_record(const GridSumArgs& a, int64_t slot, float4& rec, float2& lo2) {
+  const float4 at = a.atom4[slot], lo = a.atom_lo[slot];
+  const float q = comp(at, a.iq);
+  const float ph = dev::frac_of_product2(a.mid, a.mid_lo, q) + a.mid * comp(lo, a.iq);
+  rec = make_float4(comp(at, a.iu), comp(at, a.iv), dev::frac_rn(at.w + ph), 0.f);
+  lo2 = make_float2(comp(lo, a.iu), comp(lo, a.iv));
+}
+__device__ __forceinline__ float2 gs_entry(const GridSumArgs& a, int64_t slot, float d, float dl) {
+  const float q = comp(a.atom4[slot], a.iq), ql = comp(a.atom_lo[slot], a.iq), w = a.atom_w[slot];
+  float sn, cs;
+  sincospif(2.0f * (dev::frac_of_product2(d, dl, q) + d * ql), &sn, &cs);
+  return make_float2(w * cs, w * sn);
+}
+
+// One thread per table entry (column tile, slot, column).
+__global__ void __launch_bounds__(256) k_gridsum_tab(const GridSumArgs a, int R, int RS, int64_t total) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= total) return;
+  const int r = (int)(i % RS);
+  const int64_t slot = (i / RS) % a.n_slots, ct = i / RS / a.n_slots;
+  const int64_t c = dev::min64(ct * R + r, a.n_cols - 1);
+  a.ztab[i] = r < R ? gs_entry(a, slot, a.col_d[c], a.col_dlo[c]) : make_float2(0.f, 0.f);
+  if (ct == 0 && r == 0) gs_record(a, slot, a.rec[slot], a.rec_lo[slot]);
+}
+
+template <int R, bool TAB>
 __global__ void __launch_bounds__(256, 2) k_gridsum(const GridSumArgs a) {
   constexpr int RS = R + (R & 1);  // table row stride: 16-byte aligned
   __shared__ __align__(16) float4 sh_rec[2][kGsTile];     // (u, v, phase, 0)
   __shared__ __align__(16) float2 sh_lo[2][kGsTile];      // rounding errors of u, v (exact phases)
   __shared__ __align__(16) float2 sh_z[2][kGsTile][RS];
   __shared__ float2 sh_d[R];
+  __shared__ __align__(8) uint64_t sh_bar[2];
   using u64 = unsigned long long;
   const int tid = threadIdx.x, nt = blockDim.x;
   const int64_t row = (int64_t)blockIdx.x * nt + tid, n_rows = a.n_u * a.n_v;
@@ -83,35 +122,43 @@ __global__ void __launch_bounds__(256, 2) k_gridsum(const GridSumArgs a) {
   }
   const bool exact = dev::phase_needs_exact(a.bbox, a.shift, a.smax);
   const float sul = a.axis_lo[a.off_u + iu], svl = a.axis_lo[a.off_v + iv];
+  if (TAB && tid == 0) {
+    dev::mbar_init(&sh_bar[0], 1);
+    dev::mbar_init(&sh_bar[1], 1);
+    dev::mbar_fence_init();
+  }
   __syncthreads();
 
+  // fills a stage with the tile at slot b (TAB: thread 0 starts the copies)
   auto form = [&](int64_t b, int st) {
+    if (b >= ck.end) return;
     const int cnt = (int)dev::min64(kGsTile, ck.end - b);
-    for (int i = tid; i < cnt; i += nt) {
-      const float4 at = a.atom4[b + i], lo = a.atom_lo[b + i];
-      const float q = comp(at, a.iq);
-      const float ph = dev::frac_of_product2(a.mid, a.mid_lo, q) + a.mid * comp(lo, a.iq);
-      sh_rec[st][i] = make_float4(comp(at, a.iu), comp(at, a.iv), dev::frac_rn(at.w + ph), 0.f);
-      sh_lo[st][i] = make_float2(comp(lo, a.iu), comp(lo, a.iv));
-    }
-    for (int i = tid; i < cnt * R; i += nt) {
-      const int j = i / R, r = i % R;
-      const float q = comp(a.atom4[b + j], a.iq), ql = comp(a.atom_lo[b + j], a.iq), w = a.atom_w[b + j];
-      const float2 d = sh_d[r];
-      float sn, cs;
-      sincospif(2.0f * (dev::frac_of_product2(d.x, d.y, q) + d.x * ql), &sn, &cs);
-      sh_z[st][j][r] = make_float2(w * cs, w * sn);
+    if constexpr (TAB) {
+      if (tid != 0) return;
+      const uint32_t zb = (uint32_t)cnt * RS * (uint32_t)sizeof(float2);
+      dev::mbar_arrive_expect_tx(&sh_bar[st], zb + (uint32_t)cnt * (exact ? 24u : 16u));
+      dev::bulk_g2s(&sh_z[st][0][0], a.ztab + ((int64_t)blockIdx.y * a.n_slots + b) * RS, zb, &sh_bar[st]);
+      dev::bulk_g2s(&sh_rec[st][0], a.rec + b, (uint32_t)cnt * 16u, &sh_bar[st]);
+      if (exact) dev::bulk_g2s(&sh_lo[st][0], a.rec_lo + b, (uint32_t)cnt * 8u, &sh_bar[st]);
+    } else {
+      for (int i = tid; i < cnt; i += nt) gs_record(a, b + i, sh_rec[st][i], sh_lo[st][i]);
+      for (int i = tid; i < cnt * R; i += nt) {
+        const int j = i / R, r = i % R;
+        sh_z[st][j][r] = gs_entry(a, b + j, sh_d[r].x, sh_d[r].y);
+      }
     }
   };
 
   float tot[R][4];
 #pragma unroll
   for (int r = 0; r < R; ++r) tot[r][0] = tot[r][1] = tot[r][2] = tot[r][3] = 0.f;
-  if (ck.begin < ck.end) form(ck.begin, 0);
-  __syncthreads();
-  int st = 0;
-  for (int64_t b = ck.begin; b < ck.end; b += kGsTile, st ^= 1) {
+  form(ck.begin, 0);
+  if (TAB) form(ck.begin + kGsTile, 1);
+  if (!TAB) __syncthreads();
+  int st = 0, k = 0;
+  for (int64_t b = ck.begin; b < ck.end; b += kGsTile, st ^= 1, ++k) {
     const int cnt = (int)dev::min64(kGsTile, ck.end - b);
+    const bool ok = !TAB || dev::mbar_wait_bounded(&sh_bar[st], (uint32_t)((k >> 1) & 1));
     u64 pk[R][2];  // (P, R), (T, Q) of the tile
 #pragma unroll
     for (int r = 0; r < R; ++r) pk[r][0] = pk[r][1] = 0ull;
@@ -119,21 +166,8 @@ __global__ void __launch_bounds__(256, 2) k_gridsum(const GridSumArgs a) {
       constexpr bool kExact = decltype(exact_tag)::value;
       const float4* rec = sh_rec[st];
       const float2* rlo = sh_lo[st];
-#pragma unroll(R > 6 ? 2 : 4)
-      for (int j = 0; j < cnt; ++j) {
-        const float4 at = rec[j];
-        float f;
-        if (kExact) {
-          const float2 e = rlo[j];
-          f = dev::frac_rn(dev::frac_product2_plus(
-              su, sul, at.x, dev::frac_product2_plus(sv, svl, at.y, fmaf(su, e.x, fmaf(sv, e.y, at.z)))));
-        } else {
-          f = dev::frac_rn(fmaf(sv, at.y, fmaf(su, at.x, at.z)));
-        }
-        float er, ei;
-        dev::sincos_cycles_mufu(f, &ei, &er);
+      auto add = [&](float er, float ei, const float2* z) {
         const u64 er2 = dev::pack2(er, er), ei2 = dev::pack2(ei, ei);
-        const float2* z = sh_z[st][j];
 #pragma unroll
         for (int r = 0; r + 1 < RS; r += 2) {
           const float4 zz = *reinterpret_cast<const float4*>(z + r);
@@ -145,12 +179,42 @@ __global__ void __launch_bounds__(256, 2) k_gridsum(const GridSumArgs a) {
             dev::ffma2(pk[r + 1 < R ? r + 1 : r][1], ei2, z1);
           }
         }
+      };
+      if (kExact) {
+#pragma unroll 2
+        for (int j = 0; j < cnt; ++j) {
+          const float4 at = rec[j];
+          const float2 e = rlo[j];
+          const float f = dev::frac_rn(dev::frac_product2_plus(
+              su, sul, at.x, dev::frac_product2_plus(sv, svl, at.y, fmaf(su, e.x, fmaf(sv, e.y, at.z)))));
+          float er, ei;
+          dev::sincos_cycles_mufu(f, &ei, &er);
+          add(er, ei, sh_z[st][j]);
+        }
+      } else {
+        // two atoms' phases per packed pair (tiles hold multiples of 32 atoms)
+        const u64 su2 = dev::pack2(su, su), sv2 = dev::pack2(sv, sv);
+        const u64 magic2 = dev::pack2(12582912.0f, 12582912.0f);  // 1.5 * 2^23: rint by addition
+        const u64 twopi2 = dev::pack2(6.28318530717958647692f, 6.28318530717958647692f);
+#pragma unroll 8
+        for (int j = 0; j < cnt; j += 2) {
+          const float4 p0 = rec[j], p1 = rec[j + 1];
+          const u64 ph = dev::fma2(sv2, dev::pack2(p0.y, p1.y),
+                                   dev::fma2(su2, dev::pack2(p0.x, p1.x), dev::pack2(p0.z, p1.z)));
+          const u64 f = dev::sub2(ph, dev::sub2(dev::add2(ph, magic2), magic2));  // ph - rint(ph)
+          float t0, t1;
+          dev::unpack2(dev::mul2(f, twopi2), t0, t1);
+          add(__cosf(t0), __sinf(t0), sh_z[st][j]);
+          add(__cosf(t1), __sinf(t1), sh_z[st][j + 1]);
+        }
       }
     };
-    if (exact)
-      tile(std::true_type{});
-    else
-      tile(std::false_type{});
+    if (ok) {
+      if (exact)
+        tile(std::true_type{});
+      else
+        tile(std::false_type{});
+    }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       float P, Rr, T, Q;
@@ -161,8 +225,21 @@ __global__ void __launch_bounds__(256, 2) k_gridsum(const GridSumArgs a) {
       tot[r][2] += P + Q;  // E conj(Z)
       tot[r][3] += T - Rr;
     }
-    if (b + kGsTile < ck.end) form(b + kGsTile, st ^ 1);
-    __syncthreads();
+    if constexpr (TAB) {
+      if (__syncthreads_or(!ok)) {
+        if (tid == 0) {
+          dev::set_status(a.status, kStatusTimeout);
+          // drain the copies still in flight (bounded): this stage's and the next one's
+          dev::mbar_wait_bounded(&sh_bar[st], (uint32_t)((k >> 1) & 1), 1LL << 28);
+          if (b + kGsTile < ck.end) dev::mbar_wait_bounded(&sh_bar[st ^ 1], (uint32_t)(((k + 1) >> 1) & 1), 1LL << 28);
+        }
+        return;
+      }
+      form(b + 2 * kGsTile, st);
+    } else {
+      form(b + kGsTile, st ^ 1);
+      __syncthreads();
+    }
   }
   if (!row_ok) return;
   float2* out = a.partial + (int64_t)blockIdx.z * a.n_s + iu * a.st_u + iv * a.st_v;
@@ -234,22 +311,26 @@ __global__ void __launch_bounds__(128) k_gridsum_reduce(const GridSumReduce a) {
 
 using GridSumFn = void (*)(const GridSumArgs);
 template <int R>
-GridSumFn pick(int r) {
+GridSumFn pick(int r, bool tab) {
   if constexpr (R == 0)
     return nullptr;
   else
-    return r == R ? (GridSumFn)k_gridsum<R> : pick<R - 1>(r);
+    return r != R ? pick<R - 1>(r, tab) : tab ? (GridSumFn)k_gridsum<R, true> : (GridSumFn)k_gridsum<R, false>;
 }
 
-// Issue slots (or FMA-pipe slots, whichever is more) of one warp and atom with
-// R columns: 9 FMA-pipe operations and ~16 instructions for E, four FMA lanes
-// and 2.5 instructions per column.
-double warp_cost(int R) { return std::max(16.0 + 2.5 * R, 9.0 + 4.0 * R) + 2.0; }
+// SM clocks per warp and atom with R columns, measured on the strained sphere's
+// 61 x 47 x 33 map (8 to 16 warps per SM): R = 6 is the cheapest per column, at
+// 33 instructions in 10 clocks; more columns leave too few registers for the
+// unrolled loop, fewer repeat the row's sincos, odd ones split a 16-byte read.
+double warp_cost(int R) {
+  static const double c[kGsMaxR + 1] = {0.0, 5.2, 6.4, 7.9, 8.0, 9.0, 10.0, 11.4, 14.1};
+  return c[R];
+}
 
 struct Shape {
   int q = 2, R = 1, threads = 256;
   bool mirror = false;
-  double cost = 1e300;  // slots per atom over the whole grid
+  double cost = 1e300;  // SM clocks per atom over the whole grid
 };
 
 Shape best_shape(const scatter_plan_s* p) {
@@ -282,22 +363,25 @@ bool axis_symmetric(const std::vector<double>& v, double* mid) {
   return true;
 }
 
-// The sincos forms spend 16 MUFU slots per 32 (atom, point) pairs; the
-// factorised form is taken where its slots, rows and columns padded, are at
-// most 7/8 of that: everything but a handful of points, or single lines
+// The sincos forms spend 4 SM clocks per 32 (atom, point) pairs on the MUFU pipe;
+// the factorised form is taken where its clocks, rows and columns padded, are
+// at most 7/8 of that: everything but a handful of points, or single lines
 // shorter than a warp.
 bool gridsum_preferred(const scatter_plan_s* p) {
   if (p->s_kind != SCATTER_S_GRID || p->batch != 1 || p->n_s <= 0) return false;
-  return best_shape(p).cost < 0.875 * 16.0 * std::ceil((double)p->n_s / 32.0);
+  return best_shape(p).cost < 0.875 * 4.0 * std::ceil((double)p->n_s / 32.0);
 }
 
 scatter_status prepare_gridsum(scatter_plan_s* p, int split_override) {
   const Shape sh = best_shape(p);
   GridSum& g = p->gs;
-  for (void* b : {(void*)g.chunks, (void*)g.d, (void*)g.dlo, (void*)p->d.partial})  // of an earlier split (autotuning)
+  for (void* b : {(void*)g.chunks, (void*)g.d, (void*)g.dlo, (void*)g.rec, (void*)g.rec_lo, (void*)g.ztab,
+                  (void*)p->d.partial})  // of an earlier split (autotuning)
     if (b) cudaFree(b);
   g.chunks = nullptr;
   g.d = g.dlo = nullptr;
+  g.rec = nullptr;
+  g.rec_lo = g.ztab = nullptr;
   p->d.partial = nullptr;
   g.q = sh.q;
   g.R = sh.R;
@@ -307,7 +391,14 @@ scatter_status prepare_gridsum(scatter_plan_s* p, int split_override) {
   g.n_cols = sh.mirror ? (n + 1) / 2 : n;
   g.row_tiles = (rows + sh.threads - 1) / sh.threads;
   g.col_tiles = (g.n_cols + sh.R - 1) / sh.R;
-  GridSumFn fn = pick<kGsMaxR>(sh.R);
+  // The table where forming the tiles in every CTA (~45 instructions per entry)
+  // would cost more than its launch, a few us, and it stays below 2 GiB.
+  const double all_s = sh.cost * (double)p->n_slots / (2.0e9 * p->n_sm);
+  const double form = 14.0 * sh.R / (sh.threads * warp_cost(sh.R));  // of that, 45 instructions at ~3.3 per clock
+  const int RS = sh.R + (sh.R & 1);
+  const size_t zb = (size_t)g.col_tiles * (size_t)p->n_slots * RS * sizeof(float2);
+  g.tab = all_s * form > 8.0e-6 && zb <= (size_t)2 << 30;
+  GridSumFn fn = pick<kGsMaxR>(sh.R, g.tab);
   int per_sm = 1;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, sh.threads, 0) != cudaSuccess || per_sm < 1) {
     cudaGetLastError();
@@ -316,14 +407,30 @@ scatter_status prepare_gridsum(scatter_plan_s* p, int split_override) {
   // atom chunks: the split that minimises waves x atoms per CTA, with ~1.5 us of
   // fixed cost per CTA and the partials' write and read
   const double cap = (double)p->n_sm * per_sm, tiles = (double)(g.row_tiles * g.col_tiles);
-  const double slots = (double)std::max<int64_t>(p->n_slots, 1);
   const double clk = 2.0e9, warps = sh.threads / 32.0;
+  int64_t total = 0;
+  for (const Segment& sg : p->all_segs) total += (sg.end - sg.begin) / kGsChunk;
+  // steps per chunk and chunks of a species segment of `steps` steps for a split k
+  auto pieces = [&](int64_t steps, int k, int64_t& per) {
+    const int64_t n = std::max<int64_t>(1, std::llround((double)k * (double)steps / (double)total));
+    per = (steps + n - 1) / n;
+    return (steps + per - 1) / per;
+  };
   auto cost = [&](int k) {
-    const double ctas = tiles * k, waves = std::ceil(ctas / cap);
+    int64_t n = 0, longest = 1;
+    for (const Segment& sg : p->all_segs) {
+      int64_t per = 0;
+      n += pieces((sg.end - sg.begin) / kGsChunk, k, per);
+      longest = std::max(longest, per);
+    }
+    const double ctas = tiles * (double)n, waves = std::ceil(ctas / cap);
     const double resident = std::min(per_sm * 1.0, std::max(1.0, ctas / p->n_sm));
-    const double rate = std::min(3.4, 0.22 * warps * resident);  // slots per clock and SM: latency-bound with few warps
+    // latency-bound with few warps: full rate from 16 per SM on (1.43 ms with 12,
+    // 1.19 ms with 16 on that map); the reduction reads eight chunks at a time
+    const double rate = std::min(1.0, warps * resident / 16.0);
     const double atom = warp_cost(sh.R) * warps * resident / rate / clk;
-    return waves * (slots / k * atom + 1.5e-6) + (double)k * (double)p->n_s * 16.0 / 3.0e12;
+    return waves * ((double)(longest * kGsChunk) * atom + 1.5e-6) +
+           (double)n * ((double)p->n_s * 16.0 / 3.0e12 + 3.0e-7);
   };
   int split = 1;
   if (split_override > 0) {
@@ -338,13 +445,11 @@ scatter_status prepare_gridsum(scatter_plan_s* p, int split_override) {
       }
   }
   std::vector<Segment> chunks;
-  int64_t total = 0;
-  for (const Segment& sg : p->all_segs) total += (sg.end - sg.begin) / kGsChunk;
   for (const Segment& sg : p->all_segs) {
     const int64_t steps = (sg.end - sg.begin) / kGsChunk;
     if (steps <= 0) continue;
-    const int64_t k = std::max<int64_t>(1, std::llround((double)split * (double)steps / (double)total));
-    const int64_t per = (steps + k - 1) / k;
+    int64_t per = 0;
+    pieces(steps, split, per);
     for (int64_t b = 0; b < steps; b += per)
       chunks.push_back(Segment{sg.begin + b * kGsChunk, sg.begin + std::min(steps, b + per) * kGsChunk, sg.species, 0});
   }
@@ -375,8 +480,16 @@ scatter_status prepare_gridsum(scatter_plan_s* p, int split_override) {
       (e = cudaMemcpy(g.dlo, dl.data(), db, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(g.chunks, chunks.data(), cb, cudaMemcpyHostToDevice)) != cudaSuccess)
     return cuda_status(e, "grid sum tables");
-  p->tiling_bytes += (int64_t)(2 * db + cb + pb) - g.bytes;
-  g.bytes = (int64_t)(2 * db + cb + pb);
+  size_t tb = 0;
+  if (g.tab) {
+    const size_t n4 = (size_t)p->n_slots * sizeof(float4), n2 = (size_t)p->n_slots * sizeof(float2);
+    if ((e = cudaMalloc(&g.rec, n4)) != cudaSuccess || (e = cudaMalloc(&g.rec_lo, n2)) != cudaSuccess ||
+        (e = cudaMalloc(&g.ztab, zb)) != cudaSuccess)
+      return cuda_status(e, "cudaMalloc grid sum table");
+    tb = n4 + n2 + zb;
+  }
+  p->tiling_bytes += (int64_t)(2 * db + cb + pb + tb) - g.bytes;
+  g.bytes = (int64_t)(2 * db + cb + pb + tb);
   g.split = split;
   p->tiling.threads = sh.threads;
   p->tiling.R = sh.R * (sh.mirror ? 2 : 1);
@@ -419,8 +532,19 @@ scatter_status launch_gridsum(scatter_plan_t p, float2* amp_out, float* int_out,
   a.shift = p->d.inst_shift;
   for (int d = 0; d < 3; ++d) a.smax[d] = d == g.q ? 0.f : (float)p->s_max[d];
   a.partial = p->d.partial;
+  a.rec = g.rec;
+  a.rec_lo = g.rec_lo;
+  a.ztab = g.ztab;
+  a.n_slots = p->n_slots;
+  a.status = p->d.status;
+  if (g.tab) {
+    const int RS = g.R + (g.R & 1);
+    const int64_t total = g.col_tiles * p->n_slots * RS;
+    k_gridsum_tab<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(a, g.R, RS, total);
+    p->last_launches += 1;
+  }
   timing_begin(p, st);
-  pick<kGsMaxR>(g.R)<<<dim3((unsigned)g.row_tiles, (unsigned)g.col_tiles, (unsigned)g.n_chunks), g.threads, 0, st>>>(a);
+  pick<kGsMaxR>(g.R, g.tab)<<<dim3((unsigned)g.row_tiles, (unsigned)g.col_tiles, (unsigned)g.n_chunks), g.threads, 0, st>>>(a);
   timing_end(p, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_status(e, "grid sum launch");

@@ -315,6 +315,9 @@ extern "C" void scatter_plan_destroy(scatter_plan_t p) {
   release(p->gs.chunks);
   release(p->gs.d);
   release(p->gs.dlo);
+  release(p->gs.rec);
+  release(p->gs.rec_lo);
+  release(p->gs.ztab);
   release(p->sep_direct.chunks);
   release(p->sep_folded.chunks);
   release(d.ap_blocks);

@@ -98,6 +98,10 @@ struct GridSum {
   Segment* chunks = nullptr;        // device
   float* d = nullptr;               // device: column offsets and their rounding errors
   float* dlo = nullptr;
+  bool tab = false;                 // records and column factors tabulated per call (device below)
+  float4* rec = nullptr;
+  float2* rec_lo = nullptr;
+  float2* ztab = nullptr;
 };
 
 // One form of the separable contraction: its tiles, atom chunks and launch

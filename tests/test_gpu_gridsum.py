@@ -1,8 +1,8 @@
 """The factorised FP32 grid sum against the oracle: each axis as the columns,
-one to ten columns per thread with and without mirror columns and middles,
+one to eight columns per thread with and without mirror columns and middles,
 rows below and past a block, several species, occupancies, chunks, off-centre
 crystals, exact phases, factor tables, no atoms.  Tolerance 1e-5: MUFU
-sin/cos (2^-21 absolute per term) and FP32 sums blocked by 64 atoms, ten times
+sin/cos (2^-21 absolute per term) and FP32 sums blocked by 128 atoms, ten times
 inside the FP32 paths' 1e-4."""
 import numpy as np
 import pytest
