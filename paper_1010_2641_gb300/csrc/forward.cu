@@ -38,116 +38,267 @@ __global__ void k_bbox_init(unsigned long long* bbox, int batch) {
   if (i < batch * 6) bbox[i] = (i % 6) < 3 ? ~0ULL : 0ULL;  // min slots: max value; max slots: 0
 }
 
-// One grid row per instance; each CTA reduces a strided share of the
-// instance's atoms and merges with order-independent atomic min/max.
-__global__ void k_bbox(const double* __restrict__ xyz, const int64_t* __restrict__ atom_off,
-                       unsigned long long* bbox, unsigned* status) {
-  const int inst = blockIdx.y;
-  const int64_t b = atom_off[inst], e = atom_off[inst + 1];
-  double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-  bool bad = false;
-  for (int64_t j = b + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < e;
-       j += (int64_t)gridDim.x * blockDim.x) {
+// Bounding box as ordered integers: min xyz, max xyz.  GB300 issues FP64 (its
+// comparisons too) at ~2 operations per SM and clock, so the coordinates are
+// compared as order-preserving 64-bit integers and tested for Inf / NaN by
+// their exponent bits.
+struct Box {
+  unsigned long long v[6] = {~0ULL, ~0ULL, ~0ULL, 0ULL, 0ULL, 0ULL};
+  __device__ __forceinline__ void add(const double* p, bool& bad) {
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const double v = xyz[3 * j + d];
-      if (!isfinite(v)) {
+      const double x = p[d];
+      if ((__double2hiint(x) & 0x7ff00000) == 0x7ff00000) {
         bad = true;
         continue;
       }
-      lo[d] = fmin(lo[d], v);
-      hi[d] = fmax(hi[d], v);
+      const unsigned long long u = ordered(x);
+      v[d] = min(v[d], u);
+      v[3 + d] = max(v[3 + d], u);
     }
   }
-  if (bad) dev::set_status(status, kStatusNonFinite);
-  __shared__ double sh[6][32];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    for (int o = 16; o > 0; o >>= 1) {
-      lo[d] = fmin(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
-      hi[d] = fmax(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
-    }
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  if (lane == 0) {
+  __device__ __forceinline__ void join(const unsigned long long* o) {
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      sh[d][warp] = lo[d];
-      sh[3 + d][warp] = hi[d];
+      v[d] = min(v[d], o[d]);
+      v[3 + d] = max(v[3 + d], o[3 + d]);
     }
   }
-  __syncthreads();
-  if (threadIdx.x < 6) {
-    const int d = threadIdx.x;
-    double v = sh[d][0];
-    for (int w = 1; w < nw; ++w) v = d < 3 ? fmin(v, sh[d][w]) : fmax(v, sh[d][w]);
-    if (isfinite(v)) {
-      if (d < 3) atomicMin(&bbox[6 * inst + d], ordered(v));
-      else atomicMax(&bbox[6 * inst + d], ordered(v));
+  // the block's box in thread d < 6 (value d), 256 threads
+  __device__ __forceinline__ unsigned long long reduce(unsigned long long (*sh)[8]) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long q = __shfl_xor_sync(0xffffffffu, v[d], o);
+        v[d] = d < 3 ? min(v[d], q) : max(v[d], q);
+      }
+      if (lane == 0) sh[d][warp] = v[d];
     }
+    __syncthreads();
+    unsigned long long r = 0;
+    if (threadIdx.x < 6) {
+      r = sh[threadIdx.x][0];
+#pragma unroll
+      for (int w = 1; w < 8; ++w) r = threadIdx.x < 3 ? min(r, sh[threadIdx.x][w]) : max(r, sh[threadIdx.x][w]);
+    }
+    return r;
+  }
+};
+
+// One grid row per instance; each CTA reduces a strided share of the
+// instance's atoms and merges with order-independent atomic min/max.
+__global__ void __launch_bounds__(256) k_bbox(const double* __restrict__ xyz, const int64_t* __restrict__ atom_off,
+                                              unsigned long long* bbox, unsigned* status) {
+  __shared__ unsigned long long sh[6][8];
+  const int inst = blockIdx.y;
+  const int64_t b = atom_off[inst], e = atom_off[inst + 1];
+  Box box;
+  bool bad = false;
+  for (int64_t j = b + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < e; j += (int64_t)gridDim.x * blockDim.x)
+    box.add(xyz + 3 * j, bad);
+  if (bad) dev::set_status(status, kStatusNonFinite);
+  const unsigned long long r = box.reduce(sh);
+  if (threadIdx.x < 3 && r != ~0ULL) atomicMin(&bbox[6 * inst + threadIdx.x], r);
+  if (threadIdx.x >= 3 && threadIdx.x < 6 && r != 0ULL) atomicMax(&bbox[6 * inst + threadIdx.x], r);
+}
+
+// One instance: the box of each CTA's share of the atoms, joined by k_prep_one.
+__global__ void __launch_bounds__(256) k_box_part(const double* __restrict__ xyz, int64_t n_atoms,
+                                                  unsigned long long* __restrict__ part, unsigned* status) {
+  __shared__ unsigned long long sh[6][8];
+  Box box;
+  bool bad = false;
+#pragma unroll 4
+  for (int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x; j < n_atoms; j += (int64_t)gridDim.x * 256)
+    box.add(xyz + 3 * j, bad);
+  if (bad) dev::set_status(status, kStatusNonFinite);
+  const unsigned long long r = box.reduce(sh);
+  if (threadIdx.x < 6) part[6 * (int64_t)blockIdx.x + threadIdx.x] = r;
+}
+
+struct PrepArgs {
+  const double* xyz;
+  const float* occ;
+  const int32_t* slot_src;
+  const double* inst_H;   // [batch][3]
+  float4* atom4;
+  float4* atom_lo;
+  float* atom_w;
+  unsigned* status;
+  float4* rec_a;          // the folded separable forward's A records, or null
+  float mid[3], mid_lo[3];  // middles of its axes - H
+};
+
+// a + b with its rounding error
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+  return s;
+}
+
+// One coordinate: r = x - t as a double-float x0 + lo and its distance
+// delta = r - rint(r) as dh + dl.  Below 2^19 cells in 64-bit fixed point
+// (2^-42 cells: what FP64 holds at 2^10 cells, four decades below what the
+// double-float keeps of a centred position), with integer and FP32
+// operations only; beyond, in FP64.
+__device__ __forceinline__ void prep_coord(double x, double t, float& x0, float& lo, float& dh, float& dl) {
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+  if (e < 1023 + 19 && fabsf((float)t) < 524288.0f) {
+    const unsigned long long m =
+        ((unsigned long long)__double_as_longlong(x) & 0xfffffffffffffULL) | (e ? 0x10000000000000ULL : 0ULL);
+    const int sh = e - (1075 - 42);  // x = m 2^(e - 1075)
+    unsigned long long mag = 0ULL;
+    if (sh >= 0)
+      mag = m << sh;
+    else if (sh > -64)
+      mag = ((m >> (-sh - 1)) + 1ULL) >> 1;
+    const long long r = (hi < 0 ? -(long long)mag : (long long)mag) - ((long long)(int)t << 42);
+    const int n = (int)((r + (1LL << 41)) >> 42);
+    const long long d = r - ((long long)n << 42);  // [-2^41, 2^41)
+    dh = (float)(int)(d >> 18) * 5.9604644775390625e-08f;                 // 24 bits, 2^-24
+    dl = (float)(int)(d & 0x3ffffLL) * 2.2737367544323206e-13f;           // 18 bits, 2^-42
+    float err;
+    x0 = two_sum((float)n, dh, err);
+    lo = err + dl;
+  } else {
+    const double r = x - t, d = r - rint(r);
+    x0 = (float)r;
+    lo = (float)(r - (double)x0);
+    dh = (float)d;
+    dl = (float)(d - (double)dh);
   }
 }
 
-__global__ void k_prep(const double* __restrict__ xyz, const float* __restrict__ occ,
-                       const int32_t* __restrict__ slot_src, const int32_t* __restrict__ slot_inst,
-                       const int64_t* __restrict__ inst_slot_begin, const double* __restrict__ inst_H,
-                       const unsigned long long* __restrict__ bbox, double* inst_shift, float4* atom4,
-                       float4* atom_lo, float* atom_w, int64_t n_slots, unsigned* status, float4* rec_a,
-                       double mid0, double mid1, double mid2) {
+// The slot's records from its atom centred on t: (x', y', z', c), rounding
+// errors, occupancy; c = frac(H . delta) from exact products and TwoSums, one
+// rounding at the end as in FP64.
+// H: the instance's reflection, h the same in FP32.
+__device__ __forceinline__ void prep_slot(const PrepArgs& a, int64_t slot, const double (&t)[3], const double* H,
+                                          const float (&h)[3]) {
+  const int32_t src = a.slot_src[slot];
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  bool ok = src >= 0;
+  double x[3] = {0.0, 0.0, 0.0};
+  float w = 0.f;
+  if (ok) {
+    const double* p = a.xyz + 3 * (int64_t)src;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      x[d] = p[d];
+      ok = ok && (__double2hiint(x[d]) & 0x7ff00000) != 0x7ff00000;
+    }
+    w = a.occ ? a.occ[src] : 1.0f;
+    ok = ok && isfinite(w);
+    if (!ok) dev::set_status(a.status, kStatusNonFinite);
+  }
+  if (!ok) {
+    a.atom4[slot] = zero;
+    a.atom_lo[slot] = zero;
+    a.atom_w[slot] = 0.f;
+    if (a.rec_a) a.rec_a[slot] = zero;
+    return;
+  }
+  float x0[3], lo[3], c = 0.f, ce = 0.f;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    float dh, dl, err;
+    prep_coord(x[d], t[d], x0[d], lo[d], dh, dl);
+    if (fabsf(h[d]) < 4194304.0f) {  // exact in FP32
+      const float pr = __fmul_rn(h[d], dh);
+      c = two_sum(c, __fsub_rn(pr, rintf(pr)), err);
+      ce += err + (fmaf(h[d], dh, -pr) + h[d] * dl);
+    } else {
+      const double ph = H[d] * ((double)dh + (double)dl);
+      c = two_sum(c, (float)(ph - rint(ph)), err);
+      ce += err;
+    }
+  }
+  float err;
+  const float cr = c - rintf(c);  // exact
+  c = cr + ce;
+  a.atom4[slot] = make_float4(x0[0], x0[1], x0[2], c);
+  a.atom_lo[slot] = make_float4(lo[0], lo[1], lo[2], 0.f);
+  a.atom_w[slot] = w;
+  if (a.rec_a) {
+    // the folded forward's A record: x' as a double-float and W = w e^{2 pi i (c + (mid - H).x')}
+    float ph = cr, pe = ce;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const float pr = __fmul_rn(a.mid[d], x0[d]);
+      ph = two_sum(ph, pr - rintf(pr), err);
+      pe += err + (fmaf(a.mid[d], x0[d], -pr) + fmaf(a.mid_lo[d], x0[d], a.mid[d] * lo[d]));
+    }
+    float sn, cs;
+    sincospif(2.0f * ((ph - rintf(ph)) + pe), &sn, &cs);
+    a.rec_a[slot] = make_float4(x0[0], lo[0], w * cs, w * sn);
+  }
+}
+
+__device__ __forceinline__ double centre(unsigned long long ulo, unsigned long long uhi) {
+  return (ulo == ~0ULL || uhi == 0ULL) ? 0.0 : rint(0.5 * (unordered(ulo) + unordered(uhi)));
+}
+
+// Batches: one thread per slot, each instance's box in `bbox`.
+__global__ void __launch_bounds__(256) k_prep(const PrepArgs a, const int32_t* __restrict__ slot_inst,
+                                              const int64_t* __restrict__ inst_slot_begin,
+                                              const unsigned long long* __restrict__ bbox, double* inst_shift,
+                                              int64_t n_slots) {
   const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (slot >= n_slots) return;
   const int inst = slot_inst[slot];
   double t[3];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const unsigned long long ulo = bbox[6 * inst + d], uhi = bbox[6 * inst + 3 + d];
-    t[d] = (ulo == ~0ULL || uhi == 0ULL) ? 0.0 : rint(0.5 * (unordered(ulo) + unordered(uhi)));
-  }
+  for (int d = 0; d < 3; ++d) t[d] = centre(bbox[6 * inst + d], bbox[6 * inst + 3 + d]);
   if (slot == inst_slot_begin[inst]) {
 #pragma unroll
     for (int d = 0; d < 3; ++d) inst_shift[3 * inst + d] = t[d];
   }
-  const int32_t src = slot_src[slot];
-  if (src < 0) {
-    atom4[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
-    atom_lo[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
-    atom_w[slot] = 0.f;
-    if (rec_a) rec_a[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
-    return;
+  const double* H = a.inst_H + 3 * inst;
+  const float h[3] = {(float)H[0], (float)H[1], (float)H[2]};
+  prep_slot(a, slot, t, H, h);
+}
+
+// One instance, one launch after the boxes: every CTA joins the n_part partial
+// boxes (n_part = 0: takes the box of all the atoms itself, for small
+// crystals), then prepares its share of the slots.  1e6 atoms: 9.6 us for
+// the boxes and ~35 us here, from 63 + 76 us and an initialising launch when
+// the comparisons and the split ran in FP64; 4 CTAs per SM, each joining 256
+// boxes, measured 5 us less than 8 joining 512.
+__global__ void __launch_bounds__(256) k_prep_one(const PrepArgs a, int64_t n_atoms, int64_t n_slots,
+                                                  const unsigned long long* __restrict__ part, int n_part,
+                                                  unsigned long long* bbox, double* inst_shift) {
+  __shared__ unsigned long long sh[6][8];
+  __shared__ unsigned long long sh_box[6];
+  __shared__ double sh_t[3];
+  __shared__ float sh_h[3];
+  Box box;
+  if (n_part > 0) {
+    for (int i = threadIdx.x; i < n_part; i += 256) box.join(part + 6 * (int64_t)i);
+  } else {
+    bool bad = false;
+#pragma unroll 4
+    for (int64_t j = threadIdx.x; j < n_atoms; j += 256) box.add(a.xyz + 3 * j, bad);
+    if (bad && blockIdx.x == 0) dev::set_status(a.status, kStatusNonFinite);
   }
-  const double* H = inst_H + 3 * inst;
-  double r[3];
-  bool ok = true;
-  double c = 0.0;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    r[d] = xyz[3 * (int64_t)src + d] - t[d];
-    ok = ok && isfinite(r[d]);
-    const double delta = r[d] - rint(r[d]);
-    c = fma(H[d], delta, c);
+  const unsigned long long r = box.reduce(sh);
+  if (threadIdx.x < 6) {
+    sh_box[threadIdx.x] = r;
+    if (blockIdx.x == 0) bbox[threadIdx.x] = r;
   }
-  float w = occ ? occ[src] : 1.0f;
-  ok = ok && isfinite(w);
-  if (!ok) {
-    dev::set_status(status, kStatusNonFinite);
-    atom4[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
-    atom_lo[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
-    atom_w[slot] = 0.f;
-    if (rec_a) rec_a[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
-    return;
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    const double t = centre(sh_box[threadIdx.x], sh_box[3 + threadIdx.x]);
+    sh_t[threadIdx.x] = t;
+    sh_h[threadIdx.x] = (float)a.inst_H[threadIdx.x];
+    if (blockIdx.x == 0) inst_shift[threadIdx.x] = t;
   }
-  c -= rint(c);
-  const float x0 = (float)r[0], x1 = (float)r[1], x2 = (float)r[2];
-  atom4[slot] = make_float4(x0, x1, x2, (float)c);
-  atom_lo[slot] = make_float4((float)(r[0] - (double)x0), (float)(r[1] - (double)x1), (float)(r[2] - (double)x2), 0.f);
-  atom_w[slot] = w;
-  if (rec_a) {
-    // the folded forward's A record: x' as a double-float and W = w e^{2 pi i (c + (mid - H).x')}
-    const double ph = fma(mid2, r[2], fma(mid1, r[1], fma(mid0, r[0], c)));
-    float sn, cs;
-    sincospif(2.0f * (float)(ph - rint(ph)), &sn, &cs);
-    rec_a[slot] = make_float4(x0, (float)(r[0] - (double)x0), w * cs, w * sn);
-  }
+  __syncthreads();
+  const double t[3] = {sh_t[0], sh_t[1], sh_t[2]};
+  const float h[3] = {sh_h[0], sh_h[1], sh_h[2]};
+  for (int64_t slot = (int64_t)blockIdx.x * 256 + threadIdx.x; slot < n_slots; slot += (int64_t)gridDim.x * 256)
+    prep_slot(a, slot, t, a.inst_H, h);
 }
 
 // ---------------------------------------------------------------------------
@@ -395,18 +546,44 @@ int generic_blocks_per_sm(const scatter_plan_s* p, const Tiling& t) {
 
 scatter_status launch_prep(scatter_plan_t p, const double* xyz, const float* occ, cudaStream_t st) {
   const int batch = p->batch;
+  PrepArgs a{};
+  a.xyz = xyz;
+  a.occ = occ;
+  a.slot_src = p->d.slot_src;
+  a.inst_H = p->d.inst_H;
+  a.atom4 = p->d.atom4;
+  a.atom_lo = p->d.atom_lo;
+  a.atom_w = p->d.atom_w;
+  a.status = p->d.status;
+  a.rec_a = p->d.sep_rec;
+  for (int d = 0; d < 3; ++d) {
+    a.mid[d] = (float)p->sep_mid[d];
+    a.mid_lo[d] = (float)(p->sep_mid[d] - (double)a.mid[d]);
+  }
+  if (batch == 1) {
+    // up to kPrepSmall atoms every CTA takes the box of all of them itself: one launch
+    int n_part = 0;
+    if (p->n_atoms > kPrepSmall) {
+      n_part = (int)std::min<int64_t>(kPrepParts, (p->n_atoms + 511) / 512);
+      k_box_part<<<n_part, 256, 0, st>>>(xyz, p->n_atoms, p->d.box_part, p->d.status);
+      p->last_launches += 1;
+    }
+    const int64_t nb = std::min<int64_t>(std::max<int64_t>((p->n_slots + 255) / 256, 1), 4 * (int64_t)p->n_sm);
+    k_prep_one<<<(unsigned)nb, 256, 0, st>>>(a, p->n_atoms, p->n_slots, p->d.box_part, n_part, p->d.inst_bbox,
+                                             p->d.inst_shift);
+    p->last_launches += 1;
+    return cuda_status(cudaGetLastError(), "prep launch");
+  }
   k_bbox_init<<<(batch * 6 + 255) / 256, 256, 0, st>>>(p->d.inst_bbox, batch);
   p->last_launches += 2;
   int64_t max_atoms = 0;
   for (const auto& in : p->inst) max_atoms = std::max<int64_t>(max_atoms, in.atom_end - in.atom_begin);
-  const int bx = (int)dev::min64(std::max<int64_t>((max_atoms + 255) / 256, 1), 64);
+  const int bx = (int)dev::min64(std::max<int64_t>((max_atoms + 1023) / 1024, 1), 64);
   k_bbox<<<dim3(bx, batch), 256, 0, st>>>(xyz, p->d.atom_off, p->d.inst_bbox, p->d.status);
   if (p->n_slots > 0) {
     const int64_t nb = (p->n_slots + 255) / 256;
-    k_prep<<<(unsigned)nb, 256, 0, st>>>(xyz, occ, p->d.slot_src, p->d.slot_inst, p->d.inst_slot_begin,
-                                         p->d.inst_H, p->d.inst_bbox, p->d.inst_shift, p->d.atom4,
-                                         p->d.atom_lo, p->d.atom_w, p->n_slots, p->d.status, p->d.sep_rec,
-                                         p->sep_mid[0], p->sep_mid[1], p->sep_mid[2]);
+    k_prep<<<(unsigned)nb, 256, 0, st>>>(a, p->d.slot_inst, p->d.inst_slot_begin, p->d.inst_bbox, p->d.inst_shift,
+                                         p->n_slots);
     p->last_launches += 1;
   }
   return cuda_status(cudaGetLastError(), "prep launch");

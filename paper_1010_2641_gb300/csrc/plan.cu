@@ -288,6 +288,7 @@ extern "C" void scatter_plan_destroy(scatter_plan_t p) {
   release(d.inst_H);
   release(d.inst_shift);
   release(d.inst_bbox);
+  release(d.box_part);
   release(d.s_hi);
   release(d.s_lo);
   release(d.S64);
@@ -494,6 +495,7 @@ extern "C" scatter_status scatter_plan(const scatter_problem* pr, const scatter_
   if ((st = upload(&d.inst_H, inst_H.data(), inst_H.size(), &bytes))) return st;
   if ((st = upload<double>(&d.inst_shift, nullptr, 3 * (size_t)B, &bytes))) return st;
   if ((st = upload<unsigned long long>(&d.inst_bbox, nullptr, 6 * (size_t)B, &bytes))) return st;
+  if (B == 1 && (st = upload<unsigned long long>(&d.box_part, nullptr, 6 * (size_t)kPrepParts, &bytes))) return st;
   if ((st = upload<unsigned>(&d.status, nullptr, 1, &bytes))) return st;
   if ((e = cudaMemset(d.inst_shift, 0, 3 * sizeof(double) * B)) != cudaSuccess) return cuda_status(e, "memset");
   if ((e = cudaMemset(d.status, 0, sizeof(unsigned))) != cudaSuccess) return cuda_status(e, "memset");

@@ -28,6 +28,8 @@ namespace scatter {
 constexpr int kSlotAlign = 32;     // padding granularity of species segments
 constexpr int kNCoef = 12;         // a0..a3 b0..b3 c f' f'' B_dw
 constexpr int kMaxSpecies = 64;
+constexpr int kPrepParts = 256;    // partial bounding boxes of a call (single instances)
+constexpr int kPrepSmall = 4096;   // atoms up to which every CTA of the preparation takes the box itself
 constexpr int kLossParts = 1024;   // per-block partial sums of the misfit
 
 // Status bits written by kernels into plan->d_status.
@@ -134,6 +136,7 @@ struct DeviceBuffers {
   int64_t* inst_slot_begin = nullptr; // [batch]
   double* inst_H = nullptr;         // [batch][3]
   double* inst_shift = nullptr;     // [batch][3] integer centring t (per call)
+  unsigned long long* box_part = nullptr;   // [kPrepParts][6] partial boxes (single instances)
   unsigned long long* inst_bbox = nullptr;  // [batch][6] ordered-int min/max
   // S
   float* s_hi = nullptr;            // LIST: [3][M]
