@@ -434,16 +434,38 @@ __global__ void __launch_bounds__(THREADS) k_generic(const GenericArgs a) {
   }
 }
 
-// Sum of split-K partials in chunk order, translation phase, outputs.
-__global__ void k_reduce(GenericArgs a, int split_k, int grid_mode) {
-  const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= a.n_s) return;
+// Sum of split-K partials, translation phase, outputs.  GROUPS threads per
+// point, each over a contiguous share of the chunks in order, joined in order:
+// a short list with many chunks (atom-parallel blocks) fills the SMs and keeps
+// eight loads in flight per thread (1000 points x 245 blocks: 38 us with one
+// thread per point, 10.5 us with eight).
+template <int GROUPS>
+__global__ void __launch_bounds__(256) k_reduce(GenericArgs a, int split_k, int grid_mode) {
+  constexpr int kPts = 256 / GROUPS;
+  __shared__ float2 sh[GROUPS > 1 ? GROUPS - 1 : 1][kPts];
+  const int pt = threadIdx.x % kPts, grp = threadIdx.x / kPts;
+  const int64_t m = (int64_t)blockIdx.x * kPts + pt;
   float2 v = make_float2(0.f, 0.f);
-  for (int c = 0; c < split_k; ++c) {
-    const float2 p = a.partial[(int64_t)c * a.n_s + m];
-    v.x += p.x;
-    v.y += p.y;
+  if (m < a.n_s) {
+    const int per = (split_k + GROUPS - 1) / GROUPS, c1 = min(split_k, (grp + 1) * per);
+#pragma unroll 8
+    for (int c = grp * per; c < c1; ++c) {
+      const float2 p = a.partial[(int64_t)c * a.n_s + m];
+      v.x += p.x;
+      v.y += p.y;
+    }
   }
+  if constexpr (GROUPS > 1) {
+    if (grp > 0) sh[grp - 1][pt] = v;
+    __syncthreads();
+    if (grp > 0) return;
+#pragma unroll
+    for (int g = 0; g < GROUPS - 1; ++g) {
+      v.x += sh[g][pt].x;
+      v.y += sh[g][pt].y;
+    }
+  }
+  if (m >= a.n_s) return;
   const double* t = a.shift;
   if (t[0] != 0.0 || t[1] != 0.0 || t[2] != 0.0) {
     if (grid_mode) {
@@ -516,6 +538,17 @@ GenericArgs make_args(scatter_plan_t p) {
   a.ftab = p->d.ftab;
   a.status = p->d.status;
   return a;
+}
+
+}  // namespace
+
+namespace {
+
+void launch_reduce(const GenericArgs& a, int n_chunks, int grid_mode, cudaStream_t st) {
+  if (n_chunks >= 16 && a.n_s <= 65536)
+    k_reduce<8><<<(unsigned)((a.n_s + 31) / 32), 256, 0, st>>>(a, n_chunks, grid_mode);
+  else
+    k_reduce<1><<<(unsigned)((a.n_s + 255) / 256), 256, 0, st>>>(a, n_chunks, grid_mode);
 }
 
 }  // namespace
@@ -602,9 +635,8 @@ scatter_status launch_generic_reduce(scatter_plan_t p, int n_chunks, float2* amp
   a.partial = p->d.partial;
   a.out_amp = amp_out;
   a.out_int = int_out;
-  const int64_t nb = (p->n_s + 255) / 256;
-  if (nb > 0) {
-    k_reduce<<<(unsigned)nb, 256, 0, st>>>(a, n_chunks, mode_of(p) == kModeGrid);
+  if (p->n_s > 0) {
+    launch_reduce(a, n_chunks, mode_of(p) == kModeGrid, st);
     p->last_launches += 1;
   }
   return cuda_status(cudaGetLastError(), "generic reduction launch");
@@ -638,8 +670,7 @@ scatter_status launch_generic(scatter_plan_t p, float2* amp_out, float* int_out,
     a.partial = p->d.partial;
     a.out_amp = amp_out;
     a.out_int = int_out;
-    const int64_t nb = (p->n_s + 255) / 256;
-    k_reduce<<<(unsigned)nb, 256, 0, st>>>(a, n_chunks, mode_of(p) == kModeGrid);
+    launch_reduce(a, n_chunks, mode_of(p) == kModeGrid, st);
     p->last_launches += 1;
   }
   return cuda_status(cudaGetLastError(), "generic launch");
@@ -670,7 +701,7 @@ scatter_status launch_generic_args(GenericArgs a, int R, int threads, int n_chun
     a.partial = partial;
     a.out_amp = out_amp;
     a.out_int = out_int;
-    k_reduce<<<(unsigned)((a.n_s + 255) / 256), 256, 0, st>>>(a, n_chunks, 0);
+    launch_reduce(a, n_chunks, 0, st);
   }
   return cuda_status(cudaGetLastError(), "generic launch");
 }

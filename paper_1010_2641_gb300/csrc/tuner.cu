@@ -82,10 +82,13 @@ int best_split(const scatter_plan_s* p, const Tiling& shape) {
   const double n = (double)std::max<int64_t>(p->n_slots, 1);
   double best = 1e300;
   int best_k = 1;
+  // the fixed cost of a CTA in atoms; a small crystal's chunks may be a single
+  // 32-slot piece (320 atoms x 500 points: 34 us in one chunk, 9 us in 32-slot ones)
+  const double fixed = std::min(512.0, std::max(16.0, n / 16.0)), least = std::min(256.0, std::max(32.0, n / 32.0));
   for (int k = 1; k <= 64; ++k) {
-    if (k > 1 && n / k < 256) break;
+    if (k > 1 && n / k < least) break;
     const double waves = std::ceil((double)tiles * k / cap);
-    const double cost = waves * (n / k + 512.0) + (k > 1 ? 0.02 * k * (double)p->n_s / cap : 0.0);
+    const double cost = waves * (n / k + fixed) + (k > 1 ? 0.02 * k * (double)p->n_s / cap : 0.0);
     if (cost < best * 0.995) {
       best = cost;
       best_k = k;
