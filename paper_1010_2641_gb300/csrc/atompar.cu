@@ -45,6 +45,7 @@ struct ApArgs {
   float smax[3];                   // max |S_d - H_d| over the points
   float2* partial;        // [block][M]
   int tile;               // reflections per CTA (<= kApPts)
+  ClGate gate;            // clustered lists
 };
 
 // EXACT: the phase with its products' rounding errors restored and s and the
@@ -141,6 +142,7 @@ __global__ void __launch_bounds__(kApThreads, 2) k_atompar(const ApArgs a) {
   __shared__ float4 sh_s[kApPts];
   __shared__ float4 sh_slo[kApPts];  // rounding errors of sh_s (exact-product phases)
   __shared__ float2 sh_part[kApWarps][kApPts];
+  if (cl_gated(a.gate, 0)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const Segment blk = a.blocks[blockIdx.y];
   const int64_t p0 = (int64_t)blockIdx.x * a.tile;
@@ -336,10 +338,11 @@ scatter_status launch_atompar(scatter_plan_t p, float2* amp_out, float* int_out,
   a.shift = p->d.inst_shift;
   for (int d = 0; d < 3; ++d) a.smax[d] = (float)p->s_max[d];
   a.partial = p->d.partial;
+  a.gate = cluster_gate(p);
   a.tile = p->ap_tile > 0 ? p->ap_tile : kApPts;
   dim3 grid((unsigned)((p->n_s + a.tile - 1) / a.tile), (unsigned)p->ap_n_blocks);
   void* args[] = {&a};
-  timing_begin(p, st);
+  if (!p->cl.active) timing_begin(p, st);
   cudaError_t e = cudaLaunchKernel(fn, grid, dim3(kApThreads), args, 0, st);
   timing_end(p, st);
   if (e != cudaSuccess) return cuda_status(e, "atom-parallel kernel launch");

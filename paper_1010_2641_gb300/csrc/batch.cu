@@ -47,6 +47,7 @@ struct BatchArgs {
   float2* out_amp;
   float* out_int;
   unsigned* status;
+  ClGate gate;  // instances done by their clusters
 };
 
 template <int R, int THREADS>
@@ -57,6 +58,11 @@ __global__ void __launch_bounds__(THREADS) k_batch(const BatchArgs a) {
   __shared__ __align__(8) uint64_t sh_bar[2];
   __shared__ int sh_item;
   const int tid = threadIdx.x;
+  if (a.gate.rmax2) {  // every instance done: 3 us instead of a walk through the items
+    bool left = false;
+    for (int b = tid; b < a.gate.n; b += THREADS) left |= !cl_gated(a.gate, b);
+    if (!__syncthreads_or(left)) return;
+  }
   if (tid == 0) {
     dev::mbar_init(&sh_bar[0], 1);
     dev::mbar_init(&sh_bar[1], 1);
@@ -70,6 +76,7 @@ __global__ void __launch_bounds__(THREADS) k_batch(const BatchArgs a) {
     const int it = sh_item;
     if (it >= a.n_items) break;
     const BatchItem w = a.items[it];
+    if (cl_gated(a.gate, w.inst)) continue;
     const BatchInst in = a.inst[w.inst];
     float sx[R], sy[R], sz[R];
     bool valid[R];
@@ -133,7 +140,7 @@ __global__ void k_batch_reduce(const BatchArgs a, const int32_t* __restrict__ s_
   if (m >= a.n_s) return;
   const int b = s_inst[m];
   const BatchInst in = a.inst[b];
-  if (in.split <= 1) return;
+  if (in.split <= 1 || cl_gated(a.gate, b)) return;
   const int64_t M_b = in.s_end - in.s_begin;
   float2 v = make_float2(0.f, 0.f);
   for (int c = 0; c < in.split; ++c) {
@@ -322,6 +329,11 @@ scatter_status enqueue_batch_kernels(scatter_plan_t p, float2* amp, float* inten
   a.out_amp = amp;
   a.out_int = inten;
   a.status = p->d.status;
+  a.gate = cluster_gate(p);
+  if (p->cl.active) {
+    const scatter_status cs = launch_clusters(p, amp, inten, st);
+    if (cs != SCATTER_OK) return cs;
+  }
   cudaError_t e = cudaMemsetAsync(p->d.counter, 0, sizeof(int), st);
   if (e != cudaSuccess) return cuda_status(e, "counter reset");
   void* fn = pick_batch(p->tiling.R, p->tiling.threads);

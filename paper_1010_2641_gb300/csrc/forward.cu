@@ -33,8 +33,9 @@ namespace scatter {
 using dev::ordered;
 using dev::unordered;
 
-__global__ void k_bbox_init(unsigned long long* bbox, int batch) {
+__global__ void k_bbox_init(unsigned long long* bbox, int batch, unsigned* rmax2) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (rmax2 && i < batch) rmax2[i] = 0u;
   if (i < batch * 6) bbox[i] = (i % 6) < 3 ? ~0ULL : 0ULL;  // min slots: max value; max slots: 0
 }
 
@@ -106,8 +107,10 @@ __global__ void __launch_bounds__(256) k_bbox(const double* __restrict__ xyz, co
 
 // One instance: the box of each CTA's share of the atoms, joined by k_prep_one.
 __global__ void __launch_bounds__(256) k_box_part(const double* __restrict__ xyz, int64_t n_atoms,
-                                                  unsigned long long* __restrict__ part, unsigned* status) {
+                                                  unsigned long long* __restrict__ part, unsigned* status,
+                                                  unsigned* rmax2) {
   __shared__ unsigned long long sh[6][8];
+  if (rmax2 && blockIdx.x == 0 && threadIdx.x == 0) *rmax2 = 0u;
   Box box;
   bool bad = false;
 #pragma unroll 4
@@ -129,6 +132,7 @@ struct PrepArgs {
   unsigned* status;
   float4* rec_a;          // the folded separable forward's A records, or null
   float mid[3], mid_lo[3];  // middles of its axes - H
+  unsigned* rmax2;        // clustered lists: [batch] largest |x'|^2 (float bits, zeroed before), or null
 };
 
 // a + b with its rounding error
@@ -174,8 +178,8 @@ __device__ __forceinline__ void prep_coord(double x, double t, float& x0, float&
 // The slot's records from its atom centred on t: (x', y', z', c), rounding
 // errors, occupancy; c = frac(H . delta) from exact products and TwoSums, one
 // rounding at the end as in FP64.
-// H: the instance's reflection, h the same in FP32.
-__device__ __forceinline__ void prep_slot(const PrepArgs& a, int64_t slot, const double (&t)[3], const double* H,
+// H: the instance's reflection, h the same in FP32.  Returns |x'|^2.
+__device__ __forceinline__ float prep_slot(const PrepArgs& a, int64_t slot, const double (&t)[3], const double* H,
                                           const float (&h)[3]) {
   const int32_t src = a.slot_src[slot];
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -198,7 +202,7 @@ __device__ __forceinline__ void prep_slot(const PrepArgs& a, int64_t slot, const
     a.atom_lo[slot] = zero;
     a.atom_w[slot] = 0.f;
     if (a.rec_a) a.rec_a[slot] = zero;
-    return;
+    return 0.f;
   }
   float x0[3], lo[3], c = 0.f, ce = 0.f;
 #pragma unroll
@@ -234,6 +238,7 @@ __device__ __forceinline__ void prep_slot(const PrepArgs& a, int64_t slot, const
     sincospif(2.0f * ((ph - rintf(ph)) + pe), &sn, &cs);
     a.rec_a[slot] = make_float4(x0[0], lo[0], w * cs, w * sn);
   }
+  return x0[0] * x0[0] + x0[1] * x0[1] + x0[2] * x0[2];
 }
 
 __device__ __forceinline__ double centre(unsigned long long ulo, unsigned long long uhi) {
@@ -257,7 +262,15 @@ __global__ void __launch_bounds__(256) k_prep(const PrepArgs a, const int32_t* _
   }
   const double* H = a.inst_H + 3 * inst;
   const float h[3] = {(float)H[0], (float)H[1], (float)H[2]};
-  prep_slot(a, slot, t, H, h);
+  const unsigned r2 = __float_as_uint(prep_slot(a, slot, t, H, h));
+  if (a.rmax2) {  // n_slots is a multiple of 32: whole warps are here
+    if (__all_sync(0xffffffffu, inst == __shfl_sync(0xffffffffu, inst, 0))) {
+      const unsigned m = __reduce_max_sync(0xffffffffu, r2);
+      if ((threadIdx.x & 31) == 0) atomicMax(&a.rmax2[inst], m);
+    } else {
+      atomicMax(&a.rmax2[inst], r2);
+    }
+  }
 }
 
 // One instance, one launch after the boxes: every CTA joins the n_part partial
@@ -297,8 +310,13 @@ __global__ void __launch_bounds__(256) k_prep_one(const PrepArgs a, int64_t n_at
   __syncthreads();
   const double t[3] = {sh_t[0], sh_t[1], sh_t[2]};
   const float h[3] = {sh_h[0], sh_h[1], sh_h[2]};
+  unsigned r2 = 0u;  // |x'|^2 >= 0 orders as its bits
   for (int64_t slot = (int64_t)blockIdx.x * 256 + threadIdx.x; slot < n_slots; slot += (int64_t)gridDim.x * 256)
-    prep_slot(a, slot, t, a.inst_H, h);
+    r2 = max(r2, __float_as_uint(prep_slot(a, slot, t, a.inst_H, h)));
+  if (a.rmax2) {
+    r2 = __reduce_max_sync(0xffffffffu, r2);
+    if ((threadIdx.x & 31) == 0) atomicMax(a.rmax2, r2);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -312,6 +330,7 @@ __global__ void __launch_bounds__(THREADS) k_generic(const GenericArgs a) {
   __shared__ __align__(128) float sh_w[2][kTile];
   __shared__ __align__(8) uint64_t sh_bar[2];
 
+  if (cl_gated(a.gate, 0)) return;
   const int tid = threadIdx.x;
   const int chunk = blockIdx.y;
 
@@ -443,6 +462,7 @@ template <int GROUPS>
 __global__ void __launch_bounds__(256) k_reduce(GenericArgs a, int split_k, int grid_mode) {
   constexpr int kPts = 256 / GROUPS;
   __shared__ float2 sh[GROUPS > 1 ? GROUPS - 1 : 1][kPts];
+  if (cl_gated(a.gate, 0)) return;
   const int pt = threadIdx.x % kPts, grp = threadIdx.x / kPts;
   const int64_t m = (int64_t)blockIdx.x * kPts + pt;
   float2 v = make_float2(0.f, 0.f);
@@ -537,6 +557,7 @@ GenericArgs make_args(scatter_plan_t p) {
   for (int d = 0; d < 3; ++d) a.smax[d] = (float)p->s_max[d];
   a.ftab = p->d.ftab;
   a.status = p->d.status;
+  a.gate = cluster_gate(p);
   return a;
 }
 
@@ -589,6 +610,7 @@ scatter_status launch_prep(scatter_plan_t p, const double* xyz, const float* occ
   a.atom_w = p->d.atom_w;
   a.status = p->d.status;
   a.rec_a = p->d.sep_rec;
+  a.rmax2 = p->cl.active ? p->cl.rmax2 : nullptr;
   for (int d = 0; d < 3; ++d) {
     a.mid[d] = (float)p->sep_mid[d];
     a.mid_lo[d] = (float)(p->sep_mid[d] - (double)a.mid[d]);
@@ -596,9 +618,9 @@ scatter_status launch_prep(scatter_plan_t p, const double* xyz, const float* occ
   if (batch == 1) {
     // up to kPrepSmall atoms every CTA takes the box of all of them itself: one launch
     int n_part = 0;
-    if (p->n_atoms > kPrepSmall) {
+    if (p->n_atoms > kPrepSmall || a.rmax2) {
       n_part = (int)std::min<int64_t>(kPrepParts, (p->n_atoms + 511) / 512);
-      k_box_part<<<n_part, 256, 0, st>>>(xyz, p->n_atoms, p->d.box_part, p->d.status);
+      k_box_part<<<n_part, 256, 0, st>>>(xyz, p->n_atoms, p->d.box_part, p->d.status, a.rmax2);
       p->last_launches += 1;
     }
     const int64_t nb = std::min<int64_t>(std::max<int64_t>((p->n_slots + 255) / 256, 1), 4 * (int64_t)p->n_sm);
@@ -607,7 +629,7 @@ scatter_status launch_prep(scatter_plan_t p, const double* xyz, const float* occ
     p->last_launches += 1;
     return cuda_status(cudaGetLastError(), "prep launch");
   }
-  k_bbox_init<<<(batch * 6 + 255) / 256, 256, 0, st>>>(p->d.inst_bbox, batch);
+  k_bbox_init<<<(batch * 6 + 255) / 256, 256, 0, st>>>(p->d.inst_bbox, batch, a.rmax2);
   p->last_launches += 2;
   int64_t max_atoms = 0;
   for (const auto& in : p->inst) max_atoms = std::max<int64_t>(max_atoms, in.atom_end - in.atom_begin);
@@ -644,6 +666,10 @@ scatter_status launch_generic_reduce(scatter_plan_t p, int n_chunks, float2* amp
 
 scatter_status launch_generic(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st) {
   if (p->gs.active) return launch_gridsum(p, amp_out, int_out, st);
+  if (p->cl.active) {
+    const scatter_status cs = launch_clusters(p, amp_out, int_out, st);
+    if (cs != SCATTER_OK) return cs;
+  }
   if (p->tiling.atom_k > 0) return launch_atompar(p, amp_out, int_out, st);
   const Tiling& t = p->tiling;
   void* fn = pick_generic(mode_of(p), t.R, t.threads);
@@ -660,7 +686,7 @@ scatter_status launch_generic(scatter_plan_t p, float2* amp_out, float* int_out,
   if (tiles > 0 && n_chunks > 0) {
     dim3 grid((unsigned)tiles, (unsigned)n_chunks);
     void* args[] = {&a};
-    timing_begin(p, st);
+    if (!p->cl.active) timing_begin(p, st);
     cudaError_t e = cudaLaunchKernel(fn, grid, dim3(t.threads), args, 0, st);
     timing_end(p, st);
     if (e != cudaSuccess) return cuda_status(e, "generic kernel launch");

@@ -26,6 +26,50 @@ scatter_status launch_generic(scatter_plan_t p, float2* amp_out, float* int_out,
 scatter_status launch_generic_reduce(scatter_plan_t p, int n_chunks, float2* amp_out, float* int_out,
                                      cudaStream_t st);
 
+// Clustered S lists (cluster.cu).  Direct kernels skip an instance whose largest
+// |x'|^2 of the call (rmax2) is within lim2.
+struct ClArgs {
+  const ClInst* inst;
+  const unsigned* rmax2;
+  const float* rho;
+  const int32_t* exps;
+  const float* cen;
+  int64_t n_rows;
+  const float4* pt;
+  const int64_t* pt_out;
+  const ClItem* items;
+  const ClTabBlock* tab_blocks;
+  const ClRedBlock* red_blocks;
+  const ClEvalBlock* eval_blocks;
+  float* tab;
+  float2* partial;
+  float2* M;
+  const float4* atom4;
+  const float* atom_w;
+  const float* coef;
+  const float2* ftab;
+  int n_species;
+  float inv4a2;
+  const float* s_hi;
+  const double* S64;
+  int64_t n_s;
+  const double* inst_shift;
+  unsigned* status;
+  float2* out_amp;
+  float* out_int;
+};
+struct ClGate {
+  const unsigned* rmax2;  // null: no gate
+  const float* lim2;
+  int n;                  // instances
+};
+scatter_status prepare_clusters(scatter_plan_s* p, const double* s_list, double radius_hint);
+scatter_status launch_clusters(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st);
+void release_clusters(scatter_plan_s* p);
+inline ClGate cluster_gate(const scatter_plan_s* p) {
+  return p->cl.active ? ClGate{p->cl.rmax2, p->cl.lim2, p->batch} : ClGate{nullptr, nullptr, 0};
+}
+
 // Factorised FP32 sum on single GRID plans (gridsum.cu).
 bool gridsum_preferred(const scatter_plan_s* p);
 scatter_status prepare_gridsum(scatter_plan_s* p, int split_override);

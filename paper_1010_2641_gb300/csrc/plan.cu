@@ -313,6 +313,7 @@ extern "C" void scatter_plan_destroy(scatter_plan_t p) {
   release(d.ztab);
   release(d.sep_A);
   release(d.sep_partial);
+  release_clusters(p);
   release(p->gs.chunks);
   release(p->gs.d);
   release(p->gs.dlo);
@@ -605,6 +606,12 @@ extern "C" scatter_status scatter_plan(const scatter_problem* pr, const scatter_
     t.split_k = 1;
     if ((st = apply_tiling(p.get(), t))) return st;
   }
+  // lists of close points: clusters before the direct kernels, unless the caller
+  // asks for a tile of these
+  if (path == SCATTER_PATH_GENERIC && pr->s_kind == SCATTER_S_LIST &&
+      !(op && (op->threads || op->points_per_thread || op->split_k || op->atoms_per_thread > 0)) &&
+      (st = prepare_clusters(p.get(), pr->s_list, op ? op->radius_hint : 0.0)))
+    return st;
   if ((e = cudaDeviceSynchronize()) != cudaSuccess) return cuda_status(e, "plan synchronize");
   if (log_enabled())
     fprintf(stderr, "[scatter] plan: path=%d N=%lld slots=%lld M=%lld threads=%d R=%d split_k=%d atom_k=%d\n",

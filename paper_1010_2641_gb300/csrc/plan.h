@@ -88,6 +88,59 @@ struct Tiling {
 // more ranges, the less of the map's copy is left after the last reduction
 constexpr int kHostPieces = 16;
 
+// Clustered S lists (cluster.cu).
+struct ClInst {
+  int64_t slot_begin, n_slots;
+  float R[9];         // frame: xh = R x' (rows: the points' principal axes over X)
+  float lim2;         // X^2; -1: the instance is not clustered
+  int K, col0;        // columns, the first in exps and rho
+  int rows;           // clusters
+  int64_t row0;       // the first in cen
+  int64_t tab_off;    // floats into tab: [column tile][slot][32]
+  int64_t part_off;   // float2 into partial: [chunk][column][cluster]
+  int64_t m_off;      // float2 into M: [species][column][cluster]
+  uint64_t species;   // bit s: atoms of species s
+  float H[3];
+  double H64[3];
+};
+struct ClItem {
+  int32_t inst, row0, col_tile, species;
+  int64_t begin, end;  // slots within the instance
+  int64_t part;        // float2 offset of the chunk's partials
+};
+struct ClTabBlock {
+  int32_t inst;
+  int64_t slot;
+};
+struct ClRedBlock {
+  int32_t inst, species, c0, c1;  // chunks of the species
+  int64_t elem;                   // first of 32 (column, cluster) elements
+};
+struct ClEvalBlock {
+  int32_t inst, n;
+  int64_t p0;
+};
+struct ClState {
+  bool active = false;
+  ClInst* inst = nullptr;           // [batch]
+  float* lim2 = nullptr;            // [batch] X^2, -1: not clustered
+  unsigned* rmax2 = nullptr;        // [batch] this call's largest |x'|^2 (float bits)
+  float* rho = nullptr;             // per column: the relative radius from which it matters
+  int32_t* exps = nullptr;          // per column: exponents (4 bits each), |a| mod 4 at bit 12
+  float* cen = nullptr;             // [3][n_rows] cluster centres - H
+  float4* pt = nullptr;             // points by cluster: 2 pi X (s - centre) in the frame, cluster
+  int64_t* pt_out = nullptr;        // their output indices
+  ClItem* items = nullptr;
+  ClTabBlock* tab_blocks = nullptr;
+  ClRedBlock* red_blocks = nullptr;
+  ClEvalBlock* eval_blocks = nullptr;
+  float* tab = nullptr;
+  float2* partial = nullptr;
+  float2* M = nullptr;
+  int64_t n_rows = 0;
+  int n_items = 0, n_tab = 0, n_red = 0, n_eval = 0;
+};
+
 // The factorised FP32 grid sum (gridsum.cu).
 struct GridSum {
   bool active = false;
@@ -226,6 +279,7 @@ struct scatter_plan_s {
   int gid_mode = 0;                              // 0: on the substrate (four beams), 1: buried (one beam)
   scatter::DeviceBuffers d;
   scatter::GridSum gs;
+  scatter::ClState cl;
   int64_t base_bytes = 0;                        // tables and backward workspace
   int64_t tiling_bytes = 0;                      // chunk tables and split-K partials
   double s_max[3] = {0, 0, 0};                   // max |S - H| per axis (error model)
