@@ -18,6 +18,7 @@
 //                 sums per tile in FP32, outer sums in FP64 (the terms over
 //                 millions of S nearly cancel).  The exponentials are
 //                 recomputed, nothing of size N x M is stored.
+//                 Lists of close points: cluster_adjoint.cu in its place.
 // k_adjoint_final sums the S-chunk partials in a fixed order, scales by
 //                 -2 pi w_j and writes the caller's atom order.
 #include <cuda_runtime.h>
@@ -26,6 +27,7 @@
 #include <vector>
 #include <type_traits>
 #include "device_common.cuh"
+#include "generic_impl.cuh"
 #include "launch.h"
 
 namespace scatter {
@@ -57,6 +59,7 @@ struct LossArgs {
   float4* table;          // [n_species][M][2] (layout 0), [n_species][M] (layout 1)
   float2* gf;             // [n_species][M] (layout 2)
   double* loss_part;      // [gridDim.x]
+  ClGate gate;            // within: the clusters do the atoms, layout 2
 };
 
 // FP32 arithmetic throughout (GB300 issues FP64 at ~2 operations per SM and
@@ -75,6 +78,7 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_weights(const LossArgs a)
   }
   __syncthreads();
   const float H0 = (float)a.H[0], H1 = (float)a.H[1], H2 = (float)a.H[2];
+  const int layout = cl_gated(a.gate, 0) ? 2 : a.layout;
   dev::DFloatSum lsum;
   for (int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; m < a.n_s;
        m += (int64_t)gridDim.x * blockDim.x) {
@@ -119,9 +123,9 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_weights(const LossArgs a)
     for (int sp = 0; sp < a.n_species; ++sp) {
       const float2 F = a.ftab ? a.ftab[(int64_t)sp * a.n_s + m] : dev::form_factor(a.coef + kNCoef * sp, s2);
       const float2 gF = dev::cmul(gp, F);
-      if (a.layout == 2) {
+      if (layout == 2) {
         a.gf[(int64_t)sp * a.n_s + m] = gF;
-      } else if (a.layout == 1) {
+      } else if (layout == 1) {
         a.table[(int64_t)sp * a.n_s + m] = make_float4(sz, Sz, gF.x, gF.y);
       } else {
         float4* row = a.table + 2 * ((int64_t)sp * a.n_s + m);
@@ -167,6 +171,7 @@ struct AdjArgs {
   const double* shift;             // [3] its centring t
   float smax[3];                   // max |S_d - H_d| over the points
   unsigned* status;
+  ClGate gate;                     // within: the clusters have done the atoms
 };
 
 // Outer sums of a thread's atoms (over S tiles), double-float, in shared
@@ -209,6 +214,7 @@ struct OuterSums {
 __global__ void __launch_bounds__(kAdjThreads, 4) k_adjoint(const AdjArgs a) {
   __shared__ __align__(128) float4 sh_s[2][kSTile * 2];
   __shared__ __align__(8) uint64_t sh_bar[2];
+  if (cl_gated(a.gate, 0)) return;
   const int tid = threadIdx.x;
   const AdjBlock blk = a.blocks[blockIdx.x];
   const int chunk = blockIdx.y;
@@ -552,6 +558,7 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_adjoint_line(const AdjLineAr
 // with one thread per slot and FP64 sums, 12.5 us so).
 constexpr int kFinalVals = 64, kFinalGroups = 4;
 __global__ void __launch_bounds__(kFinalVals* kFinalGroups) k_adjoint_final(const float* __restrict__ partial, int split,
+                                                                            ClGate gate, int cl_split,
                                                                             int64_t n_slots,
                                                                             const int32_t* __restrict__ slot_src,
                                                                             const float* __restrict__ atom_w,
@@ -560,6 +567,7 @@ __global__ void __launch_bounds__(kFinalVals* kFinalGroups) k_adjoint_final(cons
   const int vi = threadIdx.x % kFinalVals, grp = threadIdx.x / kFinalVals;
   const int64_t i = (int64_t)blockIdx.x * kFinalVals + vi, n = 3 * n_slots;
   dev::DFloatSum v;
+  if (cl_gated(gate, 0)) split = cl_split;
   if (i < n) {
     const int per = (split + kFinalGroups - 1) / kFinalGroups, c1 = min(split, (grp + 1) * per);
 #pragma unroll 8
@@ -650,7 +658,10 @@ scatter_status prepare_adjoint(scatter_plan_s* p) {
   p->adj_blocks = (int)blocks.size();
   cudaError_t e;
   const size_t tab_bytes = (size_t)p->n_species * (size_t)p->n_s * 2 * sizeof(float4);
-  const size_t part_bytes = (size_t)split * (size_t)p->n_slots * 3 * sizeof(float);
+  const scatter_status cs = prepare_cluster_adjoint(p);
+  if (cs != SCATTER_OK) return cs;
+  const size_t part_bytes = (size_t)std::max<int64_t>(split, p->cl.adj.active ? p->cl.adj.split : 0) *
+                            (size_t)p->n_slots * 3 * sizeof(float);
   if (!blocks.empty()) {
     if ((e = cudaMalloc(&p->d.adj_blocks, blocks.size() * sizeof(AdjBlock))) != cudaSuccess)
       return cuda_status(e, "cudaMalloc");
@@ -707,6 +718,10 @@ scatter_status launch_backward(scatter_plan_t p, const double* xyz, const float*
   la.table = p->d.adj_table;
   la.gf = p->d.adj_gf;
   la.loss_part = p->d.loss_part;
+  const bool clustered = grad && p->cl.adj.active;
+  const ClGate gate = clustered ? cluster_gate(p) : ClGate{};
+  la.gate = gate;
+  if (clustered) la.gf = reinterpret_cast<float2*>(p->d.adj_table);  // either layout, never both
   k_loss_weights<<<kLossParts, kLossThreads, 0, st>>>(la);
   p->last_launches += 1;
   if (A && loss_out) {
@@ -727,9 +742,11 @@ scatter_status launch_backward(scatter_plan_t p, const double* xyz, const float*
     aa.shift = p->d.inst_shift;
     for (int d = 0; d < 3; ++d) aa.smax[d] = (float)p->s_max[d];
     aa.status = p->d.status;
+    aa.gate = gate;
+    if (clustered && (s = launch_cluster_adjoint(p, la.gf, p->d.adj_partial, st)) != SCATTER_OK) return s;
     if (p->adj_blocks > 0) {
       dim3 gridd((unsigned)p->adj_blocks, (unsigned)p->adj_split);
-      timing_begin(p, st);
+      if (!clustered) timing_begin(p, st);
       if (p->adj_line) {
         AdjLineArgs al{};
         al.atom4 = p->d.atom4;
@@ -753,7 +770,8 @@ scatter_status launch_backward(scatter_plan_t p, const double* xyz, const float*
       p->last_launches += 1;
     }
     const int64_t nb = (3 * p->n_slots + kFinalVals - 1) / kFinalVals;
-    k_adjoint_final<<<(unsigned)nb, kFinalVals * kFinalGroups, 0, st>>>(p->d.adj_partial, p->adj_split, p->n_slots,
+    k_adjoint_final<<<(unsigned)nb, kFinalVals * kFinalGroups, 0, st>>>(p->d.adj_partial, p->adj_split, gate,
+                                                                        p->cl.adj.split, p->n_slots,
                                                                         p->d.slot_src, p->d.atom_w, grad);
     p->last_launches += 1;
   }

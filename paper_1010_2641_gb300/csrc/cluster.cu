@@ -33,6 +33,7 @@
 #include <cmath>
 #include <cstring>
 #include <vector>
+#include "cluster_common.cuh"
 #include "device_common.cuh"
 #include "launch.h"
 
@@ -43,30 +44,9 @@ constexpr int kClCols = 16;       // columns per thread of the moments kernel
 constexpr int kClRows = 64;       // clusters per CTA (one per thread)
 constexpr int kClTile = 64;       // atoms per stage
 constexpr int kClEval = 64;       // points per CTA of the evaluation
-constexpr int kClMaxK = 320;      // columns of an instance
-constexpr int kClMaxExp = 15;     // largest exponent of an axis
 constexpr int64_t kClMaxBytes = 4LL << 30;  // workspace of a plan's clusters
 
 namespace {
-
-__device__ __forceinline__ float cl_rmax2(const ClArgs& a, int inst) { return __uint_as_float(a.rmax2[inst]); }
-
-// Columns that a crystal of this call's radius needs, 0 if it is larger than
-// the plan's X (the direct kernels then do the instance).
-__device__ __forceinline__ int cl_columns(const ClArgs& a, const ClInst& in, int inst) {
-  const float r2 = cl_rmax2(a, inst);
-  if (!(r2 <= in.lim2)) return 0;
-  const float rho = sqrtf(r2 / in.lim2) * 1.0001f;
-  int lo = 0, hi = in.K;  // columns are sorted by the radius from which they matter
-  while (lo < hi) {
-    const int m = (lo + hi) >> 1;
-    if (a.rho[in.col0 + m] < rho)
-      lo = m + 1;
-    else
-      hi = m;
-  }
-  return lo;
-}
 
 // w xh^a / a! of every column of 128 slots: a thread per slot takes the powers of its
 // three coordinates, then a thread per four columns of a slot writes 16 bytes
@@ -421,6 +401,7 @@ scatter_status prepare_clusters(scatter_plan_s* p, const double* s_list, double 
   std::vector<ClTabBlock> tab_blocks;
   std::vector<ClRedBlock> red_blocks;
   std::vector<ClEvalBlock> eval_blocks;
+  std::vector<int64_t> row_begin;  // of the last clustered instance: its clusters' points
   int64_t tab_floats = 0, part_floats = 0, m_floats = 0;
   double gain = 0.0;
   struct Framed {
@@ -614,6 +595,8 @@ scatter_status prepare_clusters(scatter_plan_s* p, const double* s_list, double 
       pt[o] = v;
       pt_out[o] = in.s_begin + i;
     }
+    row_begin.assign(1, 0);  // first[r] is now the cluster's end
+    row_begin.insert(row_begin.end(), first.begin(), first.begin() + rows);
     for (int64_t o = 0; o < M; o += kClEval)
       eval_blocks.push_back(ClEvalBlock{b, (int32_t)std::min<int64_t>(kClEval, M - o), (int64_t)p_base + o});
     for (int64_t s = 0; s < slots; s += 128) tab_blocks.push_back(ClTabBlock{b, s});
@@ -660,6 +643,11 @@ scatter_status prepare_clusters(scatter_plan_s* p, const double* s_list, double 
   cl.n_red = (int)red_blocks.size();
   cl.n_eval = (int)eval_blocks.size();
   p->base_bytes += bytes;
+  if (B == 1) {  // backward prepares its own tables from these
+    cl.first = insts[0];
+    cl.h_exps = exps;
+    cl.h_row = row_begin;
+  }
   cl.active = true;
   return SCATTER_OK;
 }
@@ -718,6 +706,7 @@ void release_clusters(scatter_plan_s* p) {
                   (void*)cl.pt_out, (void*)cl.items, (void*)cl.tab_blocks, (void*)cl.red_blocks, (void*)cl.eval_blocks,
                   (void*)cl.rmax2, (void*)cl.tab, (void*)cl.partial, (void*)cl.M})
     if (b) cudaFree(b);
+  release_cluster_adjoint(cl.adj);
   cl = ClState{};
 }
 

@@ -66,6 +66,12 @@ struct ClGate {
 scatter_status prepare_clusters(scatter_plan_s* p, const double* s_list, double radius_hint);
 scatter_status launch_clusters(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st);
 void release_clusters(scatter_plan_s* p);
+ClArgs cluster_args(scatter_plan_s* p);
+// Their adjoint (cluster_adjoint.cu): Sum_S S Im(gF e) per slot into
+// [split][n_slots][3] from gF [species][M].
+scatter_status prepare_cluster_adjoint(scatter_plan_s* p);
+scatter_status launch_cluster_adjoint(scatter_plan_t p, const float2* gf, float* partial, cudaStream_t st);
+void release_cluster_adjoint(ClAdjState& s);
 inline ClGate cluster_gate(const scatter_plan_s* p) {
   return p->cl.active ? ClGate{p->cl.rmax2, p->cl.lim2, p->batch} : ClGate{nullptr, nullptr, 0};
 }

@@ -96,7 +96,7 @@ struct ClInst {
   int K, col0;        // columns, the first in exps and rho
   int rows;           // clusters
   int64_t row0;       // the first in cen
-  int64_t tab_off;    // floats into tab: [column tile][slot][32]
+  int64_t tab_off;    // floats into tab: [column tile][slot][16]
   int64_t part_off;   // float2 into partial: [chunk][column][cluster]
   int64_t m_off;      // float2 into M: [species][column][cluster]
   uint64_t species;   // bit s: atoms of species s
@@ -120,8 +120,29 @@ struct ClEvalBlock {
   int32_t inst, n;
   int64_t p0;
 };
+struct ClGBlock {
+  int32_t row, n;  // points of one cluster
+  int64_t p0;
+};
+// Adjoint over the clusters (cluster_adjoint.cu), single instances.
+struct ClAdjState {
+  bool active = false;
+  AdjBlock* blocks = nullptr;       // atom blocks of one species
+  ClGBlock* g_blocks = nullptr;     // <= 256 points of one cluster
+  int32_t* row_blk = nullptr;       // [rows + 1] the first g_block of each cluster
+  short4* up = nullptr;             // per column: columns of a + e_d, -1: none
+  short4* down = nullptr;           //             columns of a - e_d
+  float2* g_part = nullptr;         // [g_block][species][column]
+  float* g8 = nullptr;              // [species][cluster][column][8]
+  int n_blocks = 0, n_g = 0, split = 1, rows_per_chunk = 0, smem = 0;
+  int emax[3] = {0, 0, 0};
+};
 struct ClState {
   bool active = false;
+  ClAdjState adj;
+  ClInst first;                     // the only instance, with its columns and its clusters' points
+  std::vector<int32_t> h_exps;
+  std::vector<int64_t> h_row;
   ClInst* inst = nullptr;           // [batch]
   float* lim2 = nullptr;            // [batch] X^2, -1: not clustered
   unsigned* rmax2 = nullptr;        // [batch] this call's largest |x'|^2 (float bits)
