@@ -27,7 +27,6 @@
 #include <vector>
 #include <type_traits>
 #include "device_common.cuh"
-#include "generic_impl.cuh"
 #include "launch.h"
 
 namespace scatter {
@@ -59,7 +58,7 @@ struct LossArgs {
   float4* table;          // [n_species][M][2] (layout 0), [n_species][M] (layout 1)
   float2* gf;             // [n_species][M] (layout 2)
   double* loss_part;      // [gridDim.x]
-  ClGate gate;            // within: the clusters do the atoms, layout 2
+  CallGate gate;            // within: the clusters do the atoms, layout 2
 };
 
 // FP32 arithmetic throughout (GB300 issues FP64 at ~2 operations per SM and
@@ -78,7 +77,7 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_weights(const LossArgs a)
   }
   __syncthreads();
   const float H0 = (float)a.H[0], H1 = (float)a.H[1], H2 = (float)a.H[2];
-  const int layout = cl_gated(a.gate, 0) ? 2 : a.layout;
+  const int layout = within(a.gate, 0) ? 2 : a.layout;
   dev::DFloatSum lsum;
   for (int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; m < a.n_s;
        m += (int64_t)gridDim.x * blockDim.x) {
@@ -171,7 +170,7 @@ struct AdjArgs {
   const double* shift;             // [3] its centring t
   float smax[3];                   // max |S_d - H_d| over the points
   unsigned* status;
-  ClGate gate;                     // within: the clusters have done the atoms
+  CallGate gate;                     // within: the clusters have done the atoms
 };
 
 // Outer sums of a thread's atoms (over S tiles), double-float, in shared
@@ -214,7 +213,7 @@ struct OuterSums {
 __global__ void __launch_bounds__(kAdjThreads, 4) k_adjoint(const AdjArgs a) {
   __shared__ __align__(128) float4 sh_s[2][kSTile * 2];
   __shared__ __align__(8) uint64_t sh_bar[2];
-  if (cl_gated(a.gate, 0)) return;
+  if (within(a.gate, 0)) return;
   const int tid = threadIdx.x;
   const AdjBlock blk = a.blocks[blockIdx.x];
   const int chunk = blockIdx.y;
@@ -558,7 +557,7 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_adjoint_line(const AdjLineAr
 // with one thread per slot and FP64 sums, 12.5 us so).
 constexpr int kFinalVals = 64, kFinalGroups = 4;
 __global__ void __launch_bounds__(kFinalVals* kFinalGroups) k_adjoint_final(const float* __restrict__ partial, int split,
-                                                                            ClGate gate, int cl_split,
+                                                                            CallGate gate, int cl_split,
                                                                             int64_t n_slots,
                                                                             const int32_t* __restrict__ slot_src,
                                                                             const float* __restrict__ atom_w,
@@ -567,7 +566,7 @@ __global__ void __launch_bounds__(kFinalVals* kFinalGroups) k_adjoint_final(cons
   const int vi = threadIdx.x % kFinalVals, grp = threadIdx.x / kFinalVals;
   const int64_t i = (int64_t)blockIdx.x * kFinalVals + vi, n = 3 * n_slots;
   dev::DFloatSum v;
-  if (cl_gated(gate, 0)) split = cl_split;
+  if (within(gate, 0)) split = cl_split;
   if (i < n) {
     const int per = (split + kFinalGroups - 1) / kFinalGroups, c1 = min(split, (grp + 1) * per);
 #pragma unroll 8
@@ -719,7 +718,7 @@ scatter_status launch_backward(scatter_plan_t p, const double* xyz, const float*
   la.gf = p->d.adj_gf;
   la.loss_part = p->d.loss_part;
   const bool clustered = grad && p->cl.adj.active;
-  const ClGate gate = clustered ? cluster_gate(p) : ClGate{};
+  const CallGate gate = clustered ? cluster_gate(p) : CallGate{};
   la.gate = gate;
   if (clustered) la.gf = reinterpret_cast<float2*>(p->d.adj_table);  // either layout, never both
   k_loss_weights<<<kLossParts, kLossThreads, 0, st>>>(la);

@@ -57,10 +57,14 @@ scatter_status check_inputs(scatter_plan_t p, const double* xyz, const float* oc
 // kernels, their reduction.
 scatter_status enqueue_single(scatter_plan_t p, const double* xyz, const float* occ, float2* amp, float* inten,
                               cudaStream_t st) {
-  scatter_status s = launch_prep(p, xyz, occ, st);
-  if (s != SCATTER_OK) return s;
-  if (p->path == SCATTER_PATH_SEPARABLE) return launch_separable(p, amp, inten, st);  // GRID and GID_GRID
-  return p->s_kind == SCATTER_S_GID_GRID ? launch_dwba(p, amp, inten, st) : launch_generic(p, amp, inten, st);
+  scatter_status s;
+  // the map from its nodes; what follows is for a crystal that these don't resolve
+  const bool coarse = coarse_serves(p, amp);
+  if (coarse && (s = launch_coarse(p, xyz, occ, amp, inten, st)) != SCATTER_OK) return s;
+  const CallGate gate = coarse ? coarse_gate(p) : CallGate{};
+  if ((s = launch_prep(p, xyz, occ, st, gate)) != SCATTER_OK) return s;
+  if (p->path == SCATTER_PATH_SEPARABLE) return launch_separable(p, amp, inten, st, gate);  // GRID and GID_GRID
+  return p->s_kind == SCATTER_S_GID_GRID ? launch_dwba(p, amp, inten, st) : launch_generic(p, amp, inten, st, gate);
 }
 
 // The same sequence as a CUDA graph, captured on the plan's own stream and

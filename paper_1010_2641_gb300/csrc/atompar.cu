@@ -45,7 +45,7 @@ struct ApArgs {
   float smax[3];                   // max |S_d - H_d| over the points
   float2* partial;        // [block][M]
   int tile;               // reflections per CTA (<= kApPts)
-  ClGate gate;            // clustered lists
+  CallGate gate;            // clustered lists
 };
 
 // EXACT: the phase with its products' rounding errors restored and s and the
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kApThreads, 2) k_atompar(const ApArgs a) {
   __shared__ float4 sh_s[kApPts];
   __shared__ float4 sh_slo[kApPts];  // rounding errors of sh_s (exact-product phases)
   __shared__ float2 sh_part[kApWarps][kApPts];
-  if (cl_gated(a.gate, 0)) return;
+  if (within(a.gate, 0)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const Segment blk = a.blocks[blockIdx.y];
   const int64_t p0 = (int64_t)blockIdx.x * a.tile;

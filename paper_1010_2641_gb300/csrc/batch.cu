@@ -47,7 +47,7 @@ struct BatchArgs {
   float2* out_amp;
   float* out_int;
   unsigned* status;
-  ClGate gate;  // instances done by their clusters
+  CallGate gate;  // instances done by their clusters
 };
 
 template <int R, int THREADS>
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(THREADS) k_batch(const BatchArgs a) {
   const int tid = threadIdx.x;
   if (a.gate.rmax2) {  // every instance done: 3 us instead of a walk through the items
     bool left = false;
-    for (int b = tid; b < a.gate.n; b += THREADS) left |= !cl_gated(a.gate, b);
+    for (int b = tid; b < a.gate.n; b += THREADS) left |= !within(a.gate, b);
     if (!__syncthreads_or(left)) return;
   }
   if (tid == 0) {
@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(THREADS) k_batch(const BatchArgs a) {
     const int it = sh_item;
     if (it >= a.n_items) break;
     const BatchItem w = a.items[it];
-    if (cl_gated(a.gate, w.inst)) continue;
+    if (within(a.gate, w.inst)) continue;
     const BatchInst in = a.inst[w.inst];
     float sx[R], sy[R], sz[R];
     bool valid[R];
@@ -140,7 +140,7 @@ __global__ void k_batch_reduce(const BatchArgs a, const int32_t* __restrict__ s_
   if (m >= a.n_s) return;
   const int b = s_inst[m];
   const BatchInst in = a.inst[b];
-  if (in.split <= 1 || cl_gated(a.gate, b)) return;
+  if (in.split <= 1 || within(a.gate, b)) return;
   const int64_t M_b = in.s_end - in.s_begin;
   float2 v = make_float2(0.f, 0.f);
   for (int c = 0; c < in.split; ++c) {

@@ -18,7 +18,7 @@
 // corners) or the caller's radius hint.  A call measures its atoms' largest
 // |x'|: columns that a smaller crystal does not need are skipped (they are
 // sorted by the radius from which they matter), and a larger crystal is left
-// to the direct kernels, whose launches otherwise return at once (ClGate).
+// to the direct kernels, whose launches otherwise return at once (CallGate).
 //
 //   k_cl_tab     per slot: w xh^a / a! for every column
 //   k_cl_moments 64 clusters x 16 columns x one chunk of atoms of one species

@@ -108,8 +108,9 @@ __global__ void __launch_bounds__(256) k_bbox(const double* __restrict__ xyz, co
 // One instance: the box of each CTA's share of the atoms, joined by k_prep_one.
 __global__ void __launch_bounds__(256) k_box_part(const double* __restrict__ xyz, int64_t n_atoms,
                                                   unsigned long long* __restrict__ part, unsigned* status,
-                                                  unsigned* rmax2) {
+                                                  unsigned* rmax2, const CallGate gate) {
   __shared__ unsigned long long sh[6][8];
+  if (within(gate, 0)) return;
   if (rmax2 && blockIdx.x == 0 && threadIdx.x == 0) *rmax2 = 0u;
   Box box;
   bool bad = false;
@@ -132,7 +133,9 @@ struct PrepArgs {
   unsigned* status;
   float4* rec_a;          // the folded separable forward's A records, or null
   float mid[3], mid_lo[3];  // middles of its axes - H
-  unsigned* rmax2;        // clustered lists: [batch] largest |x'|^2 (float bits, zeroed before), or null
+  unsigned* rmax2;        // [batch] largest |x'|^2 (float bits, zeroed before), or null
+  int per_axis;           // rmax2 of the largest |x'_d| instead
+  CallGate gate;          // one instance
 };
 
 // a + b with its rounding error
@@ -238,7 +241,10 @@ __device__ __forceinline__ float prep_slot(const PrepArgs& a, int64_t slot, cons
     sincospif(2.0f * ((ph - rintf(ph)) + pe), &sn, &cs);
     a.rec_a[slot] = make_float4(x0[0], lo[0], w * cs, w * sn);
   }
-  return x0[0] * x0[0] + x0[1] * x0[1] + x0[2] * x0[2];
+  const float q[3] = {x0[0] * x0[0], x0[1] * x0[1], x0[2] * x0[2]};
+  // a NaN stays one: its bits are the largest
+  if (a.per_axis) return __uint_as_float(max(max(__float_as_uint(q[0]), __float_as_uint(q[1])), __float_as_uint(q[2])));
+  return q[0] + q[1] + q[2];
 }
 
 __device__ __forceinline__ double centre(unsigned long long ulo, unsigned long long uhi) {
@@ -282,6 +288,7 @@ __global__ void __launch_bounds__(256) k_prep(const PrepArgs a, const int32_t* _
 __global__ void __launch_bounds__(256) k_prep_one(const PrepArgs a, int64_t n_atoms, int64_t n_slots,
                                                   const unsigned long long* __restrict__ part, int n_part,
                                                   unsigned long long* bbox, double* inst_shift) {
+  if (within(a.gate, 0)) return;
   __shared__ unsigned long long sh[6][8];
   __shared__ unsigned long long sh_box[6];
   __shared__ double sh_t[3];
@@ -330,7 +337,7 @@ __global__ void __launch_bounds__(THREADS) k_generic(const GenericArgs a) {
   __shared__ __align__(128) float sh_w[2][kTile];
   __shared__ __align__(8) uint64_t sh_bar[2];
 
-  if (cl_gated(a.gate, 0)) return;
+  if (within(a.gate, 0)) return;
   const int tid = threadIdx.x;
   const int chunk = blockIdx.y;
 
@@ -462,7 +469,7 @@ template <int GROUPS>
 __global__ void __launch_bounds__(256) k_reduce(GenericArgs a, int split_k, int grid_mode) {
   constexpr int kPts = 256 / GROUPS;
   __shared__ float2 sh[GROUPS > 1 ? GROUPS - 1 : 1][kPts];
-  if (cl_gated(a.gate, 0)) return;
+  if (within(a.gate, 0)) return;
   const int pt = threadIdx.x % kPts, grp = threadIdx.x / kPts;
   const int64_t m = (int64_t)blockIdx.x * kPts + pt;
   float2 v = make_float2(0.f, 0.f);
@@ -598,7 +605,8 @@ int generic_blocks_per_sm(const scatter_plan_s* p, const Tiling& t) {
   return nb > 0 ? nb : 1;
 }
 
-scatter_status launch_prep(scatter_plan_t p, const double* xyz, const float* occ, cudaStream_t st) {
+scatter_status launch_prep(scatter_plan_t p, const double* xyz, const float* occ, cudaStream_t st,
+                           const CallGate& gate) {
   const int batch = p->batch;
   PrepArgs a{};
   a.xyz = xyz;
@@ -610,7 +618,9 @@ scatter_status launch_prep(scatter_plan_t p, const double* xyz, const float* occ
   a.atom_w = p->d.atom_w;
   a.status = p->d.status;
   a.rec_a = p->d.sep_rec;
-  a.rmax2 = p->cl.active ? p->cl.rmax2 : nullptr;
+  a.rmax2 = p->cl.active ? p->cl.rmax2 : p->extent2;
+  a.per_axis = p->extent2 != nullptr;
+  a.gate = gate;
   for (int d = 0; d < 3; ++d) {
     a.mid[d] = (float)p->sep_mid[d];
     a.mid_lo[d] = (float)(p->sep_mid[d] - (double)a.mid[d]);
@@ -620,7 +630,7 @@ scatter_status launch_prep(scatter_plan_t p, const double* xyz, const float* occ
     int n_part = 0;
     if (p->n_atoms > kPrepSmall || a.rmax2) {
       n_part = (int)std::min<int64_t>(kPrepParts, (p->n_atoms + 511) / 512);
-      k_box_part<<<n_part, 256, 0, st>>>(xyz, p->n_atoms, p->d.box_part, p->d.status, a.rmax2);
+      k_box_part<<<n_part, 256, 0, st>>>(xyz, p->n_atoms, p->d.box_part, p->d.status, a.rmax2, gate);
       p->last_launches += 1;
     }
     const int64_t nb = std::min<int64_t>(std::max<int64_t>((p->n_slots + 255) / 256, 1), 4 * (int64_t)p->n_sm);
@@ -664,8 +674,8 @@ scatter_status launch_generic_reduce(scatter_plan_t p, int n_chunks, float2* amp
   return cuda_status(cudaGetLastError(), "generic reduction launch");
 }
 
-scatter_status launch_generic(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st) {
-  if (p->gs.active) return launch_gridsum(p, amp_out, int_out, st);
+scatter_status launch_generic(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st, const CallGate& gate) {
+  if (p->gs.active) return launch_gridsum(p, amp_out, int_out, st, gate);
   if (p->cl.active) {
     const scatter_status cs = launch_clusters(p, amp_out, int_out, st);
     if (cs != SCATTER_OK) return cs;

@@ -38,14 +38,8 @@ struct GenericArgs {
   float* out_int;
   float2* partial;        // split-K partials [chunk][M] (or null)
   unsigned* status;
-  ClGate gate;            // clustered lists: the instances done there
+  CallGate gate;            // clustered lists: the instances done there
 };
-
-// True where this call's atoms of the instance lie within its clusters' radius:
-// cluster.cu has done its points.
-__device__ __forceinline__ bool cl_gated(const ClGate& g, int inst) {
-  return g.rmax2 && __uint_as_float(g.rmax2[inst]) <= g.lim2[inst];
-}
 
 // LIST-mode generic kernel (+ split-K reduction) on prepared arguments.
 scatter_status launch_generic_args(GenericArgs a, int R, int threads, int n_chunks, cudaStream_t st);

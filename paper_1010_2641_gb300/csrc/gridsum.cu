@@ -69,6 +69,7 @@ struct GridSumArgs {
   float2* ztab;                // [column tile][slot][RS]
   int64_t n_slots;
   unsigned* status;
+  CallGate gate;
 };
 
 __device__ __forceinline__ float comp(const float4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : v.z; }
@@ -91,6 +92,7 @@ __device__ __forceinline__ float2 gs_entry(const GridSumArgs& a, int64_t slot, f
 
 // One thread per table entry (column tile, slot, column).
 __global__ void __launch_bounds__(256) k_gridsum_tab(const GridSumArgs a, int R, int RS, int64_t total) {
+  if (within(a.gate, 0)) return;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= total) return;
   const int r = (int)(i % RS);
@@ -102,6 +104,7 @@ __global__ void __launch_bounds__(256) k_gridsum_tab(const GridSumArgs a, int R,
 
 template <int R, bool TAB>
 __global__ void __launch_bounds__(256, 2) k_gridsum(const GridSumArgs a) {
+  if (within(a.gate, 0)) return;
   constexpr int RS = R + (R & 1);  // table row stride: 16-byte aligned
   __shared__ __align__(16) float4 sh_rec[2][kGsTile];     // (u, v, phase, 0)
   __shared__ __align__(16) float2 sh_lo[2][kGsTile];      // rounding errors of u, v (exact phases)
@@ -268,13 +271,14 @@ struct GridSumReduce {
   const double* shift;
   float2* out_amp;
   float* out_int;
+  CallGate gate;
 };
 
 // Ordered sum of the chunks with f_s(|S|) per species run, translation phase,
 // outputs; one thread per point, eight chunks' loads in flight.
 __global__ void __launch_bounds__(128) k_gridsum_reduce(const GridSumReduce a) {
   const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= a.n_s) return;
+  if (m >= a.n_s || within(a.gate, 0)) return;
   const int64_t i2 = m % a.n2, line = m / a.n2, i1 = line % a.n1, i0 = line / a.n1;
   const float Sx = a.H[0] + a.axis_s[i0], Sy = a.H[1] + a.axis_s[a.n0 + i1], Sz = a.H[2] + a.axis_s[a.n0 + a.n1 + i2];
   const float s2 = (Sx * Sx + Sy * Sy + Sz * Sz) * a.inv4a2;
@@ -498,7 +502,7 @@ scatter_status prepare_gridsum(scatter_plan_s* p, int split_override) {
   return SCATTER_OK;
 }
 
-scatter_status launch_gridsum(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st) {
+scatter_status launch_gridsum(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st, const CallGate& gate) {
   const GridSum& g = p->gs;
   const int64_t n[3] = {p->n_axis[0], p->n_axis[1], p->n_axis[2]};
   const int64_t off[3] = {0, n[0], n[0] + n[1]}, stride[3] = {n[1] * n[2], n[2], 1};
@@ -537,13 +541,14 @@ scatter_status launch_gridsum(scatter_plan_t p, float2* amp_out, float* int_out,
   a.ztab = g.ztab;
   a.n_slots = p->n_slots;
   a.status = p->d.status;
+  a.gate = gate;
   if (g.tab) {
     const int RS = g.R + (g.R & 1);
     const int64_t total = g.col_tiles * p->n_slots * RS;
     k_gridsum_tab<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(a, g.R, RS, total);
     p->last_launches += 1;
   }
-  timing_begin(p, st);
+  if (!gate.rmax2) timing_begin(p, st);
   pick<kGsMaxR>(g.R, g.tab)<<<dim3((unsigned)g.row_tiles, (unsigned)g.col_tiles, (unsigned)g.n_chunks), g.threads, 0, st>>>(a);
   timing_end(p, st);
   cudaError_t e = cudaGetLastError();
@@ -565,7 +570,8 @@ scatter_status launch_gridsum(scatter_plan_t p, float2* amp_out, float* int_out,
     r.H[d] = (float)p->inst[0].H[d];
     r.H64[d] = p->inst[0].H[d];
   }
-  r.shift = p->d.inst_shift;
+  r.shift = p->out_shift ? p->out_shift : p->d.inst_shift;
+  r.gate = gate;
   r.out_amp = amp_out;
   r.out_int = int_out;
   k_gridsum_reduce<<<(unsigned)((p->n_s + 127) / 128), 128, 0, st>>>(r);

@@ -5,10 +5,25 @@
 
 namespace scatter {
 
+// A call's choice on the device: kernels that stand by for crystals past a plan's
+// assumed radius return at once while this call's extent squared (rmax2, float
+// bits, per instance) is within lim2.
+struct CallGate {
+  const unsigned* rmax2;  // null: no gate
+  const float* lim2;
+  int n;                  // instances
+};
+#ifdef __CUDACC__
+__device__ __forceinline__ bool within(const CallGate& g, int inst) {
+  return g.rmax2 && __uint_as_float(g.rmax2[inst]) <= g.lim2[inst];
+}
+#endif
+
 // Per-call position preparation (all instances): integer centring t of each
 // instance (rint of its bounding-box centre), split r - t = n + delta,
 // c = frac(H . delta), fp32 slots.  Enqueued on `st`.
-scatter_status launch_prep(scatter_plan_t p, const double* xyz, const float* occ, cudaStream_t st);
+scatter_status launch_prep(scatter_plan_t p, const double* xyz, const float* occ, cudaStream_t st,
+                           const CallGate& gate = CallGate{});
 
 // Bounding boxes of `batch` instances (ordered-int min / max xyz, atom ranges
 // atom_off [batch+1] in device memory) into `bbox` [batch][6], which must hold
@@ -19,7 +34,8 @@ scatter_status launch_bbox_raw(const double* xyz, const int64_t* atom_off, int b
 
 // A(S) (and/or |A|^2) of every point with the generic FP32/MUFU kernel;
 // positions must have been prepared by launch_prep on the same stream.
-scatter_status launch_generic(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st);
+scatter_status launch_generic(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st,
+                              const CallGate& gate = CallGate{});
 
 // Ordered sum of n_chunks partials [chunk][M] (p->d.partial) with the
 // translation phase, into the outputs (GenericArgs reduction of forward.cu).
@@ -58,11 +74,6 @@ struct ClArgs {
   float2* out_amp;
   float* out_int;
 };
-struct ClGate {
-  const unsigned* rmax2;  // null: no gate
-  const float* lim2;
-  int n;                  // instances
-};
 scatter_status prepare_clusters(scatter_plan_s* p, const double* s_list, double radius_hint);
 scatter_status launch_clusters(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st);
 void release_clusters(scatter_plan_s* p);
@@ -72,14 +83,34 @@ ClArgs cluster_args(scatter_plan_s* p);
 scatter_status prepare_cluster_adjoint(scatter_plan_s* p);
 scatter_status launch_cluster_adjoint(scatter_plan_t p, const float2* gf, float* partial, cudaStream_t st);
 void release_cluster_adjoint(ClAdjState& s);
-inline ClGate cluster_gate(const scatter_plan_s* p) {
-  return p->cl.active ? ClGate{p->cl.rmax2, p->cl.lim2, p->batch} : ClGate{nullptr, nullptr, 0};
+inline CallGate cluster_gate(const scatter_plan_s* p) {
+  return p->cl.active ? CallGate{p->cl.rmax2, p->cl.lim2, p->batch} : CallGate{nullptr, nullptr, 0};
 }
+
+// Maps sampled far finer than the crystal's extent asks for (coarse.cu): the sum
+// at the Chebyshev nodes of each axis, interpolated to the map.
+scatter_status prepare_coarse(scatter_plan_s* p, const scatter_problem* pr, const scatter_options* op);
+scatter_status launch_coarse(scatter_plan_t p, const double* xyz, const float* occ, float2* amp_out, float* int_out,
+                             cudaStream_t st);
+void release_coarse(scatter_plan_s* p);
+// Tensor-core intensities keep the direct sum: |A|^2 doubles the difference
+// between the two (up to 2.5e-5 of the map, amplitudes 1.6e-5).
+inline bool coarse_serves(const scatter_plan_s* p, const void* amp_out) {
+  return p->coarse.sub && (amp_out || p->path != SCATTER_PATH_SEPARABLE);
+}
+inline CallGate coarse_gate(const scatter_plan_s* p) {
+  return p->coarse.sub ? CallGate{p->coarse.rmax2, p->coarse.lim2, 1} : CallGate{nullptr, nullptr, 0};
+}
+// scatter_plan without a coarse grid of its own, around H, its tensor-core
+// accumulation groups at least `group` steps (0: its own choice).
+scatter_status plan_nodes(const scatter_problem* pr, const scatter_options* op, const double (&H)[3], double group,
+                          scatter_plan_t* out);
 
 // Factorised FP32 sum on single GRID plans (gridsum.cu).
 bool gridsum_preferred(const scatter_plan_s* p);
 scatter_status prepare_gridsum(scatter_plan_s* p, int split_override);
-scatter_status launch_gridsum(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st);
+scatter_status launch_gridsum(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st,
+                              const CallGate& gate = CallGate{});
 
 // Middle of an axis that is symmetric about it: |v_i + v_{n-1-i} - 2 mid| below
 // 2e-13 of its largest value (a phase error under 1e-8 cycles for crystals of
@@ -120,7 +151,9 @@ scatter_status launch_f64_gid(scatter_plan_t p, const double* xyz, const float* 
 // error model (relative L2 of a map with uncorrelated per-term errors).
 double separable_error_model(const scatter_plan_s* p, double radius, int split, double* per_pair);
 scatter_status prepare_separable(scatter_plan_s* p, int split_override);
-scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st);
+scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st,
+                                const CallGate& gate = CallGate{});
+double sep_direct_group(const scatter_plan_s* p);
 
 // Batched persistent path (batch > 1): work list, launches (graph-captured).
 scatter_status prepare_batch(scatter_plan_s* p);

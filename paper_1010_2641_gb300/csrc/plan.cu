@@ -272,6 +272,7 @@ extern "C" void scatter_plan_destroy(scatter_plan_t p) {
   int prev = -1;
   cudaGetDevice(&prev);
   cudaSetDevice(p->device);
+  release_coarse(p);  // shares the status word and the shift
   DeviceBuffers& d = p->d;
   release(d.slot_src);
   release(d.slot_inst);
@@ -365,10 +366,10 @@ extern "C" void scatter_plan_destroy(scatter_plan_t p) {
   delete p;
 }
 
-extern "C" scatter_status scatter_plan(const scatter_problem* pr, const scatter_options* op,
-                                       scatter_plan_t* out) {
-  if (!out) return fail(SCATTER_ERR_INVALID_ARG, "out is NULL");
-  *out = nullptr;
+namespace {
+
+scatter_status make_plan(const scatter_problem* pr, const scatter_options* op, bool nodes, double group,
+                         scatter_plan_t* out) {
   scatter_status st = validate(pr, op);
   if (st != SCATTER_OK) return st;
   int dev = 0, ndev = 0;
@@ -381,6 +382,7 @@ extern "C" scatter_status scatter_plan(const scatter_problem* pr, const scatter_
 
   std::unique_ptr<scatter_plan_s, void (*)(scatter_plan_t)> p(new scatter_plan_s(), scatter_plan_destroy);
   p->device = dev;
+  p->sep_group = group;
   cudaDeviceGetAttribute(&p->n_sm, cudaDevAttrMultiProcessorCount, dev);
   p->s_kind = (scatter_s_kind)pr->s_kind;
   p->n_atoms = pr->n_atoms;
@@ -612,6 +614,7 @@ extern "C" scatter_status scatter_plan(const scatter_problem* pr, const scatter_
       !(op && (op->threads || op->points_per_thread || op->split_k || op->atoms_per_thread > 0)) &&
       (st = prepare_clusters(p.get(), pr->s_list, op ? op->radius_hint : 0.0)))
     return st;
+  if (!nodes && (st = prepare_coarse(p.get(), pr, op))) return st;
   if ((e = cudaDeviceSynchronize()) != cudaSuccess) return cuda_status(e, "plan synchronize");
   if (log_enabled())
     fprintf(stderr, "[scatter] plan: path=%d N=%lld slots=%lld M=%lld threads=%d R=%d split_k=%d atom_k=%d\n",
@@ -619,4 +622,21 @@ extern "C" scatter_status scatter_plan(const scatter_problem* pr, const scatter_
             p->tiling.R, p->tiling.split_k, p->tiling.atom_k);
   *out = p.release();
   return SCATTER_OK;
+}
+
+}  // namespace
+
+scatter_status scatter::plan_nodes(const scatter_problem* pr, const scatter_options* op, const double (&H)[3],
+                                   double group, scatter_plan_t* out) {
+  scatter_problem q = *pr;
+  q.center_mode = 1;
+  for (int d = 0; d < 3; ++d) q.center_hkl[d] = H[d];
+  return make_plan(&q, op, true, group, out);
+}
+
+extern "C" scatter_status scatter_plan(const scatter_problem* pr, const scatter_options* op,
+                                       scatter_plan_t* out) {
+  if (!out) return fail(SCATTER_ERR_INVALID_ARG, "out is NULL");
+  *out = nullptr;
+  return make_plan(pr, op, false, 0.0, out);
 }

@@ -23,6 +23,8 @@
 #include <vector>
 #include "scatter_internal.h"
 
+struct scatter_plan_s;
+
 namespace scatter {
 
 constexpr int kSlotAlign = 32;     // padding granularity of species segments
@@ -160,6 +162,24 @@ struct ClState {
   float2* M = nullptr;
   int64_t n_rows = 0;
   int n_items = 0, n_tab = 0, n_red = 0, n_eval = 0;
+};
+
+// Oversampled maps (coarse.cu).
+struct CoarseStage {
+  int axis = 0;
+  int64_t n_in = 0, n_out = 0;      // nodes, points of the axis
+  int64_t outer = 0, inner = 0;     // of the array at that stage
+  float* W = nullptr;               // [n_in][n_out], then its rounding errors
+};
+struct CoarseState {
+  scatter_plan_s* sub = nullptr;    // the sum at the nodes, without the translation phase
+  CoarseStage stage[3];
+  int n_stages = 0;
+  float2* map = nullptr;            // at the nodes
+  float2* tmp[2] = {nullptr, nullptr};
+  unsigned* rmax2 = nullptr;        // this call's largest |x'_d|^2 (float bits)
+  float* lim2 = nullptr;
+  double* no_shift = nullptr;       // [3] zeros
 };
 
 // The factorised FP32 grid sum (gridsum.cu).
@@ -301,6 +321,10 @@ struct scatter_plan_s {
   scatter::DeviceBuffers d;
   scatter::GridSum gs;
   scatter::ClState cl;
+  scatter::CoarseState coarse;
+  unsigned* extent2 = nullptr;                   // the sum at the nodes of another plan: prep writes the largest |x'_d|^2
+  const double* out_shift = nullptr;             //   its reductions' shift in place of the call's
+  double sep_group = 0.0;                        //   accumulation groups of at least this many steps
   int64_t base_bytes = 0;                        // tables and backward workspace
   int64_t tiling_bytes = 0;                      // chunk tables and split-K partials
   double s_max[3] = {0, 0, 0};                   // max |S - H| per axis (error model)

@@ -19,6 +19,7 @@ namespace scatter {
 
 constexpr int kSepFormWarps = 8;           // warps forming B rows (one N column per thread)
 constexpr int kSepThreads = 32 * (kSepFormWarps + 2);  // + the MMA warp + the copy warp
+constexpr int sep_form_warps(bool fold) { return fold ? 16 : kSepFormWarps; }  // of the one-CTA kernel
 constexpr int kSepM = 128;                 // MMA M (rows of A per CTA)
 constexpr int kSepN = 256;                 // MMA N (columns per CTA)
 constexpr int kSepStep = 16;               // K records per pipeline step (K' = 32)
@@ -55,12 +56,14 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
 
 // kind::f16: D f32, A and B f16, both K-major, N >> 3 at bit 17, M >> 4 at bit 24.
 constexpr uint32_t kSepIdesc = (1u << 4) | ((uint32_t)(kSepN >> 3) << 17) | ((uint32_t)(kSepM >> 4) << 24);
+constexpr uint32_t kSepIdescHalf = (1u << 4) | ((uint32_t)(kSepN >> 4) << 17) | ((uint32_t)(kSepM >> 4) << 24);  // N = 128
 
-__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t acc) {
+__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t acc,
+                                        uint32_t idesc = kSepIdesc) {
   asm volatile(
       "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
-      "l"(a), "l"(b), "r"(kSepIdesc), "r"(acc));
+      "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
 
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
@@ -283,6 +286,7 @@ struct SepArgs {
   int64_t n_lanes;        //   h values (fold_h: of the axis' first half) that have rows
   int flush;              // steps between TMEM flushes
   const float4* rec_a;    //   form_a: A records (x', its rounding error, Re W, Im W)
+  CallGate gate;
 };
 
 // Partials in the accumulator's own blocking.  D row m (TMEM lane of its M

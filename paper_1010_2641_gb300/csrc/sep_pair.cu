@@ -149,6 +149,7 @@ __device__ __forceinline__ void commit_pair(uint64_t* bar) {
 // (tensor pipe 73 % active, the formation's latency the rest).
 template <bool FORM_A, bool FOLD>
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(FORM_A ? 112 : 168) k_sep_pair(const SepArgs a) {
+  if (within(a.gate, 0)) return;  // both CTAs of a pair, before any barrier or allocation
   constexpr int kRec = FOLD ? kSepFoldStep : kSepStep;  // records (atoms or points) per step
   extern __shared__ __align__(1024) unsigned char pair_smem_raw[];
   __shared__ __align__(8) uint64_t bar_ready[kPairAStages];

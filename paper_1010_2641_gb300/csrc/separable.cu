@@ -65,11 +65,13 @@ struct SepTabArgs {
   int64_t n0, n1, n2;
   int64_t n_slots, n_steps, n_mt;
   uint4* A;             // [n_mt/2][n_steps][2 tiles][hi|lo][4 kb][16 mg][8 rows] of 16 B
+  CallGate gate;
 };
 
 // One thread per 16-byte row of a core matrix of the A operand (4 atoms x
 // Re/Im of one row m), hi and lo parts; the weight w_j is folded in here.
 __global__ void k_sep_tab_a(const SepTabArgs t) {
+  if (within(t.gate, 0)) return;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t total = t.n_mt * t.n_steps * 4 * kSepM;
   // total is a multiple of 512: whole warps leave here, the shuffles below
@@ -108,7 +110,9 @@ __global__ void k_sep_tab_a(const SepTabArgs t) {
 template <bool FOLD_H>
 __global__ void __launch_bounds__(256) k_sep_tab_fold(const float4* __restrict__ rec_a, const float* __restrict__ axis_d,
                                                       const float* __restrict__ axis_dlo, int64_t n0, int64_t n_lanes,
-                                                      int64_t n_steps, int64_t n_mt, uint4* __restrict__ A) {
+                                                      int64_t n_steps, int64_t n_mt, uint4* __restrict__ A,
+                                                      const CallGate gate) {
+  if (within(gate, 0)) return;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n_mt * n_steps * 128) return;  // whole warps
   const int lane = (int)(i & 31), kb = (int)((i >> 5) & 3);
@@ -137,23 +141,28 @@ __global__ void __launch_bounds__(256) k_sep_tab_fold(const float4* __restrict__
 // -------------------------------------------------------------------------
 
 
-// Warp roles: warps 0..7 form the B rows (one point per thread) and read the
-// accumulators out at every group end; warp 8 (one lane) issues the MMAs;
-// warp 9 (one lane) issues the TMA copies.  Hand-offs go through mbarriers
+// Warp roles: 8 (folded 16) formation warps form the B rows (one point per thread)
+// and read the accumulators out at every group end; the next warp (one lane)
+// issues the MMAs; the last (one lane) issues the TMA copies.  Hand-offs go through mbarriers
 // only:
 //   bar_full[a]   A block of a step arrived            (TMA, 1 arrival + bytes)
 //   bar_done[a]   MMAs of the step done (one commit per step); frees the A
 //                 stage of that step and the B stage it read
 //   bar_atom[t]   atom records of a step arrived       (TMA)
-//   bar_tempty[t] atom records read by the formation   (8 warps)
-//   bar_bfull[b]  B block of a step formed             (8 warps)
-//   bar_tfree     accumulators read out after a group end (8 warps)
+//   bar_tempty[t] atom records read by the formation   (formation warps)
+//   bar_bfull[b]  B block of a step formed             (formation warps)
+//   bar_tfree     accumulators read out after a group end (formation warps)
 // FOLD: the folded forward (sep_common.cuh): 32 atoms per step, the 256 columns
-// are the cos and sin columns of 128 mirror pairs of points; thread (p, half)
-// forms both columns of pair p over two of the four K blocks.
+// are the cos and sin columns of 128 mirror pairs of points; thread (p, kb)
+// forms both columns of pair p over one of the four K blocks.  16 warps share the
+// formation, whose latency binds a step of one M tile (64 x 64 x 24 nodes of
+// 134,009 atoms: 1.1 us a step with 8 warps, 1.0 us so).
 template <bool FOLD>
-__global__ void __maxnreg__(168) k_sep(const SepArgs a) {
+__global__ void __maxnreg__(FOLD ? 112 : 168) k_sep(const SepArgs a) {
+  if (within(a.gate, 0)) return;  // before any barrier or allocation
   constexpr int kRec = FOLD ? kSepFoldStep : kSepStep;  // records per step
+  constexpr int kForm = sep_form_warps(FOLD);
+  constexpr int kSpan = kSepN / (kForm / 4);  // columns that a formation warp reads out
   // a B stage is freed by the done barrier of the step that read it: the A
   // ring (and with it the done ring) must be at least as deep as the B ring
   static_assert(kSepBStages <= kSepAStages, "B-stage reuse is tracked on the done ring");
@@ -172,12 +181,14 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
   unsigned char* ringA = smem;
   unsigned char* ringB = smem + kSepAStages * kSepPair * kSepABytes;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool mma_warp = warp == kSepFormWarps, copy_warp = warp == kSepFormWarps + 1;
+  const bool mma_warp = warp == kForm, copy_warp = warp == kForm + 1;
   const int64_t n_mp = a.mp_count > 0 ? a.mp_count : (a.n_mt + 1) / 2;  // pairs of this launch
   const int64_t mp = a.mp_first + blockIdx.x % n_mp, nt = blockIdx.x / n_mp;
   const int ntp = 2 * mp + 1 < a.n_mt ? 2 : 1;  // M tiles of this CTA with rows
   const int chunk = blockIdx.y;
   const int64_t nbc = a.n1 * a.n2;
+  // up to 64 mirror pairs in all: 128 columns are contracted
+  const bool narrow = FOLD && a.n_pairs <= kSepFoldPairs / 2;
   // this CTA's columns [col_base, col_end) and the species of its A table
   int64_t col_base = nt * kSepN, col_end = FOLD ? sep_fold_cols(a.n_pairs) : nbc;
   int a_species = 0;
@@ -200,12 +211,12 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
     }
     for (int s = 0; s < kSepTStages; ++s) {
       dev::mbar_init(&bar_atom[s], 1);
-      dev::mbar_init(&bar_tempty[s], kSepFormWarps);
+      dev::mbar_init(&bar_tempty[s], kForm);
     }
     for (int s = 0; s < kSepBStages; ++s) {
-      dev::mbar_init(&bar_bfull[s], kSepFormWarps);
+      dev::mbar_init(&bar_bfull[s], kForm);
     }
-    dev::mbar_init(&bar_tfree, kSepFormWarps);
+    dev::mbar_init(&bar_tfree, kForm);
     s_abort = 0;
     dev::mbar_fence_init();
   }
@@ -263,6 +274,7 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
       const uint64_t dal[2] = {smem_desc(a0 + 8192, 2048, 128), smem_desc(a0 + 8192 + 4096, 2048, 128)};
       const uint64_t dbh[2] = {smem_desc(b0, 4096, 128), smem_desc(b0 + 8192, 4096, 128)};
       const uint64_t dbl[2] = {smem_desc(b0 + 16384, 4096, 128), smem_desc(b0 + 16384 + 8192, 4096, 128)};
+      const uint32_t idesc = narrow ? kSepIdescHalf : kSepIdesc;
       int64_t flushes = 0;  // groups read out before the current one
       int64_t g = 0;
       for (int64_t ks = ks_begin; ks < ks_end; ++ks, ++g) {
@@ -289,9 +301,9 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
             const uint32_t acc0 = (ks > grp.grp_start || u > 0) ? 1u : 0u;
-            mma_f16(d, dah[u] + offA, dbh[u] + offB, acc0);
-            mma_f16(d, dah[u] + offA, dbl[u] + offB, 1u);
-            mma_f16(d, dal[u] + offA, dbh[u] + offB, 1u);
+            mma_f16(d, dah[u] + offA, dbh[u] + offB, acc0, idesc);
+            mma_f16(d, dah[u] + offA, dbl[u] + offB, 1u, idesc);
+            mma_f16(d, dal[u] + offA, dbh[u] + offB, 1u, idesc);
           }
         }
         mma_commit(&bar_done[ast]);
@@ -307,7 +319,7 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
     // this thread's B row (column col of D): forward the point (b, c) with
     // offsets (s_b, s_c) from H, adjoint the atom's (y', z')
     // (folded: the first point of the thread's mirror pair)
-    const int p_loc = tid & (kSepFoldPairs - 1);
+    const int p_loc = tid & (narrow ? kSepFoldPairs / 2 - 1 : kSepFoldPairs - 1);
     const int64_t col = FOLD ? nt * kSepFoldPairs + p_loc : col_base + tid;
     const bool row_ok = col < (FOLD ? a.n_pairs : col_end);
     float sb, sc, sbl = 0.f, scl = 0.f;  // sbl, scl: low parts of a double-float s (forward)
@@ -366,9 +378,8 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
       unsigned char* sB = ringB + bst * kSepBBytes;
       const float4* at = ring_atom[tst];
       if constexpr (FOLD) {
-#pragma unroll
-        for (int kq = 0; kq < 2; ++kq) {
-          const int kb = 2 * (tid / kSepFoldPairs) + kq;
+        const int kb = tid / (narrow ? kSepFoldPairs / 2 : kSepFoldPairs);
+        if (kb < 4) {  // narrow: half of the warps
           uint4 hi[2], lo[2];
           hi[0] = hi[1] = lo[0] = lo[1] = make_uint4(0u, 0u, 0u, 0u);
           if (row_ok) {
@@ -455,11 +466,11 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
       // TMEM lane = row (2 pa + ri) of this CTA's tile: one 32 x 32 block of
       // the partials per load; padding rows and columns are written too
       const int sub = warp & 3;
-      const int col0 = (warp >> 2) * 128;
+      const int col0 = (warp >> 2) * kSpan;
       for (int tp = 0; tp < ntp; ++tp) {
         const int64_t m0 = (2 * mp + tp) * kSepM + sub * 32;
 #pragma unroll 1
-        for (int cc = 0; cc < 128; cc += 32) {
+        for (int cc = 0; cc < kSpan; cc += 32) {
           const int64_t bc0 = col_base + col0 + cc;
           if (bc0 >= col_end) break;
           float4* blk = reinterpret_cast<float4*>(part + sep_part_off(m0, bc0, a.n_cb)) + lane;
@@ -489,10 +500,10 @@ __global__ void __maxnreg__(168) k_sep(const SepArgs a) {
     if (ok && first_flush) {
       // empty chunk: its partials are zero
       const int sub = warp & 3;
-      const int col0 = (warp >> 2) * 128;
+      const int col0 = (warp >> 2) * kSpan;
       for (int tp = 0; tp < ntp; ++tp) {
         const int64_t m0 = (2 * mp + tp) * kSepM + sub * 32;
-        for (int cc = 0; cc < 128 && col_base + col0 + cc < col_end; cc += 32) {
+        for (int cc = 0; cc < kSpan && col_base + col0 + cc < col_end; cc += 32) {
           float4* blk = reinterpret_cast<float4*>(part + sep_part_off(m0, col_base + col0 + cc, a.n_cb)) + lane;
           for (int q = 0; q < 8; ++q) blk[q * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
@@ -539,7 +550,9 @@ __global__ void __launch_bounds__(256) k_sep_reduce(const float* __restrict__ pa
                                                     const float* __restrict__ axis_lo, int64_t n0, int64_t n1,
                                                     int64_t n2, float3 H, const double* __restrict__ shift,
                                                     const float* __restrict__ att, const float* __restrict__ szf,
-                                                    int64_t bm_base, float2* out_amp, float* out_int) {
+                                                    int64_t bm_base, float2* out_amp, float* out_int,
+                                                    const CallGate gate) {
+  if (within(gate, 0)) return;
   // the centring shift of the call (integers), once per block
   __shared__ float sh_t[3];
   __shared__ int sh_shifted;
@@ -643,6 +656,7 @@ struct SepFoldReduceArgs {
   int64_t l8_base;       // first block of 8 lanes of this launch
   float2* out_amp;
   float* out_int;
+  CallGate gate;
 };
 
 // The reduction of the folded forward: per species run of the chunks the
@@ -656,6 +670,7 @@ struct SepFoldReduceArgs {
 // thread per quadruple, 12.7 us with four).
 template <int GROUPS>
 __global__ void __launch_bounds__(256) k_sep_reduce_fold(const SepFoldReduceArgs a) {
+  if (within(a.gate, 0)) return;
   constexpr int kCols = 256 / GROUPS;  // threads over (alpha, quad)
   __shared__ float sh_t[3];
   __shared__ int sh_shifted;
@@ -855,7 +870,7 @@ cudaError_t sep_prepare_kernel() {
 // pair kernel's last clusters leave idle.
 static void launch_one_cta(const SepArgs& a, dim3 grid, cudaStream_t st) {
   if (a.fold)
-    k_sep<true><<<grid, kSepThreads, kSepSmem, st>>>(a);
+    k_sep<true><<<grid, 32 * (sep_form_warps(true) + 2), kSepSmem, st>>>(a);
   else
     k_sep<false><<<grid, kSepThreads, kSepSmem, st>>>(a);
 }
@@ -948,6 +963,14 @@ double sep_mean_group(const std::vector<Segment>& chunks, int step, int64_t flus
   return all > 0.0 ? sq / all : 0.0;
 }
 
+}  // namespace
+
+double sep_direct_group(const scatter_plan_s* p) {
+  return sep_mean_group(sep_chunks(p, p->sep_direct.split, kSepStep), kSepStep, kSepFlush);
+}
+
+namespace {
+
 // Atom chunks (split over K) of `steps` steps in all that minimise the waves
 // of CTAs x steps per CTA, each chunk at least min_steps long; *cost_out in
 // steps.
@@ -1031,7 +1054,7 @@ scatter_status prepare_separable(scatter_plan_s* p, int split_override) {
   fd.flush = kSepFlush;
   double cost_d = 0.0, cost_f = 0.0;
   fd.split = split_override > 0 ? split_override
-                                : sep_best_split(p, (fd.mt + 1) / 2 * fd.nt, fd.steps, 64.0, &cost_d);
+                                : sep_best_split(p, (fd.mt + 1) / 2 * fd.nt, fd.steps, std::max(64.0, p->sep_group), &cost_d);
   // The folded form, where the (k, l) axes are symmetric (evenly spaced axes)
   // and the crystal has at least kSepFoldMinSlots slots, for amplitude calls.
   // Not on grazing incidence: near the critical angle the four beams nearly
@@ -1055,7 +1078,7 @@ scatter_status prepare_separable(scatter_plan_s* p, int split_override) {
     ff.cols = sep_fold_cols(ff.pairs);
     ff.nt = (ff.cols + kSepN - 1) / kSepN;
     ff.steps = p->n_slots / kSepFoldStep;
-    const double group = 0.95 * sep_mean_group(sep_chunks(p, fd.split, kSepStep), kSepStep, kSepFlush);
+    const double group = 0.95 * (p->sep_group > 0.0 ? p->sep_group : sep_direct_group(p));
     ff.split = fd.split;
     if (split_override <= 0) {
       ff.split = sep_best_split(p, (ff.mt + 1) / 2 * ff.nt, ff.steps, group, &cost_f);
@@ -1165,7 +1188,9 @@ scatter_status prepare_separable(scatter_plan_s* p, int split_override) {
   return st == SCATTER_OK && ff.fold ? sep_prepare_side(p, ff.mt) : st;
 }
 
-scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st) {
+scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st,
+                                const CallGate& gate) {
+  const double* out_shift = p->out_shift ? p->out_shift : p->d.inst_shift;
   const SepForm& fm = p->sep_folded.fold && amp_out ? p->sep_folded : p->sep_direct;
   SepTabArgs t{};
   t.atom4 = p->d.atom4;
@@ -1180,12 +1205,13 @@ scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_ou
   t.n_steps = fm.steps;
   t.n_mt = fm.mt;
   t.A = static_cast<uint4*>(p->d.sep_A);
+  t.gate = gate;
   const int n_chunks = fm.n_chunks;
   if (fm.fold && !fm.form_a) {
     const int64_t na = fm.mt * fm.steps * 128;
     const auto kernel = fm.fold_h ? k_sep_tab_fold<true> : k_sep_tab_fold<false>;
     kernel<<<(unsigned)((na + 255) / 256), 256, 0, st>>>(p->d.sep_rec, p->d.sep_axis_d, p->d.sep_axis_dlo, p->sep_n[0],
-                                                         fm.lanes, fm.steps, fm.mt, t.A);
+                                                         fm.lanes, fm.steps, fm.mt, t.A, gate);
     p->last_launches += 1;
   } else if (p->n_slots > 0 && !fm.form_a) {
     const int64_t na = fm.mt * fm.steps * 4 * kSepM;  // real tiles; a padding tile is never read
@@ -1223,8 +1249,9 @@ scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_ou
   a.form_a = fm.form_a ? 1 : 0;
   a.rec_lo = p->d.atom_lo;
   a.rec_w = p->d.atom_w;
+  a.gate = gate;
   dim3 grid((unsigned)(((fm.mt + 1) / 2) * fm.nt), (unsigned)n_chunks);
-  timing_begin(p, st);
+  if (!gate.rmax2) timing_begin(p, st);
   const cudaError_t le = sep_launch_core(a, grid, st, p->side_stream, p->side_fork, p->side_join);
   timing_end(p, st);
   if (le != cudaSuccess) return cuda_status(le, "separable kernel launch");
@@ -1264,7 +1291,8 @@ scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_ou
       r.n_lanes = fm.lanes;
       r.fold_h = fm.fold_h ? 1 : 0;
       for (int d = 0; d < 3; ++d) r.H[d] = (float)p->inst[0].H[d];
-      r.shift = p->d.inst_shift;
+      r.shift = out_shift;
+      r.gate = gate;
       r.l8_base = b0;
       r.out_amp = amp_dst;
       r.out_int = int_dst;
@@ -1286,8 +1314,8 @@ scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_ou
           p->d.sep_partial, a.chunk_floats, n_cb, fm.chunks, n_chunks, p->d.coef, p->d.ftab,
           (float)(1.0 / (4.0 * p->lattice_a * p->lattice_a)), p->d.sep_axis_s, p->d.sep_axis_lo, p->sep_n[0],
           p->sep_n[1], p->sep_n[2],
-          make_float3((float)p->inst[0].H[0], (float)p->inst[0].H[1], (float)p->inst[0].H[2]), p->d.inst_shift,
-          p->d.sep_att, p->d.sep_szf, b0, amp_dst, int_dst);
+          make_float3((float)p->inst[0].H[0], (float)p->inst[0].H[1], (float)p->inst[0].H[2]), out_shift,
+          p->d.sep_att, p->d.sep_szf, b0, amp_dst, int_dst, gate);
     }
     p->last_launches += 1;
     if (pieces) {
