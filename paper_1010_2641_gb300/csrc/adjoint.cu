@@ -387,6 +387,7 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_adjoint(const AdjArgs a) {
 // sum v and sum S_z v, folded into double-float outer sums (FP32 pairs on
 // the FMA pipe) as S_x sum v, S_y sum v, sum S_z v.
 struct AdjLineArgs {
+  CallGate gate;
   const float4* atom4;
   const AdjBlock* blocks;
   const float4* table;      // [n_species][M]: (s_z, S_z, gF.re, gF.im)
@@ -405,6 +406,7 @@ constexpr int kReseed = 128;  // points between exact re-seeds of the recurrence
 __global__ void __launch_bounds__(kAdjThreads, 4) k_adjoint_line(const AdjLineArgs a) {
   __shared__ __align__(128) float4 sh_s[2][kSTile];
   __shared__ __align__(8) uint64_t sh_bar[2];
+  if (within(a.gate, 0)) return;
   const int tid = threadIdx.x;
   const AdjBlock blk = a.blocks[blockIdx.x];
   const int chunk = blockIdx.y;
@@ -566,7 +568,10 @@ __global__ void __launch_bounds__(kFinalVals* kFinalGroups) k_adjoint_final(cons
   const int vi = threadIdx.x % kFinalVals, grp = threadIdx.x / kFinalVals;
   const int64_t i = (int64_t)blockIdx.x * kFinalVals + vi, n = 3 * n_slots;
   dev::DFloatSum v;
-  if (within(gate, 0)) split = cl_split;
+  if (within(gate, 0)) {
+    if (cl_split == 0) return;  // the nodes have done the atoms
+    split = cl_split;
+  }
   if (i < n) {
     const int per = (split + kFinalGroups - 1) / kFinalGroups, c1 = min(split, (grp + 1) * per);
 #pragma unroll 8
@@ -597,6 +602,7 @@ scatter_status prepare_adjoint(scatter_plan_s* p) {
   scatter_status ss = prepare_adjoint_sep(p);
   if (ss != SCATTER_OK) return ss;
   if (p->adj_sep) {
+    if ((ss = prepare_coarse_adjoint(p)) != SCATTER_OK) return ss;
     p->adj_ready = true;
     return SCATTER_OK;
   }
@@ -672,8 +678,58 @@ scatter_status prepare_adjoint(scatter_plan_s* p) {
   if (part_bytes && (e = cudaMalloc(&p->d.adj_partial, part_bytes)) != cudaSuccess)
     return cuda_status(e, "cudaMalloc");
   p->base_bytes += (int64_t)(tab_bytes + part_bytes + blocks.size() * sizeof(AdjBlock));
+  if ((ss = prepare_coarse_adjoint(p)) != SCATTER_OK) return ss;
   p->adj_ready = true;
   return SCATTER_OK;
+}
+
+// The FP32 forms from the weight table, where the gate lets them.
+scatter_status launch_adjoint_tiles(scatter_plan_t p, float* grad, cudaStream_t st, const CallGate& gate) {
+  AdjArgs aa{};
+  aa.atom4 = p->d.atom4;
+  aa.blocks = p->d.adj_blocks;
+  aa.table = p->d.adj_table;
+  aa.n_s = p->n_s;
+  aa.s_per_chunk = p->adj_s_per_chunk;
+  aa.partial = p->d.adj_partial;
+  aa.n_slots = p->n_slots;
+  aa.bbox = p->d.inst_bbox;
+  aa.shift = p->d.inst_shift;
+  for (int d = 0; d < 3; ++d) aa.smax[d] = (float)p->s_max[d];
+  aa.status = p->d.status;
+  aa.gate = gate;
+  if (p->adj_blocks > 0) {
+    dim3 gridd((unsigned)p->adj_blocks, (unsigned)p->adj_split);
+    if (!gate.rmax2) timing_begin(p, st);
+    if (p->adj_line) {
+      AdjLineArgs al{};
+      al.gate = gate;
+      al.atom4 = p->d.atom4;
+      al.blocks = p->d.adj_blocks;
+      al.table = p->d.adj_table;
+      al.axis_s = p->d.axis_s;
+      for (int d = 0; d < 3; ++d) al.H[d] = (float)p->inst[0].H[d];
+      al.n0 = p->n_axis[0];
+      al.n1 = p->n_axis[1];
+      al.n2 = p->n_axis[2];
+      al.ds = p->adj_ds;
+      al.lines_per_chunk = p->adj_lines_per_chunk;
+      al.partial = p->d.adj_partial;
+      al.n_slots = p->n_slots;
+      al.status = p->d.status;
+      k_adjoint_line<<<gridd, kAdjThreads, 0, st>>>(al);
+    } else {
+      k_adjoint<<<gridd, kAdjThreads, 0, st>>>(aa);
+    }
+    timing_end(p, st);
+    p->last_launches += 1;
+  }
+  const int64_t nb = (3 * p->n_slots + kFinalVals - 1) / kFinalVals;
+  k_adjoint_final<<<(unsigned)nb, kFinalVals * kFinalGroups, 0, st>>>(p->d.adj_partial, p->adj_split, gate,
+                                                                      p->cl.adj.active ? p->cl.adj.split : 0, p->n_slots,
+                                                                      p->d.slot_src, p->d.atom_w, grad);
+  p->last_launches += 1;
+  return cuda_status(cudaGetLastError(), "backward launch");
 }
 
 scatter_status launch_backward(scatter_plan_t p, const double* xyz, const float* occ, const float2* A,
@@ -682,10 +738,18 @@ scatter_status launch_backward(scatter_plan_t p, const double* xyz, const float*
   if (p->path == SCATTER_PATH_FP64_REF)
     return fail(SCATTER_ERR_UNSUPPORTED, "backward runs on the generic path; plan with SCATTER_PATH_GENERIC");
   scatter_status s = SCATTER_OK;
+  bool coarse = false;
   if (grad) {
     if ((s = prepare_adjoint(p)) != SCATTER_OK) return s;
     // positions (and the centring t) exactly as the forward used them
-    if ((s = launch_prep(p, xyz, occ, st)) != SCATTER_OK) return s;
+    coarse = p->coarse.adjoint;
+    if (coarse) {
+      timing_begin(p, st);
+      p->coarse.sub->last_launches = 0;
+      if ((s = launch_prep(p->coarse.sub, xyz, occ, st)) != SCATTER_OK) return s;
+      p->last_launches += p->coarse.sub->last_launches;
+    }
+    if ((s = launch_prep(p, xyz, occ, st, coarse ? coarse_gate(p) : CallGate{})) != SCATTER_OK) return s;
   } else if (p->n_s > 0 && p->n_atoms > 0) {
     // loss only: the shift is not needed, but the table write is skipped too
   }
@@ -718,61 +782,20 @@ scatter_status launch_backward(scatter_plan_t p, const double* xyz, const float*
   la.gf = p->d.adj_gf;
   la.loss_part = p->d.loss_part;
   const bool clustered = grad && p->cl.adj.active;
-  const CallGate gate = clustered ? cluster_gate(p) : CallGate{};
+  const CallGate gate = clustered ? cluster_gate(p) : coarse ? coarse_gate(p) : CallGate{};
   la.gate = gate;
-  if (clustered) la.gf = reinterpret_cast<float2*>(p->d.adj_table);  // either layout, never both
+  if (clustered || (coarse && !p->adj_sep)) la.gf = reinterpret_cast<float2*>(p->d.adj_table);  // either layout, never both
   k_loss_weights<<<kLossParts, kLossThreads, 0, st>>>(la);
   p->last_launches += 1;
   if (A && loss_out) {
     k_loss_final<<<1, 256, 0, st>>>(p->d.loss_part, kLossParts, loss_out);
     p->last_launches += 1;
   }
-  if (grad && p->n_atoms > 0 && p->adj_sep) return launch_adjoint_sep(p, grad, st);
   if (grad && p->n_atoms > 0) {
-    AdjArgs aa{};
-    aa.atom4 = p->d.atom4;
-    aa.blocks = p->d.adj_blocks;
-    aa.table = p->d.adj_table;
-    aa.n_s = p->n_s;
-    aa.s_per_chunk = p->adj_s_per_chunk;
-    aa.partial = p->d.adj_partial;
-    aa.n_slots = p->n_slots;
-    aa.bbox = p->d.inst_bbox;
-    aa.shift = p->d.inst_shift;
-    for (int d = 0; d < 3; ++d) aa.smax[d] = (float)p->s_max[d];
-    aa.status = p->d.status;
-    aa.gate = gate;
+    if (coarse && (s = launch_coarse_adjoint(p, la.gf, grad, st)) != SCATTER_OK) return s;
+    if (p->adj_sep) return launch_adjoint_sep(p, grad, st, gate);
     if (clustered && (s = launch_cluster_adjoint(p, la.gf, p->d.adj_partial, st)) != SCATTER_OK) return s;
-    if (p->adj_blocks > 0) {
-      dim3 gridd((unsigned)p->adj_blocks, (unsigned)p->adj_split);
-      if (!clustered) timing_begin(p, st);
-      if (p->adj_line) {
-        AdjLineArgs al{};
-        al.atom4 = p->d.atom4;
-        al.blocks = p->d.adj_blocks;
-        al.table = p->d.adj_table;
-        al.axis_s = p->d.axis_s;
-        for (int d = 0; d < 3; ++d) al.H[d] = (float)p->inst[0].H[d];
-        al.n0 = p->n_axis[0];
-        al.n1 = p->n_axis[1];
-        al.n2 = p->n_axis[2];
-        al.ds = p->adj_ds;
-        al.lines_per_chunk = p->adj_lines_per_chunk;
-        al.partial = p->d.adj_partial;
-        al.n_slots = p->n_slots;
-        al.status = p->d.status;
-        k_adjoint_line<<<gridd, kAdjThreads, 0, st>>>(al);
-      } else {
-        k_adjoint<<<gridd, kAdjThreads, 0, st>>>(aa);
-      }
-      timing_end(p, st);
-      p->last_launches += 1;
-    }
-    const int64_t nb = (3 * p->n_slots + kFinalVals - 1) / kFinalVals;
-    k_adjoint_final<<<(unsigned)nb, kFinalVals * kFinalGroups, 0, st>>>(p->d.adj_partial, p->adj_split, gate,
-                                                                        p->cl.adj.split, p->n_slots,
-                                                                        p->d.slot_src, p->d.atom_w, grad);
-    p->last_launches += 1;
+    if ((s = launch_adjoint_tiles(p, grad, st, gate)) != SCATTER_OK) return s;
   }
   return cuda_status(cudaGetLastError(), "backward launch");
 }

@@ -75,7 +75,8 @@ __device__ __forceinline__ float scale2(float x, int k) {
 // flight, 37.7 us with 256, 7.3 us with 1024.
 __global__ void __launch_bounds__(1024) k_adj_sep_scale(const float2* __restrict__ gf, const float4* __restrict__ rec,
                                                         int64_t n0, int64_t nbc, int64_t n_k, int fold, int64_t n_s,
-                                                        int* __restrict__ sexp) {
+                                                        int* __restrict__ sexp, const CallGate gate) {
+  if (within(gate, 0)) return;
   const int64_t sp = blockIdx.x / n0, a = blockIdx.x % n0;
   const float2* row = gf + sp * n_s + a * nbc;
   float m[3] = {0.f, 0.f, 0.f};
@@ -115,11 +116,13 @@ struct AdjSepTabArgs {
   int64_t n_ksteps, n_mt, n_mp;
   int64_t total;        // threads: n_species x n_mt x n_ksteps x 512
   uint4* A;             // [species][n_mp][n_ksteps][2 tiles][hi|lo][4 kb][16 mg][8 rows] of 16 B
+  CallGate gate;
 };
 
 // One thread per 16-byte row of a core matrix (4 points x Re/Im of one A row).
 // Row 2 pa: (Pr, -Mi); row 2 pa + 1: (Pi, Mr) with P, M scaled by 2^-k.
 __global__ void k_adj_sep_tab(const AdjSepTabArgs t) {
+  if (within(t.gate, 0)) return;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= t.total) return;
   const int r = (int)(i % 8), mg = (int)((i / 8) % 16), kb = (int)((i / 128) % 4);
@@ -174,6 +177,7 @@ struct AdjSepFinalArgs {
   float H[3], H_lo[3];     // as double-floats; fold: k and l at the middles of their axes
   float mid[2], mid_lo[2]; // fold: those middles - H as double-floats, else 0
   float* grad;             // [n_atoms][3] caller order
+  CallGate gate;
 };
 
 // One warp per four atom slots: lane 2 i + ri holds row (Re or Im) of a = a0 + i
@@ -191,6 +195,7 @@ struct AdjSepFinalArgs {
 // reads were 16-byte pieces).
 constexpr int kAdjFinalWarps = 8;
 __global__ void __launch_bounds__(32 * kAdjFinalWarps) k_adj_sep_final(const AdjSepFinalArgs f) {
+  if (within(f.gate, 0)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = lane >> 1, ri = lane & 1;
   const Segment t = f.ntiles[blockIdx.x];
   const int64_t slot0 = t.begin + 4 * ((int64_t)blockIdx.y * kAdjFinalWarps + warp);
@@ -401,11 +406,11 @@ scatter_status prepare_adjoint_sep(scatter_plan_s* p) {
 
 // After k_loss_weights wrote gF (p->d.adj_gf): scales, A tables, the
 // contraction and the per-atom epilogue, all on `st`.
-scatter_status launch_adjoint_sep(scatter_plan_t p, float* grad, cudaStream_t st) {
+scatter_status launch_adjoint_sep(scatter_plan_t p, float* grad, cudaStream_t st, const CallGate& gate) {
   const int64_t n0 = p->n_axis[0], n1 = p->n_axis[1], n2 = p->n_axis[2];
   const int64_t n_mp = (p->adj_sep_mt + 1) / 2;
   k_adj_sep_scale<<<(unsigned)(p->n_species * n0), 1024, 0, st>>>(p->d.adj_gf, p->d.adj_rec, n0, n1 * n2, p->adj_sep_k,
-                                                                   p->adj_sep_fold, p->n_s, p->d.adj_sexp);
+                                                                   p->adj_sep_fold, p->n_s, p->d.adj_sexp, gate);
   AdjSepTabArgs t{};
   t.gf = p->d.adj_gf;
   t.rec = p->d.adj_rec;
@@ -420,6 +425,7 @@ scatter_status launch_adjoint_sep(scatter_plan_t p, float* grad, cudaStream_t st
   t.n_mp = n_mp;
   t.total = (int64_t)p->n_species * p->adj_sep_mt * p->adj_sep_ksteps * 512;
   t.A = static_cast<uint4*>(p->d.adj_sepA);
+  t.gate = gate;
   k_adj_sep_tab<<<(unsigned)((t.total + 255) / 256), 256, 0, st>>>(t);
   SepArgs a{};
   a.A = static_cast<const uint4*>(p->d.adj_sepA);
@@ -442,8 +448,9 @@ scatter_status launch_adjoint_sep(scatter_plan_t p, float* grad, cudaStream_t st
   a.n_mt = p->adj_sep_mt;
   a.partial = p->d.adj_sep_partial;
   a.status = p->d.status;
+  a.gate = gate;
   dim3 grid((unsigned)(n_mp * p->adj_sep_ntiles), (unsigned)p->adj_sep_chunks);
-  timing_begin(p, st);
+  if (!gate.rmax2) timing_begin(p, st);
   const cudaError_t le = sep_launch_core(a, grid, st, p->side_stream, p->side_fork, p->side_join);
   timing_end(p, st);
   if (le != cudaSuccess) return cuda_status(le, "adjoint contraction launch");
@@ -471,6 +478,7 @@ scatter_status launch_adjoint_sep(scatter_plan_t p, float* grad, cudaStream_t st
     f.mid_lo[d] = (float)(p->adj_sep_mid[d] - (double)f.mid[d]);
   }
   f.grad = grad;
+  f.gate = gate;
   k_adj_sep_final<<<dim3((unsigned)p->adj_sep_ntiles, kSepN / (4 * kAdjFinalWarps)), 32 * kAdjFinalWarps, 0, st>>>(f);
   p->last_launches += 3 + sep_core_launches(p->adj_sep_mt);
   return cuda_status(cudaGetLastError(), "adjoint launch");

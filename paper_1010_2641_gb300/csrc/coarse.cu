@@ -326,6 +326,43 @@ double form_error(const scatter_plan_s* p, int d, const Nodes& nd, double X) {
 
 }  // namespace
 
+namespace {
+
+void launch_stage(scatter_plan_t p, const InterpArgs& a, cudaStream_t st) {
+  auto tiles = [&](int64_t tile) {
+    return dim3((unsigned)((a.outer * a.inner + tile - 1) / tile), (unsigned)((a.n_out + tile - 1) / tile));
+  };
+  dim3 grid = tiles(64);
+  const bool few = (int64_t)grid.x * grid.y < 2 * p->n_sm;
+  if (few) grid = tiles(32);
+  const bool wide = p->path != SCATTER_PATH_SEPARABLE, rows = a.inner == 1 && a.axis == 2;
+  const auto kernel = wide ? (rows ? (few ? k_interp<true, true, 2> : k_interp<true, true, 4>)
+                                   : (few ? k_interp<false, true, 2> : k_interp<false, true, 4>))
+                           : (rows ? (few ? k_interp<true, false, 2> : k_interp<true, false, 4>)
+                                   : (few ? k_interp<false, false, 2> : k_interp<false, false, 4>));
+  kernel<<<grid, 256, 0, st>>>(a);
+}
+
+// The nodes' weight table of the FP32 adjoint: rows {s, gF.re | S, gF.im}, for the
+// line form (s_z, S_z, gF).
+__global__ void __launch_bounds__(256) k_node_table(const float2* __restrict__ gf, const float* __restrict__ axis_s,
+                                                    int64_t n0, int64_t n1, int64_t n2, float3 H, int64_t total,
+                                                    int line_form, float4* __restrict__ table, const CallGate gate) {
+  const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (e >= total || !within(gate, 0)) return;
+  const int64_t m = e % (n0 * n1 * n2), i2 = m % n2, line = m / n2;
+  const float sx = axis_s[line / n1], sy = axis_s[n0 + line % n1], sz = axis_s[n0 + n1 + i2];
+  const float2 g = gf[e];
+  if (line_form) {
+    table[e] = make_float4(sz, H.z + sz, g.x, g.y);
+    return;
+  }
+  table[2 * e] = make_float4(sx, sy, sz, g.x);
+  table[2 * e + 1] = make_float4(H.x + sx, H.y + sy, H.z + sz, g.y);
+}
+
+}  // namespace
+
 scatter_status prepare_coarse(scatter_plan_s* p, const scatter_problem* pr, const scatter_options* op) {
   if (p->s_kind != SCATTER_S_GRID || p->batch != 1 || pr->factor_table || p->n_atoms <= 0 || p->n_s <= 0)
     return SCATTER_OK;
@@ -427,6 +464,7 @@ scatter_status prepare_coarse(scatter_plan_s* p, const scatter_problem* pr, cons
     }
     ok = alloc(&s.W, W.size() * sizeof(float)) &&
          cudaMemcpy(s.W, W.data(), W.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
+    s.h_W = std::move(W);
     ++c.n_stages;
   }
   const float lim2 = (float)(X * X);
@@ -488,22 +526,102 @@ scatter_status launch_coarse(scatter_plan_t p, const double* xyz, const float* o
     a.inner = g.inner;
     a.outer = g.outer;
     a.axis = g.axis;
-    auto tiles = [&](int64_t tile) {
-      return dim3((unsigned)((g.outer * g.inner + tile - 1) / tile), (unsigned)((g.n_out + tile - 1) / tile));
-    };
-    dim3 grid = tiles(64);
-    const bool few = (int64_t)grid.x * grid.y < 2 * p->n_sm;
-    if (few) grid = tiles(32);
-    const bool wide = p->path != SCATTER_PATH_SEPARABLE, rows = g.axis == 2;
-    const auto kernel = wide ? (rows ? (few ? k_interp<true, true, 2> : k_interp<true, true, 4>)
-                                     : (few ? k_interp<false, true, 2> : k_interp<false, true, 4>))
-                             : (rows ? (few ? k_interp<true, false, 2> : k_interp<true, false, 4>)
-                                     : (few ? k_interp<false, false, 2> : k_interp<false, false, 4>));
-    kernel<<<grid, 256, 0, st>>>(a);
+    launch_stage(p, a, st);
     in = a.out;
     p->last_launches += 1;
   }
   return cuda_status(cudaGetLastError(), "interpolation launch");
+}
+
+// S_d e^{2 pi i S.r} is interpolated from the nodes as the wave itself is, so the
+// gradient is the nodes' own adjoint with the weights sum_S l_node(S) gF(S): the
+// interpolation's transpose, stage by stage in reverse.
+scatter_status prepare_coarse_adjoint(scatter_plan_s* p) {
+  CoarseState& c = p->coarse;
+  if (!c.sub || c.adjoint || p->n_s <= 0 || p->n_atoms <= 0) return SCATTER_OK;
+  const bool sep = p->adj_sep;
+  if (!sep && p->path == SCATTER_PATH_SEPARABLE) return SCATTER_OK;
+  // pairs per second: tensor cores 5e13 (fewer points 4e13), line recurrence
+  // 3.4e12, the nodes' tiles 2e12
+  const double pairs = (double)p->n_slots;
+  const double fine = pairs * (double)p->n_s / (sep ? 5.0e13 : p->adj_line ? 3.4e12 : 2.0e12);
+  const double few = pairs * (double)c.sub->n_s / (sep ? 4.0e13 : 2.0e12) + 60e-6 +
+                     (double)p->n_s * p->n_species * 30.0 / 4.0e12;
+  if (few > 0.75 * fine) return SCATTER_OK;
+  const int64_t before = c.sub->base_bytes;
+  if (prepare_adjoint(c.sub) != SCATTER_OK || c.sub->adj_sep != sep) return SCATTER_OK;
+  int64_t bytes = c.sub->base_bytes - before;
+  auto alloc = [&](void* ptr, size_t size) {
+    bytes += (int64_t)size;
+    return cudaMalloc(static_cast<void**>(ptr), std::max<size_t>(size, 16)) == cudaSuccess;
+  };
+  bool ok = true;
+  for (int i = 0; i < c.n_stages && ok; ++i) {
+    CoarseStage& s = c.stage[i];
+    std::vector<float> T(s.h_W.size());
+    const size_t n = (size_t)(s.n_in * s.n_out);
+    for (int part = 0; part < 2; ++part)
+      for (int64_t k = 0; k < s.n_in; ++k)
+        for (int64_t j = 0; j < s.n_out; ++j) T[part * n + j * s.n_in + k] = s.h_W[part * n + k * s.n_out + j];
+    ok = alloc(&s.Wt, T.size() * sizeof(float)) &&
+         cudaMemcpy(s.Wt, T.data(), T.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
+    // stage i leaves the input of the forward's stage i
+    const size_t out = (size_t)p->n_species * (size_t)(s.outer * s.n_in * s.inner) * sizeof(float2);
+    if (i > 0 && ok) ok = alloc(&c.adj_tmp[i - 1], out);
+    if (i == 0 && ok && !sep) ok = alloc(&c.adj_gf, out);
+  }
+  // a crystal past the nodes leaves the weights as they are: zeros at first
+  if (ok) {
+    float2* w = sep ? c.sub->d.adj_gf : c.adj_gf;
+    ok = cudaMemset(w, 0, (size_t)p->n_species * (size_t)c.sub->n_s * sizeof(float2)) == cudaSuccess &&
+         (sep || cudaMemset(c.sub->d.adj_table, 0, (size_t)p->n_species * (size_t)c.sub->n_s * 2 * sizeof(float4)) == cudaSuccess);
+  }
+  if (!ok) {
+    cudaGetLastError();
+    return SCATTER_OK;  // what was allocated goes with the plan
+  }
+  p->base_bytes += bytes;
+  c.adjoint = true;
+  return SCATTER_OK;
+}
+
+scatter_status launch_coarse_adjoint(scatter_plan_t p, const float2* gf, float* grad, cudaStream_t st) {
+  const CoarseState& c = p->coarse;
+  scatter_plan_s* sub = c.sub;
+  InterpArgs a{};
+  a.gate = coarse_gate(p);
+  a.shift = p->d.inst_shift;
+  const float2* in = gf;
+  for (int i = c.n_stages - 1; i >= 0; --i) {
+    const CoarseStage& g = c.stage[i];
+    a.in = in;
+    a.out = i > 0 ? c.adj_tmp[i - 1] : p->adj_sep ? sub->d.adj_gf : c.adj_gf;
+    a.W = g.Wt;
+    a.W_lo = g.Wt + g.n_in * g.n_out;
+    a.n_in = g.n_out;
+    a.n_out = g.n_in;
+    a.outer = p->n_species * g.outer;
+    a.inner = g.inner;
+    a.axis = g.axis;
+    launch_stage(p, a, st);
+    in = a.out;
+    p->last_launches += 1;
+  }
+  sub->last_launches = 0;
+  scatter_status s;
+  if (p->adj_sep) {
+    s = launch_adjoint_sep(sub, grad, st);
+  } else {
+    const int64_t total = (int64_t)p->n_species * sub->n_s;
+    k_node_table<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(
+        in, sub->d.axis_s, sub->n_axis[0], sub->n_axis[1], sub->n_axis[2],
+        make_float3((float)p->inst[0].H[0], (float)p->inst[0].H[1], (float)p->inst[0].H[2]), total, sub->adj_line,
+        sub->d.adj_table, a.gate);
+    p->last_launches += 1;
+    s = launch_adjoint_tiles(sub, grad, st);
+  }
+  p->last_launches += sub->last_launches;
+  return s;
 }
 
 void release_coarse(scatter_plan_s* p) {
@@ -514,8 +632,9 @@ void release_coarse(scatter_plan_s* p) {
     scatter_plan_destroy(c.sub);
   }
   for (CoarseStage& s : c.stage)
-    if (s.W) cudaFree(s.W);
-  for (void* b : {(void*)c.map, (void*)c.tmp[0], (void*)c.tmp[1], (void*)c.rmax2, (void*)c.lim2, (void*)c.no_shift})
+    for (float* w : {s.W, s.Wt})
+      if (w) cudaFree(w);
+  for (void* b : {(void*)c.adj_tmp[0], (void*)c.adj_tmp[1], (void*)c.adj_gf, (void*)c.map, (void*)c.tmp[0], (void*)c.tmp[1], (void*)c.rmax2, (void*)c.lim2, (void*)c.no_shift})
     if (b) cudaFree(b);
   c = CoarseState{};
 }

@@ -93,6 +93,9 @@ scatter_status prepare_coarse(scatter_plan_s* p, const scatter_problem* pr, cons
 scatter_status launch_coarse(scatter_plan_t p, const double* xyz, const float* occ, float2* amp_out, float* int_out,
                              cudaStream_t st);
 void release_coarse(scatter_plan_s* p);
+// The adjoint from the weights gF [species][M] contracted to the nodes.
+scatter_status prepare_coarse_adjoint(scatter_plan_s* p);
+scatter_status launch_coarse_adjoint(scatter_plan_t p, const float2* gf, float* grad, cudaStream_t st);
 // Tensor-core intensities keep the direct sum: |A|^2 doubles the difference
 // between the two (up to 2.5e-5 of the map, amplitudes 1.6e-5).
 inline bool coarse_serves(const scatter_plan_s* p, const void* amp_out) {
@@ -137,7 +140,12 @@ scatter_status launch_backward(scatter_plan_t p, const double* xyz, const float*
 // Tensor-core adjoint on grids of SEPARABLE plans (adjoint_sep.cu).
 bool adjoint_sep_applicable(const scatter_plan_s* p);
 scatter_status prepare_adjoint_sep(scatter_plan_s* p);
-scatter_status launch_adjoint_sep(scatter_plan_t p, float* grad, cudaStream_t st);
+scatter_status launch_adjoint_sep(scatter_plan_t p, float* grad, cudaStream_t st,
+                                  const CallGate& gate = CallGate{});
+// FP32 adjoint from the plan's weight table (adjoint.cu).
+scatter_status launch_adjoint_tiles(scatter_plan_t p, float* grad, cudaStream_t st,
+                                    const CallGate& gate = CallGate{});
+scatter_status prepare_adjoint(scatter_plan_s* p);
 
 // Grazing-incidence (DWBA) path: plan tables, split choice, launches.
 scatter_status prepare_gid(scatter_plan_s* p);

@@ -170,6 +170,8 @@ struct CoarseStage {
   int64_t n_in = 0, n_out = 0;      // nodes, points of the axis
   int64_t outer = 0, inner = 0;     // of the array at that stage
   float* W = nullptr;               // [n_in][n_out], then its rounding errors
+  float* Wt = nullptr;              // the adjoint's: [n_out][n_in], then its rounding errors
+  std::vector<float> h_W;           // W on the host
 };
 struct CoarseState {
   scatter_plan_s* sub = nullptr;    // the sum at the nodes, without the translation phase
@@ -180,6 +182,9 @@ struct CoarseState {
   unsigned* rmax2 = nullptr;        // this call's largest |x'_d|^2 (float bits)
   float* lim2 = nullptr;
   double* no_shift = nullptr;       // [3] zeros
+  bool adjoint = false;             // the adjoint at the nodes too
+  float2* adj_tmp[2] = {nullptr, nullptr};
+  float2* adj_gf = nullptr;         // weights at the nodes (FP32 sums)
 };
 
 // The factorised FP32 grid sum (gridsum.cu).
