@@ -738,18 +738,14 @@ scatter_status launch_backward(scatter_plan_t p, const double* xyz, const float*
   if (p->path == SCATTER_PATH_FP64_REF)
     return fail(SCATTER_ERR_UNSUPPORTED, "backward runs on the generic path; plan with SCATTER_PATH_GENERIC");
   scatter_status s = SCATTER_OK;
-  bool coarse = false;
+  int coarse = 0;  // node sets
   if (grad) {
     if ((s = prepare_adjoint(p)) != SCATTER_OK) return s;
     // positions (and the centring t) exactly as the forward used them
-    coarse = p->coarse.adjoint;
-    if (coarse) {
-      timing_begin(p, st);
-      p->coarse.sub->last_launches = 0;
-      if ((s = launch_prep(p->coarse.sub, xyz, occ, st)) != SCATTER_OK) return s;
-      p->last_launches += p->coarse.sub->last_launches;
-    }
-    if ((s = launch_prep(p, xyz, occ, st, coarse ? coarse_gate(p) : CallGate{})) != SCATTER_OK) return s;
+    coarse = p->coarse_adj_levels;
+    if (coarse) timing_begin(p, st);
+    if ((s = launch_coarse_prep(p, coarse, xyz, occ, st)) != SCATTER_OK) return s;
+    if ((s = launch_prep(p, xyz, occ, st, coarse_gate(p, coarse))) != SCATTER_OK) return s;
   } else if (p->n_s > 0 && p->n_atoms > 0) {
     // loss only: the shift is not needed, but the table write is skipped too
   }
@@ -782,7 +778,7 @@ scatter_status launch_backward(scatter_plan_t p, const double* xyz, const float*
   la.gf = p->d.adj_gf;
   la.loss_part = p->d.loss_part;
   const bool clustered = grad && p->cl.adj.active;
-  const CallGate gate = clustered ? cluster_gate(p) : coarse ? coarse_gate(p) : CallGate{};
+  const CallGate gate = clustered ? cluster_gate(p) : coarse_gate(p, coarse);
   la.gate = gate;
   if (clustered || (coarse && !p->adj_sep)) la.gf = reinterpret_cast<float2*>(p->d.adj_table);  // either layout, never both
   k_loss_weights<<<kLossParts, kLossThreads, 0, st>>>(la);

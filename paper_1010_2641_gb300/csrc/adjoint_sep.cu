@@ -321,6 +321,30 @@ bool adjoint_sep_applicable(const scatter_plan_s* p) {
          p->n_s > 0 && p->n_slots % kSepStep == 0;
 }
 
+namespace {
+
+// The (k, l) plane folds over its middle where both axes are symmetric.
+bool adj_folds(const scatter_plan_s* p, double (&mid)[2]) {
+  return !p->adj_no_fold && sep_axis_middle(p->axis_host[1], p->inst[0].H[1], &mid[0]) &&
+         sep_axis_middle(p->axis_host[2], p->inst[0].H[2], &mid[1]);
+}
+
+}  // namespace
+
+double adjoint_sep_group(const scatter_plan_s* p, bool fold) {
+  double mid[2];
+  fold = fold && adj_folds(p, mid);
+  const int64_t nbc = p->n_axis[1] * p->n_axis[2], n_k = fold ? (nbc + 1) / 2 : nbc;
+  const int64_t n_ksteps = (n_k + kSepStep - 1) / kSepStep;
+  const int64_t n_mt = (2 * 3 * p->n_axis[0] + kSepM - 1) / kSepM;
+  int64_t tiles = 0;
+  for (const Segment& sg : p->all_segs) tiles += (sg.end - sg.begin + kSepN - 1) / kSepN;
+  const int split = adj_sep_split(p, (n_mt + 1) / 2 * tiles, n_ksteps,
+                                  (size_t)sep_part_floats(n_mt, p->n_slots) * sizeof(float), fold);
+  const int64_t per = (n_ksteps + split - 1) / split, full = per / kSepFlush, rest = per % kSepFlush;
+  return (double)(full * kSepFlush * kSepFlush + rest * rest) / (double)per;
+}
+
 // Tables and tiling of the tensor-core adjoint; leaves p->adj_sep false (and
 // allocates nothing) when the map is too large for its workspace.
 scatter_status prepare_adjoint_sep(scatter_plan_s* p) {
@@ -328,10 +352,8 @@ scatter_status prepare_adjoint_sep(scatter_plan_s* p) {
   if (!adjoint_sep_applicable(p)) return SCATTER_OK;
   const int64_t n0 = p->n_axis[0], n1 = p->n_axis[1], n2 = p->n_axis[2];
   const int64_t nbc = n1 * n2;
-  // fold the (k, l) plane over its middle where both axes are symmetric
   double mid[2] = {0, 0};
-  const bool fold = sep_axis_middle(p->axis_host[1], p->inst[0].H[1], &mid[0]) &&
-                    sep_axis_middle(p->axis_host[2], p->inst[0].H[2], &mid[1]);
+  const bool fold = adj_folds(p, mid);
   const int64_t n_k = fold ? (nbc + 1) / 2 : nbc;
   const int64_t n_ksteps = (n_k + kSepStep - 1) / kSepStep;
   const int64_t n_mt = (2 * 3 * n0 + kSepM - 1) / kSepM;

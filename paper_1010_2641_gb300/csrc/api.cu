@@ -61,7 +61,7 @@ scatter_status enqueue_single(scatter_plan_t p, const double* xyz, const float* 
   // the map from its nodes; what follows is for a crystal that these don't resolve
   const bool coarse = coarse_serves(p, amp);
   if (coarse && (s = launch_coarse(p, xyz, occ, amp, inten, st)) != SCATTER_OK) return s;
-  const CallGate gate = coarse ? coarse_gate(p) : CallGate{};
+  const CallGate gate = coarse_gate(p, coarse ? p->coarse_levels : 0);
   if ((s = launch_prep(p, xyz, occ, st, gate)) != SCATTER_OK) return s;
   if (p->path == SCATTER_PATH_SEPARABLE) return launch_separable(p, amp, inten, st, gate);  // GRID and GID_GRID
   return p->s_kind == SCATTER_S_GID_GRID ? launch_dwba(p, amp, inten, st) : launch_generic(p, amp, inten, st, gate);

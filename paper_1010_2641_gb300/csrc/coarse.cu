@@ -16,10 +16,11 @@
 // translation phase e^{2 pi i s.t}, which would add |t| to the bandwidth; the
 // last interpolation stage applies it.
 //
-// X is chosen at plan time: the caller's radius hint, or 1.3 of a compact
-// crystal's radius at four atoms per cell (which holds a simple cubic cube).  A
-// call measures its largest |x'_d|; a crystal past X is left to the direct
-// kernels, whose launches otherwise return at once (CallGate).
+// X is chosen at plan time: the caller's radius hint, or up to two node sets for
+// 1.1 (a sphere, a cube, a slab) and 1.3 (a simple cubic cube) of a compact crystal's radius at
+// four atoms per cell.  A call measures its largest |x'_d|; the smallest set that
+// holds it serves, and a crystal past them is left to the direct kernels.  The
+// others' launches return at once (CallGate).
 #include <cuda_runtime.h>
 #include <algorithm>
 #include <cmath>
@@ -35,6 +36,11 @@ namespace {
 // interpolation error of one wave at |x'_d| = X (it falls a hundredfold by 0.9 X):
 // FP32 sums, tensor-core sums (3e-5 by themselves)
 constexpr double kCoarseEps = 5e-8, kCoarseEpsSep = 1e-6;
+// Truncation in the tensor cores' accumulators shrinks a gradient by up to 1.3e-7
+// per step of a group, on coherent maps.  The nodes' planes have fewer steps than
+// the map's; they are taken where that moves a gradient by less than the tensor-core
+// path's own scatter, 1.8e-5.
+constexpr double kCoarseAdjSteps = 135.0;  // 1.8e-5 / 1.3e-7
 constexpr int kIpK = 16;  // nodes per stage of the interpolation
 
 struct InterpArgs {
@@ -73,7 +79,7 @@ __global__ void __launch_bounds__(256) k_interp(const InterpArgs a) {
   __shared__ float2 sh_in[kIpK][kIpTile + (ROWS ? 1 : 0)];
   using u64 = unsigned long long;
   static_assert(T == 2 || T == 4, "outputs and columns per thread");
-  if (!within(a.gate, 0)) return;
+  if (within(a.gate, 0)) return;
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
   const int64_t b0 = (int64_t)blockIdx.x * kIpTile, i0 = (int64_t)blockIdx.y * kIpTile;
   const int64_t cols = a.outer * a.inner;
@@ -349,7 +355,7 @@ __global__ void __launch_bounds__(256) k_node_table(const float2* __restrict__ g
                                                     int64_t n0, int64_t n1, int64_t n2, float3 H, int64_t total,
                                                     int line_form, float4* __restrict__ table, const CallGate gate) {
   const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (e >= total || !within(gate, 0)) return;
+  if (e >= total || within(gate, 0)) return;
   const int64_t m = e % (n0 * n1 * n2), i2 = m % n2, line = m / n2;
   const float sx = axis_s[line / n1], sy = axis_s[n0 + line % n1], sz = axis_s[n0 + n1 + i2];
   const float2 g = gf[e];
@@ -363,19 +369,35 @@ __global__ void __launch_bounds__(256) k_node_table(const float2* __restrict__ g
 
 }  // namespace
 
-scatter_status prepare_coarse(scatter_plan_s* p, const scatter_problem* pr, const scatter_options* op) {
-  if (p->s_kind != SCATTER_S_GRID || p->batch != 1 || pr->factor_table || p->n_atoms <= 0 || p->n_s <= 0)
-    return SCATTER_OK;
-  const bool sep = p->path == SCATTER_PATH_SEPARABLE;
-  if (!sep && !(p->path == SCATTER_PATH_GENERIC && p->gs.active)) return SCATTER_OK;
-  if (op && (op->threads || op->points_per_thread || op->split_k || op->atoms_per_thread > 0)) return SCATTER_OK;
-  const double compact = std::cbrt(3.0 * (double)p->n_atoms / (16.0 * 3.14159265358979323846));
-  const double X = op && op->radius_hint > 0.0 ? op->radius_hint : 1.3 * compact + 1.0;
-  std::vector<double> nodes[3];
+namespace {
+
+// Nodes that resolve crystals with |x'_d| <= X on the map's axes.
+struct NodeSet {
+  double X = 0.0, seconds = 1e300;  // by the model
+  std::vector<double> axis[3];      // nodes, or the axis' own points
   Nodes nd[3];
+};
+
+// Time of a sum at n0 x n12 points on the plan's path.  FP32: pairs per second.
+// Tensor cores: 1 us (up to 64 mirror pairs 0.75 us) per step of 32 atoms and tile
+// of 64 lanes x 128 mirror pairs, in chunks of at least some 200 steps.
+double sum_seconds(const scatter_plan_s* p, double n0, double n12) {
+  const double N = (double)p->n_slots;
+  if (p->path != SCATTER_PATH_SEPARABLE) return N * n0 * n12 / 1.0e13;
+  const double tiles = std::ceil(n0 / 128.0) * std::ceil(n12 / 256.0), steps = N / 32.0;
+  double best = 1e300;
+  for (double k = 1.0; k <= std::max(1.0, steps / 200.0); k += 1.0)
+    best = std::min(best, std::ceil(tiles * k / p->n_sm) * (steps / k + 40.0) * (n12 <= 128.0 ? 0.75e-6 : 1e-6));
+  return best;
+}
+
+NodeSet choose_nodes(const scatter_plan_s* p, double X) {
+  NodeSet r;
+  r.X = X;
+  const bool sep = p->path == SCATTER_PATH_SEPARABLE;
   const double eps = sep ? kCoarseEpsSep : kCoarseEps;
   bool any = false;
-  double M = 1.0, Mc = 1.0;
+  double M = 1.0;
   for (int d = 0; d < 3; ++d) {
     const std::vector<double>& ax = p->axis_host[d];
     const double lo = *std::min_element(ax.begin(), ax.end()), hi = *std::max_element(ax.begin(), ax.end());
@@ -387,25 +409,56 @@ scatter_status prepare_coarse(scatter_plan_s* p, const scatter_problem* pr, cons
         const std::vector<double> tail = chebyshev_tails(c, most);
         for (n = 4; n <= most && tail[n] > eps;) ++n;
         for (; n <= most; n += 2)
-          if (form_error(p, d, nd[d] = chebyshev_nodes(lo, hi, n), X) < 2.0 * eps) break;
+          if (form_error(p, d, r.nd[d] = chebyshev_nodes(lo, hi, n), X) < 2.0 * eps) break;
         if (n > most) n = 0;
       }
     }
-    if (n > 0) {
-      nodes[d] = nd[d].x;
-      any = true;
-    } else {
-      nodes[d] = ax;
-    }
+    any = any || n > 0;
+    r.axis[d] = n > 0 ? r.nd[d].x : ax;
     M *= (double)ax.size();
-    Mc *= (double)nodes[d].size();
   }
-  // taken where the time saved by the model (pairs per second of the path, a
-  // smaller grid fills the SMs less well) is worth the extra launches
-  const double N = (double)p->n_slots;
-  const double fine = sep ? N * M / 1.5e14 : N * M / 1.0e13;
-  const double few = (sep ? N * Mc / 7.0e13 : N * Mc / 0.9e13) + 60e-6 + M * 30.0 / 4.0e12;
-  if (!any || few > 0.75 * fine || p->n_axis[0] > 4000000 || p->n_axis[1] > 4000000 || p->n_axis[2] > 4000000) return SCATTER_OK;
+  const double sum = sum_seconds(p, r.axis[0].size(), (double)r.axis[1].size() * (double)r.axis[2].size());
+  if (any) r.seconds = sum + 60e-6 + M * 30.0 / 4.0e12;
+  return r;
+}
+
+bool build_level(scatter_plan_s* p, const scatter_problem* pr, const scatter_options* op, const NodeSet& set);
+void release_level(scatter_plan_s* p, CoarseState& c);
+
+}  // namespace
+
+scatter_status prepare_coarse(scatter_plan_s* p, const scatter_problem* pr, const scatter_options* op) {
+  if (p->s_kind != SCATTER_S_GRID || p->batch != 1 || pr->factor_table || p->n_atoms <= 0 || p->n_s <= 0)
+    return SCATTER_OK;
+  const bool sep = p->path == SCATTER_PATH_SEPARABLE;
+  if (!sep && !(p->path == SCATTER_PATH_GENERIC && p->gs.active)) return SCATTER_OK;
+  if (op && (op->threads || op->points_per_thread || op->split_k || op->atoms_per_thread > 0)) return SCATTER_OK;
+  for (int d = 0; d < 3; ++d)
+    if (p->n_axis[d] > 4000000) return SCATTER_OK;
+  // taken where the time saved by the model is worth the extra launches; two sets
+  // where the tighter one saves some more (20 us of launches that return at once:
+  // 35,802 against 24,600 nodes of 61 x 47 x 33 points: 567 against 436 us)
+  const double fine = sum_seconds(p, (double)p->n_axis[0], (double)p->n_axis[1] * (double)p->n_axis[2]);
+  const double compact = std::cbrt(3.0 * (double)p->n_atoms / (16.0 * 3.14159265358979323846));
+  std::vector<NodeSet> sets;
+  if (op && op->radius_hint > 0.0) {
+    sets.push_back(choose_nodes(p, op->radius_hint));
+  } else {
+    sets.push_back(choose_nodes(p, 1.1 * compact + 1.0));
+    sets.push_back(choose_nodes(p, 1.3 * compact + 1.0));
+    if (sets[1].seconds <= 0.75 * fine && sets[0].seconds + 40e-6 > sets[1].seconds) sets.erase(sets.begin());
+  }
+  for (const NodeSet& set : sets)
+    if (set.seconds <= 0.75 * fine && !build_level(p, pr, op, set)) break;
+  return SCATTER_OK;
+}
+
+namespace {
+
+bool build_level(scatter_plan_s* p, const scatter_problem* pr, const scatter_options* op, const NodeSet& set) {
+  const bool sep = p->path == SCATTER_PATH_SEPARABLE;
+  const std::vector<double>* nodes = set.axis;
+  const Nodes* nd = set.nd;
   scatter_problem q = *pr;
   scatter_options o{};
   if (op) o = *op;
@@ -418,7 +471,7 @@ scatter_status prepare_coarse(scatter_plan_s* p, const scatter_problem* pr, cons
     q.axis[d] = nodes[d].data();
     q.n_axis[d] = (int64_t)nodes[d].size();
   }
-  CoarseState& c = p->coarse;
+  CoarseState& c = p->coarse[p->coarse_levels];
   const double H[3] = {p->inst[0].H[0], p->inst[0].H[1], p->inst[0].H[2]};
   bool ok = plan_nodes(&q, &o, H, sep ? 0.9 * sep_direct_group(p) : 0.0, &c.sub) == SCATTER_OK && (sep || c.sub->gs.active);
   // stages in the order that costs the least
@@ -467,87 +520,110 @@ scatter_status prepare_coarse(scatter_plan_s* p, const scatter_problem* pr, cons
     s.h_W = std::move(W);
     ++c.n_stages;
   }
-  const float lim2 = (float)(X * X);
-  ok = ok && alloc(&c.map, (size_t)c.sub->n_s * sizeof(float2)) && alloc(&c.rmax2, sizeof(unsigned)) &&
-       alloc(&c.lim2, sizeof(float)) && alloc(&c.no_shift, 3 * sizeof(double)) &&
-       cudaMemset(c.rmax2, 0, sizeof(unsigned)) == cudaSuccess && cudaMemset(c.no_shift, 0, 3 * sizeof(double)) == cudaSuccess &&
+  const float lim2 = (float)(set.X * set.X);
+  ok = ok && alloc(&c.map, (size_t)c.sub->n_s * sizeof(float2)) && alloc(&c.lim2, sizeof(float)) &&
+       (p->coarse_rmax2 || (alloc(&p->coarse_rmax2, sizeof(unsigned)) && alloc(&p->coarse_no_shift, 3 * sizeof(double)) &&
+                            cudaMemset(p->coarse_rmax2, 0, sizeof(unsigned)) == cudaSuccess &&
+                            cudaMemset(p->coarse_no_shift, 0, 3 * sizeof(double)) == cudaSuccess)) &&
        cudaMemcpy(c.lim2, &lim2, sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
   for (int i = 0; i < c.n_stages - 1; ++i) ok = ok && alloc(&c.tmp[i], (size_t)tmp[i] * sizeof(float2));
   if (!ok) {  // no room: the direct kernels need none of it
     cudaGetLastError();
-    release_coarse(p);
-    return SCATTER_OK;
+    release_level(p, c);
+    return false;
   }
   // the call's status word and shift are the map's own
   cudaFree(c.sub->d.status);
   cudaFree(c.sub->d.inst_shift);
   c.sub->d.status = p->d.status;
   c.sub->d.inst_shift = p->d.inst_shift;
-  c.sub->extent2 = c.rmax2;
-  c.sub->out_shift = c.no_shift;
+  c.sub->extent2 = p->coarse_levels == 0 ? p->coarse_rmax2 : nullptr;  // measured once
+  c.sub->out_shift = p->coarse_no_shift;
   p->base_bytes += bytes + c.sub->base_bytes + c.sub->tiling_bytes;
+  ++p->coarse_levels;
+  return true;
+}
+
+}  // namespace
+
+scatter_status launch_coarse_prep(scatter_plan_t p, int levels, const double* xyz, const float* occ, cudaStream_t st) {
+  for (int l = 0; l < levels; ++l) {
+    scatter_plan_s* sub = p->coarse[l].sub;
+    sub->last_launches = 0;
+    if (const scatter_status s = launch_prep(sub, xyz, occ, st, coarse_gate(p, l)); s != SCATTER_OK) return s;
+    p->last_launches += sub->last_launches;
+  }
   return SCATTER_OK;
 }
 
 scatter_status launch_coarse(scatter_plan_t p, const double* xyz, const float* occ, float2* amp_out, float* int_out,
                              cudaStream_t st) {
-  const CoarseState& c = p->coarse;
   timing_begin(p, st);  // to the end of the direct kernel, which may do the work instead
-  c.sub->last_launches = 0;
-  scatter_status s = launch_prep(c.sub, xyz, occ, st);
-  if (s == SCATTER_OK)
-    s = p->path == SCATTER_PATH_SEPARABLE ? launch_separable(c.sub, c.map, nullptr, st)
-                                          : launch_generic(c.sub, c.map, nullptr, st);
-  if (s != SCATTER_OK) return s;
-  p->last_launches += c.sub->last_launches;
-  InterpArgs a{};
-  a.axis_s = p->d.axis_s;
-  a.axis_lo = p->d.axis_lo;
-  a.axis64 = p->d.axis64;
-  for (int d = 0; d < 3; ++d) a.H64[d] = p->inst[0].H[d];
-  a.exact64 = p->path != SCATTER_PATH_SEPARABLE;
-  a.n0 = p->n_axis[0];
-  a.n1 = p->n_axis[1];
-  a.n2 = p->n_axis[2];
-  a.shift = p->d.inst_shift;
-  a.out_amp = amp_out;
-  a.out_int = int_out;
-  a.gate = coarse_gate(p);
-  const float2* in = c.map;
-  for (int i = 0; i < c.n_stages; ++i) {
-    const CoarseStage& g = c.stage[i];
-    a.in = in;
-    a.last = i + 1 == c.n_stages;
-    a.out = a.last ? nullptr : c.tmp[i];
-    a.W = g.W;
-    a.W_lo = g.W + g.n_in * g.n_out;
-    a.n_in = g.n_in;
-    a.n_out = g.n_out;
-    a.inner = g.inner;
-    a.outer = g.outer;
-    a.axis = g.axis;
-    launch_stage(p, a, st);
-    in = a.out;
-    p->last_launches += 1;
+  scatter_status s = launch_coarse_prep(p, p->coarse_levels, xyz, occ, st);
+  for (int l = 0; l < p->coarse_levels && s == SCATTER_OK; ++l) {
+    const CoarseState& c = p->coarse[l];
+    const CallGate gate = level_gate(p, l);
+    c.sub->last_launches = 0;
+    s = p->path == SCATTER_PATH_SEPARABLE ? launch_separable(c.sub, c.map, nullptr, st, gate)
+                                          : launch_generic(c.sub, c.map, nullptr, st, gate);
+    p->last_launches += c.sub->last_launches;
+    InterpArgs a{};
+    a.axis_s = p->d.axis_s;
+    a.axis_lo = p->d.axis_lo;
+    a.axis64 = p->d.axis64;
+    for (int d = 0; d < 3; ++d) a.H64[d] = p->inst[0].H[d];
+    a.exact64 = p->path != SCATTER_PATH_SEPARABLE;
+    a.n0 = p->n_axis[0];
+    a.n1 = p->n_axis[1];
+    a.n2 = p->n_axis[2];
+    a.shift = p->d.inst_shift;
+    a.out_amp = amp_out;
+    a.out_int = int_out;
+    a.gate = gate;
+    const float2* in = c.map;
+    for (int i = 0; i < c.n_stages; ++i) {
+      const CoarseStage& g = c.stage[i];
+      a.in = in;
+      a.last = i + 1 == c.n_stages;
+      a.out = a.last ? nullptr : c.tmp[i];
+      a.W = g.W;
+      a.W_lo = g.W + g.n_in * g.n_out;
+      a.n_in = g.n_in;
+      a.n_out = g.n_out;
+      a.outer = g.outer;
+      a.inner = g.inner;
+      a.axis = g.axis;
+      launch_stage(p, a, st);
+      in = a.out;
+      p->last_launches += 1;
+    }
   }
-  return cuda_status(cudaGetLastError(), "interpolation launch");
+  return s != SCATTER_OK ? s : cuda_status(cudaGetLastError(), "interpolation launch");
 }
 
 // S_d e^{2 pi i S.r} is interpolated from the nodes as the wave itself is, so the
 // gradient is the nodes' own adjoint with the weights sum_S l_node(S) gF(S): the
 // interpolation's transpose, stage by stage in reverse.
 scatter_status prepare_coarse_adjoint(scatter_plan_s* p) {
-  CoarseState& c = p->coarse;
-  if (!c.sub || c.adjoint || p->n_s <= 0 || p->n_atoms <= 0) return SCATTER_OK;
   const bool sep = p->adj_sep;
+  const int l = p->coarse_adj_levels;
+  if (l >= p->coarse_levels) return SCATTER_OK;
+  CoarseState& c = p->coarse[l];
   if (!sep && p->path == SCATTER_PATH_SEPARABLE) return SCATTER_OK;
   // pairs per second: tensor cores 5e13 (fewer points 4e13), line recurrence
   // 3.4e12, the nodes' tiles 2e12
   const double pairs = (double)p->n_slots;
   const double fine = pairs * (double)p->n_s / (sep ? 5.0e13 : p->adj_line ? 3.4e12 : 2.0e12);
-  const double few = pairs * (double)c.sub->n_s / (sep ? 4.0e13 : 2.0e12) + 60e-6 +
+  bool fold = true;
+  if (sep) {
+    const double least = adjoint_sep_group(p, false) - kCoarseAdjSteps;
+    fold = adjoint_sep_group(c.sub, true) >= least;
+    if (!fold && adjoint_sep_group(c.sub, false) < least) return SCATTER_OK;
+  }
+  const double few = pairs * (double)c.sub->n_s / (!sep ? 2.0e12 : fold ? 4.0e13 : 2.0e13) + 60e-6 +
                      (double)p->n_s * p->n_species * 30.0 / 4.0e12;
-  if (few > 0.75 * fine) return SCATTER_OK;
+  if (few > 0.75 * fine) return SCATTER_OK;  // nor any larger set
+  c.sub->adj_no_fold = !fold;
   const int64_t before = c.sub->base_bytes;
   if (prepare_adjoint(c.sub) != SCATTER_OK || c.sub->adj_sep != sep) return SCATTER_OK;
   int64_t bytes = c.sub->base_bytes - before;
@@ -570,26 +646,22 @@ scatter_status prepare_coarse_adjoint(scatter_plan_s* p) {
     if (i > 0 && ok) ok = alloc(&c.adj_tmp[i - 1], out);
     if (i == 0 && ok && !sep) ok = alloc(&c.adj_gf, out);
   }
-  // a crystal past the nodes leaves the weights as they are: zeros at first
-  if (ok) {
-    float2* w = sep ? c.sub->d.adj_gf : c.adj_gf;
-    ok = cudaMemset(w, 0, (size_t)p->n_species * (size_t)c.sub->n_s * sizeof(float2)) == cudaSuccess &&
-         (sep || cudaMemset(c.sub->d.adj_table, 0, (size_t)p->n_species * (size_t)c.sub->n_s * 2 * sizeof(float4)) == cudaSuccess);
-  }
   if (!ok) {
     cudaGetLastError();
     return SCATTER_OK;  // what was allocated goes with the plan
   }
   p->base_bytes += bytes;
-  c.adjoint = true;
-  return SCATTER_OK;
+  ++p->coarse_adj_levels;
+  return prepare_coarse_adjoint(p);  // the next set
 }
 
-scatter_status launch_coarse_adjoint(scatter_plan_t p, const float2* gf, float* grad, cudaStream_t st) {
-  const CoarseState& c = p->coarse;
+namespace {
+
+scatter_status level_adjoint(scatter_plan_t p, int l, const float2* gf, float* grad, cudaStream_t st) {
+  const CoarseState& c = p->coarse[l];
   scatter_plan_s* sub = c.sub;
   InterpArgs a{};
-  a.gate = coarse_gate(p);
+  a.gate = level_gate(p, l);
   a.shift = p->d.inst_shift;
   const float2* in = gf;
   for (int i = c.n_stages - 1; i >= 0; --i) {
@@ -610,7 +682,7 @@ scatter_status launch_coarse_adjoint(scatter_plan_t p, const float2* gf, float* 
   sub->last_launches = 0;
   scatter_status s;
   if (p->adj_sep) {
-    s = launch_adjoint_sep(sub, grad, st);
+    s = launch_adjoint_sep(sub, grad, st, a.gate);
   } else {
     const int64_t total = (int64_t)p->n_species * sub->n_s;
     k_node_table<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(
@@ -618,14 +690,23 @@ scatter_status launch_coarse_adjoint(scatter_plan_t p, const float2* gf, float* 
         make_float3((float)p->inst[0].H[0], (float)p->inst[0].H[1], (float)p->inst[0].H[2]), total, sub->adj_line,
         sub->d.adj_table, a.gate);
     p->last_launches += 1;
-    s = launch_adjoint_tiles(sub, grad, st);
+    s = launch_adjoint_tiles(sub, grad, st, a.gate);
   }
   p->last_launches += sub->last_launches;
   return s;
 }
 
-void release_coarse(scatter_plan_s* p) {
-  CoarseState& c = p->coarse;
+}  // namespace
+
+scatter_status launch_coarse_adjoint(scatter_plan_t p, const float2* gf, float* grad, cudaStream_t st) {
+  scatter_status s = SCATTER_OK;
+  for (int l = 0; l < p->coarse_adj_levels && s == SCATTER_OK; ++l) s = level_adjoint(p, l, gf, grad, st);
+  return s;
+}
+
+namespace {
+
+void release_level(scatter_plan_s* p, CoarseState& c) {
   if (c.sub) {
     if (c.sub->d.status == p->d.status) c.sub->d.status = nullptr;
     if (c.sub->d.inst_shift == p->d.inst_shift) c.sub->d.inst_shift = nullptr;
@@ -634,9 +715,20 @@ void release_coarse(scatter_plan_s* p) {
   for (CoarseStage& s : c.stage)
     for (float* w : {s.W, s.Wt})
       if (w) cudaFree(w);
-  for (void* b : {(void*)c.adj_tmp[0], (void*)c.adj_tmp[1], (void*)c.adj_gf, (void*)c.map, (void*)c.tmp[0], (void*)c.tmp[1], (void*)c.rmax2, (void*)c.lim2, (void*)c.no_shift})
+  for (void* b : {(void*)c.adj_tmp[0], (void*)c.adj_tmp[1], (void*)c.adj_gf, (void*)c.map, (void*)c.tmp[0], (void*)c.tmp[1], (void*)c.lim2})
     if (b) cudaFree(b);
   c = CoarseState{};
+}
+
+}  // namespace
+
+void release_coarse(scatter_plan_s* p) {
+  for (CoarseState& c : p->coarse) release_level(p, c);
+  for (void* b : {(void*)p->coarse_rmax2, (void*)p->coarse_no_shift})
+    if (b) cudaFree(b);
+  p->coarse_rmax2 = nullptr;
+  p->coarse_no_shift = nullptr;
+  p->coarse_levels = p->coarse_adj_levels = 0;
 }
 
 }  // namespace scatter

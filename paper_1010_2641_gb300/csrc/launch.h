@@ -7,15 +7,19 @@ namespace scatter {
 
 // A call's choice on the device: kernels that stand by for crystals past a plan's
 // assumed radius return at once while this call's extent squared (rmax2, float
-// bits, per instance) is within lim2.
+// bits, per instance) is within lim2; those of a node set also where it is not
+// within the set's own (only2, one instance).
 struct CallGate {
   const unsigned* rmax2;  // null: no gate
-  const float* lim2;
+  const float* lim2;      // null: nothing smaller serves
   int n;                  // instances
+  const float* only2;     // null: no bound of its own
 };
 #ifdef __CUDACC__
 __device__ __forceinline__ bool within(const CallGate& g, int inst) {
-  return g.rmax2 && __uint_as_float(g.rmax2[inst]) <= g.lim2[inst];
+  if (!g.rmax2) return false;
+  const float r2 = __uint_as_float(g.rmax2[inst]);
+  return (g.lim2 && r2 <= g.lim2[inst]) || (g.only2 && !(r2 <= g.only2[inst]));
 }
 #endif
 
@@ -84,7 +88,7 @@ scatter_status prepare_cluster_adjoint(scatter_plan_s* p);
 scatter_status launch_cluster_adjoint(scatter_plan_t p, const float2* gf, float* partial, cudaStream_t st);
 void release_cluster_adjoint(ClAdjState& s);
 inline CallGate cluster_gate(const scatter_plan_s* p) {
-  return p->cl.active ? CallGate{p->cl.rmax2, p->cl.lim2, p->batch} : CallGate{nullptr, nullptr, 0};
+  return p->cl.active ? CallGate{p->cl.rmax2, p->cl.lim2, p->batch, nullptr} : CallGate{};
 }
 
 // Maps sampled far finer than the crystal's extent asks for (coarse.cu): the sum
@@ -99,11 +103,18 @@ scatter_status launch_coarse_adjoint(scatter_plan_t p, const float2* gf, float* 
 // Tensor-core intensities keep the direct sum: |A|^2 doubles the difference
 // between the two (up to 2.5e-5 of the map, amplitudes 1.6e-5).
 inline bool coarse_serves(const scatter_plan_s* p, const void* amp_out) {
-  return p->coarse.sub && (amp_out || p->path != SCATTER_PATH_SEPARABLE);
+  return p->coarse_levels > 0 && (amp_out || p->path != SCATTER_PATH_SEPARABLE);
 }
-inline CallGate coarse_gate(const scatter_plan_s* p) {
-  return p->coarse.sub ? CallGate{p->coarse.rmax2, p->coarse.lim2, 1} : CallGate{nullptr, nullptr, 0};
+// Of the first `levels` node sets: crystals that one of them resolves.
+inline CallGate coarse_gate(const scatter_plan_s* p, int levels) {
+  return levels > 0 ? CallGate{p->coarse_rmax2, p->coarse[levels - 1].lim2, 1, nullptr} : CallGate{};
 }
+// Set l itself: crystals that it resolves and no smaller one does.
+inline CallGate level_gate(const scatter_plan_s* p, int l) {
+  return CallGate{p->coarse_rmax2, l > 0 ? p->coarse[l - 1].lim2 : nullptr, 1, p->coarse[l].lim2};
+}
+// Positions prepared for the first `levels` node sets, each where no smaller one serves.
+scatter_status launch_coarse_prep(scatter_plan_t p, int levels, const double* xyz, const float* occ, cudaStream_t st);
 // scatter_plan without a coarse grid of its own, around H, its tensor-core
 // accumulation groups at least `group` steps (0: its own choice).
 scatter_status plan_nodes(const scatter_problem* pr, const scatter_options* op, const double (&H)[3], double group,
@@ -140,6 +151,9 @@ scatter_status launch_backward(scatter_plan_t p, const double* xyz, const float*
 // Tensor-core adjoint on grids of SEPARABLE plans (adjoint_sep.cu).
 bool adjoint_sep_applicable(const scatter_plan_s* p);
 scatter_status prepare_adjoint_sep(scatter_plan_s* p);
+// Mean steps of the accumulation group that a step lies in, of the direct or
+// (where the plan folds) the folded form.
+double adjoint_sep_group(const scatter_plan_s* p, bool fold);
 scatter_status launch_adjoint_sep(scatter_plan_t p, float* grad, cudaStream_t st,
                                   const CallGate& gate = CallGate{});
 // FP32 adjoint from the plan's weight table (adjoint.cu).

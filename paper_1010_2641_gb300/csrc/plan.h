@@ -173,16 +173,14 @@ struct CoarseStage {
   float* Wt = nullptr;              // the adjoint's: [n_out][n_in], then its rounding errors
   std::vector<float> h_W;           // W on the host
 };
+constexpr int kCoarseLevels = 2;
 struct CoarseState {
   scatter_plan_s* sub = nullptr;    // the sum at the nodes, without the translation phase
   CoarseStage stage[3];
   int n_stages = 0;
   float2* map = nullptr;            // at the nodes
   float2* tmp[2] = {nullptr, nullptr};
-  unsigned* rmax2 = nullptr;        // this call's largest |x'_d|^2 (float bits)
-  float* lim2 = nullptr;
-  double* no_shift = nullptr;       // [3] zeros
-  bool adjoint = false;             // the adjoint at the nodes too
+  float* lim2 = nullptr;            // X^2
   float2* adj_tmp[2] = {nullptr, nullptr};
   float2* adj_gf = nullptr;         // weights at the nodes (FP32 sums)
 };
@@ -326,7 +324,11 @@ struct scatter_plan_s {
   scatter::DeviceBuffers d;
   scatter::GridSum gs;
   scatter::ClState cl;
-  scatter::CoarseState coarse;
+  scatter::CoarseState coarse[scatter::kCoarseLevels];  // by growing radius
+  int coarse_levels = 0;
+  int coarse_adj_levels = 0;                     // the first ones, with an adjoint
+  unsigned* coarse_rmax2 = nullptr;              // this call's largest |x'_d|^2 (float bits)
+  double* coarse_no_shift = nullptr;             // [3] zeros
   unsigned* extent2 = nullptr;                   // the sum at the nodes of another plan: prep writes the largest |x'_d|^2
   const double* out_shift = nullptr;             //   its reductions' shift in place of the call's
   double sep_group = 0.0;                        //   accumulation groups of at least this many steps
@@ -365,6 +367,7 @@ struct scatter_plan_s {
   float adj_ds = 0.f;               // its l step
   int64_t adj_lines_per_chunk = 0;
   bool adj_sep = false;             // SEPARABLE grid plan: the adjoint runs on k_sep
+  bool adj_no_fold = false;         // asked for: the direct form
   bool adj_sep_fold = false;        // its points folded over the middle of the (k, l) plane
   int64_t adj_sep_k = 0;            // points (mirror pairs) of a plane
   double adj_sep_mid[2] = {0, 0};   // the middles of the k and l axes - H

@@ -45,7 +45,7 @@ def _grown(plan, call):
     ("generic", 9.0, (80, 63, 48), (0.001, 0.001, 0.001), (0, 0, 0), 1),
     ("generic", 9.0, (65, 130, 9), (0.001, 0.001, 0.02), (17.3, -8.0, 40.4), 3),   # line form
     ("generic", 9.0, (1, 290, 280), (0.0, 0.0005, 0.0005), (0.4, 0.3, -0.4), 2),
-    ("separable", 12.0, (129, 130, 65), (0.001, 0.001, 0.001), (3.3, 0.2, 9.9), 2),
+    ("separable", 16.0, (400, 45, 46), (0.0005, 0.002, 0.002), (3.3, 0.2, 9.9), 2),
 ])
 def test_gradient(path, cells, shape, steps, offset, n_sp):
     c = W.fcc_sphere(radius_cells=cells, seed=401)
@@ -75,9 +75,9 @@ def test_gradient(path, cells, shape, steps, offset, n_sp):
     assert _rel(plan.vjp(x, G, w).cpu().numpy(), bare.vjp(x, G, w).cpu().numpy()) < TOL[path]
 
 
-@pytest.mark.parametrize("path, shape", [("generic", (80, 60, 50)), ("separable", (129, 130, 65))])
+@pytest.mark.parametrize("path, shape", [("generic", (80, 60, 50)), ("separable", (400, 45, 46))])
 def test_larger_crystal_is_left_to_the_direct_kernels(path, shape):
-    c = W.fcc_sphere(radius_cells=12.0 if path == "separable" else 9.0, seed=403)
+    c = W.fcc_sphere(radius_cells=16.0 if path == "separable" else 9.0, seed=403)
     axes = _axes(shape, (0.001,) * 3)
     kw = dict(axes=axes, atom_species=c.species, path=path)
     plan, bare = api.Plan(c.coef, A_LAT, len(c.xyz), **kw), api.Plan(c.coef, A_LAT, len(c.xyz), radius_hint=FAR, **kw)
