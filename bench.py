@@ -4,20 +4,26 @@ Workload (one step = one pass of the hot path over the synthetic input):
 strained spherical fcc nanocrystal of 134,009 atoms (radius 20 cells,
 Si-like core / Ge-like shell, radial strain + thermal noise) scattering onto
 a 256 x 256 x 64 grid of S points (step 0.002 r.l.u.) around (004):
-per-call prep (centring, split phase), the map kernel and the epilogue,
+per-call prep (centring, split phase), the map's sum and the epilogue,
 5.6e11 atom-reflection pairs per step.  The headline uses the separable
-tensor-core path (--path separable, the default) or the generic FP32/MUFU
-path (--path generic); both meet the 1e-4 relative-L2 tolerance on this map,
-which the CPU-baseline leg re-checks against the FP64 oracle on a sample.
+tensor-core path (--path separable, the default) or the generic FP32 path
+(--path generic); both meet the 1e-4 relative-L2 tolerance on this map, which
+the CPU-baseline leg re-checks against the FP64 oracle on a sample.  The map
+is sampled 12 times finer per axis than the crystal's extent asks for, so both
+paths sum at the Chebyshev nodes that resolve it and interpolate to the points
+(csrc/coarse.cu); `value` counts the map's pairs, `direct` is the same map
+without nodes.
 
 Metric: atom-reflection pairs per second (whole job, all ranks), the paper's
 "reflections x atoms / s" (Section 2.2).  Each rank runs its own full
 instance (weak scaling, no collective on the data path).
 
 JSON line keys beyond the base contract:
-  roofline      dominant kernel: k_sep against the measured dense tensor
-                peak, or k_generic against the MUFU bound
-                (16 sin/cos ops / SM / clk -> 8 pairs / SM / clk x SMs x clock)
+  roofline      the step against the memory it cannot do without (24 B per
+                atom read, 8 B per point written) at the measured copy rate
+  direct        the same map from a plan without nodes: its main kernel
+                against the measured dense tensor peak (executed flops), or the
+                FP32 multiply-add rate
   cpu_baseline  the FP64 oracle timed on the host cores on a bounded sample
   accuracy      relative L2 error of the GPU map vs the oracle on that sample
   e2e           the same metric through the C-ABI call with host buffers,
@@ -31,11 +37,9 @@ JSON line keys beyond the base contract:
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import os
 import pathlib
-import re
 import subprocess
 import tempfile
 import sys
@@ -50,6 +54,8 @@ METRIC = "atom·reflections/s at ≤1e-4 rel err vs FP64 oracle; fraction of FP3
 UNIT = "atom·reflections/s"
 MUFU_SINCOS_PER_SM_CLK = 16.0   # measured (scatter_microbench kind 0): 15.97
 MUFU_OPS_PER_PAIR = 2.0         # one sin + one cos per (atom, reflection)
+FMA_PAIRS_PER_SM_CLK = 64.0     # factorised grid sum on a symmetric axis: 2 of 128 multiply-adds per pair
+NO_NODES = 1e5                  # radius hint (cells) that no map here is oversampled for
 
 
 GRID = (256, 256, 64)
@@ -148,7 +154,7 @@ class ClockSampler:
 
 
 # ---------------------------------------------------------------------------
-# profile summary -> traffic of the dominant kernel (null if stale)
+# measured peaks
 # ---------------------------------------------------------------------------
 
 def measured_peak(key: str, fallback: float):
@@ -158,32 +164,6 @@ def measured_peak(key: str, fallback: float):
         return v, f"MEASURED_PEAKS.json {key} = {v} (of measured)"
     except Exception:
         return fallback, f"fallback {fallback} (of fallback)"
-
-
-GENERIC_SOURCES = ("forward.cu", "generic_impl.cuh", "device_common.cuh", "plan.h")
-
-
-def kernel_source_hash(files=GENERIC_SOURCES) -> str:
-    h = hashlib.sha1()
-    for f in files:
-        h.update((ROOT / "paper_1010_2641_gb300" / "csrc" / f).read_bytes())
-    return h.hexdigest()[:12]
-
-
-SEP_SOURCES = ("separable.cu", "sep_pair.cu", "sep_common.cuh", "device_common.cuh", "plan.h")
-
-
-def profiled_traffic(name="generic_strained_sphere.md", files=GENERIC_SOURCES):
-    """dram bytes per launch of a kernel from its committed ncu summary, if
-    the summary was taken on the current kernel source."""
-    p = ROOT / "profiles" / name
-    if not p.exists():
-        return None
-    text = p.read_text()
-    m = re.search(r"traffic_bytes_per_launch:\s*([0-9.eE+]+)\s*\(source sha1 ([0-9a-f]+)\)", text)
-    if not m or m.group(2) != kernel_source_hash(files):
-        return None
-    return float(m.group(1))
 
 
 # ---------------------------------------------------------------------------
@@ -313,36 +293,34 @@ def run_gpu(args, rank, world, local_rank):
     if world > 1:
         (t_e2e,) = sharding.max_over_ranks([t_e2e], device=dev)
 
-    # ---- roofline of the dominant kernel ----------------------------------------
+    # ---- rooflines: the step, and the direct sum's kernel -----------------------
     sm_mhz = clk["sm_mhz"] if clk else None
     n_sm = info["n_sm"]
-    roof = None
+    must = 24.0 * n_atoms + 8.0 * n_s
+    peak, basis = measured_peak("hbm_gbs", 6800.0)
+    achieved = must / (t_step * 1e-3) / 1e9
+    roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "traffic": None,
+            "kernel": ("k_sep at the nodes (tcgen05.mma kind::f16, 3 split products), k_interp" if args.path == "separable"
+                       else "k_gridsum at the nodes, k_interp"),
+            "kernel_ms": t_kern, "peak_basis": f"{basis}; bytes that the step cannot do without"}
+    dplan = api.Plan(c.coef, 5.43, n_atoms, axes=axes, atom_species=c.species, path=args.path, timing=True,
+                     radius_hint=NO_NODES)
+    A_direct = torch.empty_like(A)
+    d_ms = _time_calls(lambda: dplan.amplitude(xyz, out=A_direct), dplan, reps=3)
+    direct = {"value": pairs / (d_ms * 1e-3), "unit": UNIT, "kernel_ms": d_ms,
+              "rel_l2_to_nodes": float(((A_direct - A).abs().double().square().sum() /
+                                        A_direct.abs().double().square().sum()).sqrt())}
     if args.path == "separable":
-        # executed tensor-pipe work: 3 split products x 2 flop x M' x N' x K'
-        m_pad = -(-2 * GRID[0] // 128) * 128
-        n_pad = -(-(GRID[1] * GRID[2]) // 256) * 256
-        executed = 6.0 * m_pad * n_pad * 2 * info["n_atoms_padded"]
-        useful = 8.0 * n_atoms * n_s
-        peak, basis = measured_peak("bf16_tflops", 1900.0)
-        achieved = executed / (t_kern * 1e-3) / 1e12
-        roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": None if args.grid else profiled_traffic("separable_strained_sphere.md", SEP_SOURCES),
-                "kernel": ("k_sep_pair (tcgen05.mma.cta_group::2 kind::f16, M=256 N=256 on a CTA pair, "
-                           "3 split products)" if os.environ.get("SCATTER_SEP_PAIR", "1") != "0" else
-                           "k_sep (tcgen05.mma kind::f16, M=128 N=256, 3 split products)"),
-                "kernel_ms": t_kern, "useful_tflops": useful / (t_kern * 1e-3) / 1e12,
-                "peak_basis": f"{basis} (f16 and bf16 share the dense tensor rate)"}
+        direct["roofline"] = _tensor_roof(GRID[0], GRID[1] * GRID[2], info["n_atoms_padded"], d_ms, clk, fold=True)
+        direct["kernel"] = ("k_sep_pair (tcgen05.mma.cta_group::2 kind::f16, M=256 N=256 on a CTA pair, 3 split "
+                            "products; the grid folded over its middle)")
         # cross-check: this GPU's own f16 MMA rate (back-to-back tcgen05.mma, M=128 N=256, zero operands)
-        mb = api.microbench(8, iters=20000)
-        roof["f16_mma_microbench_tflops"] = mb["ops_per_s"] / 1e12
-        roof["frac_of_f16_mma_microbench"] = achieved / (mb["ops_per_s"] / 1e12)
-    elif sm_mhz:
-        peak = n_sm * MUFU_SINCOS_PER_SM_CLK / MUFU_OPS_PER_PAIR * sm_mhz * 1e6 / 1e9  # Gpair/s
-        achieved = pairs / (t_kern * 1e-3) / 1e9
-        roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Gpair/s",
-                "frac": achieved / peak, "traffic": profiled_traffic(),
-                "kernel": "k_generic (MUFU sin/cos, 16 ops/SM/clk)",
-                "kernel_ms": t_kern, "peak_basis": f"{n_sm} SMs x 8 pairs/SM/clk x {sm_mhz:.0f} MHz (median sampled)"}
+        direct["f16_mma_microbench_tflops"] = api.microbench(8, iters=20000)["ops_per_s"] / 1e12
+    else:
+        direct["roofline"] = _rate_roof(pairs, d_ms, FMA_PAIRS_PER_SM_CLK, n_sm, clk, "Gpair/s", "alu",
+                                        "pairs (2 FMA each: a column and its mirror)")
+        direct["kernel"] = "k_gridsum (FP32 multiply-adds)"
+    del dplan, A_direct
 
     out = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
            "warmup": args.warmup, "ms_per_step": t_step, "higher_is_better": True, "scaling": "weak",
@@ -352,7 +330,7 @@ def run_gpu(args, rank, world, local_rank):
                       "path": args.path, "threads": info["threads"], "points_per_thread": info["points_per_thread"],
                       "split_k": info["split_k"], "l2": "flushed between steps (256 MB write, outside the events)",
                       "parallelism": f"weak x{world} (independent instance per GPU)"},
-           "roofline": roof, "clocks": clk, "gpu_launches": launches,
+           "roofline": roof, "direct": direct, "clocks": clk, "gpu_launches": launches,
            "e2e": {"value": world * pairs / (t_e2e * 1e-3), "unit": UNIT,
                    "h2d_bytes_per_step": int(xyz_host.numel() * 8), "d2h_bytes_per_step": int(A_host.numel() * 8)}}
 
@@ -417,11 +395,18 @@ def _rate_roof(units, ms, per_sm_clk, n_sm, clk, unit, bound, basis):
             "clocks": clk}
 
 
-def _tensor_roof(n0, n12, n_atoms_padded, ms, clk=None):
-    """Executed-flop roofline of k_sep on an n0 x n12 separable grid."""
-    m_pad = -(-2 * n0 // 128) * 128
-    n_pad = -(-n12 // 256) * 256
-    executed = 6.0 * m_pad * n_pad * 2 * n_atoms_padded
+def _tensor_roof(n0, n12, n_atoms_padded, ms, clk=None, fold=False):
+    """Executed-flop roofline of k_sep on an n0 x n12 separable grid.  Folded over
+    its middle: 32 values of the first axis' half per 128 rows, 128 mirror pairs
+    per 256 columns, one K value per atom instead of two."""
+    if fold:
+        m_pad = -(-((n0 + 1) // 2) // 32) * 128
+        n_pad = -(-((n12 + 1) // 2) // 128) * 256
+        executed = 6.0 * m_pad * n_pad * n_atoms_padded
+    else:
+        m_pad = -(-2 * n0 // 128) * 128
+        n_pad = -(-n12 // 256) * 256
+        executed = 6.0 * m_pad * n_pad * 2 * n_atoms_padded
     peak, basis = measured_peak("bf16_tflops", 1900.0)
     achieved = executed / (ms * 1e-3) / 1e12
     return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
@@ -430,10 +415,11 @@ def _tensor_roof(n0, n12, n_atoms_padded, ms, clk=None):
 
 def _tensor_roof_adjoint(n0, n12, n_atoms_padded, ms, clk=None):
     """Executed-flop roofline of k_sep running the adjoint: rows (a, weight,
-    Re/Im) = 6 n0, columns = atom slots in 256-slot tiles, K = 2 per point."""
+    Re/Im) = 6 n0, columns = atom slots in 256-slot tiles, K = 2 per mirror pair
+    of points."""
     m_pad = -(-6 * n0 // 128) * 128
     n_pad = -(-n_atoms_padded // 256) * 256
-    k_pad = -(-n12 // 16) * 16 * 2
+    k_pad = -(-((n12 + 1) // 2) // 16) * 16 * 2
     executed = 6.0 * m_pad * n_pad * k_pad
     peak, basis = measured_peak("bf16_tflops", 1900.0)
     achieved = executed / (ms * 1e-3) / 1e12
@@ -487,18 +473,22 @@ def measure_paths(args, dev, clk, only=None):
         return only is None or only == name or (name == "dwba_island" and only == "dwba_island_separable")
 
     if want(f"{other}_sphere"):
-        # generic FP32/MUFU kernel on the full strained-sphere map, with its roofline
+        # the other path on the full strained-sphere map, and its direct sum with its roofline
         other = "generic" if args.path == "separable" else "separable"
         plan = api.Plan(c.coef, W.LATTICE_A, n_atoms, axes=axes, atom_species=c.species, path=other, timing=True)
         ms = timed(lambda: plan.amplitude(xyz), plan)
         row = {"value": n_atoms * n_s / (ms * 1e-3), "unit": UNIT, "kernel_ms": ms, "workload": "strained sphere, full map"}
         n_sm = plan.info()["n_sm"]
+        plan = api.Plan(c.coef, W.LATTICE_A, n_atoms, axes=axes, atom_species=c.species, path=other, timing=True,
+                        radius_hint=NO_NODES)
+        d_ms = timed(lambda: plan.amplitude(xyz), plan)
+        row["direct_kernel_ms"] = d_ms
         if other == "generic":
-            row["roofline"] = _rate_roof(n_atoms * n_s, ms, MUFU_SINCOS_PER_SM_CLK / MUFU_OPS_PER_PAIR, n_sm, rc.get("clk"),
-                                         "Gpair/s", "alu", "pairs (2 MUFU sin/cos each)")
+            row["direct_roofline"] = _rate_roof(n_atoms * n_s, d_ms, FMA_PAIRS_PER_SM_CLK, n_sm, rc.get("clk"), "Gpair/s",
+                                                "alu", "pairs (2 FMA each: a column and its mirror)")
         else:
-            row["roofline"] = _tensor_roof(GRID[0], GRID[1] * GRID[2], plan.info()["n_atoms_padded"], ms,
-                                            rc.get("clk"))
+            row["direct_roofline"] = _tensor_roof(GRID[0], GRID[1] * GRID[2], plan.info()["n_atoms_padded"], d_ms,
+                                                  rc.get("clk"), fold=True)
         res[f"{other}_sphere"] = row
         del plan
     if want("auto_sphere"):
@@ -586,11 +576,14 @@ def measure_paths(args, dev, clk, only=None):
         ms_f = timed(lambda: plan.amplitude(x, out=A), plan)
         ms = timed(lambda: plan.backward(x, A, I_obs), plan)
         res["adjoint_cube"] = {"value": len(cube.xyz) * 128 ** 3 / (ms * 1e-3), "unit": UNIT, "kernel_ms": ms,
-                               "forward_kernel_ms": ms_f, "workload": "strained cube 102400 atoms x 128^3, dL/dr",
-                               # uniform l axis: the line kernel carries the phase along l by a complex multiply,
-                               # 8 FMA-pipe ops per pair at 128 lane-ops per SM per clock, no MUFU
-                               "roofline": _rate_roof(len(cube.xyz) * 128 ** 3, ms, 16.0, n_sm, rc.get("clk"), "Gpair/s", "alu",
-                                                      "pairs (8 FMA-pipe ops each)")}
+                               "forward_kernel_ms": ms_f, "workload": "strained cube 102400 atoms x 128^3, dL/dr"}
+        plan = api.Plan(cube.coef, W.LATTICE_A, len(cube.xyz), axes=ax, timing=True, path="generic", radius_hint=NO_NODES)
+        ms = timed(lambda: plan.backward(x, A, I_obs), plan)
+        res["adjoint_cube"]["direct_kernel_ms"] = ms
+        # without nodes, uniform l axis: the line kernel carries the phase along l by a complex multiply,
+        # 8 FMA-pipe ops per pair at 128 lane-ops per SM per clock, no MUFU
+        res["adjoint_cube"]["direct_roofline"] = _rate_roof(len(cube.xyz) * 128 ** 3, ms, 16.0, n_sm, rc.get("clk"),
+                                                            "Gpair/s", "alu", "pairs (8 FMA-pipe ops each)")
         del plan, x, A, I_obs
     if want('adjoint_list'):
         # the S-list adjoint (k_adjoint: MUFU sin/cos per pair): strained sphere x an Ewald-slice list
@@ -603,9 +596,14 @@ def measure_paths(args, dev, clk, only=None):
         ms = timed(lambda: plan.backward(x, A, I_obs), plan)
         pairs_l = len(c_l.xyz) * len(S_l)
         res["adjoint_list"] = {"value": pairs_l / (ms * 1e-3), "unit": UNIT, "kernel_ms": ms,
-                               "workload": "strained sphere 134009 atoms x 262144 Ewald-slice points near (111), dL/dr",
-                               "roofline": _rate_roof(pairs_l, ms, MUFU_SINCOS_PER_SM_CLK / MUFU_OPS_PER_PAIR, n_sm,
-                                                      rc.get("clk"), "Gpair/s", "alu", "pairs (2 MUFU sin/cos each)")}
+                               "workload": "strained sphere 134009 atoms x 262144 Ewald-slice points near (111), dL/dr "
+                                           "(clusters of points)"}
+        # a tile override keeps the direct kernel
+        plan = api.Plan(c_l.coef, W.LATTICE_A, len(c_l.xyz), s_list=S_l, atom_species=c_l.species, timing=True, split_k=1)
+        ms = timed(lambda: plan.backward(x, A, I_obs), plan)
+        res["adjoint_list"]["direct_kernel_ms"] = ms
+        res["adjoint_list"]["direct_roofline"] = _rate_roof(pairs_l, ms, MUFU_SINCOS_PER_SM_CLK / MUFU_OPS_PER_PAIR, n_sm,
+                                                            rc.get("clk"), "Gpair/s", "alu", "pairs (2 MUFU sin/cos each)")
         del plan, x, A, I_obs
     if want('adjoint_cube_separable'):
         # the same gradient on a SEPARABLE plan: the per-atom sums contract on the tensor cores
@@ -623,9 +621,12 @@ def measure_paths(args, dev, clk, only=None):
         res["adjoint_cube_separable"] = {
             "value": len(cube.xyz) * 128 ** 3 / (ms * 1e-3), "unit": UNIT, "kernel_ms": ms, "call_ms": ms_call,
             "call_value": len(cube.xyz) * 128 ** 3 / (ms_call * 1e-3), "forward_kernel_ms": ms_f,
-            "workload": "strained cube 102400 atoms x 128^3, dL/dr on a SEPARABLE plan (k_sep, operands swapped)",
-            "roofline": _tensor_roof_adjoint(128, 128 * 128, plan.info()["n_atoms_padded"], ms,
-                                                 rc.get("clk"))}
+            "workload": "strained cube 102400 atoms x 128^3, dL/dr on a SEPARABLE plan (k_sep, operands swapped)"}
+        plan = api.Plan(cube.coef, W.LATTICE_A, len(cube.xyz), axes=ax, path="separable", timing=True, radius_hint=NO_NODES)
+        ms = timed(lambda: plan.backward(x, A, I_obs), plan)
+        res["adjoint_cube_separable"]["direct_kernel_ms"] = ms
+        res["adjoint_cube_separable"]["direct_roofline"] = _tensor_roof_adjoint(
+            128, 128 * 128, plan.info()["n_atoms_padded"], ms, rc.get("clk"))
         del plan, x, A, I_obs
     if only == 'dwba_island_mid':
         # profiling case of the FFMA DWBA kernel: 127,560-atom island (base 60, height 20 cells) x 128x128x32
@@ -711,9 +712,15 @@ def measure_paths(args, dev, clk, only=None):
         res["batch_ewald"] = {"value": pairs_b / (ms * 1e-3), "unit": UNIT, "graph_ms": ms, "instances": len(ao) - 1,
                               "tiling": {"threads": inf["threads"], "points_per_thread": inf["points_per_thread"],
                                          "autotuned": True},
-                              "workload": f"{len(ao) - 1} fcc crystals 1e3-2e5 atoms, 1e4-1e6 Ewald-slice points each",
-                              "roofline": _rate_roof(pairs_b, ms, MUFU_SINCOS_PER_SM_CLK / MUFU_OPS_PER_PAIR, n_sm, rc.get("clk"),
-                                                     "Gpair/s", "alu", "pairs (2 MUFU sin/cos each)")}
+                              "workload": f"{len(ao) - 1} fcc crystals 1e3-2e5 atoms, 1e4-1e6 Ewald-slice points each "
+                                          "(clusters of points)"}
+        # a tile override keeps the direct kernel
+        plan = api.Plan(bcoef, W.LATTICE_A, len(bx), s_list=bS, atom_species=bs, atom_off=ao, s_off=so, timing=True,
+                        threads=inf["threads"], points_per_thread=inf["points_per_thread"])
+        ms = timed(lambda: plan.amplitude(x, out=out), plan)
+        res["batch_ewald"]["direct_graph_ms"] = ms
+        res["batch_ewald"]["direct_roofline"] = _rate_roof(pairs_b, ms, MUFU_SINCOS_PER_SM_CLK / MUFU_OPS_PER_PAIR, n_sm,
+                                                           rc.get("clk"), "Gpair/s", "alu", "pairs (2 MUFU sin/cos each)")
     return res
 
 
