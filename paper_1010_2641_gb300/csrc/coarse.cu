@@ -57,6 +57,7 @@ struct InterpArgs {
   const double* axis64;       // exact64: FP64 phases, from these and H64
   double H64[3];
   int exact64;
+  int planar;                 // the last axis is not interpolated: its t is in the nodes' sum
   int64_t n0, n1, n2;
   const double* shift;
   float2* out_amp;
@@ -181,7 +182,7 @@ __global__ void __launch_bounds__(256) k_interp(const InterpArgs a) {
   }
   const bool shifted = a.last && (a.shift[0] != 0.0 || a.shift[1] != 0.0 || a.shift[2] != 0.0);
   const float ts[3] = {shifted ? (float)a.shift[0] : 0.f, shifted ? (float)a.shift[1] : 0.f,
-                       shifted ? (float)a.shift[2] : 0.f};
+                       shifted && !a.planar ? (float)a.shift[2] : 0.f};
 #pragma unroll
   for (int c = 0; c < T; ++c) {  // this thread's columns
     const int64_t b = b0 + (ROWS ? ty : tx) + 16 * c;
@@ -298,6 +299,7 @@ double form_error(const scatter_plan_s* p, int d, const Nodes& nd, double X) {
   const int64_t step = std::max<int64_t>(1, (int64_t)ax.size() / 48);
   auto pick = [&](int axis, int which) {
     const std::vector<double>& v = p->axis_host[axis];
+    if (p->s_kind == SCATTER_S_GID_GRID && axis == 2) return 0.0;  // small S_z
     return which == 0 ? v.front() : which == 1 ? v[v.size() / 2] : v.back();
   };
   std::vector<double> w(n);
@@ -384,7 +386,11 @@ struct NodeSet {
 double sum_seconds(const scatter_plan_s* p, double n0, double n12) {
   const double N = (double)p->n_slots;
   if (p->path != SCATTER_PATH_SEPARABLE) return N * n0 * n12 / 1.0e13;
-  const double tiles = std::ceil(n0 / 128.0) * std::ceil(n12 / 256.0), steps = N / 32.0;
+  double tiles = std::ceil(n0 / 128.0) * std::ceil(n12 / 256.0), steps = N / 32.0;
+  if (p->s_kind == SCATTER_S_GID_GRID) {  // four beams, the direct form: 16 atoms, 128 values x 256 columns
+    tiles = std::ceil(n0 / 128.0) * std::ceil(4.0 * n12 / 256.0);
+    steps = N / 16.0;
+  }
   double best = 1e300;
   for (double k = 1.0; k <= std::max(1.0, steps / 200.0); k += 1.0)
     best = std::min(best, std::ceil(tiles * k / p->n_sm) * (steps / k + 40.0) * (n12 <= 128.0 ? 0.75e-6 : 1e-6));
@@ -398,8 +404,14 @@ NodeSet choose_nodes(const scatter_plan_s* p, double X) {
   const double eps = sep ? kCoarseEpsSep : kCoarseEps;
   bool any = false;
   double M = 1.0;
+  const bool gid = p->s_kind == SCATTER_S_GID_GRID;
   for (int d = 0; d < 3; ++d) {
     const std::vector<double>& ax = p->axis_host[d];
+    if (gid && d == 2) {  // exit angles: four beams each, not a wave per atom
+      r.axis[d] = ax;
+      M *= (double)ax.size();
+      continue;
+    }
     const double lo = *std::min_element(ax.begin(), ax.end()), hi = *std::max_element(ax.begin(), ax.end());
     const int most = (int)std::min<int64_t>(4096, (int64_t)(0.9 * (double)ax.size()));
     int n = 0;
@@ -428,9 +440,10 @@ void release_level(scatter_plan_s* p, CoarseState& c);
 }  // namespace
 
 scatter_status prepare_coarse(scatter_plan_s* p, const scatter_problem* pr, const scatter_options* op) {
-  if (p->s_kind != SCATTER_S_GRID || p->batch != 1 || pr->factor_table || p->n_atoms <= 0 || p->n_s <= 0)
+  const bool sep = p->path == SCATTER_PATH_SEPARABLE, gid = p->s_kind == SCATTER_S_GID_GRID;
+  if (!(p->s_kind == SCATTER_S_GRID || (gid && sep && p->gid_mode == 0)) || p->batch != 1 || pr->factor_table ||
+      p->n_atoms <= 0 || p->n_s <= 0)
     return SCATTER_OK;
-  const bool sep = p->path == SCATTER_PATH_SEPARABLE;
   if (!sep && !(p->path == SCATTER_PATH_GENERIC && p->gs.active)) return SCATTER_OK;
   if (op && (op->threads || op->points_per_thread || op->split_k || op->atoms_per_thread > 0)) return SCATTER_OK;
   for (int d = 0; d < 3; ++d)
@@ -444,8 +457,9 @@ scatter_status prepare_coarse(scatter_plan_s* p, const scatter_problem* pr, cons
   if (op && op->radius_hint > 0.0) {
     sets.push_back(choose_nodes(p, op->radius_hint));
   } else {
-    sets.push_back(choose_nodes(p, 1.1 * compact + 1.0));
-    sets.push_back(choose_nodes(p, 1.3 * compact + 1.0));
+    // (flat islands reach further sideways: 1.6 and 2.3)
+    sets.push_back(choose_nodes(p, (gid ? 1.6 : 1.1) * compact + 1.0));
+    sets.push_back(choose_nodes(p, (gid ? 2.3 : 1.3) * compact + 1.0));
     if (sets[1].seconds <= 0.75 * fine && sets[0].seconds + 40e-6 > sets[1].seconds) sets.erase(sets.begin());
   }
   for (const NodeSet& set : sets)
@@ -522,9 +536,9 @@ bool build_level(scatter_plan_s* p, const scatter_problem* pr, const scatter_opt
   }
   const float lim2 = (float)(set.X * set.X);
   ok = ok && alloc(&c.map, (size_t)c.sub->n_s * sizeof(float2)) && alloc(&c.lim2, sizeof(float)) &&
-       (p->coarse_rmax2 || (alloc(&p->coarse_rmax2, sizeof(unsigned)) && alloc(&p->coarse_no_shift, 3 * sizeof(double)) &&
+       (p->coarse_rmax2 || (alloc(&p->coarse_rmax2, sizeof(unsigned)) && alloc(&p->coarse_shift, 3 * sizeof(double)) &&
                             cudaMemset(p->coarse_rmax2, 0, sizeof(unsigned)) == cudaSuccess &&
-                            cudaMemset(p->coarse_no_shift, 0, 3 * sizeof(double)) == cudaSuccess)) &&
+                            cudaMemset(p->coarse_shift, 0, 3 * sizeof(double)) == cudaSuccess)) &&
        cudaMemcpy(c.lim2, &lim2, sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
   for (int i = 0; i < c.n_stages - 1; ++i) ok = ok && alloc(&c.tmp[i], (size_t)tmp[i] * sizeof(float2));
   if (!ok) {  // no room: the direct kernels need none of it
@@ -538,7 +552,7 @@ bool build_level(scatter_plan_s* p, const scatter_problem* pr, const scatter_opt
   c.sub->d.status = p->d.status;
   c.sub->d.inst_shift = p->d.inst_shift;
   c.sub->extent2 = p->coarse_levels == 0 ? p->coarse_rmax2 : nullptr;  // measured once
-  c.sub->out_shift = p->coarse_no_shift;
+  c.sub->out_shift = p->coarse_shift;
   p->base_bytes += bytes + c.sub->base_bytes + c.sub->tiling_bytes;
   ++p->coarse_levels;
   return true;
@@ -573,6 +587,7 @@ scatter_status launch_coarse(scatter_plan_t p, const double* xyz, const float* o
     a.axis64 = p->d.axis64;
     for (int d = 0; d < 3; ++d) a.H64[d] = p->inst[0].H[d];
     a.exact64 = p->path != SCATTER_PATH_SEPARABLE;
+    a.planar = p->s_kind == SCATTER_S_GID_GRID;
     a.n0 = p->n_axis[0];
     a.n1 = p->n_axis[1];
     a.n2 = p->n_axis[2];
@@ -724,10 +739,10 @@ void release_level(scatter_plan_s* p, CoarseState& c) {
 
 void release_coarse(scatter_plan_s* p) {
   for (CoarseState& c : p->coarse) release_level(p, c);
-  for (void* b : {(void*)p->coarse_rmax2, (void*)p->coarse_no_shift})
+  for (void* b : {(void*)p->coarse_rmax2, (void*)p->coarse_shift})
     if (b) cudaFree(b);
   p->coarse_rmax2 = nullptr;
-  p->coarse_no_shift = nullptr;
+  p->coarse_shift = nullptr;
   p->coarse_levels = p->coarse_adj_levels = 0;
 }
 

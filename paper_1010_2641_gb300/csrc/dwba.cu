@@ -376,7 +376,8 @@ __global__ void __launch_bounds__(128) k_f64_gid(const double* __restrict__ xyz,
 // buried object:  A = sum_t W_t(alpha_f) T_t.  f_s(|S_t|), the translation
 // phase and (buried) the attenuation are already in T.
 __global__ void k_gid_combine(const float2* __restrict__ virt, const float2* __restrict__ w, int64_t n_hk,
-                              int64_t n_af, int n_beams, float2* out_amp, float* out_int) {
+                              int64_t n_af, int n_beams, float2* out_amp, float* out_int, const CallGate gate) {
+  if (within(gate, 0)) return;
   const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= n_hk * n_af) return;
   const int64_t af = m % n_af, hk = m / n_af;
@@ -391,10 +392,11 @@ __global__ void k_gid_combine(const float2* __restrict__ virt, const float2* __r
   if (out_int) out_int[m] = v.x * v.x + v.y * v.y;
 }
 
-scatter_status launch_gid_combine(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st) {
+scatter_status launch_gid_combine(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st,
+                                  const CallGate& gate) {
   const int64_t n_hk = p->n_axis[0] * p->n_axis[1], n_af = p->n_axis[2];
   k_gid_combine<<<(unsigned)((n_hk * n_af + 255) / 256), 256, 0, st>>>(p->d.sep_virt, p->d.gid_w, n_hk, n_af,
-                                                                      (int)p->sep_beams, amp_out, int_out);
+                                                                      (int)p->sep_beams, amp_out, int_out, gate);
   p->last_launches += 1;
   return cuda_status(cudaGetLastError(), "gid combine launch");
 }

@@ -134,7 +134,8 @@ struct PrepArgs {
   float4* rec_a;          // the folded separable forward's A records, or null
   float mid[3], mid_lo[3];  // middles of its axes - H
   unsigned* rmax2;        // [batch] largest |x'|^2 (float bits, zeroed before), or null
-  int per_axis;           // rmax2 of the largest |x'_d| instead
+  int per_axis;           // rmax2 of the largest |x'_d| of this many axes instead
+  double* z_shift;        // [3] third element: t_z, or null
   CallGate gate;          // one instance
 };
 
@@ -243,7 +244,8 @@ __device__ __forceinline__ float prep_slot(const PrepArgs& a, int64_t slot, cons
   }
   const float q[3] = {x0[0] * x0[0], x0[1] * x0[1], x0[2] * x0[2]};
   // a NaN stays one: its bits are the largest
-  if (a.per_axis) return __uint_as_float(max(max(__float_as_uint(q[0]), __float_as_uint(q[1])), __float_as_uint(q[2])));
+  if (a.per_axis)
+    return __uint_as_float(max(max(__float_as_uint(q[0]), __float_as_uint(q[1])), a.per_axis > 2 ? __float_as_uint(q[2]) : 0u));
   return q[0] + q[1] + q[2];
 }
 
@@ -313,6 +315,7 @@ __global__ void __launch_bounds__(256) k_prep_one(const PrepArgs a, int64_t n_at
     sh_t[threadIdx.x] = t;
     sh_h[threadIdx.x] = (float)a.inst_H[threadIdx.x];
     if (blockIdx.x == 0) inst_shift[threadIdx.x] = t;
+    if (blockIdx.x == 0 && threadIdx.x == 2 && a.z_shift) a.z_shift[2] = t;
   }
   __syncthreads();
   const double t[3] = {sh_t[0], sh_t[1], sh_t[2]};
@@ -619,7 +622,9 @@ scatter_status launch_prep(scatter_plan_t p, const double* xyz, const float* occ
   a.status = p->d.status;
   a.rec_a = p->d.sep_rec;
   a.rmax2 = p->cl.active ? p->cl.rmax2 : p->extent2;
-  a.per_axis = p->extent2 != nullptr;
+  const bool gid = p->s_kind == SCATTER_S_GID_GRID;
+  a.per_axis = p->extent2 ? (gid ? 2 : 3) : 0;
+  a.z_shift = gid ? p->out_shift : nullptr;
   a.gate = gate;
   for (int d = 0; d < 3; ++d) {
     a.mid[d] = (float)p->sep_mid[d];

@@ -328,9 +328,10 @@ struct scatter_plan_s {
   int coarse_levels = 0;
   int coarse_adj_levels = 0;                     // the first ones, with an adjoint
   unsigned* coarse_rmax2 = nullptr;              // this call's largest |x'_d|^2 (float bits)
-  double* coarse_no_shift = nullptr;             // [3] zeros
+  double* coarse_shift = nullptr;                // [3] the nodes' out_shift
   unsigned* extent2 = nullptr;                   // the sum at the nodes of another plan: prep writes the largest |x'_d|^2
-  const double* out_shift = nullptr;             //   its reductions' shift in place of the call's
+  double* out_shift = nullptr;                   //   its reductions' shift in place of the call's: 0 on the interpolated
+                                                 //   axes (grazing incidence: prep writes the call's t_z)
   double sep_group = 0.0;                        //   accumulation groups of at least this many steps
   int64_t base_bytes = 0;                        // tables and backward workspace
   int64_t tiling_bytes = 0;                      // chunk tables and split-K partials

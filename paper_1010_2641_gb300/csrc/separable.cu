@@ -1350,7 +1350,7 @@ scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_ou
     if (e != cudaSuccess) return cuda_status(e, "host copy completion");
   }
   if (gid) {
-    scatter_status s2 = launch_gid_combine(p, amp_out, int_out, st);
+    scatter_status s2 = launch_gid_combine(p, amp_out, int_out, st, gate);
     if (s2 != SCATTER_OK) return s2;
   }
   return cuda_status(cudaGetLastError(), "separable launch");

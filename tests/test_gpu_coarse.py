@@ -105,3 +105,29 @@ def test_larger_crystal_is_left_to_the_direct_sum(path, shape):
         assert torch.equal(p(_t(x)), q(_t(x)))
     assert torch.equal(plan.amplitude(_t(c.xyz)), small)  # and back
     plan.check()
+
+
+@pytest.mark.parametrize("shape, offset", [((150, 150, 24), (0.0, 0.0, 0.0)), ((33, 600, 24), (7.3, -4.6, 3.2))])
+def test_grazing_incidence_in_plane(shape, offset):
+    c = W.truncated_pyramid(44, 16, 14)
+    xyz = c.xyz + np.array(offset)
+    gid = dict(wavelength=W.WAVELENGTH_10KEV, alpha_i=W.GID_ALPHA_I, delta=W.GID_DELTA, beta=W.GID_BETA)
+    axes = list(W.gid_axes(*shape))
+    plan, bare = _plans(c, axes, "separable", gid=gid)
+    assert _nodes(plan, bare)
+    A, D = plan.amplitude(_t(xyz)).cpu().numpy(), bare.amplitude(_t(xyz)).cpu().numpy()
+    assert not np.array_equal(A, D)
+    assert _rel(A, D) < 5e-5  # either sum is within 5e-5 of the oracle's on such islands
+    H = plan.amplitude_host(xyz)
+    torch.cuda.synchronize()
+    assert np.array_equal(A.view(np.float32), H.numpy().reshape(-1).view(np.float32))
+    pts = W.grid_points(axes)
+    idx = np.random.default_rng(308).choice(len(pts), 150, replace=False)
+    ref = oracle.dwba(xyz, pts[idx], c.coef, A_LAT, species=c.species, **gid)
+    scale = np.sqrt(np.mean(np.abs(D) ** 2))
+    assert np.sqrt(np.mean(np.abs(A[idx] - ref) ** 2)) < 1e-4 * max(scale, np.sqrt(np.mean(np.abs(ref) ** 2)))
+    far = xyz.copy()
+    far[11, :2] *= 9.0
+    assert torch.equal(plan.amplitude(_t(far)), bare.amplitude(_t(far)))
+    assert torch.equal(plan.intensity(_t(xyz)), bare.intensity(_t(xyz)))
+    plan.check()
