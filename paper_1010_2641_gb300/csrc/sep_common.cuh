@@ -19,7 +19,7 @@ namespace scatter {
 
 constexpr int kSepFormWarps = 8;           // warps forming B rows (one N column per thread)
 constexpr int kSepThreads = 32 * (kSepFormWarps + 2);  // + the MMA warp + the copy warp
-constexpr int sep_form_warps(bool fold) { return fold ? 16 : kSepFormWarps; }  // of the one-CTA kernel
+constexpr int kSepOneWarps = 16;           // the one-CTA kernel's
 constexpr int kSepM = 128;                 // MMA M (rows of A per CTA)
 constexpr int kSepN = 256;                 // MMA N (columns per CTA)
 constexpr int kSepStep = 16;               // K records per pipeline step (K' = 32)

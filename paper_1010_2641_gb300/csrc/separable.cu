@@ -141,10 +141,10 @@ __global__ void __launch_bounds__(256) k_sep_tab_fold(const float4* __restrict__
 // -------------------------------------------------------------------------
 
 
-// Warp roles: 8 (folded 16) formation warps form the B rows (one point per thread)
-// and read the accumulators out at every group end; the next warp (one lane)
-// issues the MMAs; the last (one lane) issues the TMA copies.  Hand-offs go through mbarriers
-// only:
+// Warp roles: 16 formation warps form the B rows (two threads per point) and read
+// the accumulators out at every group end; the next warp (one lane) issues the
+// MMAs; the last (one lane) issues the TMA copies.  Hand-offs go through
+// mbarriers only:
 //   bar_full[a]   A block of a step arrived            (TMA, 1 arrival + bytes)
 //   bar_done[a]   MMAs of the step done (one commit per step); frees the A
 //                 stage of that step and the B stage it read
@@ -154,14 +154,15 @@ __global__ void __launch_bounds__(256) k_sep_tab_fold(const float4* __restrict__
 //   bar_tfree     accumulators read out after a group end (formation warps)
 // FOLD: the folded forward (sep_common.cuh): 32 atoms per step, the 256 columns
 // are the cos and sin columns of 128 mirror pairs of points; thread (p, kb)
-// forms both columns of pair p over one of the four K blocks.  16 warps share the
-// formation, whose latency binds a step of one M tile (64 x 64 x 24 nodes of
-// 134,009 atoms: 1.1 us a step with 8 warps, 1.0 us so).
+// forms both columns of pair p over one of the four K blocks.  The formation binds
+// a step of one M tile; 16 warps against 8: 43 x 43 x 31 nodes of a 127,560-atom
+// island 1.15 against 1.33 ms per call, folded 64 x 64 x 24 nodes of 134,009 atoms
+// 1.0 against 1.1 us a step; two M tiles are bound by the MMAs either way.
 template <bool FOLD>
-__global__ void __maxnreg__(FOLD ? 112 : 168) k_sep(const SepArgs a) {
+__global__ void __maxnreg__(112) k_sep(const SepArgs a) {
   if (within(a.gate, 0)) return;  // before any barrier or allocation
   constexpr int kRec = FOLD ? kSepFoldStep : kSepStep;  // records per step
-  constexpr int kForm = sep_form_warps(FOLD);
+  constexpr int kForm = kSepOneWarps;
   constexpr int kSpan = kSepN / (kForm / 4);  // columns that a formation warp reads out
   // a B stage is freed by the done barrier of the step that read it: the A
   // ring (and with it the done ring) must be at least as deep as the B ring
@@ -320,7 +321,7 @@ __global__ void __maxnreg__(FOLD ? 112 : 168) k_sep(const SepArgs a) {
     // offsets (s_b, s_c) from H, adjoint the atom's (y', z')
     // (folded: the first point of the thread's mirror pair)
     const int p_loc = tid & (narrow ? kSepFoldPairs / 2 - 1 : kSepFoldPairs - 1);
-    const int64_t col = FOLD ? nt * kSepFoldPairs + p_loc : col_base + tid;
+    const int64_t col = FOLD ? nt * kSepFoldPairs + p_loc : col_base + (tid & (kSepN - 1));
     const bool row_ok = col < (FOLD ? a.n_pairs : col_end);
     float sb, sc, sbl = 0.f, scl = 0.f;  // sbl, scl: low parts of a double-float s (forward)
     float att = 0.f;                     // buried object: 2 pi Im(sigma) of the column's beam
@@ -339,7 +340,7 @@ __global__ void __maxnreg__(FOLD ? 112 : 168) k_sep(const SepArgs a) {
         scl = a.axis_lo[a.n0 + a.n1 + rc];
       }
     }
-    const int b_row = FOLD ? (p_loc >> 6) * 128 + (p_loc & 63) : tid;  // folded: the cos column, the sin column 64 on
+    const int b_row = FOLD ? (p_loc >> 6) * 128 + (p_loc & 63) : tid & (kSepN - 1);  // folded: the cos column, the sin column 64 on
     const uint32_t b_row_off = (uint32_t)((b_row >> 3) * 128 + (b_row & 7) * 16);
     // |s_b y' + s_c z' + c| of every B element of this call stays below
     // kSepPhaseLim cycles when the centred extent is small: the exact mod-1
@@ -404,7 +405,8 @@ __global__ void __maxnreg__(FOLD ? 112 : 168) k_sep(const SepArgs a) {
         constexpr int kMode = decltype(mode_tag)::value;
         constexpr bool kAtt = decltype(att_tag)::value;
 #pragma unroll
-        for (int kb = 0; kb < 4; ++kb) {
+        for (int kq = 0; kq < 2; ++kq) {
+          const int kb = 2 * (tid / kSepN) + kq;  // two threads per column
           uint32_t hi[4] = {0u, 0u, 0u, 0u}, lo[4] = {0u, 0u, 0u, 0u};
           if (row_ok) {
 #pragma unroll
@@ -870,9 +872,9 @@ cudaError_t sep_prepare_kernel() {
 // pair kernel's last clusters leave idle.
 static void launch_one_cta(const SepArgs& a, dim3 grid, cudaStream_t st) {
   if (a.fold)
-    k_sep<true><<<grid, 32 * (sep_form_warps(true) + 2), kSepSmem, st>>>(a);
+    k_sep<true><<<grid, 32 * (kSepOneWarps + 2), kSepSmem, st>>>(a);
   else
-    k_sep<false><<<grid, kSepThreads, kSepSmem, st>>>(a);
+    k_sep<false><<<grid, 32 * (kSepOneWarps + 2), kSepSmem, st>>>(a);
 }
 
 cudaError_t sep_launch_core(const SepArgs& a, dim3 grid, cudaStream_t st, cudaStream_t side, cudaEvent_t fork,
