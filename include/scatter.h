@@ -194,10 +194,16 @@ typedef struct scatter_options {
                                 measured against the oracle, stays within the
                                 tolerance; everything else takes the generic
                                 FP32 path                                     */
-  double radius_hint;        /* SCATTER_PATH_AUTO: bound on |r_j - t| (lattice
-                                units, after the integer centring) used by
-                                that error model; 0 = a compact crystal of
-                                n_atoms at 4 atoms per cell                   */
+  double radius_hint;        /* bound on |r_j - t| (lattice units, after the
+                                integer centring); 0 = a compact crystal of
+                                n_atoms at 4 atoms per cell, with margins.
+                                SCATTER_PATH_AUTO's error model uses it, and so
+                                do grids sampled finer than the crystal's
+                                extent asks for (summed at the nodes that
+                                resolve it, interpolated) and lists of close
+                                points (clusters): a call measures its crystal,
+                                and one past the bound is summed point by point
+                                at the direct sum's speed                     */
 } scatter_options;
 
 typedef struct scatter_plan_s* scatter_plan_t;
@@ -278,9 +284,10 @@ scatter_status scatter_amplitude(scatter_plan_t plan, const double* xyz,
  * the first host call and kept until scatter_plan_destroy: 28 n_atoms + 8 n_s
  * bytes, plus a second stream and 17 events), runs the plan's forward on
  * them and copies the map back.  On a SEPARABLE plan of a GRID the final
- * reduction runs in up to 16 ranges of map rows and each range's copy to the
- * host starts on the plan's second stream as soon as that range is reduced,
- * overlapping the rest of the reduction; `stream` waits for the last copy.
+ * reduction of the direct sum runs in up to 16 ranges of map rows (4 where the
+ * grid is folded over its middle) and each range's copy to the host starts on
+ * the plan's second stream as soon as that range is reduced, overlapping the
+ * rest of the reduction; `stream` waits for the last copy.
  * Pinned host memory gives asynchronous copies; pageable memory is accepted
  * and then copied synchronously by the driver.  Errors: INVALID_ARG for a
  * NULL or device pointer (a NULL xyz or A_out is allowed only when n_atoms
