@@ -41,6 +41,7 @@ constexpr double kCoarseEps = 5e-8, kCoarseEpsSep = 1e-6;
 // the map's; they are taken where that moves a gradient by less than the tensor-core
 // path's own scatter, 1.8e-5.
 constexpr double kCoarseAdjSteps = 135.0;  // 1.8e-5 / 1.3e-7
+constexpr double kCoarseMaxWeights = 1.6e7;  // nodes x points of an axis (128 MB, 0.1 s of planning)
 constexpr int kIpK = 16;  // nodes per stage of the interpolation
 
 struct InterpArgs {
@@ -422,7 +423,7 @@ NodeSet choose_nodes(const scatter_plan_s* p, double X) {
         for (n = 4; n <= most && tail[n] > eps;) ++n;
         for (; n <= most; n += 2)
           if (form_error(p, d, r.nd[d] = chebyshev_nodes(lo, hi, n), X) < 2.0 * eps) break;
-        if (n > most) n = 0;
+        if (n > most || (double)n * (double)ax.size() > kCoarseMaxWeights) n = 0;
       }
     }
     any = any || n > 0;

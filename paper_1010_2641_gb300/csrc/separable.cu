@@ -667,9 +667,11 @@ struct SepFoldReduceArgs {
 // centring phase and |A|^2.  A thread holds one lane's rows and four pairs:
 // rows l % 8 and quad l / 8 of pairs, so a read covers 128 contiguous bytes
 // per quad, and the four row blocks and the two columns of a pair (blocks of
-// the partials that the same thread reads) combine with no exchange.  GROUPS threads share a quadruple's chunks on small maps and meet
-// in shared memory in a fixed order (64 CTAs of seven chunks: 21.5 us with one
-// thread per quadruple, 12.7 us with four).
+// the partials that the same thread reads) combine with no exchange.  GROUPS
+// threads share a quadruple's chunks on small maps and meet in shared memory in a
+// fixed order (64 CTAs of seven chunks: 21.5 us with one thread per quadruple,
+// 12.7 us with four; 51 x 51 nodes of 150 chunks: 35 us with eight,
+// 19 us with 32).
 template <int GROUPS>
 __global__ void __launch_bounds__(256) k_sep_reduce_fold(const SepFoldReduceArgs a) {
   if (within(a.gate, 0)) return;
@@ -1303,11 +1305,13 @@ scatter_status launch_separable(scatter_plan_t p, float2* amp_out, float* int_ou
       // ranges: a host call's map equals the device call's bit for bit)
       const int64_t quads = (fm.pairs + 3) / 4, range = (n_bm + max_pieces - 1) / max_pieces;
       int groups = 1;
-      while (groups < 8 && 2 * groups <= n_chunks && (quads + 31) / 32 * range * groups < p->n_sm) groups *= 2;
-      const auto kernel = groups == 1   ? k_sep_reduce_fold<1>
-                          : groups == 2 ? k_sep_reduce_fold<2>
-                          : groups == 4 ? k_sep_reduce_fold<4>
-                                        : k_sep_reduce_fold<8>;
+      while (groups < 32 && 2 * groups <= n_chunks && (quads + 31) / 32 * range * groups < p->n_sm) groups *= 2;
+      const auto kernel = groups == 1    ? k_sep_reduce_fold<1>
+                          : groups == 2  ? k_sep_reduce_fold<2>
+                          : groups == 4  ? k_sep_reduce_fold<4>
+                          : groups == 8  ? k_sep_reduce_fold<8>
+                          : groups == 16 ? k_sep_reduce_fold<16>
+                                         : k_sep_reduce_fold<32>;
       const int64_t per_cta = 32 / groups;  // quads per CTA
       kernel<<<dim3((unsigned)((quads + per_cta - 1) / per_cta), (unsigned)(b1 - b0)), 256, 0, st>>>(r);
     } else {
