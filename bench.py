@@ -580,10 +580,9 @@ def measure_paths(args, dev, clk, only=None):
         plan = api.Plan(cube.coef, W.LATTICE_A, len(cube.xyz), axes=ax, timing=True, path="generic", radius_hint=NO_NODES)
         ms = timed(lambda: plan.backward(x, A, I_obs), plan)
         res["adjoint_cube"]["direct_kernel_ms"] = ms
-        # without nodes, uniform l axis: the line kernel carries the phase along l by a complex multiply,
-        # 8 FMA-pipe ops per pair at 128 lane-ops per SM per clock, no MUFU
-        res["adjoint_cube"]["direct_roofline"] = _rate_roof(len(cube.xyz) * 128 ** 3, ms, 16.0, n_sm, rc.get("clk"),
-                                                            "Gpair/s", "alu", "pairs (8 FMA-pipe ops each)")
+        # without nodes: rows times columns, 4 multiply-adds per point of a symmetric axis at 128 per SM per clock
+        res["adjoint_cube"]["direct_roofline"] = _rate_roof(len(cube.xyz) * 128 ** 3, ms, 32.0, n_sm, rc.get("clk"),
+                                                            "Gpair/s", "alu", "pairs (4 FMA each: a column and its mirror)")
         del plan, x, A, I_obs
     if want('adjoint_list'):
         # the S-list adjoint (k_adjoint: MUFU sin/cos per pair): strained sphere x an Ewald-slice list

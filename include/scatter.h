@@ -222,9 +222,9 @@ typedef struct scatter_plan_info {
   double shift[3];           /* integer centring vector t of instance 0        */
   int32_t atoms_per_thread;  /* > 0: the atom-parallel form was chosen        */
   int32_t adjoint_form;      /* form of the gradient kernel, fixed at the first
-                              * backward: 0 none yet, 1 FP32 S tiles (lists,
-                              * non-uniform grids), 2 FP32 line recurrence
-                              * (uniform l axis), 3 tensor-core contraction
+                              * backward: 0 none yet, 1 FP32 (lists, grids with
+                              * an uneven l axis), 2 FP32 (grids with an evenly
+                              * spaced l axis), 3 tensor-core contraction
                               * (SEPARABLE grid plans)                         */
 } scatter_plan_info;
 

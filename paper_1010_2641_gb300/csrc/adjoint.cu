@@ -18,7 +18,8 @@
 //                 sums per tile in FP32, outer sums in FP64 (the terms over
 //                 millions of S nearly cancel).  The exponentials are
 //                 recomputed, nothing of size N x M is stored.
-//                 Lists of close points: cluster_adjoint.cu in its place.
+//                 Lists of close points: cluster_adjoint.cu in its place;
+//                 grids where it is cheaper: grid_adjoint.cu.
 // k_adjoint_final sums the S-chunk partials in a fixed order, scales by
 //                 -2 pi w_j and writes the caller's atom order.
 #include <cuda_runtime.h>
@@ -606,6 +607,12 @@ scatter_status prepare_adjoint(scatter_plan_s* p) {
     p->adj_ready = true;
     return SCATTER_OK;
   }
+  if ((ss = prepare_grid_adjoint(p)) != SCATTER_OK) return ss;
+  if (p->ga.active) {
+    if ((ss = prepare_coarse_adjoint(p)) != SCATTER_OK) return ss;
+    p->adj_ready = true;
+    return SCATTER_OK;
+  }
   std::vector<AdjBlock> blocks;
   const int per = kAdjThreads * kAdjRA;
   for (const Segment& s : p->all_segs)
@@ -681,6 +688,16 @@ scatter_status prepare_adjoint(scatter_plan_s* p) {
   if ((ss = prepare_coarse_adjoint(p)) != SCATTER_OK) return ss;
   p->adj_ready = true;
   return SCATTER_OK;
+}
+
+scatter_status launch_adjoint_rows(scatter_plan_t p, const float2* gf, float* grad, cudaStream_t st,
+                                   const CallGate& gate) {
+  if (const scatter_status s = launch_grid_adjoint(p, gf, st, gate); s != SCATTER_OK) return s;
+  const int64_t nb = (3 * p->n_slots + kFinalVals - 1) / kFinalVals;
+  k_adjoint_final<<<(unsigned)nb, kFinalVals * kFinalGroups, 0, st>>>(p->ga.partial, p->ga.split * p->ga.chunks, gate, 0,
+                                                                      p->n_slots, p->d.slot_src, p->d.atom_w, grad);
+  p->last_launches += 1;
+  return cuda_status(cudaGetLastError(), "backward launch");
 }
 
 // The FP32 forms from the weight table, where the gate lets them.
@@ -773,14 +790,15 @@ scatter_status launch_backward(scatter_plan_t p, const double* xyz, const float*
   la.ftab = p->d.ftab;  // Eq. 4: the block factors F_t(S) in place of f_s(|S|), held fixed
   la.n_species = grad ? p->n_species : 0;
   la.inv4a2 = (float)(1.0 / (4.0 * p->lattice_a * p->lattice_a));
-  la.layout = !grad ? 0 : (p->adj_sep ? 2 : (p->adj_line ? 1 : 0));
+  la.layout = !grad ? 0 : (p->adj_sep || p->ga.active ? 2 : (p->adj_line ? 1 : 0));
   la.table = p->d.adj_table;
   la.gf = p->d.adj_gf;
   la.loss_part = p->d.loss_part;
   const bool clustered = grad && p->cl.adj.active;
   const CallGate gate = clustered ? cluster_gate(p) : coarse_gate(p, coarse);
   la.gate = gate;
-  if (clustered || (coarse && !p->adj_sep)) la.gf = reinterpret_cast<float2*>(p->d.adj_table);  // either layout, never both
+  if (p->ga.active) la.gf = p->ga.gf;
+  else if (clustered || (coarse && !p->adj_sep)) la.gf = reinterpret_cast<float2*>(p->d.adj_table);  // either layout, never both
   k_loss_weights<<<kLossParts, kLossThreads, 0, st>>>(la);
   p->last_launches += 1;
   if (A && loss_out) {
@@ -790,6 +808,7 @@ scatter_status launch_backward(scatter_plan_t p, const double* xyz, const float*
   if (grad && p->n_atoms > 0) {
     if (coarse && (s = launch_coarse_adjoint(p, la.gf, grad, st)) != SCATTER_OK) return s;
     if (p->adj_sep) return launch_adjoint_sep(p, grad, st, gate);
+    if (p->ga.active) return launch_adjoint_rows(p, la.gf, grad, st, gate);
     if (clustered && (s = launch_cluster_adjoint(p, la.gf, p->d.adj_partial, st)) != SCATTER_OK) return s;
     if ((s = launch_adjoint_tiles(p, grad, st, gate)) != SCATTER_OK) return s;
   }

@@ -626,17 +626,17 @@ scatter_status prepare_coarse_adjoint(scatter_plan_s* p) {
   if (l >= p->coarse_levels) return SCATTER_OK;
   CoarseState& c = p->coarse[l];
   if (!sep && p->path == SCATTER_PATH_SEPARABLE) return SCATTER_OK;
-  // pairs per second: tensor cores 5e13 (fewer points 4e13), line recurrence
-  // 3.4e12, the nodes' tiles 2e12
+  // pairs per second: tensor cores 5e13 (fewer points 4e13), FP32 lanes at 2 GHz
+  const double lanes = 128.0 * p->n_sm * 2.0e9;
   const double pairs = (double)p->n_slots;
-  const double fine = pairs * (double)p->n_s / (sep ? 5.0e13 : p->adj_line ? 3.4e12 : 2.0e12);
+  const double fine = pairs * (double)p->n_s / (sep ? 5.0e13 : lanes / grid_adjoint_ops(p));
   bool fold = true;
   if (sep) {
     const double least = adjoint_sep_group(p, false) - kCoarseAdjSteps;
     fold = adjoint_sep_group(c.sub, true) >= least;
     if (!fold && adjoint_sep_group(c.sub, false) < least) return SCATTER_OK;
   }
-  const double few = pairs * (double)c.sub->n_s / (!sep ? 2.0e12 : fold ? 4.0e13 : 2.0e13) + 60e-6 +
+  const double few = pairs * (double)c.sub->n_s / (!sep ? lanes / grid_adjoint_ops(c.sub) : fold ? 4.0e13 : 2.0e13) + 60e-6 +
                      (double)p->n_s * p->n_species * 30.0 / 4.0e12;
   if (few > 0.75 * fine) return SCATTER_OK;  // nor any larger set
   c.sub->adj_no_fold = !fold;
@@ -699,6 +699,8 @@ scatter_status level_adjoint(scatter_plan_t p, int l, const float2* gf, float* g
   scatter_status s;
   if (p->adj_sep) {
     s = launch_adjoint_sep(sub, grad, st, a.gate);
+  } else if (sub->ga.active) {
+    s = launch_adjoint_rows(sub, in, grad, st, a.gate);
   } else {
     const int64_t total = (int64_t)p->n_species * sub->n_s;
     k_node_table<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(

@@ -91,6 +91,13 @@ inline CallGate cluster_gate(const scatter_plan_s* p) {
   return p->cl.active ? CallGate{p->cl.rmax2, p->cl.lim2, p->batch, nullptr} : CallGate{};
 }
 
+// FP32 adjoint on grids as rows times columns (grid_adjoint.cu): prepared where it
+// is the cheaper form; partial sums in p->ga.partial.
+scatter_status prepare_grid_adjoint(scatter_plan_s* p);
+scatter_status launch_grid_adjoint(scatter_plan_t p, const float2* gf, cudaStream_t st, const CallGate& gate);
+void release_grid_adjoint(GridAdjState& g);
+double grid_adjoint_ops(const scatter_plan_s* p);
+
 // Maps sampled far finer than the crystal's extent asks for (coarse.cu): the sum
 // at the Chebyshev nodes of each axis, interpolated to the map.
 scatter_status prepare_coarse(scatter_plan_s* p, const scatter_problem* pr, const scatter_options* op);
@@ -156,7 +163,10 @@ scatter_status prepare_adjoint_sep(scatter_plan_s* p);
 double adjoint_sep_group(const scatter_plan_s* p, bool fold);
 scatter_status launch_adjoint_sep(scatter_plan_t p, float* grad, cudaStream_t st,
                                   const CallGate& gate = CallGate{});
-// FP32 adjoint from the plan's weight table (adjoint.cu).
+// FP32 adjoint from the plan's weight table, or from gF where it runs as rows times
+// columns (adjoint.cu).
+scatter_status launch_adjoint_rows(scatter_plan_t p, const float2* gf, float* grad, cudaStream_t st,
+                                   const CallGate& gate = CallGate{});
 scatter_status launch_adjoint_tiles(scatter_plan_t p, float* grad, cudaStream_t st,
                                     const CallGate& gate = CallGate{});
 scatter_status prepare_adjoint(scatter_plan_s* p);

@@ -315,6 +315,7 @@ extern "C" void scatter_plan_destroy(scatter_plan_t p) {
   release(d.sep_A);
   release(d.sep_partial);
   release_clusters(p);
+  release_grid_adjoint(p->ga);
   release(p->gs.chunks);
   release(p->gs.d);
   release(p->gs.dlo);

@@ -164,6 +164,22 @@ struct ClState {
   int n_items = 0, n_tab = 0, n_red = 0, n_eval = 0;
 };
 
+// FP32 adjoint on grids, rows times columns (grid_adjoint.cu).
+struct GridAdjState {
+  bool active = false;
+  int q = 2, np = 0, chunks = 1, pairs = 0;  // column axis, pairs per CTA, chunks of them, pairs in all
+  bool mirror = false;
+  double mid = 0.0;                 // middle of a symmetric column axis - H
+  int64_t rows_per_split = 0;
+  int split = 1, n_blocks = 0;
+  AdjBlock* blocks = nullptr;
+  float* d = nullptr;               // column offsets, and rounding errors
+  float* dlo = nullptr;
+  float* table = nullptr;           // [species][chunk][row][np][16]
+  float* partial = nullptr;         // [split][chunk][slot][3]
+  float2* gf = nullptr;             // [species][M]
+};
+
 // Oversampled maps (coarse.cu).
 struct CoarseStage {
   int axis = 0;
@@ -324,6 +340,7 @@ struct scatter_plan_s {
   scatter::DeviceBuffers d;
   scatter::GridSum gs;
   scatter::ClState cl;
+  scatter::GridAdjState ga;
   scatter::CoarseState coarse[scatter::kCoarseLevels];  // by growing radius
   int coarse_levels = 0;
   int coarse_adj_levels = 0;                     // the first ones, with an adjoint
