@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 #include "device_common.cuh"
 #include "launch.h"
@@ -67,8 +68,9 @@ struct InterpArgs {
 };
 
 // out[o, i, b] = sum_k W[k, i] in[o, k, b], 16 T values of i x 16 T columns (o, b)
-// per CTA, T x T per thread (T = 4; 2 where that leaves the SMs idle: 61 x 47 x 33
-// points from 39 x 34 x 27 nodes: 9 us a stage, 16 us with T = 4).  ROWS: the last axis (inner = 1).  Lanes run along the
+// per CTA, T x T per thread: the largest T that gives every SM two CTAs (61 x 47 x 33
+// points from 39 x 34 x 27 nodes: 16, 9 and 6 us a stage with T = 4, 2 and 1).  ROWS:
+// the last axis (inner = 1).  Lanes run along the
 // contiguous index of the output.  Sums of 16 joined one by one in FP32; WIDE (maps
 // of FP32 sums): weights and sums as double-floats, eleven operations per term
 // instead of one, which leaves a map's error to its nodes (61 x 47 x 33 points
@@ -80,7 +82,7 @@ __global__ void __launch_bounds__(256) k_interp(const InterpArgs a) {
   __shared__ float sh_wl[WIDE ? kIpK : 1][WIDE ? kIpTile : 1];
   __shared__ float2 sh_in[kIpK][kIpTile + (ROWS ? 1 : 0)];
   using u64 = unsigned long long;
-  static_assert(T == 2 || T == 4, "outputs and columns per thread");
+  static_assert(T == 1 || T == 2 || T == 4, "outputs and columns per thread");
   if (within(a.gate, 0)) return;
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
   const int64_t b0 = (int64_t)blockIdx.x * kIpTile, i0 = (int64_t)blockIdx.y * kIpTile;
@@ -341,14 +343,19 @@ void launch_stage(scatter_plan_t p, const InterpArgs& a, cudaStream_t st) {
   auto tiles = [&](int64_t tile) {
     return dim3((unsigned)((a.outer * a.inner + tile - 1) / tile), (unsigned)((a.n_out + tile - 1) / tile));
   };
-  dim3 grid = tiles(64);
-  const bool few = (int64_t)grid.x * grid.y < 2 * p->n_sm;
-  if (few) grid = tiles(32);
+  // the largest tiles that still give every SM two CTAs
+  int T = 4;
+  while (T > 1 && (int64_t)tiles(16 * T).x * tiles(16 * T).y < 2 * p->n_sm) T /= 2;
+  const dim3 grid = tiles(16 * T);
   const bool wide = p->path != SCATTER_PATH_SEPARABLE, rows = a.inner == 1 && a.axis == 2;
-  const auto kernel = wide ? (rows ? (few ? k_interp<true, true, 2> : k_interp<true, true, 4>)
-                                   : (few ? k_interp<false, true, 2> : k_interp<false, true, 4>))
-                           : (rows ? (few ? k_interp<true, false, 2> : k_interp<true, false, 4>)
-                                   : (few ? k_interp<false, false, 2> : k_interp<false, false, 4>));
+  auto pick = [&](auto t) {
+    constexpr int kT = decltype(t)::value;
+    return wide ? (rows ? k_interp<true, true, kT> : k_interp<false, true, kT>)
+                : (rows ? k_interp<true, false, kT> : k_interp<false, false, kT>);
+  };
+  const auto kernel = T == 4   ? pick(std::integral_constant<int, 4>{})
+                      : T == 2 ? pick(std::integral_constant<int, 2>{})
+                               : pick(std::integral_constant<int, 1>{});
   kernel<<<grid, 256, 0, st>>>(a);
 }
 
