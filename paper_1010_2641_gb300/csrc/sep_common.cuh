@@ -30,7 +30,7 @@ constexpr int kSepFlush = 256;             // steps between TMEM flushes
 constexpr uint32_t kSepABytes = 16384;     // A block of one M tile: hi + lo, 128 x 32 f16 each
 constexpr int kSepPair = 2;                // M tiles per CTA (one formed B tile feeds both)
 constexpr uint32_t kSepBBytes = 32768;     // B block: hi + lo, 256 x 32 f16 each
-constexpr int kSepAStages = 4;             // A ring (full / empty barrier per stage)
+constexpr int kSepALog = 2, kSepAStages = 1 << kSepALog;  // A ring (full / empty barrier per stage)
 constexpr int kSepBStages = 2;             // B ring: formation of step k+1 overlaps MMAs of k
 constexpr int kSepTStages = 8;             // K-record ring (256 B per step)
 constexpr size_t kSepSmem = kSepAStages * kSepPair * kSepABytes + kSepBStages * kSepBBytes + 1024;  // + align

@@ -168,8 +168,8 @@ __global__ void __maxnreg__(112) k_sep(const SepArgs a) {
   // ring (and with it the done ring) must be at least as deep as the B ring
   static_assert(kSepBStages <= kSepAStages, "B-stage reuse is tracked on the done ring");
   extern __shared__ __align__(1024) unsigned char sep_smem_raw[];
-  __shared__ __align__(8) uint64_t bar_full[kSepAStages];
-  __shared__ __align__(8) uint64_t bar_done[kSepAStages];
+  __shared__ __align__(8) uint64_t bar_full[2 * kSepAStages];
+  __shared__ __align__(8) uint64_t bar_done[2 * kSepAStages];
   __shared__ __align__(8) uint64_t bar_atom[kSepTStages];
   __shared__ __align__(8) uint64_t bar_tempty[kSepTStages];
   __shared__ __align__(8) uint64_t bar_bfull[kSepBStages];
@@ -186,6 +186,10 @@ __global__ void __maxnreg__(112) k_sep(const SepArgs a) {
   const int64_t n_mp = a.mp_count > 0 ? a.mp_count : (a.n_mt + 1) / 2;  // pairs of this launch
   const int64_t mp = a.mp_first + blockIdx.x % n_mp, nt = blockIdx.x / n_mp;
   const int ntp = 2 * mp + 1 < a.n_mt ? 2 : 1;  // M tiles of this CTA with rows
+  // one M tile: twice the A stages, of half the bytes (127,560-atom island, 43 x 43 x
+  // 31 nodes: 1.26 ms per call with three stages, 1.148 with four, 1.134 with eight;
+  // the bytes in two more B stages instead: 1.20)
+  const int la = ntp == 1 ? kSepALog + 1 : kSepALog, n_a = 1 << la;
   const int chunk = blockIdx.y;
   const int64_t nbc = a.n1 * a.n2;
   // up to 64 mirror pairs in all: 128 columns are contracted
@@ -206,7 +210,7 @@ __global__ void __maxnreg__(112) k_sep(const SepArgs a) {
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int s = 0; s < kSepAStages; ++s) {
+    for (int s = 0; s < n_a; ++s) {
       dev::mbar_init(&bar_full[s], 1);
       dev::mbar_init(&bar_done[s], 1);
     }
@@ -245,7 +249,7 @@ __global__ void __maxnreg__(112) k_sep(const SepArgs a) {
           ok = false;
           break;
         }
-        const int tst = (int)(g % kSepTStages), ast = (int)(g % kSepAStages);
+        const int tst = (int)(g % kSepTStages), ast = (int)(g & (n_a - 1));
         if (g >= kSepTStages &&
             !dev::mbar_wait_bounded(&bar_tempty[tst], (uint32_t)(((g - kSepTStages) / kSepTStages) & 1))) {
           ok = false;
@@ -254,13 +258,12 @@ __global__ void __maxnreg__(112) k_sep(const SepArgs a) {
         dev::mbar_arrive_expect_tx(&bar_atom[tst], kRec * sizeof(float4));
         dev::bulk_g2s(&ring_atom[tst][0], a.rec + ks * kRec, kRec * sizeof(float4), &bar_atom[tst]);
         t_issued = g + 1;
-        if (g >= kSepAStages &&
-            !dev::mbar_wait_bounded(&bar_done[ast], (uint32_t)(((g - kSepAStages) / kSepAStages) & 1))) {
+        if (g >= n_a && !dev::mbar_wait_bounded(&bar_done[ast], (uint32_t)(((g - n_a) >> la) & 1))) {
           ok = false;
           break;
         }
         dev::mbar_arrive_expect_tx(&bar_full[ast], a_bytes);
-        dev::bulk_g2s(ringA + ast * kSepPair * kSepABytes, Ablk + ks * (kSepPair * kSepABytes / 16), a_bytes,
+        dev::bulk_g2s(ringA + ast * ntp * kSepABytes, Ablk + ks * (kSepPair * kSepABytes / 16), a_bytes,
                       &bar_full[ast]);
         a_issued = g + 1;
       }
@@ -288,8 +291,8 @@ __global__ void __maxnreg__(112) k_sep(const SepArgs a) {
           ok = false;
           break;
         }
-        const int ast = (int)(g % kSepAStages), bst = (int)(g % kSepBStages);
-        if (!dev::mbar_wait_bounded(&bar_full[ast], (uint32_t)((g / kSepAStages) & 1)) ||
+        const int ast = (int)(g & (n_a - 1)), bst = (int)(g % kSepBStages);
+        if (!dev::mbar_wait_bounded(&bar_full[ast], (uint32_t)((g >> la) & 1)) ||
             !dev::mbar_wait_bounded(&bar_bfull[bst], (uint32_t)((g / kSepBStages) & 1))) {
           ok = false;
           break;
@@ -297,7 +300,7 @@ __global__ void __maxnreg__(112) k_sep(const SepArgs a) {
         tc_fence_after();
         const uint64_t offB = (uint64_t)((bst * kSepBBytes) >> 4);
         for (int tp = 0; tp < ntp; ++tp) {
-          const uint64_t offA = (uint64_t)(((ast * kSepPair + tp) * kSepABytes) >> 4);
+          const uint64_t offA = (uint64_t)(((ast * ntp + tp) * kSepABytes) >> 4);
           const uint32_t d = tmem + (uint32_t)(tp * kSepN);
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
@@ -368,8 +371,7 @@ __global__ void __maxnreg__(112) k_sep(const SepArgs a) {
       // every lane waits, the warp agrees on the outcome
       bool w = !s_abort;
       if (w && g >= kSepBStages)
-        w = dev::mbar_wait_bounded(&bar_done[(g - kSepBStages) % kSepAStages],
-                                   (uint32_t)(((g - kSepBStages) / kSepAStages) & 1));
+        w = dev::mbar_wait_bounded(&bar_done[(g - kSepBStages) & (n_a - 1)], (uint32_t)(((g - kSepBStages) >> la) & 1));
       if (w) w = dev::mbar_wait_bounded(&bar_atom[tst], (uint32_t)((g / kSepTStages) & 1));
       if (!__all_sync(0xffffffffu, w)) {
         ok = false;
@@ -459,7 +461,7 @@ __global__ void __maxnreg__(112) k_sep(const SepArgs a) {
 
       // ---- group end: TMEM -> blocked partials -------------------------------
       // the commit of step g covers every earlier MMA of the group
-      w = dev::mbar_wait_bounded(&bar_done[g % kSepAStages], (uint32_t)((g / kSepAStages) & 1));
+      w = dev::mbar_wait_bounded(&bar_done[g & (n_a - 1)], (uint32_t)((g >> la) & 1));
       if (!__all_sync(0xffffffffu, w)) {
         ok = false;
         break;
@@ -521,11 +523,11 @@ __global__ void __maxnreg__(112) k_sep(const SepArgs a) {
   // releasing TMEM and shared memory; phases already complete return at once
   if (mma_warp && lane == 0 && s_abort && g_committed > 0) {
     const int64_t gl = g_committed - 1;
-    dev::mbar_wait_bounded(&bar_done[gl % kSepAStages], (uint32_t)((gl / kSepAStages) & 1), 1LL << 28);
+    dev::mbar_wait_bounded(&bar_done[gl & (n_a - 1)], (uint32_t)((gl >> la) & 1), 1LL << 28);
   }
   if (copy_warp && lane == 0 && s_abort) {
-    for (int64_t s = a_issued > kSepAStages ? a_issued - kSepAStages : 0; s < a_issued; ++s)
-      dev::mbar_wait_bounded(&bar_full[s % kSepAStages], (uint32_t)((s / kSepAStages) & 1), 1LL << 28);
+    for (int64_t s = a_issued > n_a ? a_issued - n_a : 0; s < a_issued; ++s)
+      dev::mbar_wait_bounded(&bar_full[s & (n_a - 1)], (uint32_t)((s >> la) & 1), 1LL << 28);
     for (int64_t s = t_issued > kSepTStages ? t_issued - kSepTStages : 0; s < t_issued; ++s)
       dev::mbar_wait_bounded(&bar_atom[s % kSepTStages], (uint32_t)((s / kSepTStages) & 1), 1LL << 28);
   }
