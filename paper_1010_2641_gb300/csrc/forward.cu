@@ -17,6 +17,7 @@
 //   reduce   split-K partials summed in a fixed order (deterministic), then
 //            the translation phase e^{2 pi i s.t} and |A|^2 if requested.
 #include <cuda_runtime.h>
+#include <cmath>
 #include <cstdint>
 #include <cstdio>
 #include "device_common.cuh"
@@ -136,8 +137,15 @@ struct PrepArgs {
   unsigned* rmax2;        // [batch] largest |x'|^2 (float bits, zeroed before), or null
   int per_axis;           // rmax2 of the largest |x'_d| of this many axes instead
   double* z_shift;        // [3] third element: t_z, or null
+  int wide;               // |S| past kPrepFixedS: the split in FP64 throughout
   CallGate gate;          // one instance
 };
+
+// Positions in 2^-42 fixed point err by up to 2^-43 cells, a phase by |S| times as
+// much: 2^-31 cycles at |S| = 2^12, a 64th of the rounding of c itself.  Longer S go
+// with coordinates that are small numbers (crystals in metres: S of 1e10, positions of
+// 1e-8, of which fixed point keeps four digits) and take FP64.
+constexpr double kPrepFixedS = 4096.0;
 
 // a + b with its rounding error
 __device__ __forceinline__ float two_sum(float a, float b, float& err) {
@@ -165,8 +173,9 @@ __device__ __forceinline__ void prep_coord(double x, double t, float& x0, float&
     const long long r = (hi < 0 ? -(long long)mag : (long long)mag) - ((long long)(int)t << 42);
     const int n = (int)((r + (1LL << 41)) >> 42);
     const long long d = r - ((long long)n << 42);  // [-2^41, 2^41)
-    dh = (float)(int)(d >> 18) * 5.9604644775390625e-08f;                 // 24 bits, 2^-24
-    dl = (float)(int)(d & 0x3ffffLL) * 2.2737367544323206e-13f;           // 18 bits, 2^-42
+    // 24 bits of 2^-24 and 18 of 2^-42, joined to the nearest float and the rest: a
+    // small coordinate keeps its digits
+    dh = two_sum((float)(int)(d >> 18) * 5.9604644775390625e-08f, (float)(int)(d & 0x3ffffLL) * 2.2737367544323206e-13f, dl);
     float err;
     x0 = two_sum((float)n, dh, err);
     lo = err + dl;
@@ -208,24 +217,32 @@ __device__ __forceinline__ float prep_slot(const PrepArgs& a, int64_t slot, cons
     if (a.rec_a) a.rec_a[slot] = zero;
     return 0.f;
   }
-  float x0[3], lo[3], c = 0.f, ce = 0.f;
+  float x0[3], lo[3], cr, ce = 0.f, err;
+  if (a.wide) {
+    double c = 0.0;
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    float dh, dl, err;
-    prep_coord(x[d], t[d], x0[d], lo[d], dh, dl);
-    if (fabsf(h[d]) < 4194304.0f) {  // exact in FP32
+    for (int d = 0; d < 3; ++d) {
+      const double r = x[d] - t[d];
+      x0[d] = (float)r;
+      lo[d] = (float)(r - (double)x0[d]);
+      c = fma(H[d], r - rint(r), c);
+    }
+    c -= rint(c);
+    cr = (float)c;
+    ce = (float)(c - (double)cr);
+  } else {
+    float c = 0.f;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      float dh, dl;
+      prep_coord(x[d], t[d], x0[d], lo[d], dh, dl);
       const float pr = __fmul_rn(h[d], dh);
       c = two_sum(c, __fsub_rn(pr, rintf(pr)), err);
       ce += err + (fmaf(h[d], dh, -pr) + h[d] * dl);
-    } else {
-      const double ph = H[d] * ((double)dh + (double)dl);
-      c = two_sum(c, (float)(ph - rint(ph)), err);
-      ce += err;
     }
+    cr = c - rintf(c);  // exact
   }
-  float err;
-  const float cr = c - rintf(c);  // exact
-  c = cr + ce;
+  const float c = cr + ce;
   a.atom4[slot] = make_float4(x0[0], x0[1], x0[2], c);
   a.atom_lo[slot] = make_float4(lo[0], lo[1], lo[2], 0.f);
   a.atom_w[slot] = w;
@@ -625,6 +642,8 @@ scatter_status launch_prep(scatter_plan_t p, const double* xyz, const float* occ
   const bool gid = p->s_kind == SCATTER_S_GID_GRID;
   a.per_axis = p->extent2 ? (gid ? 2 : 3) : 0;
   a.z_shift = gid ? p->out_shift : nullptr;
+  for (const Instance& in : p->inst)
+    for (int d = 0; d < 3; ++d) a.wide |= std::fabs(in.H[d]) + p->s_max[d] > kPrepFixedS;
   a.gate = gate;
   for (int d = 0; d < 3; ++d) {
     a.mid[d] = (float)p->sep_mid[d];
