@@ -41,6 +41,7 @@ namespace {
 constexpr int kGsTile = 128;   // atoms per stage
 constexpr int kGsMaxR = 8;     // columns per thread
 constexpr int kGsChunk = 32;   // chunk granularity (slots)
+constexpr int64_t kGsMaxTiles = 65535;  // column tiles and chunks: y and z of the launch grid
 
 struct GridSumArgs {
   const float4* atom4;
@@ -344,12 +345,14 @@ Shape best_shape(const scatter_plan_s* p) {
     double mid;
     const bool mirror = axis_symmetric(p->axis_host[q], &mid);
     const int64_t cols = mirror ? (n + 1) / 2 : n, rows = p->n_s / n;
-    for (int R = 1; R <= kGsMaxR; ++R)
+    for (int R = 1; R <= kGsMaxR; ++R) {
+      if ((cols + R - 1) / R > kGsMaxTiles) continue;  // a long axis: more columns per thread, or rows
       for (int th : {64, 128, 256}) {
         const double warps = std::ceil((double)rows / th) * (th / 32);
         const double c = warps * std::ceil((double)cols / R) * warp_cost(R);
         if (c < best.cost * 0.999) best = Shape{q, R, th, mirror, c};
       }
+    }
   }
   return best;
 }
@@ -376,17 +379,20 @@ bool gridsum_preferred(const scatter_plan_s* p) {
   return best_shape(p).cost < 0.875 * 4.0 * std::ceil((double)p->n_s / 32.0);
 }
 
-scatter_status prepare_gridsum(scatter_plan_s* p, int split_override) {
-  const Shape sh = best_shape(p);
+void release_gridsum(scatter_plan_s* p) {
   GridSum& g = p->gs;
   for (void* b : {(void*)g.chunks, (void*)g.d, (void*)g.dlo, (void*)g.rec, (void*)g.rec_lo, (void*)g.ztab,
-                  (void*)p->d.partial})  // of an earlier split (autotuning)
+                  (void*)p->d.partial})
     if (b) cudaFree(b);
-  g.chunks = nullptr;
-  g.d = g.dlo = nullptr;
-  g.rec = nullptr;
-  g.rec_lo = g.ztab = nullptr;
   p->d.partial = nullptr;
+  p->tiling_bytes -= g.bytes;
+  g = GridSum{};
+}
+
+scatter_status prepare_gridsum(scatter_plan_s* p, int split_override) {
+  const Shape sh = best_shape(p);
+  release_gridsum(p);  // of an earlier split (autotuning)
+  GridSum& g = p->gs;
   g.q = sh.q;
   g.R = sh.R;
   g.threads = sh.threads;
@@ -458,7 +464,7 @@ scatter_status prepare_gridsum(scatter_plan_s* p, int split_override) {
       chunks.push_back(Segment{sg.begin + b * kGsChunk, sg.begin + std::min(steps, b + per) * kGsChunk, sg.species, 0});
   }
   if (chunks.empty()) chunks.push_back(Segment{0, 0, 0, 0});  // no atoms: one empty chunk, zero partials
-  if (chunks.size() > 65535 || g.col_tiles > 65535)
+  if ((int64_t)chunks.size() > kGsMaxTiles || g.col_tiles > kGsMaxTiles)
     return fail(SCATTER_ERR_UNSUPPORTED, "grid sum: %zu chunks or %lld column tiles exceed the launch grid",
                 chunks.size(), (long long)g.col_tiles);
   g.n_chunks = (int)chunks.size();
@@ -477,8 +483,11 @@ scatter_status prepare_gridsum(scatter_plan_s* p, int split_override) {
   cudaError_t e;
   const size_t db = d.size() * sizeof(float), cb = chunks.size() * sizeof(Segment);
   const size_t pb = chunks.size() * (size_t)p->n_s * sizeof(float2);
-  if ((e = cudaMalloc(&g.d, db)) != cudaSuccess || (e = cudaMalloc(&g.dlo, db)) != cudaSuccess ||
-      (e = cudaMalloc(&g.chunks, cb)) != cudaSuccess || (e = cudaMalloc(&p->d.partial, pb)) != cudaSuccess)
+  auto alloc = [](auto** dst, size_t size) {
+    return injected_alloc_failure() ? cudaErrorMemoryAllocation : cudaMalloc((void**)dst, size);
+  };
+  if ((e = alloc(&g.d, db)) != cudaSuccess || (e = alloc(&g.dlo, db)) != cudaSuccess ||
+      (e = alloc(&g.chunks, cb)) != cudaSuccess || (e = alloc(&p->d.partial, pb)) != cudaSuccess)
     return cuda_status(e, "cudaMalloc grid sum");
   if ((e = cudaMemcpy(g.d, d.data(), db, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(g.dlo, dl.data(), db, cudaMemcpyHostToDevice)) != cudaSuccess ||
@@ -487,13 +496,13 @@ scatter_status prepare_gridsum(scatter_plan_s* p, int split_override) {
   size_t tb = 0;
   if (g.tab) {
     const size_t n4 = (size_t)p->n_slots * sizeof(float4), n2 = (size_t)p->n_slots * sizeof(float2);
-    if ((e = cudaMalloc(&g.rec, n4)) != cudaSuccess || (e = cudaMalloc(&g.rec_lo, n2)) != cudaSuccess ||
-        (e = cudaMalloc(&g.ztab, zb)) != cudaSuccess)
+    if ((e = alloc(&g.rec, n4)) != cudaSuccess || (e = alloc(&g.rec_lo, n2)) != cudaSuccess ||
+        (e = alloc(&g.ztab, zb)) != cudaSuccess)
       return cuda_status(e, "cudaMalloc grid sum table");
     tb = n4 + n2 + zb;
   }
-  p->tiling_bytes += (int64_t)(2 * db + cb + pb + tb) - g.bytes;
   g.bytes = (int64_t)(2 * db + cb + pb + tb);
+  p->tiling_bytes += g.bytes;
   g.split = split;
   p->tiling.threads = sh.threads;
   p->tiling.R = sh.R * (sh.mirror ? 2 : 1);

@@ -130,6 +130,7 @@ scatter_status plan_nodes(const scatter_problem* pr, const scatter_options* op, 
 // Factorised FP32 sum on single GRID plans (gridsum.cu).
 bool gridsum_preferred(const scatter_plan_s* p);
 scatter_status prepare_gridsum(scatter_plan_s* p, int split_override);
+void release_gridsum(scatter_plan_s* p);
 scatter_status launch_gridsum(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st,
                               const CallGate& gate = CallGate{});
 

@@ -316,12 +316,7 @@ extern "C" void scatter_plan_destroy(scatter_plan_t p) {
   release(d.sep_partial);
   release_clusters(p);
   release_grid_adjoint(p->ga);
-  release(p->gs.chunks);
-  release(p->gs.d);
-  release(p->gs.dlo);
-  release(p->gs.rec);
-  release(p->gs.rec_lo);
-  release(p->gs.ztab);
+  release_gridsum(p);
   release(p->sep_direct.chunks);
   release(p->sep_folded.chunks);
   release(d.ap_blocks);
@@ -581,27 +576,36 @@ scatter_status make_plan(const scatter_problem* pr, const scatter_options* op, b
     if ((st = apply_tiling(p.get(), t))) return st;
   } else if (path == SCATTER_PATH_GENERIC) {
     // single grids: the factorised sum, unless the caller asks for a tile of the
-    // sincos forms or the grid is too small for it
+    // sincos forms or the grid is too small for it; where it finds no room (it keeps
+    // a map per chunk, at least one per species) the sincos form, which needs none
     const bool tile_asked = op && (op->threads || op->points_per_thread || op->atoms_per_thread > 0);
-    const bool factorised = !tile_asked && gridsum_preferred(p.get());
-    Tiling t = factorised ? Tiling{} : heuristic_tiling(p.get());
-    if (op && op->threads) t.threads = op->threads;
-    if (op && op->points_per_thread) t.R = op->points_per_thread;
-    if (op && op->split_k && !factorised) t.split_k = op->split_k;
-    if (op && (op->threads || op->points_per_thread || op->split_k || op->atoms_per_thread < 0)) t.atom_k = 0;
-    if (op && op->atoms_per_thread > 0) t.atom_k = op->atoms_per_thread;
-    if (!generic_tiling_supported(t))
-      return fail(SCATTER_ERR_INVALID_ARG, "unsupported tile override (threads=%d R=%d)", t.threads, t.R);
-    if ((st = apply_tiling(p.get(), t))) return st;
+    bool factorised = !tile_asked && gridsum_preferred(p.get());
     if (factorised) {
-      if ((st = prepare_gridsum(p.get(), op ? op->split_k : 0))) return st;
-      if (op && op->autotune && !op->split_k && (st = autotune_gridsum(p.get(), op->tune_cache))) return st;
-    } else if (pr->batch > 1) {
+      if ((st = apply_tiling(p.get(), Tiling{}))) return st;
+      st = prepare_gridsum(p.get(), op ? op->split_k : 0);
+      if (st == SCATTER_OK && op && op->autotune && !op->split_k) st = autotune_gridsum(p.get(), op->tune_cache);
+      if (st != SCATTER_OK && st != SCATTER_ERR_OOM && st != SCATTER_ERR_UNSUPPORTED) return st;
+      factorised = st == SCATTER_OK;
+      if (!factorised) release_gridsum(p.get());
+    }
+    if (!factorised) {
+      Tiling t = heuristic_tiling(p.get());
+      if (op && op->threads) t.threads = op->threads;
+      if (op && op->points_per_thread) t.R = op->points_per_thread;
+      if (op && op->split_k) t.split_k = op->split_k;
+      if (op && (op->threads || op->points_per_thread || op->split_k || op->atoms_per_thread < 0)) t.atom_k = 0;
+      if (op && op->atoms_per_thread > 0) t.atom_k = op->atoms_per_thread;
+      if (!generic_tiling_supported(t))
+        return fail(SCATTER_ERR_INVALID_ARG, "unsupported tile override (threads=%d R=%d)", t.threads, t.R);
+      if ((st = apply_tiling(p.get(), t))) return st;
+    }
+    if (pr->batch > 1) {
       if ((st = prepare_batch(p.get()))) return st;
       if (op && op->autotune && !(op->threads || op->points_per_thread) &&
           (st = autotune_batch(p.get(), op->tune_cache)))
         return st;
-    } else if (op && op->autotune && !(op->threads || op->points_per_thread || op->split_k || op->atoms_per_thread)) {
+    } else if (!factorised && op && op->autotune &&
+               !(op->threads || op->points_per_thread || op->split_k || op->atoms_per_thread)) {
       if ((st = autotune_generic(p.get(), op->tune_cache))) return st;
     }
   } else {
