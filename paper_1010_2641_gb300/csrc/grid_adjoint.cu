@@ -38,6 +38,7 @@ constexpr int kGaThreads = 128;
 constexpr int kGaAtoms = 2 * kGaThreads;
 constexpr int kGaRows = 16;   // rows per stage
 constexpr int kGaMaxNP = 16;  // pairs per CTA
+constexpr int kGaMaxY = 65535;  // row ranges x chunks of pairs: y of the launch grid
 
 struct GridAdjArgs {
   const float4* atom4;
@@ -238,7 +239,7 @@ GaShape ga_shape(const scatter_plan_s* p) {
     s.q = q;
     s.mirror = axis_symmetric(p->axis_host[q], &s.mid);
     const int64_t n = p->n_axis[q], pairs = s.mirror ? (n + 1) / 2 : n;
-    if (pairs > (1 << 20)) continue;
+    if (pairs > (int64_t)kGaMaxNP * kGaMaxY) continue;
     s.pairs = (int)pairs;
     s.chunks = (s.pairs + kGaMaxNP - 1) / kGaMaxNP;
     s.np = 2 * ((s.pairs + 2 * s.chunks - 1) / (2 * s.chunks));
@@ -291,7 +292,7 @@ scatter_status prepare_grid_adjoint(scatter_plan_s* p) {
   // rows per CTA: waves x (rows + some 20 rows' worth of table and output)
   double best = 1e300;
   const double cap = (double)p->n_sm * bps, base = (double)blocks.size() * s.chunks;
-  for (int64_t split = 1; split <= std::min<int64_t>(n_rows, 4096) && split * s.chunks <= 65535; ++split) {
+  for (int64_t split = 1; split <= std::min<int64_t>(n_rows, 4096) && split * s.chunks <= kGaMaxY; ++split) {
     const int64_t per = (n_rows + split - 1) / split, n = (n_rows + per - 1) / per;
     const double cost = std::ceil(base * (double)n / cap) * ((double)per + 20.0) + 0.02 * (double)n;
     if (cost < best * 0.999) {
