@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(kFinalVals* kFinalGroups) k_adjoint_final(cons
   const int64_t slot = i / 3;
   const int32_t src = slot_src[slot];
   if (src < 0) return;
-  grad[3 * (int64_t)src + (i - 3 * slot)] = -6.28318530717958647692f * atom_w[slot] * v.value();
+  grad[3 * (int64_t)src + (i - 3 * slot)] = v.times_minus_two_pi(atom_w[slot]);
 }
 
 // ---------------------------------------------------------------------------

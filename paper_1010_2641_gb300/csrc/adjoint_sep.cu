@@ -273,14 +273,14 @@ __global__ void __launch_bounds__(32 * kAdjFinalWarps) k_adj_sep_final(const Adj
     if (src < 0) continue;
     // -2 pi w (H_d V + W_d) in double-floats (an FP64 operation of two lanes
     // costs the whole warp's 19 cycles here), H_d exact in two floats
-    const float scale = -6.28318530717958647692f * f.atom_w[slot + u];
+    const float w = f.atom_w[slot + u];
     const dev::DFloatSum v = sum[u][0];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       dev::DFloatSum g = sum[u][d + 1];
       g.add_product(f.H[d], v.hi);
       g.lo = __fadd_rn(g.lo, fmaf(f.H[d], v.lo, f.H_lo[d] * v.hi));
-      f.grad[3 * (int64_t)src + d] = scale * g.value();
+      f.grad[3 * (int64_t)src + d] = g.times_minus_two_pi(w);
     }
   }
 }

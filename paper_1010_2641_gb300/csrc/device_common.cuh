@@ -121,6 +121,17 @@ struct DFloatSum {
     lo = __fadd_rn(lo, e);
   }
   __device__ __forceinline__ float value() const { return __fadd_rn(hi, lo); }
+  // -2 pi w times the sum, rounded once: the product of two double-floats
+  // (a gradient's last step; 13 FP32 operations, FP64 would take the slow pipe)
+  __device__ __forceinline__ float times_minus_two_pi(float w) const {
+    const float c = 6.28318530717958647692f, c_lo = -1.7484556e-7f;  // 2 pi
+    const float p = __fmul_rn(c, w), p_lo = __fmaf_rn(c, w, -p) + c_lo * w;
+    const float s = __fadd_rn(hi, lo), bb = __fsub_rn(s, hi);
+    const float s_lo = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(lo, bb));
+    const float r = __fmul_rn(p, s);
+    const float e = __fmaf_rn(p, s, -r) + fmaf(p, s_lo, p_lo * s);
+    return isfinite(r) ? -__fadd_rn(r, e) : -r;
+  }
 };
 
 // sin and cos of 2*pi*f for |f| <= 1/2 (cycles) on the MUFU pipe
