@@ -198,8 +198,15 @@ scatter_status autotune_generic(scatter_plan_s* p, const char* cache_path) {
 
 scatter_status autotune_gridsum(scatter_plan_s* p, const char* cache_path) {
   if (p->n_s == 0 || p->n_slots == 0) return SCATTER_OK;
+  // what the number of chunks goes with: the launch's shape, which depends on all three
+  // axes and on their symmetry, and the number of slots
   std::string key = cache_key(p);
   key.replace(0, 7, "gridsum");
+  const GridSum& g = p->gs;
+  char shape[128];
+  snprintf(shape, sizeof(shape), "|q%d|R%d|t%d|m%d|r%lld|c%lld|tab%d", g.q, g.R, g.threads, (int)g.mirror,
+           (long long)g.row_tiles, (long long)g.col_tiles, (int)g.tab);
+  key += shape;
   Tiling t;
   if (cache_lookup(cache_path, key, &t)) return prepare_gridsum(p, t.split_k);
   cudaEvent_t e0, e1;
