@@ -128,6 +128,7 @@ scatter_status plan_nodes(const scatter_problem* pr, const scatter_options* op, 
                           scatter_plan_t* out);
 
 // Factorised FP32 sum on single GRID plans (gridsum.cu).
+constexpr int kGridSumMaxSplit = 2048;  // chunks that a tuned plan may ask for
 bool gridsum_preferred(const scatter_plan_s* p);
 scatter_status prepare_gridsum(scatter_plan_s* p, int split_override);
 void release_gridsum(scatter_plan_s* p);

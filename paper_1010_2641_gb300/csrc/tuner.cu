@@ -33,7 +33,7 @@ std::string cache_key(const scatter_plan_s* p) {
   return buf;
 }
 
-bool cache_lookup(const char* path, const std::string& key, Tiling* t) {
+bool cache_lookup(const char* path, const std::string& key, Tiling* t, int most_split = 256) {
   if (!path) return false;
   FILE* f = fopen(path, "r");
   if (!f) return false;
@@ -55,7 +55,7 @@ bool cache_lookup(const char* path, const std::string& key, Tiling* t) {
       const char* d = strstr(line, "\"atom_k\":");  // absent in older caches: S-parallel
       int ak = 0;
       if (d && sscanf(d, "\"atom_k\": %d", &ak) == 1 && ak >= 0 && ak <= 16) cand.atom_k = ak;
-      if (generic_tiling_supported(cand) && k >= 1 && k <= 256) {
+      if (generic_tiling_supported(cand) && k >= 1 && k <= most_split) {
         *t = cand;
         found = true;
       }
@@ -208,13 +208,13 @@ scatter_status autotune_gridsum(scatter_plan_s* p, const char* cache_path) {
            (long long)g.row_tiles, (long long)g.col_tiles, (int)g.tab);
   key += shape;
   Tiling t;
-  if (cache_lookup(cache_path, key, &t)) return prepare_gridsum(p, t.split_k);
+  if (cache_lookup(cache_path, key, &t, kGridSumMaxSplit)) return prepare_gridsum(p, t.split_k);
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   const int start = p->gs.split;
   double best_ms = 1e30;
-  for (int k : {start, std::max(1, start / 2), 2 * start}) {
+  for (int k : {start, std::max(1, start / 2), std::min(kGridSumMaxSplit, 2 * start)}) {
     if (prepare_gridsum(p, k) != SCATTER_OK) continue;
     launch_gridsum(p, p->d.amp, nullptr, nullptr);  // warm-up
     for (int i = 0; i < 2; ++i) {

@@ -1,4 +1,5 @@
-"""Tuned FP32 grids: a cache entry serves plans of its launch shape only.  Maps against the oracle at the FP32 sums'
+"""Tuned FP32 grids: a cache entry serves plans of its launch shape only, and every
+entry that is written is found again.  Maps against the oracle at the FP32 sums'
 1e-5."""
 import numpy as np
 import pytest
@@ -37,3 +38,13 @@ def test_entries_serve_their_own_shape(tmp_path):
         A = plan.amplitude(torch.tensor(c.xyz, device="cuda:0")).cpu().numpy()
         ref = oracle.amplitude(c.xyz, W.grid_points(axes), c.coef, A_LAT, species=c.species)
         assert np.linalg.norm(A - ref) < 1e-5 * np.linalg.norm(ref)
+
+
+def test_many_chunks_are_found_again(tmp_path):
+    cache = tmp_path / "tune.jsonl"
+    n = 1000000
+    axes = _axes((16, 16, 2), False)
+    for _ in range(2):
+        plan = api.Plan(W.unit_species()[None], A_LAT, n, axes=axes, path="generic", autotune=True, tune_cache=str(cache))
+        assert plan.info()["split_k"] > 256
+        assert cache.read_text().count("\n") == 1
