@@ -1126,55 +1126,73 @@ scatter_status prepare_separable(scatter_plan_s* p, int split_override) {
     p->d.partial = nullptr;
   }
   cudaError_t e;
-  size_t a_bytes = 0, part_bytes = 0, chunk_bytes = 0;
-  for (SepForm* f : {&fd, &ff}) {
-    if (f == &ff && !ff.fold) break;
-    const std::vector<float>& off = f->fold ? dvals : alls;  // offsets that the kernels form phases from
-    for (int64_t i = 0; i < p->sep_n[1]; ++i) f->smax[0] = std::max(f->smax[0], std::fabs(off[p->sep_n[0] + i]));
-    for (int64_t i = 0; i < p->sep_n[2]; ++i)
-      f->smax[1] = std::max(f->smax[1], std::fabs(off[p->sep_n[0] + p->sep_n[1] + i]));
-    // With one N tile every A tile is read by one cluster only: the CTA pair
-    // then forms its A tiles itself from the atom records (the same arithmetic
-    // as k_sep_tab_a), and the table, written and read once, is not kept.
-    // With several N tiles that formation would repeat per tile, so the table
-    // stays; an odd pair count runs its last pair on the one-CTA kernel, which
-    // reads the table.
-    const int64_t n_mp = (f->mt + 1) / 2;
-    f->form_a = sep_pair_enabled() && n_mp % 2 == 0 && f->nt == 1;
-    if (!f->form_a)
-      a_bytes = std::max(a_bytes, (size_t)(2 * n_mp) * (size_t)std::max<int64_t>(f->steps, 1) * kSepABytes);
-    std::vector<Segment> chunks = sep_chunks(p, f->split, f->fold ? kSepFoldStep : kSepStep);
-    if (chunks.empty()) chunks.push_back(Segment{0, 0, 0, 0});  // no atoms: one empty chunk, zero partials
-    f->n_chunks = (int32_t)chunks.size();
-    part_bytes = std::max(part_bytes, (size_t)f->n_chunks * (size_t)sep_part_floats(f->mt, f->cols) * sizeof(float));
-    const size_t cb = chunks.size() * sizeof(Segment);
-    if ((e = cudaMalloc(&f->chunks, cb)) != cudaSuccess) return cuda_status(e, "cudaMalloc chunks");
-    cudaMemcpy(f->chunks, chunks.data(), cb, cudaMemcpyHostToDevice);
-    chunk_bytes += cb;
+  size_t bytes = 0;
+  auto alloc = [&](auto** dst, size_t size) {
+    bytes += size;
+    return injected_alloc_failure() ? cudaErrorMemoryAllocation : cudaMalloc((void**)dst, size);
+  };
+  auto put = [&](auto** dst, const auto& v) {
+    const size_t size = v.size() * sizeof(v[0]);
+    const cudaError_t r = alloc(dst, size);
+    return r != cudaSuccess ? r : cudaMemcpy(*dst, v.data(), size, cudaMemcpyHostToDevice);
+  };
+  // Chunk tables, A table, partials and offsets of the direct form, and of the folded one
+  auto make = [&](bool fold) {
+    cudaError_t r = cudaSuccess;
+    size_t a_bytes = 0, part_bytes = 0;
+    for (SepForm* f : {&fd, &ff}) {
+      if (f == &ff && !fold) break;
+      const std::vector<float>& off = f->fold ? dvals : alls;  // offsets that the kernels form phases from
+      for (int64_t i = 0; i < p->sep_n[1]; ++i) f->smax[0] = std::max(f->smax[0], std::fabs(off[p->sep_n[0] + i]));
+      for (int64_t i = 0; i < p->sep_n[2]; ++i)
+        f->smax[1] = std::max(f->smax[1], std::fabs(off[p->sep_n[0] + p->sep_n[1] + i]));
+      // With one N tile every A tile is read by one cluster only: the CTA pair
+      // then forms its A tiles itself from the atom records (the same arithmetic
+      // as k_sep_tab_a), and the table, written and read once, is not kept.
+      // With several N tiles that formation would repeat per tile, so the table
+      // stays; an odd pair count runs its last pair on the one-CTA kernel, which
+      // reads the table.
+      const int64_t n_mp = (f->mt + 1) / 2;
+      f->form_a = sep_pair_enabled() && n_mp % 2 == 0 && f->nt == 1;
+      if (!f->form_a)
+        a_bytes = std::max(a_bytes, (size_t)(2 * n_mp) * (size_t)std::max<int64_t>(f->steps, 1) * kSepABytes);
+      std::vector<Segment> chunks = sep_chunks(p, f->split, f->fold ? kSepFoldStep : kSepStep);
+      if (chunks.empty()) chunks.push_back(Segment{0, 0, 0, 0});  // no atoms: one empty chunk, zero partials
+      f->n_chunks = (int32_t)chunks.size();
+      part_bytes = std::max(part_bytes, (size_t)f->n_chunks * (size_t)sep_part_floats(f->mt, f->cols) * sizeof(float));
+      if ((r = put(&f->chunks, chunks)) != cudaSuccess) return r;
+    }
+    if (a_bytes) {
+      // tiles past the last row are never written by the table kernel (the
+      // CTA-pair kernel streams the second tile of a pair always; its rows are
+      // never read): zero them once
+      if ((r = alloc(&p->d.sep_A, a_bytes)) != cudaSuccess) return r;
+      if ((r = cudaMemset(p->d.sep_A, 0, a_bytes)) != cudaSuccess) return r;
+    }
+    if ((r = alloc(&p->d.sep_partial, part_bytes)) != cudaSuccess) return r;
+    if (!fold) return cudaSuccess;
+    if ((r = alloc(&p->d.sep_rec, (size_t)p->n_slots * sizeof(float4))) != cudaSuccess) return r;
+    if ((r = put(&p->d.sep_axis_d, dvals)) != cudaSuccess) return r;
+    return put(&p->d.sep_axis_dlo, dvals_lo);
+  };
+  e = make(ff.fold);
+  if (e == cudaErrorMemoryAllocation && ff.fold) {  // no room: the direct form may have no table, or a smaller one
+    cudaGetLastError();
+    for (void* b : {(void*)fd.chunks, (void*)ff.chunks, (void*)p->d.sep_A, (void*)p->d.sep_partial, (void*)p->d.sep_rec,
+                    (void*)p->d.sep_axis_d, (void*)p->d.sep_axis_dlo})
+      if (b) cudaFree(b);
+    ff = SepForm{};
+    fd.chunks = nullptr;
+    p->d.sep_A = nullptr;
+    p->d.sep_partial = p->d.sep_axis_d = p->d.sep_axis_dlo = nullptr;
+    p->d.sep_rec = nullptr;
+    for (double& m : p->sep_mid) m = 0.0;
+    bytes = 0;
+    e = make(false);
   }
-  if (a_bytes) {
-    if ((e = cudaMalloc(&p->d.sep_A, a_bytes)) != cudaSuccess) return cuda_status(e, "cudaMalloc separable A");
-    // tiles past the last row are never written by the table kernel (the
-    // CTA-pair kernel streams the second tile of a pair always; its rows are
-    // never read): zero them once
-    if ((e = cudaMemset(p->d.sep_A, 0, a_bytes)) != cudaSuccess) return cuda_status(e, "memset separable A");
-  }
-  if ((e = cudaMalloc(&p->d.sep_partial, part_bytes)) != cudaSuccess)
-    return cuda_status(e, "cudaMalloc separable partials");
-  if ((e = cudaMalloc(&p->d.sep_axis_s, alls.size() * sizeof(float))) != cudaSuccess) return cuda_status(e, "axes");
-  if ((e = cudaMalloc(&p->d.sep_axis_lo, alls_lo.size() * sizeof(float))) != cudaSuccess) return cuda_status(e, "axes");
-  cudaMemcpy(p->d.sep_axis_s, alls.data(), alls.size() * sizeof(float), cudaMemcpyHostToDevice);
-  cudaMemcpy(p->d.sep_axis_lo, alls_lo.data(), alls_lo.size() * sizeof(float), cudaMemcpyHostToDevice);
-  size_t fold_bytes = 0;
-  if (ff.fold) {
-    const size_t rb = (size_t)p->n_slots * sizeof(float4), db = dvals.size() * sizeof(float);
-    if ((e = cudaMalloc(&p->d.sep_rec, rb)) != cudaSuccess) return cuda_status(e, "cudaMalloc folded records");
-    if ((e = cudaMalloc(&p->d.sep_axis_d, db)) != cudaSuccess) return cuda_status(e, "folded axes");
-    if ((e = cudaMalloc(&p->d.sep_axis_dlo, db)) != cudaSuccess) return cuda_status(e, "folded axes");
-    cudaMemcpy(p->d.sep_axis_d, dvals.data(), db, cudaMemcpyHostToDevice);
-    cudaMemcpy(p->d.sep_axis_dlo, dvals_lo.data(), db, cudaMemcpyHostToDevice);
-    fold_bytes = rb + 2 * db;
-  }
+  if (e != cudaSuccess) return cuda_status(e, "separable tables");
+  if ((e = put(&p->d.sep_axis_s, alls)) != cudaSuccess || (e = put(&p->d.sep_axis_lo, alls_lo)) != cudaSuccess)
+    return cuda_status(e, "separable axes");
   size_t virt_bytes = 0;
   if (gid) {
     virt_bytes = (size_t)p->sep_ns * sizeof(float2);
@@ -1188,7 +1206,7 @@ scatter_status prepare_separable(scatter_plan_s* p, int split_override) {
     cudaMemcpy(p->d.sep_szf, szf.data(), tb, cudaMemcpyHostToDevice);
     virt_bytes += 2 * tb;
   }
-  p->base_bytes += (int64_t)(a_bytes + part_bytes + chunk_bytes + virt_bytes + fold_bytes);
+  p->base_bytes += (int64_t)(bytes + virt_bytes);
   if ((e = sep_prepare_kernel()) != cudaSuccess) return cuda_status(e, "separable shared memory attribute");
   st = sep_prepare_side(p, fd.mt);
   return st == SCATTER_OK && ff.fold ? sep_prepare_side(p, ff.mt) : st;
