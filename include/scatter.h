@@ -376,10 +376,16 @@ scatter_status scatter_check(scatter_plan_t plan, void* stream);
  *  per_pair      out: bound on |computed - exact| of one term
  *                exp(2 i pi S.r_j), relative to its weight |w_j f|: phase
  *                reduction in FP32 (c + s.x' with |c| <= 1/2), the 2 pi
- *                scaling and the MUFU sin/cos error.
+ *                scaling and the MUFU sin/cos error.  Where the plan may sum
+ *                over clusters of points or at Chebyshev nodes (radius_hint),
+ *                the neglected terms of their series and their roundings at the
+ *                worst are added; errors at nodes count times the
+ *                interpolation's Lebesgue constants, and weights are then the
+ *                map's largest.
  *  rel_l2_random out: the relative L2 error of a map whose per-pair errors
- *                are uncorrelated, including blocked FP32 accumulation
- *                (per_pair plus the summation term); correlated (coherent)
+ *                are uncorrelated, including blocked FP32 accumulation and the
+ *                neglected terms (the per-pair error without those worst cases
+ *                plus the summation term); correlated (coherent)
  *                errors are bounded by per_pair * sum_j |w_j f| / |A|.
  */
 scatter_status scatter_error_bound(scatter_plan_t plan, double radius, double* per_pair,

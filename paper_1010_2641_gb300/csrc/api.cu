@@ -303,8 +303,15 @@ extern "C" scatter_status scatter_error_bound(scatter_plan_t p, double radius, d
     return fail(SCATTER_ERR_INVALID_ARG, "bad argument");
   const double u = std::ldexp(1.0, -24);  // fp32 unit roundoff
   const double pi = 3.14159265358979323846;
+  // sums at nodes or over clusters, where they may serve: their truncated series in
+  // both results; their roundings at the worst, node errors amplified by the
+  // interpolation's Lebesgue constants, in the bound of one term alone
+  double truncation = 0.0, rounding = 0.0, amplify = 1.0;
+  if (p->cl.active) cluster_error(p, radius, &truncation, &rounding);
+  if (p->coarse_levels > 0) coarse_error(p, radius, &truncation, &rounding, &amplify);
   if (p->path == SCATTER_PATH_SEPARABLE) {
-    *rel_l2_random = separable_error_model(p, radius, p->tiling.split_k, per_pair);
+    *rel_l2_random = separable_error_model(p, radius, p->tiling.split_k, per_pair) + truncation;
+    *per_pair = *per_pair * amplify + truncation + rounding;
     return SCATTER_OK;
   }
   if (p->path == SCATTER_PATH_FP64_REF) {
@@ -323,7 +330,8 @@ extern "C" scatter_status scatter_error_bound(scatter_plan_t p, double radius, d
   // blocked FP32 accumulation: tiles of 256 atoms, then tiles summed
   const double per_seg = (double)std::max<int64_t>(p->n_slots, 1) / 256.0;
   const double acc = u * std::sqrt(256.0 + per_seg + (double)p->tiling.split_k);
-  *rel_l2_random = *per_pair + acc;
+  *rel_l2_random = *per_pair + truncation + acc;
+  *per_pair = *per_pair * amplify + truncation + rounding;
   return SCATTER_OK;
 }
 

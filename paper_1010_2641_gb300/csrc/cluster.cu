@@ -401,6 +401,7 @@ scatter_status prepare_clusters(scatter_plan_s* p, const double* s_list, double 
   std::vector<ClTabBlock> tab_blocks;
   std::vector<ClRedBlock> red_blocks;
   std::vector<ClEvalBlock> eval_blocks;
+  std::vector<ClExtent> extents;
   std::vector<int64_t> row_begin;  // of the last clustered instance: its clusters' points
   int64_t tab_floats = 0, part_floats = 0, m_floats = 0;
   double gain = 0.0;
@@ -616,6 +617,7 @@ scatter_status prepare_clusters(scatter_plan_s* p, const double* s_list, double 
     part_floats += more_part;
     m_floats += (int64_t)p->n_species * ci.K * rows;
     lim[b] = ci.lim2;
+    extents.push_back(ClExtent{X, {th[0], th[1], th[2]}});
     gain += direct - best;
   }
   // worth the extra launches (~30 us)
@@ -648,8 +650,58 @@ scatter_status prepare_clusters(scatter_plan_s* p, const double* s_list, double 
     cl.h_exps = exps;
     cl.h_row = row_begin;
   }
+  cl.extents = std::move(extents);
   cl.active = true;
   return SCATTER_OK;
+}
+
+void cluster_error(const scatter_plan_s* p, double radius, double* truncation, double* rounding) {
+  *truncation = *rounding = 0.0;
+  for (const ClExtent& e : p->cl.extents) {
+    const double r = std::min(1.0, radius / e.X), u = std::ldexp(1.0, -24);
+    if (!(r > 0.0)) continue;
+    // Every term above 1e-12 with the relative radius from which it is a column (past 1
+    // never).  A crystal of relative radius q leaves out those past q: of degree n at most
+    // their largest values over the ball, and at most all terms' (|th| q)^n / n!.
+    // The sum is largest just before a column joins, or at r.
+    constexpr int kTop = 40;
+    struct Term {
+      double t, rho;
+      int n;
+    };
+    std::vector<Term> terms;
+    double ax[3][kTop + 1], lf = 0.0;
+    for (int i = 0; i <= kTop; ++i) {
+      if (i) lf += std::log((double)i);
+      for (int d = 0; d < 3; ++d)
+        ax[d][i] = i ? i * (std::log(std::max(e.th[d], 1e-12)) + 0.5 * std::log((double)i)) - lf : 0.0;
+    }
+    for (int a = 0; a <= kTop; ++a)
+      for (int b = 0; a + b <= kTop; ++b)
+        for (int c = 0; a + b + c <= kTop; ++c) {
+          const int n = a + b + c;
+          if (n == 0) continue;
+          const double t = ax[0][a] + ax[1][b] + ax[2][c] - 0.5 * n * std::log((double)n);
+          if (t > -27.6) terms.push_back({t, std::exp((std::log(kClEps) - t) / n), n});
+        }
+    const double len = std::sqrt(e.th[0] * e.th[0] + e.th[1] * e.th[1] + e.th[2] * e.th[2]);
+    auto neglected = [&](double q) {
+      double by[kTop + 1] = {0.0}, sum = 0.0, all = 1.0;
+      for (const Term& m : terms)
+        if (m.rho >= q) by[m.n] += std::exp(m.t + m.n * std::log(q));
+      for (int n = 1; n <= kTop; ++n) {
+        all *= len * q / n;
+        sum += std::min(by[n], all);
+      }
+      return sum;
+    };
+    double worst = neglected(r);
+    for (const Term& m : terms)
+      if (m.rho < r) worst = std::max(worst, neglected(m.rho));
+    *truncation = std::max(*truncation, worst);
+    // a column of degree n carries 4 n + 5 roundings; the columns' absolute sum is below e^(|th| r)
+    *rounding = std::max(*rounding, u * std::exp(len * r) * (4.0 * len * r + 5.0));
+  }
 }
 
 ClArgs cluster_args(scatter_plan_s* p) {

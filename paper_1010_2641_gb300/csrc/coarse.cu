@@ -561,12 +561,46 @@ bool build_level(scatter_plan_s* p, const scatter_problem* pr, const scatter_opt
   c.sub->d.inst_shift = p->d.inst_shift;
   c.sub->extent2 = p->coarse_levels == 0 ? p->coarse_rmax2 : nullptr;  // measured once
   c.sub->out_shift = p->coarse_shift;
+  c.X = set.X;
   p->base_bytes += bytes + c.sub->base_bytes + c.sub->tiling_bytes;
   ++p->coarse_levels;
   return true;
 }
 
 }  // namespace
+
+void coarse_error(const scatter_plan_s* p, double radius, double* truncation, double* rounding, double* amplify) {
+  *truncation = *rounding = 0.0;
+  *amplify = 1.0;
+  const double u = std::ldexp(1.0, -24);
+  for (int l = 0; l < p->coarse_levels; ++l) {
+    const CoarseState& c = p->coarse[l];
+    const double X = std::min(radius, c.X);
+    // Lebesgue constants: 2/pi ln n + 1 bounds those of n Chebyshev nodes
+    double product = 1.0;
+    auto lebesgue = [](double n) { return 0.63661977236758134 * std::log(n) + 1.0; };
+    for (int i = 0; i < c.n_stages; ++i) product *= lebesgue((double)c.stage[i].n_in);
+    // A wave has |x'| <= X in all: past 0.9 X along one axis it stays within 0.44 X along
+    // the others, whose tails are then nothing.
+    double one = 0.0, near = 0.0, round = 0.0;
+    for (int i = 0; i < c.n_stages; ++i) {
+      const CoarseStage& s = c.stage[i];
+      const std::vector<double>& ax = p->axis_host[s.axis];
+      const double lo = *std::min_element(ax.begin(), ax.end()), hi = *std::max_element(ax.begin(), ax.end());
+      const int n = (int)s.n_in;
+      const double others = product / lebesgue((double)n), c1 = 3.14159265358979323846 * X * (hi - lo);
+      // waves, and waves times form factors
+      const double form = form_error(p, s.axis, chebyshev_nodes(lo, hi, n), X);
+      one = std::max(one, others * (chebyshev_tails(c1, n)[n] + form));
+      near += others * (chebyshev_tails(0.9 * c1, n)[n] + form);
+      // WIDE: double-float weights and sums; else n products in sums of 16
+      round += product * u * (p->path == SCATTER_PATH_SEPARABLE ? 18.0 + (double)n / 16.0 : 1.0);
+    }
+    *truncation = std::max(*truncation, one + near);
+    *rounding = std::max(*rounding, round);
+    *amplify = std::max(*amplify, product);
+  }
+}
 
 scatter_status launch_coarse_prep(scatter_plan_t p, int levels, const double* xyz, const float* occ, cudaStream_t st) {
   for (int l = 0; l < levels; ++l) {

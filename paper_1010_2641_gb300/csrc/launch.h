@@ -82,6 +82,9 @@ scatter_status prepare_clusters(scatter_plan_s* p, const double* s_list, double 
 scatter_status launch_clusters(scatter_plan_t p, float2* amp_out, float* int_out, cudaStream_t st);
 void release_clusters(scatter_plan_s* p);
 ClArgs cluster_args(scatter_plan_s* p);
+// Of one term, for crystals within `radius`: the neglected columns, and the roundings of
+// the columns' powers and sums.
+void cluster_error(const scatter_plan_s* p, double radius, double* truncation, double* rounding);
 // Their adjoint (cluster_adjoint.cu): Sum_S S Im(gF e) per slot into
 // [split][n_slots][3] from gF [species][M].
 scatter_status prepare_cluster_adjoint(scatter_plan_s* p);
@@ -104,6 +107,9 @@ scatter_status prepare_coarse(scatter_plan_s* p, const scatter_problem* pr, cons
 scatter_status launch_coarse(scatter_plan_t p, const double* xyz, const float* occ, float2* amp_out, float* int_out,
                              cudaStream_t st);
 void release_coarse(scatter_plan_s* p);
+// Of one term, for crystals within `radius`: the interpolation's own error, its
+// roundings, and the factor by which it can amplify errors at the nodes.
+void coarse_error(const scatter_plan_s* p, double radius, double* truncation, double* rounding, double* amplify);
 // The adjoint from the weights gF [species][M] contracted to the nodes.
 scatter_status prepare_coarse_adjoint(scatter_plan_s* p);
 scatter_status launch_coarse_adjoint(scatter_plan_t p, const float2* gf, float* grad, cudaStream_t st);

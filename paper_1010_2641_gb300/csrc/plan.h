@@ -139,9 +139,15 @@ struct ClAdjState {
   int n_blocks = 0, n_g = 0, split = 1, rows_per_chunk = 0, smem = 0;
   int emax[3] = {0, 0, 0};
 };
+// A clustered instance's radius and its clusters' largest corner phases, for the
+// error bound.
+struct ClExtent {
+  double X, th[3];
+};
 struct ClState {
   bool active = false;
   ClAdjState adj;
+  std::vector<ClExtent> extents;
   ClInst first;                     // the only instance, with its columns and its clusters' points
   std::vector<int32_t> h_exps;
   std::vector<int64_t> h_row;
@@ -192,6 +198,7 @@ struct CoarseStage {
 constexpr int kCoarseLevels = 2;
 struct CoarseState {
   scatter_plan_s* sub = nullptr;    // the sum at the nodes, without the translation phase
+  double X = 0.0;                   // |x'_d| that they resolve
   CoarseStage stage[3];
   int n_stages = 0;
   float2* map = nullptr;            // at the nodes
