@@ -445,6 +445,9 @@ scatter_status prepare_clusters(scatter_plan_s* p, const double* s_list, double 
     }
     const double compact = std::cbrt(3.0 * (double)N / (16.0 * 3.14159265358979323846));
     const double X = radius_hint > 0.0 ? radius_hint : 1.45 * compact + 1.0;
+    // a hint whose square is no float: a crystal of one point would be within it, and no
+    // column matter
+    if (!((float)(X * X) > 0.0f)) continue;
     // phases s.x' below the bound past which the direct kernels take exact products
     if (0.5 + (p->s_max[0] + p->s_max[1] + p->s_max[2]) * (X + 1.0) > 100.0) continue;
     // candidates for the cell side (corner phase th0) by the model, in clocks of
