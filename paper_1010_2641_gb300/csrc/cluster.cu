@@ -39,7 +39,6 @@
 
 namespace scatter {
 
-constexpr double kClEps = 2e-6;   // columns with a largest term below this are left out
 constexpr int kClCols = 16;       // columns per thread of the moments kernel
 constexpr int kClRows = 64;       // clusters per CTA (one per thread)
 constexpr int kClTile = 64;       // atoms per stage

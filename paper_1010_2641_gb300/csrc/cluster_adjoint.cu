@@ -332,6 +332,34 @@ scatter_status prepare_cluster_adjoint(scatter_plan_s* p) {
     upv[c] = make_short4(u[0], u[1], u[2], 0);
     dnv[c] = make_short4(v[0], v[1], v[2], 0);
   }
+  // A column of degree n and largest term t counts for the sum from the radius at which
+  // t r^n passes kClEps, and for a derivative from n t r^(n - 1) = kClEps of the whole
+  // phase gradient, 2 pi X |H| and the corner's own: of a crystal that is a point the first
+  // degree is left (dropped, the gradient kept |S| at the clusters' centres: 3e-2 off).
+  // The columns in use are the first ones, so each takes the least radius behind it.
+  const ClExtent& ext = cl.extents[0];
+  const double* H = p->inst[0].H;
+  const double corner = std::sqrt(ext.th[0] * ext.th[0] + ext.th[1] * ext.th[1] + ext.th[2] * ext.th[2]);
+  const double scale = std::max(corner, 6.283185307179586 * ext.X * std::sqrt(H[0] * H[0] + H[1] * H[1] + H[2] * H[2]));
+  std::vector<float> rho(K);
+  for (int c = K - 1; c >= 0; --c) {
+    int n = 0;
+    double t = 0.0;
+    for (int d = 0; d < 3; ++d) {
+      const int x = (cl.h_exps[c] >> (4 * d)) & 15;
+      n += x;
+      if (x) t += x * (std::log(std::max(ext.th[d], 1e-12)) + 0.5 * std::log((double)x)) - std::lgamma(x + 1.0);
+    }
+    double r = -1.0;
+    if (n > 0) {
+      t -= 0.5 * n * std::log((double)n);
+      const double own = (std::log(kClEps) - t) / n, der = std::log(kClEps * scale / n) - t;
+      r = std::exp(n > 1 ? std::min(own, der / (n - 1)) : own);
+      if (n == 1 && der < 0.0) r = -1.0;
+    }
+    rho[c] = (float)r;
+    if (c + 1 < K) rho[c] = std::min(rho[c], rho[c + 1]);
+  }
   std::vector<ClGBlock> gb;
   std::vector<int32_t> row_blk(rows + 1);
   for (int r = 0; r < rows; ++r) {
@@ -367,7 +395,7 @@ scatter_status prepare_cluster_adjoint(scatter_plan_s* p) {
     }
   }
   const bool ok = up_host(&s.up, upv) && up_host(&s.down, dnv) && up_host(&s.g_blocks, gb) &&
-                  up_host(&s.row_blk, row_blk) && up_host(&s.blocks, blocks) &&
+                  up_host(&s.row_blk, row_blk) && up_host(&s.blocks, blocks) && up_host(&s.rho, rho) &&
                   cudaMalloc(&s.g_part, (size_t)part * sizeof(float2)) == cudaSuccess &&
                   cudaMalloc(&s.g8, (size_t)g8 * sizeof(float)) == cudaSuccess;
   if (!ok) {  // no room: the direct kernel needs none of it
@@ -377,7 +405,7 @@ scatter_status prepare_cluster_adjoint(scatter_plan_s* p) {
   }
   s.n_blocks = (int)blocks.size();
   s.n_g = (int)gb.size();
-  p->base_bytes += part * 8 + g8 * 4 + (int64_t)(K * 16 + gb.size() * sizeof(ClGBlock) + rows * 4 + blocks.size() * sizeof(AdjBlock));
+  p->base_bytes += part * 8 + g8 * 4 + (int64_t)(K * 20 + gb.size() * sizeof(ClGBlock) + rows * 4 + blocks.size() * sizeof(AdjBlock));
   s.active = true;
   return SCATTER_OK;
 }
@@ -386,6 +414,7 @@ scatter_status launch_cluster_adjoint(scatter_plan_t p, const float2* gf, float*
   const ClAdjState& s = p->cl.adj;
   ClAdjArgs a{};
   a.c = cluster_args(p);
+  a.c.rho = s.rho;
   a.gf = gf;
   a.g_blocks = s.g_blocks;
   a.row_blk = s.row_blk;
@@ -407,8 +436,8 @@ scatter_status launch_cluster_adjoint(scatter_plan_t p, const float2* gf, float*
 }
 
 void release_cluster_adjoint(ClAdjState& s) {
-  for (void* b : {(void*)s.blocks, (void*)s.g_blocks, (void*)s.row_blk, (void*)s.up, (void*)s.down, (void*)s.g_part,
-                  (void*)s.g8})
+  for (void* b : {(void*)s.blocks, (void*)s.g_blocks, (void*)s.row_blk, (void*)s.up, (void*)s.down, (void*)s.rho,
+                  (void*)s.g_part, (void*)s.g8})
     if (b) cudaFree(b);
   s = ClAdjState{};
 }

@@ -5,6 +5,7 @@
 
 namespace scatter {
 
+constexpr double kClEps = 2e-6;   // columns with a largest term below this are left out
 constexpr int kClMaxK = 320;      // columns of an instance
 constexpr int kClMaxExp = 15;     // largest exponent of an axis
 

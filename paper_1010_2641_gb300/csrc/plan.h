@@ -134,6 +134,7 @@ struct ClAdjState {
   int32_t* row_blk = nullptr;       // [rows + 1] the first g_block of each cluster
   short4* up = nullptr;             // per column: columns of a + e_d, -1: none
   short4* down = nullptr;           //             columns of a - e_d
+  float* rho = nullptr;             // per column: the relative radius from which it or its derivative matters
   float2* g_part = nullptr;         // [g_block][species][column]
   float* g8 = nullptr;              // [species][cluster][column][8]
   int n_blocks = 0, n_g = 0, split = 1, rows_per_chunk = 0, smem = 0;
