@@ -15,8 +15,8 @@
 // k_adjoint       atom-parallel (the paper's alternative decomposition,
 //                 Section 2.2): each thread holds RA atoms in registers, S
 //                 tiles are staged in shared memory by the TMA engine; inner
-//                 sums per tile in FP32, outer sums in FP64 (the terms over
-//                 millions of S nearly cancel).  The exponentials are
+//                 sums per tile in FP32, outer sums in double-float FP32 (the
+//                 terms over millions of S nearly cancel).  The exponentials are
 //                 recomputed, nothing of size N x M is stored.
 //                 Lists of close points: cluster_adjoint.cu in its place;
 //                 grids where it is cheaper: grid_adjoint.cu.
@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_adjoint_line(const AdjLineAr
       const u64 one2 = dev::pack2(1.f, 1.f), zero2 = 0ull;
       const float4* sv4 = sh_s[st];
       for (int jb = 0; jb < cnt; jb += kReseed) {
-        // exact exponential at the first point of every 64
+        // exact exponential at the first point of every kReseed
         const float qz = sv4[jb].x;
 #pragma unroll
         for (int r = 0; r < kAdjRA; ++r)

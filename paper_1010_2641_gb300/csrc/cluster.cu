@@ -537,7 +537,7 @@ scatter_status prepare_clusters(scatter_plan_s* p, const double* s_list, double 
     std::sort(cols.begin(), cols.end(), [](const Column& x, const Column& y) {
       return x.rho != y.rho ? x.rho < y.rho : std::lexicographical_compare(x.e, x.e + 3, y.e, y.e + 3);
     });
-    // chunks of one species: at most 512 atoms, fewer where the SMs would idle
+    // chunks of one species: at most 256 atoms, fewer where the SMs would idle
     const int row_tiles = (rows + kClRows - 1) / kClRows, col_tiles = ((int)cols.size() + kClCols - 1) / kClCols;
     int64_t len = 256;
     while (len > 64 && (double)row_tiles * std::max(1, col_tiles * 2 / 3) * std::ceil((double)slots / (double)len) * B <

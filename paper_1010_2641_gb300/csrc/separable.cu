@@ -19,21 +19,23 @@
 // k_sep: CTA = a pair of 128-row M tiles (two 128 x 256 FP32
 // accumulators filling the 512 TMEM columns) x one 256-point N tile x one
 // atom chunk; per 16-atom step the TMA engine copies the pair's A blocks
-// and the step's 16 atom records (y', z', c), every thread computes its
-// point's row of B from them (FP32 phase, exact reduction mod 1, MUFU
+// and the step's 16 atom records (y', z', c), two threads per point compute its
+// row of B from them (FP32 phase, exact reduction mod 1, MUFU
 // sincos, f16 split) into shared memory once for both tiles, and one
 // thread issues 12 tcgen05.mma (2 tiles x 2 K16 sub-steps x 3 products,
-// M=128 N=256).  Warp roles: eight warps form B (and read the accumulators
+// M=128 N=256).  Warp roles: sixteen warps form B (and read the accumulators
 // out), one warp issues the MMAs, one warp issues the copies (a 32 KB bulk
 // copy holds its issuing thread for ~1000 cycles, so it must not be the MMA
-// thread).  A four-stage ring for the A blocks, an eight-stage ring for the
+// thread).  A ring for the A blocks (four stages, eight where the CTA has one
+// M tile), an eight-stage ring for the
 // atom records and a two-stage ring for the B blocks, each stage with a
 // full and an empty mbarrier, keep the formation of step k+1 and the copies
 // of later steps overlapped with the MMAs of step k.  The MMAs read ~96 B/clk of shared memory on their own;
 // computing B from the atom records, instead of loading tabulated factors
 // through L1, keeps the rest of the shared-memory traffic to the A copies
 // and the B stores.
-// Atom chunks (grid y) hold one species each.  Every 256 steps and at the
+// Atom chunks (grid y) hold one species each.  Every kSepFlush steps (folded:
+// the form's own interval) and at the
 // end of the chunk the accumulator is read from TMEM (tcgen05.ld) and added
 // into FP32 partials owned by the CTA, in the accumulator's 32 x 32 blocks
 // (sep_part_off; shorter groups keep the
