@@ -203,7 +203,13 @@ typedef struct scatter_options {
                                 resolve it, interpolated) and lists of close
                                 points (clusters): a call measures its crystal,
                                 and one past the bound is summed point by point
-                                at the direct sum's speed                     */
+                                at the direct sum's speed.  0 takes, for R =
+                                (3 n_atoms / 16 pi)^(1/3), largest |x'_d| up to
+                                1.3 R + 1 on grids (grazing incidence, in the
+                                plane: 2.3 R + 1) and |x'| up to 1.45 R + 1 on
+                                lists: wires, films, simple cubic spheres and
+                                parts of a larger crystal (sharded atoms) need
+                                a hint                                        */
 } scatter_options;
 
 typedef struct scatter_plan_s* scatter_plan_t;
@@ -300,7 +306,11 @@ scatter_status scatter_amplitude_host(scatter_plan_t plan, const double* xyz,
 /*
  * scatter_intensity — I(S) = |A(S)|^2 (the quantity of the paper's maps,
  * Section 2.3).  Same inputs as scatter_amplitude; I_out is device float32
- * [n_s].  A is formed in the plan's workspace.
+ * [n_s].  A is formed in the plan's workspace.  On SEPARABLE plans intensities
+ * are summed at every point, while amplitudes may come from a grid folded over
+ * its middle or from nodes: the two calls then agree within the path's error (up
+ * to ~2.5e-5 of the map), not bit for bit, and squaring an amplitude map is the
+ * faster way to one's intensities.
  */
 scatter_status scatter_intensity(scatter_plan_t plan, const double* xyz,
                                  const float* occ, float* I_out, void* stream);

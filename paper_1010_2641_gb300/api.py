@@ -66,6 +66,9 @@ class Plan:
         enough and its error model (with a measured margin) meets `tolerance`
         (relative L2 of the map, 0 = 1e-4) for crystals of `radius_hint`
         lattice units around their centre (0 = compact); otherwise generic.
+    radius_hint : also the extent up to which oversampled grids are summed at
+        nodes and lists of close points over clusters (0 = compact, with margins);
+        crystals past it take the direct sum.
     """
 
     def __init__(self, coef, lattice_a: float, n_atoms: int, *, s_list=None, axes: Sequence | None = None,
@@ -216,6 +219,8 @@ class Plan:
         return out
 
     def intensity(self, xyz, occ=None, out=None, stream=None) -> torch.Tensor:
+        """|A(S)|^2.  On the separable path it is summed at every point and agrees with
+        the square of amplitude() within the path's error, not bit for bit."""
         xyz, occ = self._xyz(xyz), self._occ(occ)
         if out is None:
             out = torch.empty(self.n_s, dtype=torch.float32, device=xyz.device)

@@ -21,7 +21,7 @@
 //   k_cl_adj   256 atoms x a range of clusters, four clusters at a time
 // A crystal past the clusters' radius is left to k_adjoint, whose launch
 // otherwise returns at once.
-// 28,953 atoms x 100,003 points of a detector patch (64 clusters): 0.13 ms per
+// 28,953 atoms x 100,003 points of a detector patch (64 clusters): 0.13-0.16 ms per
 // call against 1.47 ms; relative error against FP64 1.8e-7 against 2.6e-7.
 #include <cuda_runtime.h>
 #include <algorithm>

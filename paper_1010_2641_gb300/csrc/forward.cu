@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(256) k_prep(const PrepArgs a, const int32_t* _
 // One instance, one launch after the boxes: every CTA joins the n_part partial
 // boxes (n_part = 0: takes the box of all the atoms itself, for small
 // crystals), then prepares its share of the slots.  1e6 atoms: 9.6 us for
-// the boxes and ~35 us here, from 63 + 76 us and an initialising launch when
+// the boxes and ~20 us here, from 63 + 76 us and an initialising launch when
 // the comparisons and the split ran in FP64; 4 CTAs per SM, each joining 256
 // boxes, measured 5 us less than 8 joining 512.
 __global__ void __launch_bounds__(256) k_prep_one(const PrepArgs a, int64_t n_atoms, int64_t n_slots,

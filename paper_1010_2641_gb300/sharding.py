@@ -97,7 +97,11 @@ class AtomShardedPlan:
     reflection; each rank centres its own atoms).  amplitude() returns the
     full A on every rank (one all-reduce); backward() returns the misfit L
     (the same on every rank) and dL/dr of this rank's atoms, computed from
-    the full A with no further exchange."""
+    the full A with no further exchange.
+
+    A rank's part reaches further than a compact crystal of its atom count: pass
+    `radius_hint`, the whole crystal's radius, where oversampled maps or lists of
+    close points should be summed at nodes or over clusters."""
 
     def __init__(self, coef, lattice_a: float, n_atoms: int, *, world: int, rank: int, atom_species=None,
                  group=None, **plan_kw):
