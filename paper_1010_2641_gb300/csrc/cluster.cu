@@ -669,7 +669,7 @@ void cluster_error(const scatter_plan_s* p, double radius, double* truncation, d
     // The sum is largest just before a column joins, or at r.
     constexpr int kTop = 40;
     struct Term {
-      double t, rho;
+      double value, rho;  // over the whole ball
       int n;
     };
     std::vector<Term> terms;
@@ -685,16 +685,17 @@ void cluster_error(const scatter_plan_s* p, double radius, double* truncation, d
           const int n = a + b + c;
           if (n == 0) continue;
           const double t = ax[0][a] + ax[1][b] + ax[2][c] - 0.5 * n * std::log((double)n);
-          if (t > -27.6) terms.push_back({t, std::exp((std::log(kClEps) - t) / n), n});
+          if (t > -27.6) terms.push_back({std::exp(t), std::exp((std::log(kClEps) - t) / n), n});
         }
     const double len = std::sqrt(e.th[0] * e.th[0] + e.th[1] * e.th[1] + e.th[2] * e.th[2]);
     auto neglected = [&](double q) {
-      double by[kTop + 1] = {0.0}, sum = 0.0, all = 1.0;
+      double by[kTop + 1] = {0.0}, sum = 0.0, all = 1.0, power = 1.0;
       for (const Term& m : terms)
-        if (m.rho >= q) by[m.n] += std::exp(m.t + m.n * std::log(q));
+        if (m.rho >= q) by[m.n] += m.value;
       for (int n = 1; n <= kTop; ++n) {
         all *= len * q / n;
-        sum += std::min(by[n], all);
+        power *= q;
+        sum += std::min(by[n] * power, all);
       }
       return sum;
     };
